@@ -101,6 +101,7 @@ struct nbody_ctx {
     double *stage = nullptr;  // 6 n doubles: external forces / AoS staging
     void *partials = nullptr;
     size_t partials_cap = 0;
+    void *sym_buf = nullptr;  // scratch of the force by unordered pairs (sym_scratch_bytes), on first use
     void *sched_scratch = nullptr;
     SchedOut *sched_out = nullptr;
     DevStatus *st = nullptr;
@@ -145,7 +146,7 @@ void release(nbody_ctx *c)
     if (c->step_graph) cudaGraphExecDestroy(c->step_graph);
     void *dev[] = {c->state, c->t, c->level, c->jbuf, c->act_force, c->act_corr, c->act_sched,
                    c->f_acc, c->f_jerk, c->f_pot, c->stage, c->partials, c->sched_scratch,
-                   c->sched_out, c->st, c->phi, c->e_out, c->trange, c->graph_fits, c->loop_dev, c->grid_buf};
+                   c->sched_out, c->st, c->phi, c->e_out, c->trange, c->graph_fits, c->loop_dev, c->grid_buf, c->sym_buf};
     for (void *d : dev)
         if (d) cudaFree(d);
     void *host[] = {c->sched_host, c->st_host, c->e_host, c->trange_host, c->loop_host};
@@ -221,22 +222,63 @@ int ensure_partials(nbody_ctx *c, size_t bytes)
     return NBODY_OK;
 }
 
+// Scratch of the force by unordered pairs (cfg), or false where the device has no room for it.
+bool sym_room(nbody_ctx *c, const ForceConfig &cfg, int64_t n_act)
+{
+    if (!c->sym_buf && dev_alloc(&c->sym_buf, sym_scratch_bytes(c->n)) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return ensure_partials(c, force_partial_bytes(c->p.mode, cfg, n_act)) == NBODY_OK;
+}
+
 // Force on a device list already in act_force.  With for_step, a shape whose
 // partials the corrector adds (force_partials_fused) skips the reduction;
-// fused_split then tells correct_internal to read them.
-int force_internal(nbody_ctx *c, int64_t n_act, bool for_step = false)
+// fused_split then tells correct_internal to read them.  `ascending`: the list
+// is the library's own (a schedule's, or all particles), so its particles are
+// distinct; a caller's list is checked on the device, and one that repeats a
+// particle takes the one-sided kernels.
+int force_internal(nbody_ctx *c, int64_t n_act, bool for_step = false, bool ascending = true)
 {
+    auto choose = [&](ForceConfig *cfg, bool pairs) {
+        return force_choose(c->p.mode, n_act, c->n_pad, c->sm_count, c->p.j_tile, c->p.i_block, c->p.j_split, cfg,
+                            c->p.j_sub, pairs && c->J.soa ? c->n : 0);
+    };
     ForceConfig cfg{};
-    const int r = force_choose(c->p.mode, n_act, c->n_pad, c->sm_count, c->p.j_tile, c->p.i_block, c->p.j_split,
-                               &cfg, c->p.j_sub);
+    int r = choose(&cfg, true);
+    if (r == NBODY_OK && cfg.sym_sb > 0 && !sym_room(c, cfg, n_act)) r = choose(&cfg, false);
     if (r != NBODY_OK) return fail(r, "unsupported force shape: %d threads x %d i per thread", c->p.j_tile, c->p.i_block);
-    const int rp = ensure_partials(c, force_partial_bytes(c->p.mode, cfg, n_act));
-    if (rp != NBODY_OK) return rp;
     int64_t launches = 0;
-    const bool fused = for_step && force_partials_fused(c->p.mode, cfg);
-    NB_CUDA(force_launch(c->p.mode, c->J, c->n, c->act_force, n_act, c->eps2, cfg,
-                         c->f_acc, c->f_jerk, c->f_pot, c->partials, c->st, c->s, &launches, nullptr, !fused),
-            "force kernel launch");
+    bool fused = false;
+    if (cfg.sym_sb > 0) {
+        const long long *rows_general = nullptr;
+        ForceConfig general{};
+        if (!ascending) {
+            r = choose(&general, false);
+            if (r != NBODY_OK) return r;
+            r = ensure_partials(c, force_partial_bytes(c->p.mode, general, n_act));
+            if (r != NBODY_OK) return r;
+        }
+        NB_CUDA(force_sym_launch(c->p.mode, c->J, c->n, c->act_force, n_act, c->eps2, cfg, ascending, c->f_acc,
+                                 c->f_jerk, c->f_pot, c->partials, c->sym_buf, &rows_general, c->st, c->s, &launches),
+                "force kernel launch");
+        if (rows_general) {  // (nothing to do for a list of distinct particles: ~5 us)
+            NB_CUDA(force_launch(c->p.mode, c->J, c->n, c->act_force, n_act, c->eps2, general, c->f_acc, c->f_jerk,
+                                 c->f_pot, c->partials, c->st, c->s, &launches, rows_general, false),
+                    "force kernel launch");
+            if (general.split > 1)
+                NB_CUDA(force_sym_reduce_launch(c->p.mode, static_cast<float *>(c->partials), general.split, n_act,
+                                                c->f_acc, c->f_jerk, c->f_pot, rows_general, true, c->s, &launches),
+                        "force kernel launch");
+        }
+    } else {
+        r = ensure_partials(c, force_partial_bytes(c->p.mode, cfg, n_act));
+        if (r != NBODY_OK) return r;
+        fused = for_step && force_partials_fused(c->p.mode, cfg);
+        NB_CUDA(force_launch(c->p.mode, c->J, c->n, c->act_force, n_act, c->eps2, cfg,
+                             c->f_acc, c->f_jerk, c->f_pot, c->partials, c->st, c->s, &launches, nullptr, !fused),
+                "force kernel launch");
+    }
     c->fused_split = fused ? cfg.split : 0;
     c->stats.kernel_launches += launches;
     c->stats.force_calls += 1;
@@ -683,7 +725,7 @@ int nbody_force(nbody_ctx *c, const int32_t *active, int64_t n_act, double *acc,
     if (!c->pred_valid) return fail(NBODY_ESTATE, "nbody_force: no prediction since the last correction");
     const size_t na = static_cast<size_t>(n_act);
     NB_CUDA(to_device(c->act_force, active, na * sizeof(int32_t), c->s), "active list upload");
-    int r = force_internal(c, n_act);
+    int r = force_internal(c, n_act, false, false);
     if (r != NBODY_OK) return r;
     bool host_out = false;
     if (acc) {

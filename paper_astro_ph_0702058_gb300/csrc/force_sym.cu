@@ -1,0 +1,294 @@
+// Launch of the force by unordered pairs (kernel in force_sym.cuh): when a block
+// takes it, how it is cut, the rows and the particles outside the block as
+// contiguous arrays, and the sum over the slots.
+#include <cmath>
+
+#include "force_sym.cuh"
+
+namespace nb {
+
+namespace {
+
+constexpr int kSymMaxSb = 128;             // superblocks
+constexpr int64_t kSymMinRows = 8192;      // rows from which a block may take pairs
+constexpr int64_t kSymPartCap = int64_t(8) << 30;  // bytes of its slots
+constexpr int kSymThreads = 256;
+constexpr int kSymScan = 4 * kSymThreads;  // particles of a block of the compaction
+
+// Resident warps per SM, and the unroll factor of the pair loop: at n = 262144
+// 12 warps (168 registers) x 4 against 16 (128) x 2 took 44.2 against 45.2 ms in
+// plain mode, 55.2 against 54.4 in compensated mode (128 registers spill there,
+// yet the fourth warp of a scheduler gains more); one-warp CTAs (n <= 32768)
+// are faster with 12 x 4 in both.
+template <int MODE, int W>
+struct SymShape {
+    static constexpr bool wide = MODE == kModeComp && W > 1;
+    static constexpr int unroll = wide ? 2 : 4, warps = wide ? 16 : 12;
+};
+
+template <int MODE, int W>
+cudaError_t sym_launch(const SymParams &P, const ForceConfig &cfg, cudaStream_t s)
+{
+    using Sh = SymShape<MODE, W>;
+    const int units = cfg.sym_sb * (cfg.sym_sb + 1) / 2 + cfg.sym_sb * cfg.sym_ranges;
+    force_sym_kernel<MODE, W, Sh::unroll, Sh::warps><<<units, 32 * W, 0, s>>>(P);
+    return cudaGetLastError();
+}
+
+// Row q <- particle list[q] (a list with an index outside [0, n) or with a
+// particle twice sets *rows_general to n_act); marks the block's particles.
+__global__ void __launch_bounds__(kSymThreads)
+    sym_gather_kernel(const float *__restrict__ soa, const long long stride, const int arrays,
+                      const int32_t *__restrict__ list, const int n_act, const int n, float *__restrict__ rows,
+                      const long long rows_stride, int *__restrict__ mark, long long *rows_general, DevStatus *st)
+{
+    const int q = blockIdx.x * kSymThreads + threadIdx.x;
+    if (q >= n_act) return;
+    const int idx = list[q];
+    if (idx < 0 || idx >= n) {
+        atomicOr(&st->flags, static_cast<unsigned>(kFlagBadIndex));
+        st->bad_index = q;
+        *rows_general = n_act;
+        return;
+    }
+    if (atomicExch(mark + idx, 1) != 0) *rows_general = n_act;
+    for (int a = 0; a < arrays; ++a) rows[a * rows_stride + q] = soa[a * stride + idx];
+}
+
+// counts[b] <- particles of block b's kSymScan that are not marked.
+__global__ void __launch_bounds__(kSymThreads) sym_count_kernel(const int *__restrict__ mark, const int n, int *counts)
+{
+    __shared__ int sh[kSymThreads / 32];
+    int k = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const int i = blockIdx.x * kSymScan + e * kSymThreads + threadIdx.x;
+        k += i < n && mark[i] == 0;
+    }
+    k = __reduce_add_sync(0xffffffffu, k);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = k;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int t = 0;
+        for (int w = 0; w < kSymThreads / 32; ++w) t += sh[w];
+        counts[blockIdx.x] = t;
+    }
+}
+
+// The particles that are not marked, ascending, as contiguous arrays of at most n_out.
+__global__ void __launch_bounds__(kSymThreads)
+    sym_compact_kernel(const float *__restrict__ soa, const long long stride, const int arrays,
+                       const int *__restrict__ mark, const int n, const int *__restrict__ counts,
+                       float *__restrict__ out, const long long out_stride, const int n_out)
+{
+    __shared__ int sh[kSymThreads / 32];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    int before = 0;  // particles of the blocks before this one
+    for (int b = t; b < static_cast<int>(blockIdx.x); b += kSymThreads) before += counts[b];
+    before = __reduce_add_sync(0xffffffffu, before);
+    if (lane == 0) sh[w] = before;
+    __syncthreads();
+    int base = 0;
+    for (int k = 0; k < kSymThreads / 32; ++k) base += sh[k];
+    for (int e = 0; e < 4; ++e) {
+        const int i = blockIdx.x * kSymScan + e * kSymThreads + t;
+        const bool hit = i < n && mark[i] == 0;
+        const unsigned m = __ballot_sync(0xffffffffu, hit);
+        __syncthreads();
+        if (lane == 0) sh[w] = __popc(m);
+        __syncthreads();
+        int pos = base + __popc(m & ((1u << lane) - 1u));
+        for (int k = 0; k < kSymThreads / 32; ++k) {
+            if (k < w) pos += sh[k];
+            base += sh[k];
+        }
+        if (hit && pos < n_out)  // (a list with a particle twice leaves more)
+            for (int a = 0; a < arrays; ++a) out[a * out_stride + pos] = soa[a * stride + i];
+    }
+}
+
+// The sums of a row over the slots, in slot order: one thread per row and
+// component, reads coalesced over the rows; double-single on the FP32 pipe.
+template <int MODE>
+__global__ void __launch_bounds__(256)
+    force_sym_reduce_kernel(const float *__restrict__ part, const int slots, const int n, double *__restrict__ acc,
+                            double *__restrict__ jerk, double *__restrict__ pot, const long long *rows_general,
+                            const bool general)
+{
+    constexpr int NC = MODE == kModeComp ? 14 : 7;
+    if (rows_general && (*rows_general != 0) != general) return;  // the other path's rows
+    const int q = blockIdx.x * 256 + threadIdx.x;
+    const int c = blockIdx.y;
+    if (q >= n) return;
+    float h = 0.0f, l = 0.0f;
+#pragma unroll 8
+    for (int s = 0; s < slots; ++s) {
+        const float *b = part + (static_cast<size_t>(s) * NC + c) * n + q;
+        ds2_add(h, l, b[0], MODE == kModeComp ? b[static_cast<size_t>(7) * n] : 0.0f);
+    }
+    const double t = static_cast<double>(h) + static_cast<double>(l);
+    if (c < 3)
+        acc[3 * static_cast<size_t>(q) + c] = t;
+    else if (c < 6)
+        jerk[3 * static_cast<size_t>(q) + c - 3] = t;
+    else
+        pot[q] = t;
+}
+
+// Scratch of a context: the general path's row count, the marks, the
+// compaction's counts, then the rows and the other particles (together n).
+struct SymScratch {
+    long long *rows_general;
+    int *mark, *counts;
+    float *rows;
+};
+int64_t up4(const int64_t n) { return (n + 3) / 4 * 4; }
+SymScratch sym_scratch(void *p, const int64_t n)
+{
+    SymScratch S;
+    char *b = static_cast<char *>(p);
+    S.rows_general = reinterpret_cast<long long *>(b);
+    S.mark = reinterpret_cast<int *>(b + 16);
+    S.counts = S.mark + up4(n);
+    S.rows = reinterpret_cast<float *>(S.counts + up4(n / kSymScan + 1));
+    return S;
+}
+
+}  // namespace
+
+size_t sym_scratch_bytes(int64_t n)
+{
+    return 16 + sizeof(int) * (up4(n) + up4(n / kSymScan + 1)) + sizeof(float) * kSoaArrays * (n + 8);
+}
+
+// A block takes pairs from 8192 rows on (full forces at n = 8192, 4096 measured 1.23
+// and 1.0 times the one-sided kernel's rate), when it holds enough of the particles:
+// only pairs within the block are shared, and the one-sided units run at 0.88 of
+// force_kernel_x2's rate (four rows per lane, 12 warps).  Measured, one-sided
+// kernel -> pairs, us: compensated 33536 of 65536 rows 2270 -> 2193, 22000: 1512 ->
+// 1500, 16384: 1142 -> 1140, 40001 of 100003: 4035 -> 4091; plain 40001 of 100003
+// 3396 -> 3242.  So half of the particles compensated, three eighths plain.
+// Superblocks are as small as 128 of them allow, for many units (8256 against 2080
+// of twice the size: 4-5 % at n = 65536 and 262144), up to 8 GiB of slots (2^20
+// compensated: 889 ms with 7.6 GB, 920 with 4.3); CTAs of one warp up to 32768
+// rows, of four above (n = 16384: 194 against 240 us plain; 65536: 2894 against 2804).
+bool sym_plan(int mode, int64_t n_act, int64_t n, int sm_count, ForceConfig *cfg)
+{
+    if (!NB_PACKED || (mode != kModePlain && mode != kModeComp)) return false;
+    if (n_act < kSymMinRows || n_act > n || (mode == kModeComp ? 2 : 8.0 / 3.0) * n_act < n) return false;
+    const int nc = two_word_sums(mode) ? 14 : 7;
+    const int W = n_act <= 32768 ? 1 : 4;
+    const int64_t bt = static_cast<int64_t>(W) * kSymRows;
+    const int64_t n_out = n - n_act;
+    const int64_t slot_bytes = static_cast<int64_t>(nc) * n_act * sizeof(float);
+    const int res = (mode == kModeComp && W > 1 ? 16 : 12) / W;  // resident CTAs per SM (SymShape)
+    const int64_t slots = static_cast<int64_t>(res) * sm_count;
+    const int64_t t_min = (n_act + bt * kSymMaxSb - 1) / (bt * kSymMaxSb);
+    bool found = false;
+    double best = 0.0;
+    for (int64_t tiles = t_min; !found || tiles <= t_min + t_min / 4; ++tiles) {
+        const int64_t sb = (n_act + bt * tiles - 1) / (bt * tiles);
+        // outside ranges: about two units for every resident CTA
+        int64_t ranges = 0, len = 0;
+        if (n_out > 0) {
+            const int64_t want = (2 * slots + sb - 1) / sb;
+            len = ((n_out + want - 1) / want + bt - 1) / bt * bt;
+            ranges = (n_out + len - 1) / len;
+        }
+        const int64_t units = sb * (sb + 1) / 2;
+        if (units + sb * ranges < slots) break;  // too few units
+        if ((sb + 1 + ranges) * slot_bytes > kSymPartCap) continue;
+        // the last, partly filled wave: an SM that holds k of res CTAs works at
+        // about 0.6, 0.87 and 0.97 of its rate with 1/4, 1/2 and 3/4 of them
+        const double waves = static_cast<double>(units) / slots, whole = std::floor(waves);
+        const double fill = waves - whole;
+        const double last = fill == 0.0 ? 0.0 : fill <= 0.25 ? 0.42 : fill <= 0.5 ? 0.57 : fill <= 0.75 ? 0.77 : 1.0;
+        const double cost = (whole + last) * static_cast<double>(tiles) * tiles;
+        if (found && cost >= 0.99 * best) continue;
+        found = true;
+        best = cost;
+        cfg->threads = 32 * W;
+        cfg->ipt = 4;
+        cfg->jsub = 1;
+        cfg->slice = 0;
+        cfg->n_iblk = static_cast<int>(sb);
+        cfg->split = static_cast<int>(sb + 1 + ranges);
+        cfg->tiles_per_split = static_cast<int>(tiles);
+        cfg->sym_sb = static_cast<int>(sb);
+        cfg->sym_ranges = static_cast<int>(ranges);
+        cfg->sym_out_len = static_cast<int>(len);
+    }
+    return found;
+}
+
+cudaError_t force_sym_launch(int mode, const JStream &js, int64_t n, const int32_t *active, int64_t n_act,
+                             double eps2, const ForceConfig &cfg, bool ascending, double *acc, double *jerk,
+                             double *pot, void *partials, void *scratch, const long long **rows_general,
+                             DevStatus *st, cudaStream_t s, int64_t *launches)
+{
+    const SymScratch X = sym_scratch(scratch, n);
+    const int na = static_cast<int>(n_act), nn = static_cast<int>(n), n_out = nn - na;
+    const int arrays = mode == kModeComp ? 10 : 7;
+    SymParams P{};
+    P.n = na;
+    P.n_sb = cfg.sym_sb;
+    P.tiles = cfg.tiles_per_split;
+    P.n_out = n_out;
+    P.out_len = cfg.sym_out_len;
+    P.eps2 = static_cast<float>(eps2);
+    P.part = static_cast<float *>(partials);
+    P.soa = js.soa;
+    P.stride = js.n_pad;
+    P.st = st;
+    *rows_general = nullptr;
+    if (!ascending || n_out > 0) {
+        cudaError_t e = cudaMemsetAsync(scratch, 0, 16 + sizeof(int) * up4(n), s);
+        if (e != cudaSuccess) return e;
+        P.soa = X.rows;
+        P.stride = up4(n_act);
+        sym_gather_kernel<<<(na + kSymThreads - 1) / kSymThreads, kSymThreads, 0, s>>>(
+            js.soa, js.n_pad, arrays, active, na, nn, X.rows, P.stride, X.mark, X.rows_general, st);
+        ++*launches;
+        if (!ascending) {
+            P.skip = X.rows_general;
+            *rows_general = X.rows_general;
+        }
+        if (n_out > 0) {
+            float *out = X.rows + kSoaArrays * P.stride;
+            P.out_soa = out;
+            P.out_stride = up4(n_out);
+            const int nb = (nn + kSymScan - 1) / kSymScan;
+            sym_count_kernel<<<nb, kSymThreads, 0, s>>>(X.mark, nn, X.counts);
+            sym_compact_kernel<<<nb, kSymThreads, 0, s>>>(js.soa, js.n_pad, arrays, X.mark, nn, X.counts, out,
+                                                          P.out_stride, n_out);
+            *launches += 2;
+        }
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    cudaError_t e;
+    if (mode == kModeComp)
+        e = cfg.threads == 32 ? sym_launch<kModeComp, 1>(P, cfg, s) : sym_launch<kModeComp, 4>(P, cfg, s);
+    else
+        e = cfg.threads == 32 ? sym_launch<kModePlain, 1>(P, cfg, s) : sym_launch<kModePlain, 4>(P, cfg, s);
+    if (e != cudaSuccess) return e;
+    ++*launches;
+    return force_sym_reduce_launch(mode, P.part, cfg.split, n_act, acc, jerk, pot, P.skip, false, s, launches);
+}
+
+cudaError_t force_sym_reduce_launch(int mode, const float *part, int slots, int64_t n_act, double *acc, double *jerk,
+                                    double *pot, const long long *rows_general, bool general, cudaStream_t s,
+                                    int64_t *launches)
+{
+    const int na = static_cast<int>(n_act);
+    const dim3 grid((na + 255) / 256, 7);
+    if (mode == kModeComp)
+        force_sym_reduce_kernel<kModeComp><<<grid, 256, 0, s>>>(part, slots, na, acc, jerk, pot, rows_general, general);
+    else
+        force_sym_reduce_kernel<kModePlain><<<grid, 256, 0, s>>>(part, slots, na, acc, jerk, pot, rows_general,
+                                                                 general);
+    ++*launches;
+    return cudaGetLastError();
+}
+
+}  // namespace nb

@@ -110,6 +110,10 @@ struct ForceConfig {
     int n_iblk;           // i-blocks (gridDim.x)
     int jsub = 1;         // threads per row, each taking 1/jsub of every tile (1 or 4)
     int slice = 0;        // 1: the slice shape (one CTA per SM, split = CTAs; force_slice.cuh)
+    int sym_sb = 0;       // > 0: by unordered pairs (force_sym.cuh): superblocks of tiles_per_split x threads x ipt
+                          // rows, split = slots
+    int sym_ranges = 0;   // ranges of the particles outside the block, of sym_out_len each
+    int sym_out_len = 0;
 };
 // The j-subgroup shape: 256 threads, 64 rows of 4 subgroups (packed plain and compensated modes).
 constexpr int kJSubThreads = 256;
@@ -123,8 +127,10 @@ extern int g_skip_first_copy;  // test hook: force kernels leave out their first
 // Picks the launch shape for n_act active particles against n_pad j.
 // req_* > 0 override the automatic choice.
 // req_jsub: 0 automatic, 1 one thread per row, 4 four (256 threads, one i each).
+// n_pairs: the particles the block belongs to when it may take the force by
+// unordered pairs (force_sym_launch), else 0.
 int force_choose(int mode, int64_t n_act, int64_t n_pad, int sm_count, int req_threads,
-                 int req_ipt, int req_split, ForceConfig *cfg, int req_jsub = 0);
+                 int req_ipt, int req_split, ForceConfig *cfg, int req_jsub = 0, int64_t n_pairs = 0);
 // Whether this mode's force kernels honour ForceParams::n_act_dev (the packed kernels).
 bool force_reads_device_rows(int mode);
 // Scratch bytes needed for partial sums when cfg.split > 1 (0 otherwise).
@@ -145,6 +151,25 @@ cudaError_t force_launch(int mode, const JStream &js, int64_t n, const int32_t *
 constexpr int kFusedSplitMax = 8;
 // Whether a block step of this mode and shape hands its partials to the corrector.
 bool force_partials_fused(int mode, const ForceConfig &cfg);
+
+// ---- force_sym.cu ----
+// Whether a block of n_act of n particles takes the force by unordered pairs, and how (into cfg).
+bool sym_plan(int mode, int64_t n_act, int64_t n, int sm_count, ForceConfig *cfg);
+size_t sym_scratch_bytes(int64_t n);
+// Launches it: partials of force_partial_bytes, scratch of sym_scratch_bytes(n).  `ascending`: the
+// list is known to be the ascending list of distinct particles (a schedule, or all of them);
+// otherwise a list with a particle twice or an index out of range computes nothing here and
+// **rows_general, on the device, is n_act (else 0): the rows a general force of the same list
+// has to compute (force_launch's n_act_dev).  NULL for an ascending list.
+cudaError_t force_sym_launch(int mode, const JStream &js, int64_t n, const int32_t *active, int64_t n_act,
+                             double eps2, const ForceConfig &cfg, bool ascending, double *acc, double *jerk,
+                             double *pot, void *partials, void *scratch, const long long **rows_general,
+                             DevStatus *st, cudaStream_t s, int64_t *launches);
+// acc, jerk, pot <- the sums of the rows' slots; with rows_general only where it is not zero
+// (general) or zero (!general).
+cudaError_t force_sym_reduce_launch(int mode, const float *part, int slots, int64_t n_act, double *acc, double *jerk,
+                                    double *pot, const long long *rows_general, bool general, cudaStream_t s,
+                                    int64_t *launches);
 
 // ---- force_ds.cu ----
 int force_occupancy_ds();

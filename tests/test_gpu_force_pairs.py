@@ -1,0 +1,115 @@
+"""Large blocks by unordered pairs (csrc/force_sym.cuh) against the FP64 oracle and the one-sided kernel."""
+import numpy as np
+import pytest
+
+import oracle
+from synthetic import active_subset, plummer_sphere
+from tests.gpu_common import EPS2, check_force, gpu_force, need_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch():
+    return need_gpu()
+
+
+def _sim(m, x, v, eps2, mode, **kw):
+    from paper_astro_ph_0702058_gb300 import Simulation
+    return Simulation(m, x, v, eps2, mode=mode, **kw)
+
+
+def _masses(n, seed):
+    w = np.random.default_rng(seed).uniform(0.1, 10.0, n)
+    return w / w.sum()
+
+
+def _check(mode, m, x, v, eps2, act, got, st, what):
+    assert st["last_i_per_thread"] == 4, st  # the pairs took it
+    rows = np.unique(np.concatenate([np.arange(130), np.linspace(0, len(act) - 1, 400).astype(int),
+                                     np.arange(len(act) - 130, len(act))]))
+    ref = oracle.force(m, x, v, eps2, act[rows])
+    assert all(np.all(np.isfinite(g)) for g in got)
+    check_force(mode, m, x, v, eps2, act[rows], tuple(g[rows] for g in got), ref, what)
+
+
+# one-warp CTAs up to 32768 rows, four-warp ones above; one and several tiles per superblock; a last superblock
+# of one row, of one chunk and of a part of a chunk
+@pytest.mark.parametrize("mode", ["plain", "comp"])
+@pytest.mark.parametrize("n,eps2", [(8192, EPS2), (8193, EPS2), (16384, 0.0), (16385, EPS2), (32768, EPS2),
+                                    (33000, 0.0), (65536, EPS2), (70001, EPS2)])
+def test_all_particles(torch, mode, n, eps2):
+    m, x, v = plummer_sphere(n, 3)
+    m = _masses(n, 3)
+    with _sim(m, x, v, eps2, mode) as sim:  # (its set-up takes the pairs of the whole stream)
+        st0 = sim.stats()
+        assert st0["last_i_per_thread"] == 4, st0
+        s = {k: np.zeros((n, 3)) for k in ("a", "k")}
+        sim.get_state(**s)
+        sim.predict(0.0)
+        act = np.random.default_rng(1).permutation(n).astype(np.int32)  # any order of the list
+        got = gpu_force(sim, act)
+        st = sim.stats()
+        assert np.array_equal(got[0], gpu_force(sim, act)[0])  # repeats bit for bit
+    _check(mode, m, x, v, eps2, act, got, st, f"pairs n={n}")
+    every = np.arange(n, dtype=np.int32)
+    _check(mode, m, x, v, eps2, every, (s["a"], s["k"], got[2][np.argsort(act)]), st0, f"set-up n={n}")
+
+
+# blocks of three eighths (plain) or half of the particles on, the others outside (ragged ranges)
+@pytest.mark.parametrize("mode,n,n_act", [(mode, n, n_act) for mode in ("plain", "comp") for n, n_act in
+                                          ((8200, 8192), (16384, 8192), (15001, 8195), (65536, 33000))] +
+                         [("plain", 21845, 8192), ("plain", 100003, 40001)])
+def test_part_of_the_particles(torch, mode, n, n_act):
+    m, x, v = plummer_sphere(n, 4)
+    m = _masses(n, 4)
+    act = active_subset(n, n_act, 5)
+    with _sim(m, x, v, EPS2, mode) as sim:
+        sim.predict(0.0)
+        got = gpu_force(sim, act)
+        st = sim.stats()
+    _check(mode, m, x, v, EPS2, act, got, st, f"pairs n={n} n_act={n_act}")
+
+
+@pytest.mark.parametrize("mode", ["plain", "comp"])
+def test_lists_that_repeat_a_particle(torch, mode):
+    """A caller's list may hold a particle twice: every row is its particle's force, as from the one-sided kernel."""
+    n = 9000
+    m, x, v = plummer_sphere(n, 6)
+    act = np.arange(n, dtype=np.int32)[:8500].copy()
+    act[17] = act[8000]
+    with _sim(m, x, v, EPS2, mode) as sim, _sim(m, x, v, EPS2, mode, j_tile=256, i_block=1) as one:
+        for s in (sim, one):
+            s.predict(0.0)
+        got, ref = gpu_force(sim, act), gpu_force(one, act)
+        for g, r in zip(got, ref):
+            assert np.array_equal(g[17], g[8000])
+            np.testing.assert_allclose(g, r, rtol=0, atol=1e-4 * np.abs(r).max())
+        full = np.zeros(n, dtype=np.int32)  # the same particle in every row
+        got = gpu_force(sim, full)
+        assert np.all(got[0] == got[0][0]) and np.all(got[2] == got[2][0])
+    rows = np.array([0, 17, 8000])
+    check_force(mode, m, x, v, EPS2, act[rows], tuple(g[rows] for g in gpu_force_again(m, x, v, mode, act)),
+                oracle.force(m, x, v, EPS2, act[rows]), "repeated")
+
+
+def gpu_force_again(m, x, v, mode, act):
+    with _sim(m, x, v, EPS2, mode) as sim:
+        sim.predict(0.0)
+        return gpu_force(sim, act)
+
+
+def test_bad_index(torch):
+    from paper_astro_ph_0702058_gb300 import NBodyError
+    n = 9000
+    m, x, v = plummer_sphere(n, 7)
+    act = np.arange(n, dtype=np.int32)
+    act[5000] = n
+    with _sim(m, x, v, EPS2, "comp") as sim:
+        sim.predict(0.0)
+        with pytest.raises(NBodyError) as e:
+            gpu_force(sim, act)
+        assert e.value.code == -1
+        got = gpu_force(sim, np.arange(n, dtype=np.int32))
+        st = sim.stats()
+    _check("comp", m, x, v, EPS2, np.arange(n, dtype=np.int32), got, st, "after a bad index")
