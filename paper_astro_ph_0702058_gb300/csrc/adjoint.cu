@@ -13,7 +13,10 @@
 // p both of its roles combine linearly: with G_a = m_p g_a,q - m_q g_a,p and
 // G_k likewise, one evaluation per pair (p, q) gives p's position and
 // velocity gradients.
+#include <algorithm>
+
 #include "force_impl.cuh"  // fold_ds_rn; nbody_internal.cuh, ptx.cuh
+#include "step_impl.cuh"
 
 namespace nb {
 
@@ -191,45 +194,71 @@ __global__ void adj_init_kernel(DiffGrads G, int n)
 }
 
 // Loss L = sum |x|^2 + E_pot (FP64) and its gradient at the final state:
-// dL/dx_i = 2 x_i - m_i a_i, dL/dm_i = phi_i; per-particle loss terms in lval.
-__global__ void loss_kernel(const State S, double eps2, DiffGrads G, double *__restrict__ lval)
+// dL/dx_i = 2 x_i - m_i a_i, dL/dm_i = phi_i.  Grid (i-blocks, j-ranges): the FP64
+// sums (phi, a) of 128 rows over a range of whole 128-particle tiles go to
+// part[range][4][n].  FP64-bound (one unit per SM, ~19 cycles per warp
+// instruction): 18 operations per pair with rsqrt_f64, about 45 with an IEEE
+// root and division, and ranges spread a small n over every SM; n = 4096: 4.2 ms
+// in 32 blocks -> 0.7.
+__global__ void __launch_bounds__(128)
+    loss_pairs_kernel(const State S, double eps2, int tiles_per_range, double *__restrict__ part)
 {
     __shared__ double sx[128], sy[128], sz[128], sm[128];
-    const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    const int64_t i = blockIdx.x * 128ll + threadIdx.x;
     const bool live = i < S.n;
     const double xi = live ? S.x[0][i] : 0.0, yi = live ? S.x[1][i] : 0.0, zi = live ? S.x[2][i] : 0.0;
     double phi = 0.0, a0 = 0.0, a1 = 0.0, a2 = 0.0;
-    for (int64_t j0 = 0; j0 < S.n; j0 += 128) {
+    const int64_t j_begin = static_cast<int64_t>(blockIdx.y) * tiles_per_range * 128;
+    const int64_t j_end = j_begin + static_cast<int64_t>(tiles_per_range) * 128 < S.n
+                              ? j_begin + static_cast<int64_t>(tiles_per_range) * 128
+                              : S.n;
+    for (int64_t j0 = j_begin; j0 < j_end; j0 += 128) {
         __syncthreads();
-        for (int t = threadIdx.x; t < 128; t += blockDim.x) {
-            const int64_t j = j0 + t;
-            const bool ok = j < S.n;
-            sx[t] = ok ? S.x[0][j] : 0.0;
-            sy[t] = ok ? S.x[1][j] : 0.0;
-            sz[t] = ok ? S.x[2][j] : 0.0;
-            sm[t] = ok ? S.m[j] : 0.0;
+        const int64_t j = j0 + threadIdx.x;
+        if (j < j_end) {
+            sx[threadIdx.x] = S.x[0][j];
+            sy[threadIdx.x] = S.x[1][j];
+            sz[threadIdx.x] = S.x[2][j];
+            sm[threadIdx.x] = S.m[j];
         }
         __syncthreads();
-        const int jn = static_cast<int>(S.n - j0 < 128 ? S.n - j0 : 128);
+        const int jn = static_cast<int>(j_end - j0 < 128 ? j_end - j0 : 128);
+#pragma unroll 2
         for (int t = 0; t < jn; ++t) {
             if (j0 + t == i) continue;
             const double dx = sx[t] - xi, dy = sy[t] - yi, dz = sz[t] - zi;
-            const double r2 = eps2 + dx * dx + dy * dy + dz * dz;
-            const double rinv = 1.0 / sqrt(r2);
-            const double r3 = rinv * rinv * rinv;
-            phi -= sm[t] * rinv;
-            a0 += sm[t] * dx * r3;
-            a1 += sm[t] * dy * r3;
-            a2 += sm[t] * dz * r3;
+            const double y = rsqrt_f64(__fma_rn(dz, dz, __fma_rn(dy, dy, __fma_rn(dx, dx, eps2))));
+            const double my = sm[t] * y, w = my * (y * y);
+            phi -= my;
+            a0 = __fma_rn(w, dx, a0);
+            a1 = __fma_rn(w, dy, a1);
+            a2 = __fma_rn(w, dz, a2);
         }
     }
     if (!live) return;
-    const double mi = S.m[i];
-    G.gx[0][i] = 2.0 * xi - mi * a0;
-    G.gx[1][i] = 2.0 * yi - mi * a1;
-    G.gx[2][i] = 2.0 * zi - mi * a2;
-    G.gm[i] = phi;
-    lval[i] = xi * xi + yi * yi + zi * zi + 0.5 * mi * phi;
+    double *b = part + static_cast<size_t>(blockIdx.y) * 4 * S.n + i;
+    b[0] = phi;
+    b[S.n] = a0;
+    b[2 * S.n] = a1;
+    b[3 * S.n] = a2;
+}
+
+// Adds the ranges in ascending order; per-particle loss terms in lval.
+__global__ void loss_finish_kernel(const State S, const double *__restrict__ part, int ranges, DiffGrads G,
+                                   double *__restrict__ lval)
+{
+    const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    if (i >= S.n) return;
+    double t[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int y = 0; y < ranges; ++y)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) t[c] += part[(static_cast<size_t>(y) * 4 + c) * S.n + i];
+    const double xi = S.x[0][i], yi = S.x[1][i], zi = S.x[2][i], mi = S.m[i];
+    G.gx[0][i] = 2.0 * xi - mi * t[1];
+    G.gx[1][i] = 2.0 * yi - mi * t[2];
+    G.gx[2][i] = 2.0 * zi - mi * t[3];
+    G.gm[i] = t[0];
+    lval[i] = xi * xi + yi * yi + zi * zi + 0.5 * mi * t[0];
 }
 
 __global__ void sum_kernel(const double *__restrict__ v, int64_t n, double *out)
@@ -317,12 +346,32 @@ cudaError_t adj_init_launch(const DiffGrads &G, int64_t n, cudaStream_t s, int64
     return cudaGetLastError();
 }
 
-cudaError_t loss_launch(const State &S, double eps2, const DiffGrads &G, double *lval, double *loss, cudaStream_t s,
-                        int64_t *launches)
+namespace {
+// j-ranges of the loss (about four CTAs per SM) and tiles per range.
+int loss_ranges(int64_t n, int sm_count, int *tiles_per_range)
 {
-    loss_kernel<<<blocks_of(S.n, 128), 128, 0, s>>>(S, eps2, G, lval);
+    const int bx = blocks_of(n, 128);
+    const int want = std::max(1, std::min((4 * sm_count + bx - 1) / bx, bx));
+    *tiles_per_range = (bx + want - 1) / want;
+    return (bx + *tiles_per_range - 1) / *tiles_per_range;
+}
+}  // namespace
+
+size_t loss_scratch_doubles(int64_t n, int sm_count)
+{
+    int tpr;
+    return static_cast<size_t>(loss_ranges(n, sm_count, &tpr)) * 4 * static_cast<size_t>(n);
+}
+
+cudaError_t loss_launch(const State &S, double eps2, const DiffGrads &G, int sm_count, double *scratch, double *lval,
+                        double *loss, cudaStream_t s, int64_t *launches)
+{
+    int tpr;
+    const int r = loss_ranges(S.n, sm_count, &tpr);
+    loss_pairs_kernel<<<dim3(blocks_of(S.n, 128), r), 128, 0, s>>>(S, eps2, tpr, scratch);
+    loss_finish_kernel<<<blocks_of(S.n, 64), 64, 0, s>>>(S, scratch, r, G, lval);
     sum_kernel<<<1, 1024, 0, s>>>(lval, S.n, loss);
-    *launches += 2;
+    *launches += 3;
     return cudaGetLastError();
 }
 

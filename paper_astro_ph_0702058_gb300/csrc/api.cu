@@ -357,18 +357,16 @@ int check_params(const nbody_params *p)
 int energy_common(nbody_ctx *c, double *ekin, double *epot, bool ds_potential)
 {
     NB_CUDA(time_range_launch(c->S, c->trange, c->s, &c->stats.kernel_launches), "time-range kernel");
+    NB_CUDA(energy_launch(c->S, c->eps2, c->phi, c->trange, c->e_out, c->s, &c->stats.kernel_launches, ds_potential),
+            "energy kernels");
     NB_CUDA(cudaMemcpyAsync(c->trange_host, c->trange, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->s),
             "time-range read-back");
-    int r = sync_and_check(c);
+    NB_CUDA(cudaMemcpyAsync(c->e_host, c->e_out, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->s), "energy read-back");
+    const int r = sync_and_check(c);
     if (r != NBODY_OK) return r;
     if (c->trange_host[0] != c->trange_host[1])
         return fail(NBODY_ENOTSYNC, "particles are at different times (%llu .. %llu ticks)", c->trange_host[0],
                     c->trange_host[1]);
-    NB_CUDA(energy_launch(c->S, c->eps2, c->phi, c->e_out, c->s, &c->stats.kernel_launches, ds_potential),
-            "energy kernels");
-    NB_CUDA(cudaMemcpyAsync(c->e_host, c->e_out, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->s), "energy read-back");
-    r = sync_and_check(c);
-    if (r != NBODY_OK) return r;
     *ekin = c->e_host[0];
     *epot = c->e_host[1];
     return NBODY_OK;
@@ -452,7 +450,8 @@ int rollout_impl(const char *who, int64_t n, const double *m, const double *x0, 
     NB_DR(dev_alloc(reinterpret_cast<void **>(&lval), nd * sizeof(double)), "loss terms");
     NB_DR(dev_alloc(reinterpret_cast<void **>(&dloss), sizeof(double)), "loss");
     NB_DR(dev_alloc(reinterpret_cast<void **>(&g4), 2 * npad * sizeof(float4)), "force upstream");
-    const size_t vjp_doubles = vjp_scratch_doubles(n, c->n_pad, c->sm_count);
+    const size_t vjp_doubles = std::max(vjp_scratch_doubles(n, c->n_pad, c->sm_count),
+                                        seed_loss ? loss_scratch_doubles(n, c->sm_count) : size_t(0));
     if (vjp_doubles) NB_DR(dev_alloc(reinterpret_cast<void **>(&vjp), vjp_doubles * sizeof(double)), "adjoint scratch");
     NB_DR(cudaMemsetAsync(gbuf, 0, 19 * nd * sizeof(double), s), "memset");
     NB_DR(cudaMemsetAsync(g4, 0, 2 * npad * sizeof(float4), s), "memset");
@@ -496,7 +495,7 @@ int rollout_impl(const char *who, int64_t n, const double *m, const double *x0, 
     r = copy_final();  // before the backward sweep overwrites the state
     if (r != NBODY_OK) return done(r);
     if (seed_loss) {
-        NB_DR(loss_launch(c->S, eps2, G, lval, dloss, s, L), "loss kernels");
+        NB_DR(loss_launch(c->S, eps2, G, c->sm_count, vjp, lval, dloss, s, L), "loss kernels");
     } else {  // the cotangents of the final x, v seed the sweep (row-major n x 3 -> components)
         if (g_xT) {
             NB_DR(to_device(c->stage, g_xT, 3 * nd * sizeof(double), s), "cotangent upload");
@@ -624,7 +623,7 @@ int nbody_init(nbody_ctx **out, int64_t n, const double *m, const double *x, con
     NB_INIT(dev_alloc(&c->sched_scratch, sched_scratch_bytes(n)), "scheduler scratch allocation");
     NB_INIT(dev_alloc(reinterpret_cast<void **>(&c->sched_out), sizeof(SchedOut)), "scheduler allocation");
     NB_INIT(dev_alloc(reinterpret_cast<void **>(&c->st), sizeof(DevStatus)), "status allocation");
-    NB_INIT(dev_alloc(reinterpret_cast<void **>(&c->phi), nd * sizeof(double)), "energy scratch allocation");
+    NB_INIT(dev_alloc(reinterpret_cast<void **>(&c->phi), (nd + kEnergyPad) * sizeof(double)), "energy scratch allocation");
     NB_INIT(dev_alloc(reinterpret_cast<void **>(&c->e_out), 2 * sizeof(double)), "energy allocation");
     NB_INIT(dev_alloc(reinterpret_cast<void **>(&c->trange), 2 * sizeof(unsigned long long)), "time-range allocation");
     NB_INIT(host_alloc(reinterpret_cast<void **>(&c->sched_host), sizeof(SchedOut)), "pinned allocation");

@@ -483,9 +483,7 @@ __global__ void ens_phi_kernel(const EnsDev E, double eps2, double *__restrict__
         for (int64_t j = E.off[c]; j < E.off[c + 1]; ++j) {
             if (j == i) continue;
             const double dx = E.S.x[0][j] - xi, dy = E.S.x[1][j] - yi, dz = E.S.x[2][j] - zi;
-            const double r2 = __dadd_rn(__dadd_rn(__dadd_rn(eps2, __dmul_rn(dx, dx)), __dmul_rn(dy, dy)),
-                                        __dmul_rn(dz, dz));
-            p = __dsub_rn(p, __ddiv_rn(E.S.m[j], __dsqrt_rn(r2)));
+            p = __fma_rn(-E.S.m[j], rsqrt_f64(__fma_rn(dz, dz, __fma_rn(dy, dy, __fma_rn(dx, dx, eps2)))), p);
         }
         phi[i] = p;
     }

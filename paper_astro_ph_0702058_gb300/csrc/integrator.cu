@@ -343,68 +343,6 @@ __global__ void step_loop_kernel(const SchedOut *next, const LoopArgs la)
     loop_decide(la, next->t_blk, next->n_act);
 }
 
-// ------------------------------------------------------------------ energy
-// phi_i = -sum_{j != i} m_j / sqrt(r^2 + eps^2) in FP64, j in ascending order.
-constexpr int kETile = 128;
-
-__global__ void phi_kernel(const State S, double eps2, double *__restrict__ phi)
-{
-    __shared__ double sx[kETile], sy[kETile], sz[kETile], sm[kETile];
-    const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-    const bool live = i < S.n;
-    const double xi = live ? S.x[0][i] : 0.0;
-    const double yi = live ? S.x[1][i] : 0.0;
-    const double zi = live ? S.x[2][i] : 0.0;
-    double p = 0.0;
-    for (int64_t j0 = 0; j0 < S.n; j0 += kETile) {
-        __syncthreads();
-        for (int t = threadIdx.x; t < kETile; t += blockDim.x) {
-            const int64_t j = j0 + t;
-            const bool ok = j < S.n;
-            sx[t] = ok ? S.x[0][j] : 0.0;
-            sy[t] = ok ? S.x[1][j] : 0.0;
-            sz[t] = ok ? S.x[2][j] : 0.0;
-            sm[t] = ok ? S.m[j] : 0.0;
-        }
-        __syncthreads();
-        const int jn = static_cast<int>(S.n - j0 < kETile ? S.n - j0 : kETile);
-        for (int t = 0; t < jn; ++t) {
-            if (j0 + t == i) continue;
-            const double dx = sx[t] - xi, dy = sy[t] - yi, dz = sz[t] - zi;
-            const double r2 = __dadd_rn(__dadd_rn(__dadd_rn(eps2, __dmul_rn(dx, dx)), __dmul_rn(dy, dy)),
-                                        __dmul_rn(dz, dz));
-            p = __dsub_rn(p, __ddiv_rn(sm[t], __dsqrt_rn(r2)));
-        }
-    }
-    if (live) phi[i] = p;
-}
-
-// One block: E_kin = sum m v^2 / 2, E_pot = sum m phi / 2 (fixed summation order).
-__global__ void energy_sum_kernel(const State S, const double *__restrict__ phi, double *out)
-{
-    __shared__ double sk[1024], sp[1024];
-    double k = 0.0, p = 0.0;
-    for (int64_t i = threadIdx.x; i < S.n; i += blockDim.x) {
-        const double vx = S.v[0][i], vy = S.v[1][i], vz = S.v[2][i];
-        k += 0.5 * S.m[i] * (vx * vx + vy * vy + vz * vz);
-        p += 0.5 * S.m[i] * phi[i];
-    }
-    sk[threadIdx.x] = k;
-    sp[threadIdx.x] = p;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (static_cast<int>(threadIdx.x) < s) {
-            sk[threadIdx.x] += sk[threadIdx.x + s];
-            sp[threadIdx.x] += sp[threadIdx.x + s];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        out[0] = sk[0];
-        out[1] = sp[0];
-    }
-}
-
 __global__ void time_range_kernel(const State S, unsigned long long *out)
 {
     __shared__ unsigned long long sh[32];
@@ -568,21 +506,6 @@ cudaError_t schedule_loop_launch(const State &S, int lmax, int32_t *active, Sche
     cudaError_t e = schedule_launch(S, lmax, active, out, scratch, s, launches);
     if (e != cudaSuccess) return e;
     step_loop_kernel<<<1, 1, 0, s>>>(out, la);
-    ++*launches;
-    return cudaGetLastError();
-}
-
-cudaError_t energy_launch(const State &S, double eps2, double *phi, double *out, cudaStream_t s,
-                          int64_t *launches, bool ds_potential)
-{
-    if (ds_potential) {
-        const cudaError_t e = phi_ds_launch(S, eps2, phi, s, launches);
-        if (e != cudaSuccess) return e;
-    } else {
-        phi_kernel<<<blocks_for(S.n, kETile), kETile, 0, s>>>(S, eps2, phi);
-        ++*launches;
-    }
-    energy_sum_kernel<<<1, 1024, 0, s>>>(S, phi, out);
     ++*launches;
     return cudaGetLastError();
 }

@@ -274,13 +274,13 @@ cudaError_t grid_step_launch(int mode, const State &S, const JStream &J, double 
                              DevStatus *st, SchedOut *sched_out, StepLoop *L, int32_t *act_out, void *buf,
                              cudaStream_t s, int64_t *launches);
 
-// E_kin and E_pot (phi scratch: n doubles; out: 2 doubles); the potential in
-// FP64 or, with ds_potential, in double-single arithmetic (energy_ds.cu).
-cudaError_t energy_launch(const State &S, double eps2, double *phi_scratch, double *out,
+// ---- energy.cu ----
+// E_kin and E_pot (scratch: n + kEnergyPad doubles; out: 2 doubles) of a system whose times are
+// all alike, trange[0] == trange[1] (else nothing is computed); the potential in FP64 or, with
+// ds_potential, in double-single arithmetic.
+constexpr int kEnergyPad = 64;
+cudaError_t energy_launch(const State &S, double eps2, double *scratch, const unsigned long long *trange, double *out,
                           cudaStream_t s, int64_t *launches, bool ds_potential = false);
-// ---- energy_ds.cu ----
-// phi_i = -sum_{j != i} m_j / sqrt(eps2 + |x_j - x_i|^2) in double-single arithmetic (n doubles).
-cudaError_t phi_ds_launch(const State &S, double eps2, double *phi, cudaStream_t s, int64_t *launches);
 // min and max of t over all particles (out: 2 unsigned long long).
 cudaError_t time_range_launch(const State &S, unsigned long long *out, cudaStream_t s,
                               int64_t *launches);
@@ -311,8 +311,9 @@ cudaError_t force_vjp_launch(const JStream &J, const DiffGrads &G, int64_t n, fl
 cudaError_t adj_correct_launch(const DiffGrads &G, int64_t n, double dt, cudaStream_t s, int64_t *launches);
 cudaError_t adj_predict_launch(const DiffGrads &G, int64_t n, double dt, cudaStream_t s, int64_t *launches);
 cudaError_t adj_init_launch(const DiffGrads &G, int64_t n, cudaStream_t s, int64_t *launches);
-cudaError_t loss_launch(const State &S, double eps2, const DiffGrads &G, double *lval, double *loss,
-                        cudaStream_t s, int64_t *launches);
+size_t loss_scratch_doubles(int64_t n, int sm_count);
+cudaError_t loss_launch(const State &S, double eps2, const DiffGrads &G, int sm_count, double *scratch, double *lval,
+                        double *loss, cudaStream_t s, int64_t *launches);
 cudaError_t set_time_launch(const State &S, int64_t tick, int level, cudaStream_t s, int64_t *launches);
 
 // Row-major n x 3 <-> three component arrays.

@@ -58,6 +58,21 @@ __device__ __forceinline__ double f2d(const float f)
     return __longlong_as_double(static_cast<long long>(bits));
 }
 
+// x^(-1/2) in FP64 with 5 operations on the FP64 pipe: the MUFU's approximation y0
+// (relative error below 2^-20) times the binomial series of (1 - e)^(-1/2) in
+// e = 1 - x y0^2 to second order; the third, 5 e^3/16, is below 2^-61.  y0 has 21
+// significant bits at most, so y0^2 is exact.  Arguments outside [2^-900, 2^900]
+// (zero, subnormal, infinite, NaN) take the IEEE root and division.
+__device__ __forceinline__ double rsqrt_f64(const double x)
+{
+    const unsigned int ex = (static_cast<unsigned int>(__double2hiint(x)) >> 20) - 123u;  // (sign: out of range)
+    if (ex > 1800u) return __ddiv_rn(1.0, __dsqrt_rn(x));
+    double y0;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
+    const double e = __fma_rn(-x, __dmul_rn(y0, y0), 1.0);
+    return __fma_rn(__dmul_rn(y0, e), __fma_rn(0.375, e, 0.5), y0);
+}
+
 __device__ __forceinline__ double norm3(const double *u)
 {
     return sqrt(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
@@ -238,6 +253,9 @@ struct MinOp {
 };
 struct MaxOp {
     __device__ unsigned long long operator()(unsigned long long a, unsigned long long b) const { return a > b ? a : b; }
+};
+struct AddOp {
+    __device__ double operator()(double a, double b) const { return a + b; }
 };
 struct SumOp {
     __device__ long long operator()(long long a, long long b) const { return a + b; }
