@@ -313,9 +313,11 @@ void nbody_debug_step_graphs(int level);
  * initial positions, velocities (n x 3) and masses (n) to g_x0, g_v0, g_m
  * (host or device).  The adjoint transposes the predictor and corrector and
  * applies a hand-written vector-Jacobian product of the pair force (FP32
- * pair math, FP64 totals); states are checkpointed every checkpoint_every
- * steps (<= 0: 16) and each segment is recomputed forward during the
- * backward sweep.  eps2 must be > 0.  Allocates its own scratch; waits.
+ * pair math, FP64 totals).  The states of the run are kept where 1 GiB holds
+ * them (96 n bytes each); otherwise they are checkpointed every
+ * checkpoint_every steps (<= 0: 16) and each segment is recomputed forward
+ * during the backward sweep, with the same results.  eps2 must be > 0.
+ * Allocates its own scratch; waits.
  * Errors: EINVAL, ENOMEM, ECUDA, ENONFINITE. */
 int nbody_diff_rollout(int64_t n, const double *m, const double *x0, const double *v0, double eps2,
                        int level, int64_t steps, int64_t checkpoint_every, int mode, double *loss,

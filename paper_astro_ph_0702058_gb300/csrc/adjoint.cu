@@ -14,6 +14,7 @@
 // G_k likewise, one evaluation per pair (p, q) gives p's position and
 // velocity gradients.
 #include <algorithm>
+#include <cmath>
 
 #include "force_impl.cuh"  // fold_ds_rn; nbody_internal.cuh, ptx.cuh
 #include "step_impl.cuh"
@@ -26,13 +27,12 @@ constexpr int kVjpThreads = 128;
 constexpr int kVjpTile = 128;
 
 // grid (i-blocks, j-ranges): block (x, y) takes the particles p of i-block x
-// against the j-tiles of range y.  With one range it adds its totals to the
-// gradients; with several it writes them to part[y][7][n] and
-// vjp_reduce_kernel adds the ranges in ascending order (deterministic).
+// against the j-tiles of range y and writes its totals to part[y][7][n]; the
+// kernel that follows adds the ranges in ascending order (deterministic).
 __global__ void __launch_bounds__(kVjpThreads)
     force_vjp_kernel(const float4 *__restrict__ posm, const float4 *__restrict__ vel,
                      const float4 *__restrict__ gA, const float4 *__restrict__ gK, int n, int n_pad, float eps2,
-                     int tiles_per_range, double *__restrict__ part, DiffGrads G)
+                     int tiles_per_range, double *__restrict__ part)
 {
     __shared__ float4 sp[kVjpTile], sv[kVjpTile], sa[kVjpTile], sk[kVjpTile];
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
@@ -101,22 +101,13 @@ __global__ void __launch_bounds__(kVjpThreads)
         tv[c] = static_cast<double>(hv[c]) + static_cast<double>(lv[c]);
     }
     const double tm = static_cast<double>(hm) + static_cast<double>(lm);
-    if (gridDim.y == 1) {
+    double *b = part + static_cast<size_t>(blockIdx.y) * 7 * n + p;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            G.gxp[c][p] += tx[c];
-            G.gvp[c][p] += tv[c];
-        }
-        G.gm[p] += tm;
-    } else {
-        double *b = part + static_cast<size_t>(blockIdx.y) * 7 * n + p;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            b[static_cast<size_t>(c) * n] = tx[c];
-            b[static_cast<size_t>(3 + c) * n] = tv[c];
-        }
-        b[static_cast<size_t>(6) * n] = tm;
+    for (int c = 0; c < 3; ++c) {
+        b[static_cast<size_t>(c) * n] = tx[c];
+        b[static_cast<size_t>(3 + c) * n] = tv[c];
     }
+    b[static_cast<size_t>(6) * n] = tm;
 }
 
 // One thread per (particle, component): adds the component's ranges in order.
@@ -136,61 +127,119 @@ __global__ void vjp_reduce_kernel(const double *__restrict__ part, int ranges, i
         G.gm[p] += t;
 }
 
-// Transposed corrector: from the gradients of the corrected state (gx, gv, ga,
-// gk) to those of the predicted state (gxp, gvp), of the force (gA, gK, FP32)
-// and of the start-of-step a, k (left in ga, gk).
-__global__ void adj_correct_kernel(DiffGrads G, int n, double dt)
+// One forward step's end and the next one's start, one thread per (component,
+// particle): the force on the particle (its j-range partials, or acc and jerk),
+// the corrector from the state at src to the state at dst, and (predict) the
+// j-stream at the prediction from there.  src, dst: x[3], v[3], a[3], k[3] of n
+// doubles each.  A shared step has no criterion or level, so the components are
+// independent: three short FP64 chains in parallel instead of the general
+// corrector's one with its roots and division, and no kernel boundary between
+// the reduction, the corrector, the copy of the state and the predictor
+// (n = 4096: 7.5 + 11.0 + 2 + 4.7 us before).
+template <bool DSW>
+__global__ void roll_step_kernel(const double *src, double *dst, const int n, const double *__restrict__ acc,
+                                 const double *__restrict__ jerk, const float *__restrict__ part, const int split,
+                                 const CorrDt d, const bool predict, const JStream J, DevStatus *st)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const double c1 = dt * dt * dt * dt / 24.0, c2 = dt * dt * dt * dt * dt / 120.0;
-    const double c3 = dt * dt * dt / 6.0, c4 = dt * dt * dt * dt / 24.0;
-    float ap[3], kp[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const double gx = G.gx[c][i], gv = G.gv[c][i];
-        const double g2 = c1 * gx + c3 * gv, g3 = c2 * gx + c4 * gv;
-        ap[c] = static_cast<float>(6.0 / (dt * dt) * g2 - 12.0 / (dt * dt * dt) * g3 + G.ga[c][i]);
-        kp[c] = static_cast<float>(-2.0 / dt * g2 + 6.0 / (dt * dt) * g3 + G.gk[c][i]);
-        G.ga[c][i] = -6.0 / (dt * dt) * g2 + 12.0 / (dt * dt * dt) * g3;
-        G.gk[c][i] = -4.0 / dt * g2 + 6.0 / (dt * dt) * g3;
-        G.gxp[c][i] = gx;
-        G.gvp[c][i] = gv;
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= 3 * n) return;
+    const int c = idx / n, i = idx - c * n;
+    double ap, kp;
+    if (part) {
+        constexpr int NC = DSW ? 14 : 7;
+        float ah = 0.0f, al = 0.0f, kh = 0.0f, kl = 0.0f;
+        const float *b = part + static_cast<size_t>(c) * n + i;
+#pragma unroll 4
+        for (int r = 0; r < split; ++r, b += static_cast<size_t>(NC) * n) {
+            ds2_add(ah, al, b[0], DSW ? b[static_cast<size_t>(7) * n] : 0.0f);
+            ds2_add(kh, kl, b[static_cast<size_t>(3) * n], DSW ? b[static_cast<size_t>(10) * n] : 0.0f);
+        }
+        ap = f2d(ah) + f2d(al);
+        kp = f2d(kh) + f2d(kl);
+    } else {
+        ap = acc[3 * static_cast<size_t>(i) + c];
+        kp = jerk[3 * static_cast<size_t>(i) + c];
     }
-    G.gA[i] = make_float4(ap[0], ap[1], ap[2], 0.f);
-    G.gK[i] = make_float4(kp[0], kp[1], kp[2], 0.f);
+    const size_t e = static_cast<size_t>(idx), n3 = 3 * static_cast<size_t>(n);
+    double xn, vn, a2e, a3;
+    corr_dim(src[e], src[n3 + e], src[2 * n3 + e], src[3 * n3 + e], ap, kp, d, xn, vn, a2e, a3);
+    if (!(isfinite(xn) && isfinite(vn) && isfinite(ap) && isfinite(kp))) {
+        atomicOr(&st->flags, static_cast<unsigned>(kFlagNonfinite));
+        atomicAdd(&st->nonfinite, 1ull);
+    }
+    dst[e] = xn;
+    dst[n3 + e] = vn;
+    dst[2 * n3 + e] = ap;
+    dst[3 * n3 + e] = kp;
+    if (!predict) return;
+    double xp, vp;
+    predict_dim(xn, vn, ap, kp, d.pd, xp, vp);
+    const float h = d2f_rn(xp);
+    J.soa[static_cast<size_t>(c) * J.n_pad + i] = h;
+    J.soa[static_cast<size_t>(4 + c) * J.n_pad + i] = d2f_rn(vp);
+    if (DSW) J.soa[static_cast<size_t>(7 + c) * J.n_pad + i] = d2f_rn(xp - f2d(h));
 }
 
-// Transposed predictor: gradients of the start-of-step state.
-__global__ void adj_predict_kernel(DiffGrads G, int n, double dt)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const double gxp = G.gxp[c][i], gvp = G.gvp[c][i];
-        G.gx[c][i] = gxp;
-        G.gv[c][i] = gxp * dt + gvp;
-        G.ga[c][i] += gxp * dt * dt / 2.0 + gvp * dt;
-        G.gk[c][i] += gxp * dt * dt * dt / 6.0 + gvp * dt * dt / 2.0;
-    }
-}
+// Coefficients of the transposed corrector and predictor of a step dt.
+struct AdjDt {
+    double dt, dt2h, dt3s;      // dt, dt^2 / 2, dt^3 / 6
+    double c1, c2, c3, c4;      // dt^4 / 24, dt^5 / 120, dt^3 / 6, dt^4 / 24
+    double i1, i2, i3;          // 1 / dt, 1 / dt^2, 1 / dt^3
+    PredDt pd;
+};
 
-// Start of the rollout: the upstream of the t = 0 force is (ga, gk) itself.
-__global__ void adj_init_kernel(DiffGrads G, int n)
+// Between two force adjoints of the backward sweep, one thread per (component,
+// particle).  With `after` (> 0) the totals of the last one (its `after` ranges
+// of part) join the gradients of the predicted state and the masses, and the
+// transposed predictor leads to the gradients of the state the step began
+// with.  Then, with `corrector`, the transposed corrector of the step before:
+// from the gradients of the corrected state (gx, gv, ga, gk) to those of the
+// predicted one (gxp, gvp), of the force (gA, gK, FP32) and of the start's a, k
+// (left in ga, gk); without it the force at t = 0, whose upstream is (ga, gk)
+// itself.  Last, the j-stream the force adjoint reads, at the prediction of
+// that step from its state `src` (dt = 0 at t = 0).
+__global__ void adj_step_kernel(const double *__restrict__ part, const int after, const DiffGrads G, const int n,
+                                const AdjDt d, const bool corrector, const double *__restrict__ src, const JStream J)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float ap[3], kp[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        ap[c] = static_cast<float>(G.ga[c][i]);
-        kp[c] = static_cast<float>(G.gk[c][i]);
-        G.gxp[c][i] = G.gx[c][i];
-        G.gvp[c][i] = G.gv[c][i];
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= 3 * n) return;
+    const int c = idx / n, i = idx - c * n;
+    const size_t e = static_cast<size_t>(idx), n3 = 3 * static_cast<size_t>(n);
+    // (the component arrays of each gradient are contiguous: gx[0][e] is component c of particle i)
+    double gx = G.gx[0][e], gv = G.gv[0][e], ga = G.ga[0][e], gk = G.gk[0][e];
+    if (after > 0) {
+        double tx = 0.0, tv = 0.0, tm = 0.0;
+        for (int y = 0; y < after; ++y) {
+            const double *b = part + static_cast<size_t>(y) * 7 * n + e;
+            tx += b[0];
+            tv += b[n3];
+            if (c == 0) tm += b[2 * n3];
+        }
+        if (c == 0) G.gm[i] += tm;
+        const double gxp = G.gxp[0][e] + tx, gvp = G.gvp[0][e] + tv;
+        gx = gxp;
+        gv = gxp * d.dt + gvp;
+        ga += gxp * d.dt2h + gvp * d.dt;
+        gk += gxp * d.dt3s + gvp * d.dt2h;
     }
-    G.gA[i] = make_float4(ap[0], ap[1], ap[2], 0.f);
-    G.gK[i] = make_float4(kp[0], kp[1], kp[2], 0.f);
+    float ap = static_cast<float>(ga), kp = static_cast<float>(gk);
+    if (corrector) {
+        const double g2 = d.c1 * gx + d.c3 * gv, g3 = d.c2 * gx + d.c4 * gv;
+        ap = static_cast<float>(6.0 * d.i2 * g2 - 12.0 * d.i3 * g3 + ga);
+        kp = static_cast<float>(-2.0 * d.i1 * g2 + 6.0 * d.i2 * g3 + gk);
+        ga = -6.0 * d.i2 * g2 + 12.0 * d.i3 * g3;
+        gk = -4.0 * d.i1 * g2 + 6.0 * d.i2 * g3;
+    }
+    G.gxp[0][e] = gx;
+    G.gvp[0][e] = gv;
+    G.ga[0][e] = ga;
+    G.gk[0][e] = gk;
+    reinterpret_cast<float *>(G.gA + i)[c] = ap;
+    reinterpret_cast<float *>(G.gK + i)[c] = kp;
+    double xp = src[e], vp = src[n3 + e];
+    if (corrector) predict_dim(xp, vp, src[2 * n3 + e], src[3 * n3 + e], d.pd, xp, vp);
+    reinterpret_cast<float *>(J.posm + i)[c] = d2f_rn(xp);
+    reinterpret_cast<float *>(J.vel + i)[c] = d2f_rn(vp);
 }
 
 // Loss L = sum |x|^2 + E_pot (FP64) and its gradient at the final state:
@@ -275,16 +324,6 @@ __global__ void sum_kernel(const double *__restrict__ v, int64_t n, double *out)
     if (threadIdx.x == 0) *out = s[0];
 }
 
-// Shared step: every particle's time is `tick` and level `level`.
-__global__ void set_time_kernel(const State S, int64_t tick, int level)
-{
-    for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < S.n;
-         i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        S.t[i] = tick;
-        S.level[i] = static_cast<int8_t>(level);
-    }
-}
-
 int blocks_of(int64_t n, int t) { return static_cast<int>((n + t - 1) / t); }
 
 }  // namespace
@@ -302,46 +341,72 @@ int vjp_ranges(int64_t n, int64_t n_pad, int sm_count)
 
 size_t vjp_scratch_doubles(int64_t n, int64_t n_pad, int sm_count)
 {
-    const int r = vjp_ranges(n, n_pad, sm_count);
-    return r > 1 ? static_cast<size_t>(r) * 7 * static_cast<size_t>(n) : 0;
+    return static_cast<size_t>(vjp_ranges(n, n_pad, sm_count)) * 7 * static_cast<size_t>(n);
 }
 
 cudaError_t force_vjp_launch(const JStream &J, const DiffGrads &G, int64_t n, float eps2, int sm_count,
-                             double *scratch, cudaStream_t s, int64_t *launches)
+                             double *scratch, int *ranges, cudaStream_t s, int64_t *launches)
 {
     const int tiles = static_cast<int>(J.n_pad / kVjpTile);
     const int r = vjp_ranges(n, J.n_pad, sm_count);
     const int tpr = (tiles + r - 1) / r;
     const dim3 grid(blocks_of(n, kVjpThreads), r);
     force_vjp_kernel<<<grid, kVjpThreads, 0, s>>>(J.posm, J.vel, G.gA, G.gK, static_cast<int>(n),
-                                                  static_cast<int>(J.n_pad), eps2, tpr, scratch, G);
+                                                  static_cast<int>(J.n_pad), eps2, tpr, scratch);
     ++*launches;
-    if (r > 1) {
-        vjp_reduce_kernel<<<blocks_of(7 * n, 256), 256, 0, s>>>(scratch, r, static_cast<int>(n), G);
-        ++*launches;
-    }
+    *ranges = r;
     return cudaGetLastError();
 }
 
-cudaError_t adj_correct_launch(const DiffGrads &G, int64_t n, double dt, cudaStream_t s, int64_t *launches)
+cudaError_t vjp_finish_launch(const DiffGrads &G, int64_t n, const double *scratch, int ranges, cudaStream_t s,
+                              int64_t *launches)
 {
-    const int t = n >= 152 * 256 ? 256 : 32;  // FP64-heavy rows: spread small n over more SMs
-    adj_correct_kernel<<<blocks_of(n, t), t, 0, s>>>(G, static_cast<int>(n), dt);
+    vjp_reduce_kernel<<<blocks_of(7 * n, 256), 256, 0, s>>>(scratch, ranges, static_cast<int>(n), G);
     ++*launches;
     return cudaGetLastError();
 }
 
-cudaError_t adj_predict_launch(const DiffGrads &G, int64_t n, double dt, cudaStream_t s, int64_t *launches)
+namespace {
+// Threads of the per-(component, particle) kernels: FP64 chains, so a small n is
+// spread over all SMs.
+int elem_threads(int64_t n) { return 3 * n >= 152 * 512 ? 256 : 32; }
+}  // namespace
+
+cudaError_t roll_step_launch(const double *src, double *dst, int64_t n, const double *acc, const double *jerk,
+                             const float *part, int split, bool two_word, int level, bool predict, const JStream &J,
+                             DevStatus *st, cudaStream_t s, int64_t *launches)
 {
-    const int t = n >= 152 * 256 ? 256 : 32;
-    adj_predict_kernel<<<blocks_of(n, t), t, 0, s>>>(G, static_cast<int>(n), dt);
+    const double dt = std::ldexp(1.0, -level);
+    CorrDt d;
+    d.dt = dt;
+    d.idt = 1.0 / dt;  // (powers of two: every one of these is exact but the third)
+    d.idt2 = d.idt * d.idt;
+    d.dt3 = dt * dt * dt;
+    d.dt4 = d.dt3 * dt;
+    d.pd = {dt, 0.5 * dt, dt * (1.0 / 3.0)};
+    const int t = elem_threads(n);
+    auto *kernel = two_word ? roll_step_kernel<true> : roll_step_kernel<false>;
+    kernel<<<blocks_of(3 * n, t), t, 0, s>>>(src, dst, static_cast<int>(n), acc, jerk, part, split, d, predict, J, st);
     ++*launches;
     return cudaGetLastError();
 }
 
-cudaError_t adj_init_launch(const DiffGrads &G, int64_t n, cudaStream_t s, int64_t *launches)
+cudaError_t adj_step_launch(const double *scratch, int after, const DiffGrads &G, int64_t n, double dt, bool corrector,
+                            const double *src, const JStream &J, cudaStream_t s, int64_t *launches)
 {
-    adj_init_kernel<<<blocks_of(n, 256), 256, 0, s>>>(G, static_cast<int>(n));
+    AdjDt d;
+    d.dt = dt;
+    d.dt2h = dt * dt / 2.0;
+    d.dt3s = dt * dt * dt / 6.0;
+    d.c1 = d.c4 = dt * dt * dt * dt / 24.0;
+    d.c2 = dt * dt * dt * dt * dt / 120.0;
+    d.c3 = d.dt3s;
+    d.i1 = 1.0 / dt;
+    d.i2 = d.i1 * d.i1;
+    d.i3 = d.i2 * d.i1;
+    d.pd = {dt, 0.5 * dt, dt * (1.0 / 3.0)};
+    const int t = elem_threads(n);
+    adj_step_kernel<<<blocks_of(3 * n, t), t, 0, s>>>(scratch, after, G, static_cast<int>(n), d, corrector, src, J);
     ++*launches;
     return cudaGetLastError();
 }
@@ -372,13 +437,6 @@ cudaError_t loss_launch(const State &S, double eps2, const DiffGrads &G, int sm_
     loss_finish_kernel<<<blocks_of(S.n, 64), 64, 0, s>>>(S, scratch, r, G, lval);
     sum_kernel<<<1, 1024, 0, s>>>(lval, S.n, loss);
     *launches += 3;
-    return cudaGetLastError();
-}
-
-cudaError_t set_time_launch(const State &S, int64_t tick, int level, cudaStream_t s, int64_t *launches)
-{
-    set_time_kernel<<<blocks_of(S.n, 256) < 1024 ? blocks_of(S.n, 256) : 1024, 256, 0, s>>>(S, tick, level);
-    ++*launches;
     return cudaGetLastError();
 }
 

@@ -24,6 +24,7 @@ int g_fail_alloc = 0;    // allocation-failure injection countdown (test hook)
 // replay per block, 2 a device-side loop of blocks in each replay
 int g_step_graphs = 3;
 constexpr int64_t kLoopCap = 1024;  // blocks one replay of the loop may run
+constexpr int64_t kRollKeep = int64_t(1) << 30;  // bytes of states a gradient keeps instead of running steps again
 constexpr int64_t kClusterCap = 4096;  // blocks one launch of the cluster or the grid kernel may run
 #ifndef NB_GRID_ROWS
 #define NB_GRID_ROWS 4095
@@ -394,11 +395,8 @@ int rollout_impl(const char *who, int64_t n, const double *m, const double *x0, 
     nbody_ctx *c = nullptr;
     int r = nbody_init(&c, n, m, x0, v0, eps2, &p);
     if (r != NBODY_OK) return r;
-    c->J.aos = true;  // the force's vector-Jacobian product reads the float4 j-stream
     const size_t nd = static_cast<size_t>(n);
     const size_t npad = static_cast<size_t>(c->n_pad);
-    const int64_t n_ck = steps / checkpoint_every + 1;
-    const size_t state_doubles = 12 * nd;  // x, v, a, k (contiguous after m)
     double *ck = nullptr, *seg = nullptr, *gbuf = nullptr, *lval = nullptr, *dloss = nullptr, *vjp = nullptr;
     float4 *g4 = nullptr;
     DiffGrads G{};
@@ -432,27 +430,78 @@ int rollout_impl(const char *who, int64_t n, const double *m, const double *x0, 
         }
         return NBODY_OK;
     };
-    if (!backward) {
-        NB_DR(iota_launch(c->act_force, n, s, L), "index kernel");
-        for (int64_t k = 0; k < steps; ++k) {
-            r = predict_internal(c, k + 1);
-            if (r == NBODY_OK) r = force_internal(c, n);
-            if (r == NBODY_OK) r = correct_internal(c, c->act_force, n, c->f_acc, c->f_jerk);
-            if (r != NBODY_OK) return done(r);
+    double *xvak = c->state + nd;  // x[3], v[3], a[3], k[3]
+    const size_t state_doubles = 12 * nd;
+    NB_DR(iota_launch(c->act_force, n, s, L), "index kernel");
+    const bool packed = force_reads_device_rows(c->p.mode);
+    // `count` shared steps from the state at `first`; state k + 1 goes to dst(k).  In the packed modes the
+    // kernel that ends a step also predicts the next one; the others go through the context's own state.
+    auto run = [&](const double *first, int64_t count, auto &&dst) -> int {
+        if (count <= 0) return NBODY_OK;
+        if (first != xvak)
+            NB_CUDA(cudaMemcpyAsync(xvak, first, state_doubles * sizeof(double), cudaMemcpyDeviceToDevice, s), "state copy");
+        NB_CUDA(cudaMemsetAsync(c->t, 0, nd * sizeof(int64_t), s), "memset");  // the steps' times are relative to `first`
+        c->t_max = 0;
+        const double *src = first;
+        for (int64_t k = 0; k < count; ++k) {
+            double *to = dst(k);
+            if (k == 0 || !packed) {
+                if (k > 0) {
+                    if (src != xvak)
+                        NB_CUDA(cudaMemcpyAsync(xvak, src, state_doubles * sizeof(double), cudaMemcpyDeviceToDevice, s),
+                                "state copy");
+                    c->t_max = 0;
+                }
+                const int rr = predict_internal(c, 1);
+                if (rr != NBODY_OK) return rr;
+            }
+            ForceConfig cfg{};
+            const bool parts = packed && force_choose(c->p.mode, n, c->n_pad, c->sm_count, 0, 0, 0, &cfg, 0, n) == NBODY_OK &&
+                               cfg.sym_sb == 0 && cfg.split > 1;
+            if (parts) {
+                const int rr = ensure_partials(c, force_partial_bytes(c->p.mode, cfg, n));
+                if (rr != NBODY_OK) return rr;
+                NB_CUDA(force_launch(c->p.mode, c->J, n, c->act_force, n, c->eps2, cfg, c->f_acc, c->f_jerk, c->f_pot,
+                                     c->partials, c->st, s, L, nullptr, false),
+                        "force kernel launch");
+            } else {
+                const int rr = force_internal(c, n);
+                if (rr != NBODY_OK) return rr;
+            }
+            NB_CUDA(roll_step_launch(src, to, n, c->f_acc, c->f_jerk, parts ? static_cast<float *>(c->partials) : nullptr,
+                                     cfg.split, two_word_sums(c->p.mode), level, packed && k + 1 < count, c->J, c->st, s, L),
+                    "step kernel");
+            src = to;
         }
-        r = copy_final();
+        return NBODY_OK;
+    };
+    if (!backward) {
+        r = run(xvak, steps, [&](int64_t) { return xvak; });
+        if (r == NBODY_OK) r = copy_final();
         if (r == NBODY_OK) r = sync_and_check(c);
         return done(r);
     }
+    // Every state is kept where kRollKeep holds them; else checkpoints every checkpoint_every steps, and the
+    // steps of a segment run again before its backward sweep.  The same bits either way.
+    bool keep = static_cast<double>(steps) * state_doubles * sizeof(double) <= static_cast<double>(kRollKeep);
+    if (keep && dev_alloc(reinterpret_cast<void **>(&seg), std::max<int64_t>(steps, 1) * state_doubles * sizeof(double)) !=
+                    cudaSuccess) {
+        cudaGetLastError();
+        seg = nullptr;
+        keep = false;
+    }
+    const int64_t seg_len = keep ? std::max<int64_t>(steps, 1) : checkpoint_every;
+    const int64_t n_ck = keep ? 1 : steps / seg_len + 1;
+    if (!keep)
+        NB_DR(dev_alloc(reinterpret_cast<void **>(&seg), seg_len * state_doubles * sizeof(double)), "segment");
     NB_DR(dev_alloc(reinterpret_cast<void **>(&ck), n_ck * state_doubles * sizeof(double)), "checkpoints");
-    NB_DR(dev_alloc(reinterpret_cast<void **>(&seg), checkpoint_every * state_doubles * sizeof(double)), "segment");
     NB_DR(dev_alloc(reinterpret_cast<void **>(&gbuf), 19 * nd * sizeof(double)), "gradients");
     NB_DR(dev_alloc(reinterpret_cast<void **>(&lval), nd * sizeof(double)), "loss terms");
     NB_DR(dev_alloc(reinterpret_cast<void **>(&dloss), sizeof(double)), "loss");
     NB_DR(dev_alloc(reinterpret_cast<void **>(&g4), 2 * npad * sizeof(float4)), "force upstream");
     const size_t vjp_doubles = std::max(vjp_scratch_doubles(n, c->n_pad, c->sm_count),
                                         seed_loss ? loss_scratch_doubles(n, c->sm_count) : size_t(0));
-    if (vjp_doubles) NB_DR(dev_alloc(reinterpret_cast<void **>(&vjp), vjp_doubles * sizeof(double)), "adjoint scratch");
+    NB_DR(dev_alloc(reinterpret_cast<void **>(&vjp), vjp_doubles * sizeof(double)), "adjoint scratch");
     NB_DR(cudaMemsetAsync(gbuf, 0, 19 * nd * sizeof(double), s), "memset");
     NB_DR(cudaMemsetAsync(g4, 0, 2 * npad * sizeof(float4), s), "memset");
     for (int q = 0; q < 3; ++q) {
@@ -466,31 +515,26 @@ int rollout_impl(const char *who, int64_t n, const double *m, const double *x0, 
     G.gm = gbuf + 18 * nd;
     G.gA = g4;
     G.gK = g4 + npad;
-    double *xvak = c->state + nd;  // x[3], v[3], a[3], k[3]
-    NB_DR(iota_launch(c->act_force, n, s, L), "index kernel");
-    // one shared Hermite step from tick s0 to s0 + 1 (all particles in the block)
-    auto step = [&](int64_t s0) -> int {
-        int rr = predict_internal(c, s0 + 1);
-        if (rr != NBODY_OK) return rr;
-        rr = force_internal(c, n);
-        if (rr != NBODY_OK) return rr;
-        return correct_internal(c, c->act_force, n, c->f_acc, c->f_jerk);
-    };
-    auto restore = [&](const double *src, int64_t tick) -> int {
-        NB_CUDA(cudaMemcpyAsync(xvak, src, state_doubles * sizeof(double), cudaMemcpyDeviceToDevice, s), "restore");
-        NB_CUDA(set_time_launch(c->S, tick, level, s, L), "time kernel");
-        c->t_max = tick;
+    auto seg_state = [&](int64_t k) { return seg + k * state_doubles; };  // k within the segment
+    auto copy_state = [&](double *to, const double *from) -> int {
+        NB_CUDA(cudaMemcpyAsync(to, from, state_doubles * sizeof(double), cudaMemcpyDeviceToDevice, s), "state copy");
         return NBODY_OK;
     };
-    // forward with checkpoints
-    NB_DR(cudaMemcpyAsync(ck, xvak, state_doubles * sizeof(double), cudaMemcpyDeviceToDevice, s), "checkpoint");
-    for (int64_t k = 0; k < steps; ++k) {
-        r = step(k);
+    // forward: the final state in the context's
+    r = copy_state(ck, xvak);
+    if (r != NBODY_OK) return done(r);
+    if (keep) {
+        r = copy_state(seg, xvak);
+        if (r == NBODY_OK)
+            r = run(seg, steps, [&](int64_t k) { return k + 1 < steps ? seg_state(k + 1) : xvak; });
         if (r != NBODY_OK) return done(r);
-        if ((k + 1) % checkpoint_every == 0)
-            NB_DR(cudaMemcpyAsync(ck + ((k + 1) / checkpoint_every) * state_doubles, xvak,
-                                  state_doubles * sizeof(double), cudaMemcpyDeviceToDevice, s),
-                  "checkpoint");
+    } else {
+        for (int64_t k0 = 0; k0 < steps; k0 += seg_len) {
+            const int64_t count = std::min(seg_len, steps - k0);
+            r = run(xvak, count, [&](int64_t) { return xvak; });
+            if (r == NBODY_OK && (k0 + count) % seg_len == 0) r = copy_state(ck + (k0 + count) / seg_len * state_doubles, xvak);
+            if (r != NBODY_OK) return done(r);
+        }
     }
     r = copy_final();  // before the backward sweep overwrites the state
     if (r != NBODY_OK) return done(r);
@@ -506,38 +550,24 @@ int rollout_impl(const char *who, int64_t n, const double *m, const double *x0, 
             NB_DR(aos_to_soa_launch(c->stage + 3 * nd, G.gv[0], G.gv[1], G.gv[2], n, s, L), "layout kernel");
         }
     }
-    // backward, one checkpoint segment at a time
-    for (int64_t seg0 = (steps - 1) / checkpoint_every * checkpoint_every; steps > 0 && seg0 >= 0;
-         seg0 -= checkpoint_every) {
-        const int64_t seg1 = std::min(seg0 + checkpoint_every, steps);
-        r = restore(ck + (seg0 / checkpoint_every) * state_doubles, seg0);
-        if (r != NBODY_OK) return done(r);
-        for (int64_t k = seg0; k < seg1; ++k) {
-            NB_DR(cudaMemcpyAsync(seg + (k - seg0) * state_doubles, xvak, state_doubles * sizeof(double),
-                                  cudaMemcpyDeviceToDevice, s),
-                  "segment");
-            if (k + 1 < seg1) {
-                r = step(k);
-                if (r != NBODY_OK) return done(r);
-            }
+    // backward, one segment at a time
+    int ranges = 0;  // of the last force adjoint (0: none yet)
+    for (int64_t seg0 = steps > 0 ? (steps - 1) / seg_len * seg_len : -1; seg0 >= 0; seg0 -= seg_len) {
+        const int64_t count = std::min(seg_len, steps - seg0);
+        if (!keep) {
+            r = copy_state(seg, ck + seg0 / seg_len * state_doubles);
+            if (r == NBODY_OK) r = run(seg, count - 1, [&](int64_t k) { return seg_state(k + 1); });
+            if (r != NBODY_OK) return done(r);
         }
-        for (int64_t k = seg1 - 1; k >= seg0; --k) {
-            r = restore(seg + (k - seg0) * state_doubles, k);
-            if (r != NBODY_OK) return done(r);
-            r = predict_internal(c, k + 1);  // j-stream at the predicted state of step k
-            if (r != NBODY_OK) return done(r);
-            NB_DR(adj_correct_launch(G, n, dt, s, L), "adjoint corrector");
-            NB_DR(force_vjp_launch(c->J, G, n, e2, c->sm_count, vjp, s, L), "force adjoint");
-            NB_DR(adj_predict_launch(G, n, dt, s, L), "adjoint predictor");
+        for (int64_t k = count - 1; k >= 0; --k) {
+            NB_DR(adj_step_launch(vjp, ranges, G, n, dt, true, seg_state(k), c->J, s, L), "adjoint step");
+            NB_DR(force_vjp_launch(c->J, G, n, e2, c->sm_count, vjp, &ranges, s, L), "force adjoint");
         }
     }
     // the t = 0 force
-    r = restore(ck, 0);
-    if (r != NBODY_OK) return done(r);
-    r = predict_internal(c, 0);
-    if (r != NBODY_OK) return done(r);
-    NB_DR(adj_init_launch(G, n, s, L), "adjoint init");
-    NB_DR(force_vjp_launch(c->J, G, n, e2, c->sm_count, vjp, s, L), "force adjoint");
+    NB_DR(adj_step_launch(vjp, ranges, G, n, dt, false, ck, c->J, s, L), "adjoint step");
+    NB_DR(force_vjp_launch(c->J, G, n, e2, c->sm_count, vjp, &ranges, s, L), "force adjoint");
+    NB_DR(vjp_finish_launch(G, n, vjp, ranges, s, L), "adjoint reduction");
     if (seed_loss && loss) NB_DR(cudaMemcpyAsync(loss, dloss, sizeof(double), cudaMemcpyDefault, s), "loss copy");
     if (g_x0) {
         NB_DR(soa_to_aos_launch(G.gxp[0], G.gxp[1], G.gxp[2], c->stage, n, s, L), "layout");

@@ -304,17 +304,27 @@ struct DiffGrads {
     double *gm;                             // gradient of the masses
     float4 *gA, *gK;                        // upstream of the force (n_pad, zero padded)
 };
-// Doubles of scratch the force VJP needs for its j-range partial sums (0: none).
+// (each of gx .. gvp three contiguous arrays of n)
+// Doubles of scratch the force VJP needs for its j-range totals.
 size_t vjp_scratch_doubles(int64_t n, int64_t n_pad, int sm_count);
+// The force's vector-Jacobian product: totals of *ranges ranges to scratch, for adj_step_launch
+// (`after`) or vjp_finish_launch, which adds them to gxp, gvp and gm.
 cudaError_t force_vjp_launch(const JStream &J, const DiffGrads &G, int64_t n, float eps2, int sm_count,
-                             double *scratch, cudaStream_t s, int64_t *launches);
-cudaError_t adj_correct_launch(const DiffGrads &G, int64_t n, double dt, cudaStream_t s, int64_t *launches);
-cudaError_t adj_predict_launch(const DiffGrads &G, int64_t n, double dt, cudaStream_t s, int64_t *launches);
-cudaError_t adj_init_launch(const DiffGrads &G, int64_t n, cudaStream_t s, int64_t *launches);
+                             double *scratch, int *ranges, cudaStream_t s, int64_t *launches);
+cudaError_t vjp_finish_launch(const DiffGrads &G, int64_t n, const double *scratch, int ranges, cudaStream_t s,
+                              int64_t *launches);
+// Ends a shared step of 2^-level (state at src -> state at dst, x[3], v[3], a[3], k[3] of n doubles
+// each) with the force in part ([split][7 or 14][n] partial sums; two_word: hi and lo) or in acc and
+// jerk, and predicts the j-stream of the next one.
+cudaError_t roll_step_launch(const double *src, double *dst, int64_t n, const double *acc, const double *jerk,
+                             const float *part, int split, bool two_word, int level, bool predict, const JStream &J,
+                             DevStatus *st, cudaStream_t s, int64_t *launches);
+// From one force VJP to the next of the backward sweep (see adj_step_kernel).
+cudaError_t adj_step_launch(const double *scratch, int after, const DiffGrads &G, int64_t n, double dt, bool corrector,
+                            const double *src, const JStream &J, cudaStream_t s, int64_t *launches);
 size_t loss_scratch_doubles(int64_t n, int sm_count);
 cudaError_t loss_launch(const State &S, double eps2, const DiffGrads &G, int sm_count, double *scratch, double *lval,
                         double *loss, cudaStream_t s, int64_t *launches);
-cudaError_t set_time_launch(const State &S, int64_t tick, int level, cudaStream_t s, int64_t *launches);
 
 // Row-major n x 3 <-> three component arrays.
 cudaError_t aos_to_soa_launch(const double *aos, double *c0, double *c1, double *c2, int64_t n,

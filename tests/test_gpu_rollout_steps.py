@@ -1,0 +1,69 @@
+"""The fused steps of a shared-step rollout (csrc/adjoint.cu) against the library's own block-step calls."""
+import numpy as np
+import pytest
+
+from synthetic import plummer_sphere
+from tests.gpu_common import need_gpu
+
+pytestmark = pytest.mark.gpu
+EPS2, LEVEL = (1.0 / 128) ** 2, 9
+
+
+# one particle, blocks of 32 (component, particle) threads and their edges, several j-ranges, pairs (8192)
+@pytest.mark.parametrize("n,mode", [(1, "plain"), (2, "comp"), (11, "plain"), (33, "comp"), (257, "plain"), (1500, "comp"),
+                                    (8191, "plain"), (8192, "comp"), (20000, "plain"), (300, "ds"), (300, "sumcheck"),
+                                    (100, "sorted")])
+def test_rollout_equals_block_steps(n, mode):
+    """x_T and v_T of three steps against predict, force and correct called one by one.  Both add the same FP32
+    partial sums; only the order of the last additions (to ~2^-48) may differ, so x and v agree to ~1e-13."""
+    need_gpu()
+    from paper_astro_ph_0702058_gb300 import MODES, Simulation
+    from paper_astro_ph_0702058_gb300._lib import nbody_rollout
+    m, x, v = plummer_sphere(n, 50 + n)
+    xT, vT = np.zeros((n, 3)), np.zeros((n, 3))
+    nbody_rollout(n, m, x, v, EPS2, LEVEL, 3, MODES[mode], xT, vT)
+    every = np.arange(n, dtype=np.int32)
+    with Simulation(m, x, v, EPS2, lmin=LEVEL, lmax=LEVEL, mode=mode) as sim:
+        for k in range(3):
+            sim.predict((k + 1) * 2.0 ** -LEVEL)
+            sim.force(every)
+            sim.correct(every)
+        s = {k: np.zeros((n, 3)) for k in ("x", "v")}
+        sim.get_state(**s)
+    np.testing.assert_allclose(xT, s["x"], rtol=0, atol=1e-13 * np.abs(s["x"]).max())
+    np.testing.assert_allclose(vT, s["v"], rtol=0, atol=1e-12 * max(np.abs(s["v"]).max(), 1e-30))
+
+
+@pytest.mark.parametrize("steps", [0, 1])
+def test_shortest_rollouts(steps):
+    need_gpu()
+    from paper_astro_ph_0702058_gb300._lib import nbody_rollout_vjp
+    n = 40
+    m, x, v = plummer_sphere(n, 9)
+    g = np.random.default_rng(1).standard_normal((2, n, 3))
+    out = [np.zeros((n, 3)), np.zeros((n, 3)), np.zeros(n)]
+    nbody_rollout_vjp(n, m, x, v, EPS2, LEVEL, steps, 16, 0, g[0], g[1], *out)
+    from oracle import adjoint
+    dt = 2.0 ** -LEVEL
+    ref = adjoint.rollout_vjp(m, x, v, EPS2, dt, steps, g[0], g[1])[2:]
+    # The force adjoint runs at FP32 positions: a separation is off by 2^-24 (|x_i| + |x_j|), which moves
+    # da/dx by at most 6 m / eps^4 of it, and the step weighs the force by ~dt^2 (x) of the cotangents; twice that
+    # for the jerk's part and the two forces of a step.
+    tol = 2 * 2.0 ** -24 * 2 * np.abs(x).max() * dt ** 2 * 6 * m.max() / EPS2 ** 2 * np.abs(g).max()
+    for o, r in zip(out, ref):
+        np.testing.assert_allclose(o, r, rtol=0, atol=tol)
+
+
+def test_segments_where_the_states_are_too_many_to_keep():
+    """20000 particles x 600 steps are 1.15 GB of states: segments run again, their length without effect."""
+    need_gpu()
+    from paper_astro_ph_0702058_gb300._lib import nbody_rollout_vjp
+    n, steps = 20000, 600
+    m, x, v = plummer_sphere(n, 10)
+    g = np.random.default_rng(2).standard_normal((2, n, 3))
+    out = []
+    for every in (16, 50):
+        out.append([np.zeros((n, 3)), np.zeros((n, 3)), np.zeros(n)])
+        nbody_rollout_vjp(n, m, x, v, EPS2, LEVEL, steps, every, 0, g[0], g[1], *out[-1])
+    for a, b in zip(*out):
+        assert np.all(np.isfinite(a)) and np.array_equal(a, b)
