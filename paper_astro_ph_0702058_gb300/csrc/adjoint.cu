@@ -12,123 +12,296 @@
 // upstream gradients of particle i's acceleration and jerk.  For one particle
 // p both of its roles combine linearly: with G_a = m_p g_a,q - m_q g_a,p and
 // G_k likewise, one evaluation per pair (p, q) gives p's position and
-// velocity gradients.
+// velocity gradients, and minus them q's.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
-#include "force_impl.cuh"  // fold_ds_rn; nbody_internal.cuh, ptx.cuh
+#include "force_x2.cuh"  // packed FP32; fold_ds_rn, ds2_add
 #include "step_impl.cuh"
 
 namespace nb {
 
 namespace {
 
-constexpr int kVjpThreads = 128;
-constexpr int kVjpTile = 128;
+constexpr int kVjpRows = 64;  // rows of a warp
 
-// grid (i-blocks, j-ranges): block (x, y) takes the particles p of i-block x
-// against the j-tiles of range y and writes its totals to part[y][7][n]; the
-// kernel that follows adds the ranges in ascending order (deterministic).
-__global__ void __launch_bounds__(kVjpThreads)
-    force_vjp_kernel(const float4 *__restrict__ posm, const float4 *__restrict__ vel,
-                     const float4 *__restrict__ gA, const float4 *__restrict__ gK, int n, int n_pad, float eps2,
-                     int tiles_per_range, double *__restrict__ part)
+// Sums of a pair that both of its particles need.  Row data packed for two rows
+// (force_x2.cuh's packed FP32), the j's values twice.
+struct VjpRow {
+    f2_t x[3], m, v[3], a[3], k[3];  // position, mass, velocity, upstream of acceleration and jerk
+};
+struct VjpSum {
+    f2_t x[3], v[3], m;
+};
+
+__device__ __forceinline__ f2_t dot3(const f2_t (&a)[3], const f2_t (&b)[3])
 {
-    __shared__ float4 sp[kVjpTile], sv[kVjpTile], sa[kVjpTile], sk[kVjpTile];
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    const int pl = p < n ? p : 0;
-    const float4 xi = posm[pl], vi = vel[pl], ga = gA[pl], gk = gK[pl];
-    const float mp = xi.w;
-    // running totals over the tiles as double-single pairs on the FP32 pipe (fold_ds_rn;
-    // GB300's FP64 unit takes ~19 cycles per warp instruction), hi + lo in FP64 at the end
-    float hx[3] = {0, 0, 0}, lx[3] = {0, 0, 0}, hv[3] = {0, 0, 0}, lv[3] = {0, 0, 0}, hm = 0.f, lm = 0.f;
-    const int j_begin = blockIdx.y * tiles_per_range * kVjpTile;
-    const int j_end = min(j_begin + tiles_per_range * kVjpTile, n_pad);
-    for (int j0 = j_begin; j0 < j_end; j0 += kVjpTile) {
-        __syncthreads();
-        for (int t = threadIdx.x; t < kVjpTile; t += blockDim.x) {
-            sp[t] = posm[j0 + t];
-            sv[t] = vel[j0 + t];
-            sa[t] = gA[j0 + t];
-            sk[t] = gK[j0 + t];
+    return f2_fma(a[2], b[2], f2_fma(a[1], b[1], f2_mul(a[0], b[0])));
+}
+
+// The pair (p, q): p's share to P, q's to Q.  Exchanging p and q turns d, e, G_a
+// and G_k over, so the position and velocity gradients of q are minus p's; the
+// mass gradients take the other particle's upstream each.
+template <bool DIAG>
+__device__ __forceinline__ void vjp_pair(const VjpRow &p, const VjpRow &q, const f2_t E2, const bool ma, const bool mb,
+                                         VjpSum &P, VjpSum &Q)
+{
+    f2_t d[3], e[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        d[c] = f2_sub(p.x[c], q.x[c]);
+        e[c] = f2_sub(p.v[c], q.v[c]);
+    }
+    const f2_t r2 = f2_fma(d[2], d[2], f2_fma(d[1], d[1], f2_fma(d[0], d[0], E2)));
+    float a, b;
+    f2_unpack(r2, a, b);
+    if (DIAG) {  // pairs to leave out: r^-1 = 0
+        a = ma ? INFINITY : a;
+        b = mb ? INFINITY : b;
+    }
+    const f2_t R = f2_pack(rsqrt_mufu(a), rsqrt_mufu(b));
+    const f2_t R2 = f2_mul(R, R), R3 = f2_mul(R2, R);
+    const f2_t t5 = f2_mul(f2_mul(R3, R2), f2_pack(-3.0f, -3.0f));  // -3 R^5
+    const f2_t de = dot3(d, e);
+    const f2_t aq = dot3(d, q.a), ap = dot3(d, p.a), bq = dot3(e, q.k), bp = dot3(e, p.k);
+    const f2_t cq = dot3(d, q.k), cp = dot3(d, p.k);
+    const f2_t nmq = f2_sub(0ull, q.m);
+    const f2_t sq = f2_add(aq, bq), sp = f2_add(ap, bp);
+    const f2_t dAeK = f2_fma(nmq, sp, f2_mul(p.m, sq));  // d.G_a + e.G_k
+    const f2_t dK = f2_fma(nmq, cp, f2_mul(p.m, cq));
+    const f2_t cg = f2_mul(t5, de), ce = f2_mul(t5, dK);
+    const f2_t w = f2_mul(f2_mul(R2, cg), f2_pack(-5.0f, -5.0f));  // 15 R^7 (d.e)
+    const f2_t cd = f2_fma(w, dK, f2_mul(t5, dAeK));
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const f2_t A = f2_fma(nmq, p.a[c], f2_mul(p.m, q.a[c])), K = f2_fma(nmq, p.k[c], f2_mul(p.m, q.k[c]));
+        const f2_t gx = f2_fma(cg, K, f2_fma(ce, e[c], f2_fma(cd, d[c], f2_mul(R3, A))));
+        const f2_t gv = f2_fma(ce, d[c], f2_mul(R3, K));
+        P.x[c] = f2_add(P.x[c], gx);
+        Q.x[c] = f2_sub(Q.x[c], gx);
+        P.v[c] = f2_add(P.v[c], gv);
+        Q.v[c] = f2_sub(Q.v[c], gv);
+    }
+    P.m = f2_fma(R3, sq, f2_fma(cg, cq, P.m));
+    Q.m = f2_sub(Q.m, f2_fma(R3, sp, f2_mul(cg, cp)));
+}
+
+__device__ __forceinline__ f2_t &vjp_at(VjpSum &s, const int c) { return c < 3 ? s.x[c] : c < 6 ? s.v[c - 3] : s.m; }
+
+// Adds x to the total of component c at p (component stride n): FP32 where a slot
+// holds one sum of 64 terms, else a double-single pair (lo words 7 further on).
+template <bool FOLD>
+__device__ __forceinline__ void vjp_fold(float *p, const size_t n, const int c, const float x, const bool first)
+{
+    float *h = p + static_cast<size_t>(c) * n;
+    if (!FOLD) {
+        *h = x;
+        return;
+    }
+    float *l = p + static_cast<size_t>(7 + c) * n;
+    float hi = first ? 0.0f : *h, lo = first ? 0.0f : *l;
+    fold_ds_rn(hi, lo, x);
+    *h = hi;
+    *l = lo;
+}
+
+// Force adjoint by unordered pairs: the structure of force_sym_kernel
+// (force_sym.cuh) with one warp per CTA and 64 rows per warp.  Superblocks of 64
+// (FOLD: 64 x tiles) rows; one CTA per unordered pair (I, J) of them and per
+// j-part h of H (H = 2: the two halves of J's 64, FOLD: J whole, H = 1).  Lane l
+// holds rows l and l + 32 of a packed pair and takes j = (l + s) mod 32 in step s;
+// the j's sums go down one lane per step.  Slots of part: rows of I in J H + h,
+// those of J in I H, the second side of (I, I) in S H.
+// One pair costs 96 packed FP32 operations for both particles, 40 of them with
+// three different registers (3 cycles each, not 2: force_sym.cuh), where the
+// one-sided scalar loop took about 85 per particle: n = 4096 59.8 -> 41.2 us,
+// 1500 12.8 -> 9.0 us.
+template <int H, bool FOLD>
+__global__ void __launch_bounds__(32, 12)
+    vjp_pairs_kernel(const float4 *__restrict__ posm, const float4 *__restrict__ vel, const float4 *__restrict__ gA,
+                     const float4 *__restrict__ gK, const int n, const float eps2, const int S, const int tiles,
+                     float *__restrict__ part)
+{
+    static_assert(!FOLD || H == 1, "tiles of a superblock whole");
+    constexpr int NC = FOLD ? 14 : 7;
+    __shared__ float4 sj[4][32];
+    const int lane = threadIdx.x;
+    const int u = blockIdx.x / H, h = blockIdx.x % H;
+    int J = static_cast<int>((sqrtf(8.0f * u + 1.0f) - 1.0f) * 0.5f);
+    while ((J + 1) * (J + 2) / 2 <= u) ++J;
+    while (J * (J + 1) / 2 > u) --J;
+    const int I = u - J * (J + 1) / 2;
+    const bool diag = I == J;
+    const size_t slot = static_cast<size_t>(NC) * n;
+    float *pi_out = part + slot * (J * H + h), *pj_out = part + slot * (diag ? S * H : I * H);
+    const int sb = tiles * kVjpRows;
+    const int j_end = min(n, (J + 1) * sb);
+    const f2_t E2 = f2_pack(eps2, eps2);
+    const float4 far = make_float4(kPadPosition, kPadPosition, kPadPosition, 0.f), zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i0 = I * sb; i0 < min(n, (I + 1) * sb); i0 += kVjpRows) {
+        const int r0 = i0 + lane, r1 = r0 + 32;
+        VjpRow p;
+        {
+            const float4 x0 = r0 < n ? posm[r0] : far, x1 = r1 < n ? posm[r1] : far;
+            const float4 v0 = r0 < n ? vel[r0] : zero, v1 = r1 < n ? vel[r1] : zero;
+            const float4 a0 = r0 < n ? gA[r0] : zero, a1 = r1 < n ? gA[r1] : zero;
+            const float4 k0 = r0 < n ? gK[r0] : zero, k1 = r1 < n ? gK[r1] : zero;
+            p.x[0] = f2_pack(x0.x, x1.x);
+            p.x[1] = f2_pack(x0.y, x1.y);
+            p.x[2] = f2_pack(x0.z, x1.z);
+            p.m = f2_pack(x0.w, x1.w);
+            p.v[0] = f2_pack(v0.x, v1.x);
+            p.v[1] = f2_pack(v0.y, v1.y);
+            p.v[2] = f2_pack(v0.z, v1.z);
+            p.a[0] = f2_pack(a0.x, a1.x);
+            p.a[1] = f2_pack(a0.y, a1.y);
+            p.a[2] = f2_pack(a0.z, a1.z);
+            p.k[0] = f2_pack(k0.x, k1.x);
+            p.k[1] = f2_pack(k0.y, k1.y);
+            p.k[2] = f2_pack(k0.z, k1.z);
         }
-        __syncthreads();
-        float px[3] = {0, 0, 0}, pv[3] = {0, 0, 0}, pm = 0.f;
+        bool ifirst = true;
+        for (int t0 = diag ? i0 : J * sb; t0 < j_end; t0 += kVjpRows) {  // a tile of 64 j
+            VjpSum P;
+#pragma unroll
+            for (int c = 0; c < 7; ++c) vjp_at(P, c) = 0ull;
+            for (int j0 = t0 + 32 * h; j0 < min(j_end, H == 2 ? t0 + 32 * h + 32 : t0 + 64); j0 += 32) {
+                __syncwarp();
+                const int j = j0 + lane;
+                sj[0][lane] = j < n ? posm[j] : far;
+                sj[1][lane] = j < n ? vel[j] : zero;
+                sj[2][lane] = j < n ? gA[j] : zero;
+                sj[3][lane] = j < n ? gK[j] : zero;
+                __syncwarp();
+                VjpSum Q;
+#pragma unroll
+                for (int c = 0; c < 7; ++c) vjp_at(Q, c) = 0ull;
+                auto turn = [&](auto own) {
+#pragma unroll 1
+                    for (int s = 0; s < 32; ++s) {
+                        const int jl = (lane + s) & 31;
+                        const float4 x = sj[0][jl], v = sj[1][jl], a = sj[2][jl], k = sj[3][jl];
+                        VjpRow q;
+                        q.x[0] = f2_pack(x.x, x.x);
+                        q.x[1] = f2_pack(x.y, x.y);
+                        q.x[2] = f2_pack(x.z, x.z);
+                        q.m = f2_pack(x.w, x.w);
+                        q.v[0] = f2_pack(v.x, v.x);
+                        q.v[1] = f2_pack(v.y, v.y);
+                        q.v[2] = f2_pack(v.z, v.z);
+                        q.a[0] = f2_pack(a.x, a.x);
+                        q.a[1] = f2_pack(a.y, a.y);
+                        q.a[2] = f2_pack(a.z, a.z);
+                        q.k[0] = f2_pack(k.x, k.x);
+                        q.k[1] = f2_pack(k.y, k.y);
+                        q.k[2] = f2_pack(k.z, k.z);
+                        constexpr bool OWN = decltype(own)::value;
+                        vjp_pair<OWN>(p, q, E2, OWN && j0 + jl <= r0, OWN && j0 + jl <= r1, P, Q);
+#pragma unroll
+                        for (int c = 0; c < 7; ++c) {
+                            float a0, a1;
+                            f2_unpack(vjp_at(Q, c), a0, a1);
+                            a0 = __shfl_sync(0xffffffffu, a0, (lane + 1) & 31);
+                            a1 = __shfl_sync(0xffffffffu, a1, (lane + 1) & 31);
+                            vjp_at(Q, c) = f2_pack(a0, a1);
+                        }
+                    }
+                };
+                if (diag && t0 == i0)
+                    turn(std::true_type());
+                else
+                    turn(std::false_type());
+                if (j < j_end) {
+#pragma unroll
+                    for (int c = 0; c < 7; ++c) {
+                        float a0, a1;
+                        f2_unpack(vjp_at(Q, c), a0, a1);
+                        vjp_fold<FOLD>(pj_out + j, n, c, a0 + a1, i0 == I * sb);
+                    }
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < 7; ++c) {
+                float a0, a1;
+                f2_unpack(vjp_at(P, c), a0, a1);
+                if (r0 < n) vjp_fold<FOLD>(pi_out + r0, n, c, a0, ifirst);
+                if (r1 < n) vjp_fold<FOLD>(pi_out + r1, n, c, a1, ifirst);
+            }
+            ifirst = false;
+        }
+    }
+}
+
+// The per-(component, particle) kernels: blocks of 32 columns (a warp's width of
+// one component's particles) x kLanes warps.  The sums over slots or j-ranges of
+// a column are spread over the warps (warp w takes w, w + kLanes, ...), added in
+// double-single and then in warp order; warp 0 goes on alone with the column's
+// FP64 work.  One thread per column instead took 45 us (65 slots) and 20 us (16
+// ranges) at n = 4096, nearly all of it the latency of its own loads.
+constexpr int kLanes = 8;
+
+// Sums of NV values over count of them per column: at(s, v, hi, lo) loads value v
+// of entry s.  Every thread of the block calls; warp 0 gets the sums.
+template <int NV, class At>
+__device__ __forceinline__ void column_sums(const int count, At &&at, double (&sum)[NV])
+{
+    __shared__ float2 sh[NV][kLanes][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    float h[NV], l[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) h[v] = l[v] = 0.0f;
 #pragma unroll 4
-        for (int t = 0; t < kVjpTile; ++t) {
-            const float4 xq = sp[t], vq = sv[t], gaq = sa[t], gkq = sk[t];
-            const float mq = xq.w;
-            const float d0 = xi.x - xq.x, d1 = xi.y - xq.y, d2 = xi.z - xq.z;  // d = x_p - x_q
-            const float e0 = vi.x - vq.x, e1 = vi.y - vq.y, e2 = vi.z - vq.z;
-            const float r2 = fmaf(d2, d2, fmaf(d1, d1, fmaf(d0, d0, eps2)));
-            const float R = rsqrt_mufu(r2);
-            const float R2 = R * R, R3 = R2 * R, R5 = R3 * R2, R7 = R5 * R2;
-            const float A0 = fmaf(-mq, ga.x, mp * gaq.x), A1 = fmaf(-mq, ga.y, mp * gaq.y),
-                        A2 = fmaf(-mq, ga.z, mp * gaq.z);
-            const float K0 = fmaf(-mq, gk.x, mp * gkq.x), K1 = fmaf(-mq, gk.y, mp * gkq.y),
-                        K2 = fmaf(-mq, gk.z, mp * gkq.z);
-            const float dA = fmaf(d2, A2, fmaf(d1, A1, d0 * A0));
-            const float eK = fmaf(e2, K2, fmaf(e1, K1, e0 * K0));
-            const float dK = fmaf(d2, K2, fmaf(d1, K1, d0 * K0));
-            const float de = fmaf(d2, e2, fmaf(d1, e1, d0 * e0));
-            const float cd = fmaf(15.0f * R7 * de, dK, -3.0f * R5 * (dA + eK));
-            const float ce = -3.0f * R5 * dK;
-            const float cg = -3.0f * R5 * de;
-            px[0] += fmaf(cg, K0, fmaf(ce, e0, fmaf(cd, d0, R3 * A0)));
-            px[1] += fmaf(cg, K1, fmaf(ce, e1, fmaf(cd, d1, R3 * A1)));
-            px[2] += fmaf(cg, K2, fmaf(ce, e2, fmaf(cd, d2, R3 * A2)));
-            pv[0] += fmaf(ce, d0, R3 * K0);
-            pv[1] += fmaf(ce, d1, R3 * K1);
-            pv[2] += fmaf(ce, d2, R3 * K2);
-            // p as the source of q's force: d . g_a,q etc.
-            const float dga = fmaf(d2, gaq.z, fmaf(d1, gaq.y, d0 * gaq.x));
-            const float egk = fmaf(e2, gkq.z, fmaf(e1, gkq.y, e0 * gkq.x));
-            const float dgk = fmaf(d2, gkq.z, fmaf(d1, gkq.y, d0 * gkq.x));
-            pm += fmaf(R3, dga + egk, -3.0f * R5 * de * dgk);
+    for (int s = w; s < count; s += kLanes)
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            float a = 0.0f, b = 0.0f;
+            at(s, v, a, b);
+            ds2_add(h[v], l[v], a, b);
         }
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            fold_ds_rn(hx[c], lx[c], px[c]);
-            fold_ds_rn(hv[c], lv[c], pv[c]);
+    for (int v = 0; v < NV; ++v) sh[v][w][lane] = make_float2(h[v], l[v]);
+    __syncthreads();
+    if (w == 0)
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+#pragma unroll
+            for (int k = 1; k < kLanes; ++k) ds2_add(h[v], l[v], sh[v][k][lane].x, sh[v][k][lane].y);
+            sum[v] = f2d(h[v]) + f2d(l[v]);
         }
-        fold_ds_rn(hm, lm, pm);
-    }
-    if (p >= n) return;
-    double tx[3], tv[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        tx[c] = static_cast<double>(hx[c]) + static_cast<double>(lx[c]);
-        tv[c] = static_cast<double>(hv[c]) + static_cast<double>(lv[c]);
-    }
-    const double tm = static_cast<double>(hm) + static_cast<double>(lm);
-    double *b = part + static_cast<size_t>(blockIdx.y) * 7 * n + p;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        b[static_cast<size_t>(c) * n] = tx[c];
-        b[static_cast<size_t>(3 + c) * n] = tv[c];
-    }
-    b[static_cast<size_t>(6) * n] = tm;
 }
 
-// One thread per (particle, component): adds the component's ranges in order.
-__global__ void vjp_reduce_kernel(const double *__restrict__ part, int ranges, int n, DiffGrads G)
+// Value of component c of particle i in slot s (zero where the slot has none).
+__device__ __forceinline__ void vjp_at_slot(const float *__restrict__ part, const VjpSlots V, const int n, const int c,
+                                            const int i, const int s, float &a, float &b)
 {
-    const int64_t idx = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-    if (idx >= 7LL * n) return;
-    const int c = static_cast<int>(idx / n);
-    const int p = static_cast<int>(idx - static_cast<int64_t>(c) * n);
-    double t = 0.0;
-    for (int y = 0; y < ranges; ++y) t += part[(static_cast<size_t>(y) * 7 + c) * n + p];
-    if (c < 3)
-        G.gxp[c][p] += t;
-    else if (c < 6)
-        G.gvp[c - 3][p] += t;
-    else
-        G.gm[p] += t;
+    if (V.parts == 2 && s < 2 * (i / V.rows) && (s & 1)) return;  // (as the j of an earlier superblock: one slot)
+    const float *p = part + (static_cast<size_t>(s) * (V.two_word ? 14 : 7) + c) * n + i;
+    a = p[0];
+    if (V.two_word) b = p[static_cast<size_t>(7) * n];
 }
 
-// One forward step's end and the next one's start, one thread per (component,
-// particle): the force on the particle (its j-range partials, or acc and jerk),
+// Adds the totals to the gradients.
+__global__ void __launch_bounds__(32 * kLanes)
+    vjp_reduce_kernel(const float *__restrict__ part, const VjpSlots V, int n, DiffGrads G)
+{
+    const int64_t idx = blockIdx.x * 32ll + (threadIdx.x & 31);
+    const bool live = idx < 7ll * n;
+    const int c = live ? static_cast<int>(idx / n) : 0;
+    const int p = live ? static_cast<int>(idx - static_cast<int64_t>(c) * n) : 0;
+    double t[1];
+    column_sums(V.sb * V.parts + 1, [&](int s, int, float &a, float &b) { vjp_at_slot(part, V, n, c, p, s, a, b); }, t);
+    if (threadIdx.x >= 32 || !live) return;
+    if (c < 3)
+        G.gxp[c][p] += t[0];
+    else if (c < 6)
+        G.gvp[c - 3][p] += t[0];
+    else
+        G.gm[p] += t[0];
+}
+
+// One forward step's end and the next one's start, per (component, particle):
+// the force on the particle (its j-range partials, or acc and jerk),
 // the corrector from the state at src to the state at dst, and (predict) the
 // j-stream at the prediction from there.  src, dst: x[3], v[3], a[3], k[3] of n
 // doubles each.  A shared step has no criterion or level, so the components are
@@ -137,26 +310,27 @@ __global__ void vjp_reduce_kernel(const double *__restrict__ part, int ranges, i
 // the reduction, the corrector, the copy of the state and the predictor
 // (n = 4096: 7.5 + 11.0 + 2 + 4.7 us before).
 template <bool DSW>
-__global__ void roll_step_kernel(const double *src, double *dst, const int n, const double *__restrict__ acc,
+__global__ void __launch_bounds__(32 * kLanes) roll_step_kernel(const double *src, double *dst, const int n, const double *__restrict__ acc,
                                  const double *__restrict__ jerk, const float *__restrict__ part, const int split,
                                  const CorrDt d, const bool predict, const JStream J, DevStatus *st)
 {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= 3 * n) return;
-    const int c = idx / n, i = idx - c * n;
+    const int idx = blockIdx.x * 32 + (threadIdx.x & 31);
+    const bool live = idx < 3 * n;
+    const int c = live ? idx / n : 0, i = live ? idx - c * n : 0;
     double ap, kp;
     if (part) {
         constexpr int NC = DSW ? 14 : 7;
-        float ah = 0.0f, al = 0.0f, kh = 0.0f, kl = 0.0f;
-        const float *b = part + static_cast<size_t>(c) * n + i;
-#pragma unroll 4
-        for (int r = 0; r < split; ++r, b += static_cast<size_t>(NC) * n) {
-            ds2_add(ah, al, b[0], DSW ? b[static_cast<size_t>(7) * n] : 0.0f);
-            ds2_add(kh, kl, b[static_cast<size_t>(3) * n], DSW ? b[static_cast<size_t>(10) * n] : 0.0f);
-        }
-        ap = f2d(ah) + f2d(al);
-        kp = f2d(kh) + f2d(kl);
-    } else {
+        double f[2];
+        column_sums(split, [&](int r, int v, float &a, float &b) {
+            const float *q = part + (static_cast<size_t>(r) * NC + 3 * v + c) * n + i;
+            a = q[0];
+            if (DSW) b = q[static_cast<size_t>(7) * n];
+        }, f);
+        ap = f[0];
+        kp = f[1];
+    }
+    if (threadIdx.x >= 32 || !live) return;
+    if (!part) {
         ap = acc[3 * static_cast<size_t>(i) + c];
         kp = jerk[3 * static_cast<size_t>(i) + c];
     }
@@ -188,9 +362,9 @@ struct AdjDt {
     PredDt pd;
 };
 
-// Between two force adjoints of the backward sweep, one thread per (component,
-// particle).  With `after` (> 0) the totals of the last one (its `after` ranges
-// of part) join the gradients of the predicted state and the masses, and the
+// Between two force adjoints of the backward sweep, per (component, particle).
+// After the first one (V.sb > 0) the totals of the last one, in the
+// slots of part, join the gradients of the predicted state and the masses, and the
 // transposed predictor leads to the gradients of the state the step began
 // with.  Then, with `corrector`, the transposed corrector of the step before:
 // from the gradients of the corrected state (gx, gv, ga, gk) to those of the
@@ -198,23 +372,23 @@ struct AdjDt {
 // (left in ga, gk); without it the force at t = 0, whose upstream is (ga, gk)
 // itself.  Last, the j-stream the force adjoint reads, at the prediction of
 // that step from its state `src` (dt = 0 at t = 0).
-__global__ void adj_step_kernel(const double *__restrict__ part, const int after, const DiffGrads G, const int n,
+__global__ void __launch_bounds__(32 * kLanes) adj_step_kernel(const float *__restrict__ part, const VjpSlots V, const DiffGrads G, const int n,
                                 const AdjDt d, const bool corrector, const double *__restrict__ src, const JStream J)
 {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= 3 * n) return;
-    const int c = idx / n, i = idx - c * n;
+    const int idx = blockIdx.x * 32 + (threadIdx.x & 31);
+    const bool live = idx < 3 * n;
+    const int c = live ? idx / n : 0, i = live ? idx - c * n : 0;
+    double t[3];
+    if (V.sb > 0)
+        column_sums(V.sb * V.parts + 1, [&](int s, int v, float &a, float &b) {
+            if (v < 2 || c == 0) vjp_at_slot(part, V, n, v < 2 ? 3 * v + c : 6, i, s, a, b);
+        }, t);
+    if (threadIdx.x >= 32 || !live) return;
     const size_t e = static_cast<size_t>(idx), n3 = 3 * static_cast<size_t>(n);
     // (the component arrays of each gradient are contiguous: gx[0][e] is component c of particle i)
     double gx = G.gx[0][e], gv = G.gv[0][e], ga = G.ga[0][e], gk = G.gk[0][e];
-    if (after > 0) {
-        double tx = 0.0, tv = 0.0, tm = 0.0;
-        for (int y = 0; y < after; ++y) {
-            const double *b = part + static_cast<size_t>(y) * 7 * n + e;
-            tx += b[0];
-            tv += b[n3];
-            if (c == 0) tm += b[2 * n3];
-        }
+    if (V.sb > 0) {
+        const double tx = t[0], tv = t[1], tm = t[2];
         if (c == 0) G.gm[i] += tm;
         const double gxp = G.gxp[0][e] + tx, gvp = G.gvp[0][e] + tv;
         gx = gxp;
@@ -328,49 +502,48 @@ int blocks_of(int64_t n, int t) { return static_cast<int>((n + t - 1) / t); }
 
 }  // namespace
 
-int vjp_ranges(int64_t n, int64_t n_pad, int sm_count)
+// Superblocks of 64 rows up to n = 8192 (128 of them), each pair of them in two
+// parts while that leaves fewer warps than the GPU holds (n = 4096 and below);
+// more tiles per superblock beyond, their sums folded in double-single.
+VjpSlots vjp_slots(int64_t n, int sm_count)
 {
-    // enough blocks for about four per SM; ranges of whole tiles
-    const int bx = blocks_of(n, kVjpThreads);
-    const int tiles = static_cast<int>(n_pad / kVjpTile);
-    const int want = (4 * sm_count + bx - 1) / bx;
-    const int r = want < 1 ? 1 : (want > tiles ? tiles : want);
-    const int tpr = (tiles + r - 1) / r;
-    return (tiles + tpr - 1) / tpr;
+    VjpSlots V{};
+    const int64_t tiles = (n + 64 * kVjpRows * 2 - 1) / (64 * kVjpRows * 2);
+    V.rows = static_cast<int>(tiles) * kVjpRows;
+    V.sb = static_cast<int>((n + V.rows - 1) / V.rows);
+    V.two_word = tiles > 1;
+    V.parts = tiles == 1 && static_cast<int64_t>(V.sb) * (V.sb + 1) / 2 < 12LL * sm_count ? 2 : 1;
+    return V;
 }
 
-size_t vjp_scratch_doubles(int64_t n, int64_t n_pad, int sm_count)
+size_t vjp_scratch_bytes(int64_t n, int sm_count)
 {
-    return static_cast<size_t>(vjp_ranges(n, n_pad, sm_count)) * 7 * static_cast<size_t>(n);
+    const VjpSlots V = vjp_slots(n, sm_count);
+    return (static_cast<size_t>(V.sb) * V.parts + 1) * (V.two_word ? 14 : 7) * static_cast<size_t>(n) * sizeof(float);
 }
 
 cudaError_t force_vjp_launch(const JStream &J, const DiffGrads &G, int64_t n, float eps2, int sm_count,
-                             double *scratch, int *ranges, cudaStream_t s, int64_t *launches)
+                             void *scratch, VjpSlots *slots, cudaStream_t s, int64_t *launches)
 {
-    const int tiles = static_cast<int>(J.n_pad / kVjpTile);
-    const int r = vjp_ranges(n, J.n_pad, sm_count);
-    const int tpr = (tiles + r - 1) / r;
-    const dim3 grid(blocks_of(n, kVjpThreads), r);
-    force_vjp_kernel<<<grid, kVjpThreads, 0, s>>>(J.posm, J.vel, G.gA, G.gK, static_cast<int>(n),
-                                                  static_cast<int>(J.n_pad), eps2, tpr, scratch);
+    const VjpSlots V = vjp_slots(n, sm_count);
+    const unsigned units = static_cast<unsigned>(static_cast<int64_t>(V.sb) * (V.sb + 1) / 2 * V.parts);
+    auto *kernel = V.two_word ? vjp_pairs_kernel<1, true> : V.parts == 2 ? vjp_pairs_kernel<2, false>
+                                                                         : vjp_pairs_kernel<1, false>;
+    kernel<<<units, 32, 0, s>>>(J.posm, J.vel, G.gA, G.gK, static_cast<int>(n), eps2, V.sb, V.rows / kVjpRows,
+                                static_cast<float *>(scratch));
     ++*launches;
-    *ranges = r;
+    *slots = V;
     return cudaGetLastError();
 }
 
-cudaError_t vjp_finish_launch(const DiffGrads &G, int64_t n, const double *scratch, int ranges, cudaStream_t s,
+cudaError_t vjp_finish_launch(const DiffGrads &G, int64_t n, const void *scratch, const VjpSlots &slots, cudaStream_t s,
                               int64_t *launches)
 {
-    vjp_reduce_kernel<<<blocks_of(7 * n, 256), 256, 0, s>>>(scratch, ranges, static_cast<int>(n), G);
+    vjp_reduce_kernel<<<blocks_of(7 * n, 32), 32 * kLanes, 0, s>>>(static_cast<const float *>(scratch), slots,
+                                                            static_cast<int>(n), G);
     ++*launches;
     return cudaGetLastError();
 }
-
-namespace {
-// Threads of the per-(component, particle) kernels: FP64 chains, so a small n is
-// spread over all SMs.
-int elem_threads(int64_t n) { return 3 * n >= 152 * 512 ? 256 : 32; }
-}  // namespace
 
 cudaError_t roll_step_launch(const double *src, double *dst, int64_t n, const double *acc, const double *jerk,
                              const float *part, int split, bool two_word, int level, bool predict, const JStream &J,
@@ -384,14 +557,13 @@ cudaError_t roll_step_launch(const double *src, double *dst, int64_t n, const do
     d.dt3 = dt * dt * dt;
     d.dt4 = d.dt3 * dt;
     d.pd = {dt, 0.5 * dt, dt * (1.0 / 3.0)};
-    const int t = elem_threads(n);
     auto *kernel = two_word ? roll_step_kernel<true> : roll_step_kernel<false>;
-    kernel<<<blocks_of(3 * n, t), t, 0, s>>>(src, dst, static_cast<int>(n), acc, jerk, part, split, d, predict, J, st);
+    kernel<<<blocks_of(3 * n, 32), 32 * kLanes, 0, s>>>(src, dst, static_cast<int>(n), acc, jerk, part, split, d, predict, J, st);
     ++*launches;
     return cudaGetLastError();
 }
 
-cudaError_t adj_step_launch(const double *scratch, int after, const DiffGrads &G, int64_t n, double dt, bool corrector,
+cudaError_t adj_step_launch(const void *scratch, const VjpSlots &slots, const DiffGrads &G, int64_t n, double dt, bool corrector,
                             const double *src, const JStream &J, cudaStream_t s, int64_t *launches)
 {
     AdjDt d;
@@ -405,8 +577,8 @@ cudaError_t adj_step_launch(const double *scratch, int after, const DiffGrads &G
     d.i2 = d.i1 * d.i1;
     d.i3 = d.i2 * d.i1;
     d.pd = {dt, 0.5 * dt, dt * (1.0 / 3.0)};
-    const int t = elem_threads(n);
-    adj_step_kernel<<<blocks_of(3 * n, t), t, 0, s>>>(scratch, after, G, static_cast<int>(n), d, corrector, src, J);
+    adj_step_kernel<<<blocks_of(3 * n, 32), 32 * kLanes, 0, s>>>(static_cast<const float *>(scratch), slots, G, static_cast<int>(n), d,
+                                                   corrector, src, J);
     ++*launches;
     return cudaGetLastError();
 }

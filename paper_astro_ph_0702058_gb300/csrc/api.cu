@@ -499,9 +499,9 @@ int rollout_impl(const char *who, int64_t n, const double *m, const double *x0, 
     NB_DR(dev_alloc(reinterpret_cast<void **>(&lval), nd * sizeof(double)), "loss terms");
     NB_DR(dev_alloc(reinterpret_cast<void **>(&dloss), sizeof(double)), "loss");
     NB_DR(dev_alloc(reinterpret_cast<void **>(&g4), 2 * npad * sizeof(float4)), "force upstream");
-    const size_t vjp_doubles = std::max(vjp_scratch_doubles(n, c->n_pad, c->sm_count),
-                                        seed_loss ? loss_scratch_doubles(n, c->sm_count) : size_t(0));
-    NB_DR(dev_alloc(reinterpret_cast<void **>(&vjp), vjp_doubles * sizeof(double)), "adjoint scratch");
+    const size_t vjp_bytes = std::max(vjp_scratch_bytes(n, c->sm_count),
+                                      seed_loss ? loss_scratch_doubles(n, c->sm_count) * sizeof(double) : size_t(0));
+    NB_DR(dev_alloc(reinterpret_cast<void **>(&vjp), vjp_bytes), "adjoint scratch");
     NB_DR(cudaMemsetAsync(gbuf, 0, 19 * nd * sizeof(double), s), "memset");
     NB_DR(cudaMemsetAsync(g4, 0, 2 * npad * sizeof(float4), s), "memset");
     for (int q = 0; q < 3; ++q) {
@@ -551,7 +551,7 @@ int rollout_impl(const char *who, int64_t n, const double *m, const double *x0, 
         }
     }
     // backward, one segment at a time
-    int ranges = 0;  // of the last force adjoint (0: none yet)
+    VjpSlots slots{};  // of the last force adjoint (none yet)
     for (int64_t seg0 = steps > 0 ? (steps - 1) / seg_len * seg_len : -1; seg0 >= 0; seg0 -= seg_len) {
         const int64_t count = std::min(seg_len, steps - seg0);
         if (!keep) {
@@ -560,14 +560,14 @@ int rollout_impl(const char *who, int64_t n, const double *m, const double *x0, 
             if (r != NBODY_OK) return done(r);
         }
         for (int64_t k = count - 1; k >= 0; --k) {
-            NB_DR(adj_step_launch(vjp, ranges, G, n, dt, true, seg_state(k), c->J, s, L), "adjoint step");
-            NB_DR(force_vjp_launch(c->J, G, n, e2, c->sm_count, vjp, &ranges, s, L), "force adjoint");
+            NB_DR(adj_step_launch(vjp, slots, G, n, dt, true, seg_state(k), c->J, s, L), "adjoint step");
+            NB_DR(force_vjp_launch(c->J, G, n, e2, c->sm_count, vjp, &slots, s, L), "force adjoint");
         }
     }
     // the t = 0 force
-    NB_DR(adj_step_launch(vjp, ranges, G, n, dt, false, ck, c->J, s, L), "adjoint step");
-    NB_DR(force_vjp_launch(c->J, G, n, e2, c->sm_count, vjp, &ranges, s, L), "force adjoint");
-    NB_DR(vjp_finish_launch(G, n, vjp, ranges, s, L), "adjoint reduction");
+    NB_DR(adj_step_launch(vjp, slots, G, n, dt, false, ck, c->J, s, L), "adjoint step");
+    NB_DR(force_vjp_launch(c->J, G, n, e2, c->sm_count, vjp, &slots, s, L), "force adjoint");
+    NB_DR(vjp_finish_launch(G, n, vjp, slots, s, L), "adjoint reduction");
     if (seed_loss && loss) NB_DR(cudaMemcpyAsync(loss, dloss, sizeof(double), cudaMemcpyDefault, s), "loss copy");
     if (g_x0) {
         NB_DR(soa_to_aos_launch(G.gxp[0], G.gxp[1], G.gxp[2], c->stage, n, s, L), "layout");

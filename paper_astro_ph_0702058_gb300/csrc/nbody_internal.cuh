@@ -305,13 +305,17 @@ struct DiffGrads {
     float4 *gA, *gK;                        // upstream of the force (n_pad, zero padded)
 };
 // (each of gx .. gvp three contiguous arrays of n)
-// Doubles of scratch the force VJP needs for its j-range totals.
-size_t vjp_scratch_doubles(int64_t n, int64_t n_pad, int sm_count);
-// The force's vector-Jacobian product: totals of *ranges ranges to scratch, for adj_step_launch
-// (`after`) or vjp_finish_launch, which adds them to gxp, gvp and gm.
+// Slots that hold the totals of a force VJP: superblocks of `rows` rows, `parts` slots of each.
+struct VjpSlots {
+    int sb, rows, parts;  // sb = 0: none yet
+    int two_word;
+};
+size_t vjp_scratch_bytes(int64_t n, int sm_count);
+// The force's vector-Jacobian product: totals to scratch, for adj_step_launch or vjp_finish_launch,
+// which adds them to gxp, gvp and gm.
 cudaError_t force_vjp_launch(const JStream &J, const DiffGrads &G, int64_t n, float eps2, int sm_count,
-                             double *scratch, int *ranges, cudaStream_t s, int64_t *launches);
-cudaError_t vjp_finish_launch(const DiffGrads &G, int64_t n, const double *scratch, int ranges, cudaStream_t s,
+                             void *scratch, VjpSlots *slots, cudaStream_t s, int64_t *launches);
+cudaError_t vjp_finish_launch(const DiffGrads &G, int64_t n, const void *scratch, const VjpSlots &slots, cudaStream_t s,
                               int64_t *launches);
 // Ends a shared step of 2^-level (state at src -> state at dst, x[3], v[3], a[3], k[3] of n doubles
 // each) with the force in part ([split][7 or 14][n] partial sums; two_word: hi and lo) or in acc and
@@ -320,7 +324,7 @@ cudaError_t roll_step_launch(const double *src, double *dst, int64_t n, const do
                              const float *part, int split, bool two_word, int level, bool predict, const JStream &J,
                              DevStatus *st, cudaStream_t s, int64_t *launches);
 // From one force VJP to the next of the backward sweep (see adj_step_kernel).
-cudaError_t adj_step_launch(const double *scratch, int after, const DiffGrads &G, int64_t n, double dt, bool corrector,
+cudaError_t adj_step_launch(const void *scratch, const VjpSlots &slots, const DiffGrads &G, int64_t n, double dt, bool corrector,
                             const double *src, const JStream &J, cudaStream_t s, int64_t *launches);
 size_t loss_scratch_doubles(int64_t n, int sm_count);
 cudaError_t loss_launch(const State &S, double eps2, const DiffGrads &G, int sm_count, double *scratch, double *lval,
