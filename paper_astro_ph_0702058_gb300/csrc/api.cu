@@ -12,6 +12,7 @@
 #include <new>
 #include <vector>
 
+#include "arena.h"
 #include "nbody_internal.cuh"
 
 using namespace nb;
@@ -93,6 +94,7 @@ struct nbody_ctx {
     cudaStream_t s = nullptr;
     int sm_count = 0;
 
+    void *dev_base = nullptr, *host_base = nullptr;  // the allocations that hold the fixed buffers below
     double *state = nullptr;  // 13 n doubles: m, x[3], v[3], a[3], k[3]
     int64_t *t = nullptr;
     int8_t *level = nullptr;
@@ -145,14 +147,10 @@ namespace {
 void release(nbody_ctx *c)
 {
     if (c->step_graph) cudaGraphExecDestroy(c->step_graph);
-    void *dev[] = {c->state, c->t, c->level, c->jbuf, c->act_force, c->act_corr, c->act_sched,
-                   c->f_acc, c->f_jerk, c->f_pot, c->stage, c->partials, c->sched_scratch,
-                   c->sched_out, c->st, c->phi, c->e_out, c->trange, c->graph_fits, c->loop_dev, c->grid_buf, c->sym_buf};
+    void *dev[] = {c->dev_base, c->partials, c->graph_fits, c->grid_buf, c->sym_buf};
     for (void *d : dev)
         if (d) cudaFree(d);
-    void *host[] = {c->sched_host, c->st_host, c->e_host, c->trange_host, c->loop_host};
-    for (void *h : host)
-        if (h) cudaFreeHost(h);
+    if (c->host_base) cudaFreeHost(c->host_base);
     delete c;
 }
 
@@ -399,6 +397,7 @@ int rollout_impl(const char *who, int64_t n, const double *m, const double *x0, 
     const size_t npad = static_cast<size_t>(c->n_pad);
     double *ck = nullptr, *seg = nullptr, *gbuf = nullptr, *lval = nullptr, *dloss = nullptr, *vjp = nullptr;
     float4 *g4 = nullptr;
+    void *mem_base = nullptr;  // holds them all
     DiffGrads G{};
     const double dt = std::ldexp(1.0, -level);
     const float e2 = static_cast<float>(eps2);
@@ -406,9 +405,7 @@ int rollout_impl(const char *who, int64_t n, const double *m, const double *x0, 
     int64_t *L = &c->stats.kernel_launches;
     auto done = [&](int code) {
         cudaStreamSynchronize(s);
-        void *bufs[] = {ck, seg, gbuf, lval, dloss, g4, vjp};
-        for (void *b : bufs)
-            if (b) cudaFree(b);
+        if (mem_base) cudaFree(mem_base);
         nbody_free(c);
         return code;
     };
@@ -483,25 +480,29 @@ int rollout_impl(const char *who, int64_t n, const double *m, const double *x0, 
     }
     // Every state is kept where kRollKeep holds them; else checkpoints every checkpoint_every steps, and the
     // steps of a segment run again before its backward sweep.  The same bits either way.
-    bool keep = static_cast<double>(steps) * state_doubles * sizeof(double) <= static_cast<double>(kRollKeep);
-    if (keep && dev_alloc(reinterpret_cast<void **>(&seg), std::max<int64_t>(steps, 1) * state_doubles * sizeof(double)) !=
-                    cudaSuccess) {
-        cudaGetLastError();
-        seg = nullptr;
-        keep = false;
-    }
-    const int64_t seg_len = keep ? std::max<int64_t>(steps, 1) : checkpoint_every;
-    const int64_t n_ck = keep ? 1 : steps / seg_len + 1;
-    if (!keep)
-        NB_DR(dev_alloc(reinterpret_cast<void **>(&seg), seg_len * state_doubles * sizeof(double)), "segment");
-    NB_DR(dev_alloc(reinterpret_cast<void **>(&ck), n_ck * state_doubles * sizeof(double)), "checkpoints");
-    NB_DR(dev_alloc(reinterpret_cast<void **>(&gbuf), 19 * nd * sizeof(double)), "gradients");
-    NB_DR(dev_alloc(reinterpret_cast<void **>(&lval), nd * sizeof(double)), "loss terms");
-    NB_DR(dev_alloc(reinterpret_cast<void **>(&dloss), sizeof(double)), "loss");
-    NB_DR(dev_alloc(reinterpret_cast<void **>(&g4), 2 * npad * sizeof(float4)), "force upstream");
     const size_t vjp_bytes = std::max(vjp_scratch_bytes(n, c->sm_count),
                                       seed_loss ? loss_scratch_doubles(n, c->sm_count) * sizeof(double) : size_t(0));
-    NB_DR(dev_alloc(reinterpret_cast<void **>(&vjp), vjp_bytes), "adjoint scratch");
+    bool keep = static_cast<double>(steps) * state_doubles * sizeof(double) <= static_cast<double>(kRollKeep);
+    auto room = [&]() -> cudaError_t {
+        const int64_t len = keep ? std::max<int64_t>(steps, 1) : checkpoint_every;
+        Arena mem;
+        mem.add(&seg, len * state_doubles * sizeof(double));
+        mem.add(&ck, (keep ? 1 : steps / len + 1) * state_doubles * sizeof(double));
+        mem.add(&gbuf, 19 * nd * sizeof(double));
+        mem.add(&lval, nd * sizeof(double));
+        mem.add(&dloss, sizeof(double));
+        mem.add(&g4, 2 * npad * sizeof(float4));
+        mem.add(&vjp, vjp_bytes);
+        return mem.commit(&mem_base, dev_alloc);
+    };
+    cudaError_t er = room();
+    if (er == cudaErrorMemoryAllocation && keep) {
+        cudaGetLastError();
+        keep = false;
+        er = room();
+    }
+    NB_DR(er, "rollout scratch");
+    const int64_t seg_len = keep ? std::max<int64_t>(steps, 1) : checkpoint_every;
     NB_DR(cudaMemsetAsync(gbuf, 0, 19 * nd * sizeof(double), s), "memset");
     NB_DR(cudaMemsetAsync(g4, 0, 2 * npad * sizeof(float4), s), "memset");
     for (int q = 0; q < 3; ++q) {
@@ -638,31 +639,33 @@ int nbody_init(nbody_ctx **out, int64_t n, const double *m, const double *x, con
     NB_INIT(cudaGetDevice(&dev), "cudaGetDevice");
     NB_INIT(cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, dev), "SM count");
     const size_t nd = static_cast<size_t>(n);
-    NB_INIT(dev_alloc(reinterpret_cast<void **>(&c->state), 13 * nd * sizeof(double)), "state allocation");
-    NB_INIT(dev_alloc(reinterpret_cast<void **>(&c->t), nd * sizeof(int64_t)), "time allocation");
-    NB_INIT(dev_alloc(reinterpret_cast<void **>(&c->level), nd), "level allocation");
+    Arena dev_mem, host_mem;
+    dev_mem.add(&c->state, 13 * nd * sizeof(double));
+    dev_mem.add(&c->t, nd * sizeof(int64_t));
+    dev_mem.add(&c->level, nd);
     const size_t jbytes = static_cast<size_t>(c->n_pad) * (4 * sizeof(float4) + kSoaArrays * sizeof(float));
-    NB_INIT(dev_alloc(reinterpret_cast<void **>(&c->jbuf), jbytes), "j-stream allocation");
-    NB_INIT(dev_alloc(reinterpret_cast<void **>(&c->act_force), nd * sizeof(int32_t)), "list allocation");
-    NB_INIT(dev_alloc(reinterpret_cast<void **>(&c->act_corr), nd * sizeof(int32_t)), "list allocation");
-    NB_INIT(dev_alloc(reinterpret_cast<void **>(&c->act_sched), nd * sizeof(int32_t)), "list allocation");
-    NB_INIT(dev_alloc(reinterpret_cast<void **>(&c->f_acc), 3 * nd * sizeof(double)), "force allocation");
-    NB_INIT(dev_alloc(reinterpret_cast<void **>(&c->f_jerk), 3 * nd * sizeof(double)), "force allocation");
-    NB_INIT(dev_alloc(reinterpret_cast<void **>(&c->f_pot), nd * sizeof(double)), "force allocation");
-    NB_INIT(dev_alloc(reinterpret_cast<void **>(&c->stage), 6 * nd * sizeof(double)), "staging allocation");
-    NB_INIT(dev_alloc(&c->sched_scratch, sched_scratch_bytes(n)), "scheduler scratch allocation");
-    NB_INIT(dev_alloc(reinterpret_cast<void **>(&c->sched_out), sizeof(SchedOut)), "scheduler allocation");
-    NB_INIT(dev_alloc(reinterpret_cast<void **>(&c->st), sizeof(DevStatus)), "status allocation");
-    NB_INIT(dev_alloc(reinterpret_cast<void **>(&c->phi), (nd + kEnergyPad) * sizeof(double)), "energy scratch allocation");
-    NB_INIT(dev_alloc(reinterpret_cast<void **>(&c->e_out), 2 * sizeof(double)), "energy allocation");
-    NB_INIT(dev_alloc(reinterpret_cast<void **>(&c->trange), 2 * sizeof(unsigned long long)), "time-range allocation");
-    NB_INIT(host_alloc(reinterpret_cast<void **>(&c->sched_host), sizeof(SchedOut)), "pinned allocation");
-    NB_INIT(host_alloc(reinterpret_cast<void **>(&c->st_host), sizeof(DevStatus)), "pinned allocation");
-    NB_INIT(host_alloc(reinterpret_cast<void **>(&c->e_host), 2 * sizeof(double)), "pinned allocation");
-    NB_INIT(host_alloc(reinterpret_cast<void **>(&c->trange_host), 2 * sizeof(unsigned long long)),
-            "pinned allocation");
-    NB_INIT(dev_alloc(reinterpret_cast<void **>(&c->loop_dev), sizeof(StepLoop)), "loop control allocation");
-    NB_INIT(host_alloc(reinterpret_cast<void **>(&c->loop_host), sizeof(StepLoop)), "pinned allocation");
+    dev_mem.add(&c->jbuf, jbytes);
+    dev_mem.add(&c->act_force, nd * sizeof(int32_t));
+    dev_mem.add(&c->act_corr, nd * sizeof(int32_t));
+    dev_mem.add(&c->act_sched, nd * sizeof(int32_t));
+    dev_mem.add(&c->f_acc, 3 * nd * sizeof(double));
+    dev_mem.add(&c->f_jerk, 3 * nd * sizeof(double));
+    dev_mem.add(&c->f_pot, nd * sizeof(double));
+    dev_mem.add(&c->stage, 6 * nd * sizeof(double));
+    dev_mem.add(&c->sched_scratch, sched_scratch_bytes(n));
+    dev_mem.add(&c->sched_out, sizeof(SchedOut));
+    dev_mem.add(&c->st, sizeof(DevStatus));
+    dev_mem.add(&c->phi, (nd + kEnergyPad) * sizeof(double));
+    dev_mem.add(&c->e_out, 2 * sizeof(double));
+    dev_mem.add(&c->trange, 2 * sizeof(unsigned long long));
+    host_mem.add(&c->sched_host, sizeof(SchedOut));
+    host_mem.add(&c->st_host, sizeof(DevStatus));
+    host_mem.add(&c->e_host, 2 * sizeof(double));
+    host_mem.add(&c->trange_host, 2 * sizeof(unsigned long long));
+    dev_mem.add(&c->loop_dev, sizeof(StepLoop));
+    host_mem.add(&c->loop_host, sizeof(StepLoop));
+    NB_INIT(dev_mem.commit(&c->dev_base, dev_alloc), "context allocation");
+    NB_INIT(host_mem.commit(&c->host_base, host_alloc), "pinned allocation");
     std::memset(c->st_host, 0, sizeof(DevStatus));
 
     State &S = c->S;

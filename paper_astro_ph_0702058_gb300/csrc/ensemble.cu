@@ -28,6 +28,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "arena.h"
 #include "force_x2.cuh"
 #include "step_impl.cuh"
 
@@ -634,7 +635,8 @@ struct nbody_ens {
     int s_max = 8;
     int threads = 64, ipt = 1, tiles_per_range = 4;
     std::vector<int64_t> off_h;
-    // device memory
+    // device memory, in one allocation, and pinned memory in another
+    void *dev_base = nullptr, *host_base = nullptr;
     double *state = nullptr;
     int64_t *t = nullptr;
     int8_t *level = nullptr;
@@ -685,13 +687,8 @@ int ecuda(cudaError_t e, const char *what)
 void ens_release(nbody_ens *e)
 {
     if (e->graph) cudaGraphExecDestroy(e->graph);
-    void *dev[] = {e->state, e->t, e->level, e->jbuf, e->off, e->joff, e->cl_of, e->act, e->t_blk, e->item_pfx,
-                   e->row_pfx, e->blocks, e->pairs, e->n_act, e->nsplit, e->tpr, e->live, e->work, e->part, e->st, e->phi,
-                   e->e_out, e->stage, e->trange};
-    for (void *d : dev)
-        if (d) cudaFree(d);
-    if (e->live_h) cudaFreeHost(e->live_h);
-    if (e->st_h) cudaFreeHost(e->st_h);
+    if (e->dev_base) cudaFree(e->dev_base);
+    if (e->host_base) cudaFreeHost(e->host_base);
     if (e->own_stream && e->s) cudaStreamDestroy(e->s);
     delete e;
 }
@@ -812,33 +809,36 @@ int nbody_ens_init(nbody_ens **out, int64_t n_clusters, const int64_t *sizes, co
     NB_EI(cudaDeviceGetAttribute(&e->sm_count, cudaDevAttrMultiProcessorCount, dev), "SM count");
     const size_t nd = static_cast<size_t>(n), nc = static_cast<size_t>(n_clusters);
     const size_t NC = prm.mode == NBODY_MODE_COMP ? 14 : 7;
-    NB_EI(cudaMalloc(&e->state, 13 * nd * sizeof(double)), "state allocation");
-    NB_EI(cudaMalloc(&e->t, nd * sizeof(int64_t)), "time allocation");
-    NB_EI(cudaMalloc(&e->level, nd), "level allocation");
+    Arena dev_mem, host_mem;
+    dev_mem.add(&e->state, 13 * nd * sizeof(double));
+    dev_mem.add(&e->t, nd * sizeof(int64_t));
+    dev_mem.add(&e->level, nd);
     const size_t jbytes = static_cast<size_t>(jt) * (3 * sizeof(float4) + kSoaArrays * sizeof(float));
-    NB_EI(cudaMalloc(&e->jbuf, jbytes), "j-stream allocation");
-    NB_EI(cudaMalloc(&e->off, (nc + 1) * sizeof(int64_t)), "offsets");
-    NB_EI(cudaMalloc(&e->joff, nc * sizeof(int64_t)), "offsets");
-    NB_EI(cudaMalloc(&e->cl_of, nd * sizeof(int32_t)), "cluster map");
-    NB_EI(cudaMalloc(&e->act, nd * sizeof(int32_t)), "block lists");
-    NB_EI(cudaMalloc(&e->t_blk, nc * sizeof(long long)), "cluster times");
-    NB_EI(cudaMalloc(&e->item_pfx, (nc + 1) * sizeof(long long)), "plan");
-    NB_EI(cudaMalloc(&e->row_pfx, (nc + 1) * sizeof(long long)), "plan");
-    NB_EI(cudaMalloc(&e->blocks, nc * sizeof(long long)), "block counters");
-    NB_EI(cudaMalloc(&e->pairs, nc * sizeof(long long)), "pair counters");
-    NB_EI(cudaMalloc(&e->n_act, nc * sizeof(int)), "plan");
-    NB_EI(cudaMalloc(&e->nsplit, nc * sizeof(int)), "plan");
-    NB_EI(cudaMalloc(&e->tpr, nc * sizeof(int)), "plan");
-    NB_EI(cudaMalloc(&e->live, 2 * sizeof(int)), "plan");
-    NB_EI(cudaMalloc(&e->work, sizeof(unsigned int)), "work counter");
-    NB_EI(cudaMalloc(&e->part, nd * e->s_max * NC * sizeof(float)), "partial sums");
-    NB_EI(cudaMalloc(&e->st, sizeof(DevStatus)), "status");
-    NB_EI(cudaMalloc(&e->phi, nd * sizeof(double)), "energy scratch");
-    NB_EI(cudaMalloc(&e->e_out, 2 * nc * sizeof(double)), "energy");
-    NB_EI(cudaMalloc(&e->stage, 3 * nd * sizeof(double)), "staging");
-    NB_EI(cudaMalloc(&e->trange, 2 * nc * sizeof(long long)), "time range");
-    NB_EI(cudaMallocHost(&e->live_h, 2 * sizeof(int)), "pinned");
-    NB_EI(cudaMallocHost(&e->st_h, sizeof(DevStatus)), "pinned");
+    dev_mem.add(&e->jbuf, jbytes);
+    dev_mem.add(&e->off, (nc + 1) * sizeof(int64_t));
+    dev_mem.add(&e->joff, nc * sizeof(int64_t));
+    dev_mem.add(&e->cl_of, nd * sizeof(int32_t));
+    dev_mem.add(&e->act, nd * sizeof(int32_t));
+    dev_mem.add(&e->t_blk, nc * sizeof(long long));
+    dev_mem.add(&e->item_pfx, (nc + 1) * sizeof(long long));
+    dev_mem.add(&e->row_pfx, (nc + 1) * sizeof(long long));
+    dev_mem.add(&e->blocks, nc * sizeof(long long));
+    dev_mem.add(&e->pairs, nc * sizeof(long long));
+    dev_mem.add(&e->n_act, nc * sizeof(int));
+    dev_mem.add(&e->nsplit, nc * sizeof(int));
+    dev_mem.add(&e->tpr, nc * sizeof(int));
+    dev_mem.add(&e->live, 2 * sizeof(int));
+    dev_mem.add(&e->work, sizeof(unsigned int));
+    dev_mem.add(&e->part, nd * e->s_max * NC * sizeof(float));
+    dev_mem.add(&e->st, sizeof(DevStatus));
+    dev_mem.add(&e->phi, nd * sizeof(double));
+    dev_mem.add(&e->e_out, 2 * nc * sizeof(double));
+    dev_mem.add(&e->stage, 3 * nd * sizeof(double));
+    dev_mem.add(&e->trange, 2 * nc * sizeof(long long));
+    host_mem.add(&e->live_h, 2 * sizeof(int));
+    host_mem.add(&e->st_h, sizeof(DevStatus));
+    NB_EI(dev_mem.commit(&e->dev_base, [](void **p, size_t b) { return cudaMalloc(p, b); }), "ensemble allocation");
+    NB_EI(host_mem.commit(&e->host_base, [](void **p, size_t b) { return cudaMallocHost(p, b); }), "pinned allocation");
     std::vector<int32_t> clmap(nd);
     for (size_t c = 0; c < nc; ++c)
         for (int64_t i = off[c]; i < off[c + 1]; ++i) clmap[static_cast<size_t>(i)] = static_cast<int32_t>(c);
