@@ -211,10 +211,10 @@ cudaError_t force_launch(int mode, const JStream &js, int64_t n, const int32_t *
     if (n_act <= 0) return cudaSuccess;
     const float eps2 = static_cast<float>(eps2_d);
     if (mode == kModeDS) {
-        cudaError_t e = force_ds_launch(js, n, active, n_act, eps2_d, cfg, acc, jerk, pot, partials, st, s);
+        cudaError_t e = force_ds_launch(js, n, active, n_act, eps2_d, cfg, acc, jerk, pot, partials, st, s, n_act_dev);
         if (e != cudaSuccess) return e;
         ++*launches;
-        if (cfg.split > 1) {
+        if (cfg.split > 1 && reduce) {
             e = reduce_comp(static_cast<float *>(partials), cfg.split, static_cast<int>(n_act), acc, jerk, pot, s,
                             nullptr);
             if (e != cudaSuccess) return e;

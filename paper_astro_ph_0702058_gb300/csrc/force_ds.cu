@@ -42,10 +42,12 @@ struct DsParams {
     double *__restrict__ acc, *__restrict__ jerk, *__restrict__ pot;
     float *__restrict__ part;  // [split][14][n_act] when split > 1
     DevStatus *st;
+    const long long *run;  // when set and zero: nothing to do
 };
 
 __global__ void __launch_bounds__(kDsThreads) force_ds_kernel(const DsParams P)
 {
+    if (P.run && *P.run == 0) return;
     __shared__ float4 sp[kJTile], sl[kJTile], sv[kJTile], svl[kJTile];
     const int tid = threadIdx.x;
     const int q = blockIdx.x * kDsThreads + tid;
@@ -116,9 +118,10 @@ int force_occupancy_ds()
 
 cudaError_t force_ds_launch(const JStream &js, int64_t n, const int32_t *active, int64_t n_act, double eps2,
                             const ForceConfig &cfg, double *acc, double *jerk, double *pot, void *partials,
-                            DevStatus *st, cudaStream_t s)
+                            DevStatus *st, cudaStream_t s, const long long *run)
 {
     DsParams P;
+    P.run = run;
     P.posm = js.posm;
     P.poslo = js.poslo;
     P.vel = js.vel;

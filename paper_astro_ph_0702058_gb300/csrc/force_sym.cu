@@ -2,8 +2,11 @@
 // takes it, how it is cut, the rows and the particles outside the block as
 // contiguous arrays, and the sum over the slots.
 #include <cmath>
+#include <type_traits>
 
+#include "ds_arith.cuh"
 #include "force_sym.cuh"
+#include "force_sym_ds.cuh"
 
 namespace nb {
 
@@ -11,6 +14,7 @@ namespace {
 
 constexpr int kSymMaxSb = 128;             // superblocks
 constexpr int64_t kSymMinRows = 8192;      // rows from which a block may take pairs
+constexpr int64_t kSymDsMin = 4096;        // particles from which the double-single force may
 constexpr int64_t kSymPartCap = int64_t(8) << 30;  // bytes of its slots
 constexpr int kSymThreads = 256;
 constexpr int kSymScan = 4 * kSymThreads;  // particles of a block of the compaction
@@ -53,6 +57,27 @@ __global__ void __launch_bounds__(kSymThreads)
     }
     if (atomicExch(mark + idx, 1) != 0) *rows_general = n_act;
     for (int a = 0; a < arrays; ++a) rows[a * rows_stride + q] = soa[a * stride + idx];
+}
+
+// The float4 streams of the rows (double-single mode), likewise.
+__global__ void __launch_bounds__(kSymThreads)
+    sym_gather_ds_kernel(const JStream J, const int32_t *__restrict__ list, const int n_act, const int n,
+                         float4 *__restrict__ rows, int *__restrict__ mark, long long *rows_general, DevStatus *st)
+{
+    const int q = blockIdx.x * kSymThreads + threadIdx.x;
+    if (q >= n_act) return;
+    const int idx = list[q];
+    if (idx < 0 || idx >= n) {
+        atomicOr(&st->flags, static_cast<unsigned>(kFlagBadIndex));
+        st->bad_index = q;
+        *rows_general = n_act;
+        return;
+    }
+    if (atomicExch(mark + idx, 1) != 0) *rows_general = n_act;
+    rows[q] = J.posm[idx];
+    rows[n_act + q] = J.poslo[idx];
+    rows[2ll * n_act + q] = J.vel[idx];
+    rows[3ll * n_act + q] = J.vello[idx];
 }
 
 // counts[b] <- particles of block b's kSymScan that are not marked.
@@ -125,6 +150,11 @@ __global__ void __launch_bounds__(256)
     for (int s = 0; s < slots; ++s) {
         const float *b = part + (static_cast<size_t>(s) * NC + c) * n + q;
         ds2_add(h, l, b[0], MODE == kModeComp ? b[static_cast<size_t>(7) * n] : 0.0f);
+        if (MODE == kModeComp) {  // (double-single mode: a low word left to grow would cost ~2 of its 46 bits)
+            const dsa::ds r = dsa::fast_two_sum(h, l);
+            h = r.h;
+            l = r.l;
+        }
     }
     const double t = static_cast<double>(h) + static_cast<double>(l);
     if (c < 3)
@@ -158,7 +188,7 @@ SymScratch sym_scratch(void *p, const int64_t n)
 
 size_t sym_scratch_bytes(int64_t n)
 {
-    return 16 + sizeof(int) * (up4(n) + up4(n / kSymScan + 1)) + sizeof(float) * kSoaArrays * (n + 8);
+    return 16 + sizeof(int) * (up4(n) + up4(n / kSymScan + 1)) + sizeof(float) * 16 * (n + 8);
 }
 
 // A block takes pairs from 8192 rows on (full forces at n = 8192, 4096 measured 1.23
@@ -174,6 +204,25 @@ size_t sym_scratch_bytes(int64_t n)
 // rows, of four above (n = 16384: 194 against 240 us plain; 65536: 2894 against 2804).
 bool sym_plan(int mode, int64_t n_act, int64_t n, int sm_count, ForceConfig *cfg)
 {
+    if (mode == kModeDS) {
+        // all particles only, from 4096 on (one unit per resident warp and more: 303 -> 196 us there);
+        // 64-row tiles, one-warp CTAs
+        if (n_act != n || n < kSymDsMin) return false;
+        const int64_t slot = 14 * n * static_cast<int64_t>(sizeof(float));
+        int64_t tiles = (n + kSymDsRows * kSymMaxSb - 1) / (kSymDsRows * kSymMaxSb), sb;
+        while (sb = (n + kSymDsRows * tiles - 1) / (kSymDsRows * tiles), (sb + 1) * slot > kSymPartCap) ++tiles;
+        if (sb * (sb + 1) / 2 < 12LL * sm_count) return false;
+        cfg->threads = 32;
+        cfg->ipt = 2;
+        cfg->jsub = 1;
+        cfg->slice = 0;
+        cfg->n_iblk = static_cast<int>(sb);
+        cfg->split = static_cast<int>(sb + 1);
+        cfg->tiles_per_split = static_cast<int>(tiles);
+        cfg->sym_sb = static_cast<int>(sb);
+        cfg->sym_ranges = cfg->sym_out_len = 0;
+        return true;
+    }
     if (!NB_PACKED || (mode != kModePlain && mode != kModeComp)) return false;
     if (n_act < kSymMinRows || n_act > n || (mode == kModeComp ? 2 : 8.0 / 3.0) * n_act < n) return false;
     const int nc = two_word_sums(mode) ? 14 : 7;
@@ -229,6 +278,40 @@ cudaError_t force_sym_launch(int mode, const JStream &js, int64_t n, const int32
     const SymScratch X = sym_scratch(scratch, n);
     const int na = static_cast<int>(n_act), nn = static_cast<int>(n), n_out = nn - na;
     const int arrays = mode == kModeComp ? 10 : 7;
+    if (mode == kModeDS) {
+        SymDsParams D{};
+        D.posm = js.posm;
+        D.poslo = js.poslo;
+        D.vel = js.vel;
+        D.vello = js.vello;
+        D.n = na;
+        D.n_sb = cfg.sym_sb;
+        D.tiles = cfg.tiles_per_split;
+        D.eps2 = static_cast<float>(eps2);
+        D.eps2_lo = static_cast<float>(eps2 - static_cast<double>(D.eps2));
+        D.part = static_cast<float *>(partials);
+        D.sign = 0x8000000080000000ull;
+        *rows_general = nullptr;
+        if (!ascending) {
+            const cudaError_t e = cudaMemsetAsync(scratch, 0, 16 + sizeof(int) * up4(n), s);
+            if (e != cudaSuccess) return e;
+            float4 *rows = reinterpret_cast<float4 *>(X.rows);
+            sym_gather_ds_kernel<<<(na + kSymThreads - 1) / kSymThreads, kSymThreads, 0, s>>>(
+                js, active, na, nn, rows, X.mark, X.rows_general, st);
+            ++*launches;
+            D.posm = rows;
+            D.poslo = rows + n_act;
+            D.vel = rows + 2 * n_act;
+            D.vello = rows + 3 * n_act;
+            D.skip = X.rows_general;
+            *rows_general = X.rows_general;
+        }
+        force_sym_ds_kernel<<<cfg.sym_sb * (cfg.sym_sb + 1) / 2, 32, 0, s>>>(D);
+        ++*launches;
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        return force_sym_reduce_launch(mode, D.part, cfg.split, n_act, acc, jerk, pot, D.skip, false, s, launches);
+    }
     SymParams P{};
     P.n = na;
     P.n_sb = cfg.sym_sb;
@@ -282,7 +365,7 @@ cudaError_t force_sym_reduce_launch(int mode, const float *part, int slots, int6
 {
     const int na = static_cast<int>(n_act);
     const dim3 grid((na + 255) / 256, 7);
-    if (mode == kModeComp)
+    if (two_word_sums(mode))
         force_sym_reduce_kernel<kModeComp><<<grid, 256, 0, s>>>(part, slots, na, acc, jerk, pot, rows_general, general);
     else
         force_sym_reduce_kernel<kModePlain><<<grid, 256, 0, s>>>(part, slots, na, acc, jerk, pot, rows_general,

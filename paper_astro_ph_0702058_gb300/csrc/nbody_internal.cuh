@@ -175,7 +175,7 @@ cudaError_t force_sym_reduce_launch(int mode, const float *part, int slots, int6
 int force_occupancy_ds();
 cudaError_t force_ds_launch(const JStream &js, int64_t n, const int32_t *active, int64_t n_act, double eps2,
                             const ForceConfig &cfg, double *acc, double *jerk, double *pot, void *partials,
-                            DevStatus *st, cudaStream_t s);
+                            DevStatus *st, cudaStream_t s, const long long *run = nullptr);
 
 // ---- force_sorted.cu ----
 // One block per active row; terms sorted by size and added in FP32 (n <= kSortedMaxN).

@@ -4,7 +4,7 @@ import pytest
 
 import oracle
 from synthetic import active_subset, plummer_sphere
-from tests.gpu_common import EPS2, check_force, gpu_force, need_gpu
+from tests.gpu_common import EPS2, check_force, errors, gpu_force, need_gpu
 
 pytestmark = pytest.mark.gpu
 
@@ -113,3 +113,25 @@ def test_bad_index(torch):
         got = gpu_force(sim, np.arange(n, dtype=np.int32))
         st = sim.stats()
     _check("comp", m, x, v, EPS2, np.arange(n, dtype=np.int32), got, st, "after a bad index")
+
+
+# one and several 64-row tiles per superblock, a last superblock of one row
+@pytest.mark.parametrize("n,eps2", [(4096, EPS2), (4097, 0.0), (8192, EPS2), (8193, EPS2), (16000, 0.0)])
+def test_double_single(torch, n, eps2):
+    """The double-single force by pairs: the mode's 1e-10 per row (max over the rows of the relative errors)."""
+    m, x, v = plummer_sphere(n, 8)
+    m = _masses(n, 8)
+    act = np.random.default_rng(2).permutation(n).astype(np.int32)
+    with _sim(m, x, v, eps2, "ds") as sim:
+        sim.predict(0.0)
+        got = gpu_force(sim, act)
+        assert sim.stats()["last_i_per_thread"] == 2
+        twice = act.copy()
+        twice[5] = twice[n - 7]
+        rep = gpu_force(sim, twice)  # a repeated particle: the one-sided kernel, each row its particle's force
+        assert all(np.array_equal(r[5], r[n - 7]) for r in rep)
+    rows = np.unique(np.concatenate([np.arange(70), np.linspace(0, n - 1, 300).astype(int), np.arange(n - 70, n)]))
+    for g, a in ((got, act), (rep, twice)):
+        e = errors(*(u[rows] for u in g), *oracle.force(m, x, v, eps2, a[rows]))
+        for k in ("acc", "jerk", "pot"):
+            assert e[k].max() <= 1e-10, (k, e[k].max())
