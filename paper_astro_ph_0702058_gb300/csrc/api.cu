@@ -79,6 +79,12 @@ bool is_device_ptr(const void *p)
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Whether a and b, of na and nb doubles, share bytes.
+bool overlap(const double *a, const size_t na, const double *b, const size_t nb)
+{
+    return a && b && a < b + nb && b < a + na;
+}
+
 }  // namespace
 
 int nb::report_error(int code, const char *msg)
@@ -93,6 +99,7 @@ struct nbody_ctx {
     nbody_params p{};
     cudaStream_t s = nullptr;
     int sm_count = 0;
+    int dev = 0;
 
     void *dev_base = nullptr, *host_base = nullptr;  // the allocations that hold the fixed buffers below
     double *state = nullptr;  // 13 n doubles: m, x[3], v[3], a[3], k[3]
@@ -221,6 +228,18 @@ int ensure_partials(nbody_ctx *c, size_t bytes)
     return NBODY_OK;
 }
 
+// Device memory of the context's GPU, aligned to `align` bytes: what a kernel may use as it is.
+bool own_device_ptr(const nbody_ctx *c, const void *p, const uintptr_t align)
+{
+    if (!p || reinterpret_cast<uintptr_t>(p) % align != 0) return false;
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == c->dev;
+}
+
 // Scratch of the force by unordered pairs (cfg), or false where the device has no room for it.
 bool sym_room(nbody_ctx *c, const ForceConfig &cfg, int64_t n_act)
 {
@@ -237,11 +256,14 @@ bool sym_room(nbody_ctx *c, const ForceConfig &cfg, int64_t n_act)
 // is the library's own (a schedule's, or all particles), so its particles are
 // distinct; a caller's list is checked on the device, and one that repeats a
 // particle takes the one-sided kernels.
-int force_internal(nbody_ctx *c, int64_t n_act, bool for_step = false, bool ascending = true)
+// user_list, user: a caller's list, not yet in act_force, and device buffers (a
+// force on its own); *user_done tells that the results are in them.
+int force_internal(nbody_ctx *c, int64_t n_act, bool for_step = false, bool ascending = true,
+                   const int32_t *user_list = nullptr, const ForceUser *user = nullptr, bool *user_done = nullptr)
 {
     auto choose = [&](ForceConfig *cfg, bool pairs) {
         return force_choose(c->p.mode, n_act, c->n_pad, c->sm_count, c->p.j_tile, c->p.i_block, c->p.j_split, cfg,
-                            c->p.j_sub, pairs && c->J.soa ? c->n : 0);
+                            c->p.j_sub, pairs && c->J.soa ? c->n : 0, user && n_act > 0);
     };
     ForceConfig cfg{};
     int r = choose(&cfg, true);
@@ -249,6 +271,14 @@ int force_internal(nbody_ctx *c, int64_t n_act, bool for_step = false, bool asce
     if (r != NBODY_OK) return fail(r, "unsupported force shape: %d threads x %d i per thread", c->p.j_tile, c->p.i_block);
     int64_t launches = 0;
     bool fused = false;
+    const int32_t *list = c->act_force;
+    // many ranges: the rows' list is read by the first kernel and the results written by the second
+    const bool direct = user && n_act > 0 && cfg.sym_sb == 0 && cfg.split >= 8 && force_reads_device_rows(c->p.mode);
+    if (direct && user->list)
+        list = user->list;
+    else if (user)
+        NB_CUDA(to_device(c->act_force, user_list, static_cast<size_t>(n_act) * sizeof(int32_t), c->s),
+                "active list upload");
     if (cfg.sym_sb > 0) {
         const long long *rows_general = nullptr;
         ForceConfig general{};
@@ -274,9 +304,15 @@ int force_internal(nbody_ctx *c, int64_t n_act, bool for_step = false, bool asce
         r = ensure_partials(c, force_partial_bytes(c->p.mode, cfg, n_act));
         if (r != NBODY_OK) return r;
         fused = for_step && force_partials_fused(c->p.mode, cfg);
-        NB_CUDA(force_launch(c->p.mode, c->J, c->n, c->act_force, n_act, c->eps2, cfg,
-                             c->f_acc, c->f_jerk, c->f_pot, c->partials, c->st, c->s, &launches, nullptr, !fused),
+        NB_CUDA(force_launch(c->p.mode, c->J, c->n, list, n_act, c->eps2, cfg, c->f_acc, c->f_jerk, c->f_pot,
+                             c->partials, c->st, c->s, &launches, nullptr, !fused && !direct),
                 "force kernel launch");
+        if (direct) {
+            NB_CUDA(force_out_launch(c->p.mode, static_cast<float *>(c->partials), cfg.split, n_act, c->f_acc,
+                                     c->f_jerk, c->f_pot, *user, c->s, &launches),
+                    "force reduction launch");
+            *user_done = true;
+        }
     }
     c->fused_split = fused ? cfg.split : 0;
     c->stats.kernel_launches += launches;
@@ -635,9 +671,8 @@ int nbody_init(nbody_ctx **out, int64_t n, const double *m, const double *x, con
         if (e_ != cudaSuccess) return bail(cuda_fail(e_, what)); \
     } while (0)
 
-    int dev = 0;
-    NB_INIT(cudaGetDevice(&dev), "cudaGetDevice");
-    NB_INIT(cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, dev), "SM count");
+    NB_INIT(cudaGetDevice(&c->dev), "cudaGetDevice");
+    NB_INIT(cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->dev), "SM count");
     const size_t nd = static_cast<size_t>(n);
     Arena dev_mem, host_mem;
     dev_mem.add(&c->state, 13 * nd * sizeof(double));
@@ -756,22 +791,28 @@ int nbody_force(nbody_ctx *c, const int32_t *active, int64_t n_act, double *acc,
     if (n_act > 0 && !active) return fail(NBODY_EINVAL, "nbody_force: null active list");
     if (!c->pred_valid) return fail(NBODY_ESTATE, "nbody_force: no prediction since the last correction");
     const size_t na = static_cast<size_t>(n_act);
-    NB_CUDA(to_device(c->act_force, active, na * sizeof(int32_t), c->s), "active list upload");
-    int r = force_internal(c, n_act, false, false);
+    ForceUser user{};
+    if (own_device_ptr(c, active, 4)) user.list = active;
+    // outputs that overlap one another are copied one after the other
+    if (!overlap(acc, 3 * na, jerk, 3 * na) && !overlap(acc, 3 * na, pot, na) && !overlap(jerk, 3 * na, pot, na)) {
+        if (own_device_ptr(c, acc, 8)) user.acc = acc;
+        if (own_device_ptr(c, jerk, 8)) user.jerk = jerk;
+        if (own_device_ptr(c, pot, 8)) user.pot = pot;
+    }
+    bool done = false;
+    int r = force_internal(c, n_act, false, false, active, &user, &done);
     if (r != NBODY_OK) return r;
     bool host_out = false;
-    if (acc) {
-        NB_CUDA(cudaMemcpyAsync(acc, c->f_acc, 3 * na * sizeof(double), cudaMemcpyDefault, c->s), "acc copy");
-        host_out |= !is_device_ptr(acc);
-    }
-    if (jerk) {
-        NB_CUDA(cudaMemcpyAsync(jerk, c->f_jerk, 3 * na * sizeof(double), cudaMemcpyDefault, c->s), "jerk copy");
-        host_out |= !is_device_ptr(jerk);
-    }
-    if (pot) {
-        NB_CUDA(cudaMemcpyAsync(pot, c->f_pot, na * sizeof(double), cudaMemcpyDefault, c->s), "pot copy");
-        host_out |= !is_device_ptr(pot);
-    }
+    auto copy_out = [&](double *to, const double *user_to, const double *from, size_t count) -> int {
+        if (!to || (done && user_to)) return NBODY_OK;
+        NB_CUDA(cudaMemcpyAsync(to, from, count * sizeof(double), cudaMemcpyDefault, c->s), "force copy");
+        host_out |= !is_device_ptr(to);
+        return NBODY_OK;
+    };
+    r = copy_out(acc, user.acc, c->f_acc, 3 * na);
+    if (r == NBODY_OK) r = copy_out(jerk, user.jerk, c->f_jerk, 3 * na);
+    if (r == NBODY_OK) r = copy_out(pot, user.pot, c->f_pot, na);
+    if (r != NBODY_OK) return r;
     if (host_out) {
         r = sync_and_check(c);
         if (r != NBODY_OK) return r;

@@ -86,8 +86,9 @@ __device__ __forceinline__ void rows_sums_x2(const float *jsm, const int stride_
 // `stride` floats each (STRIDE when it is positive, else stride_rt; x, y, z, m,
 // vx, vy, vz, and the lo parts of x, y, z in
 // compensated mode), or in the double-single mode four float4 arrays (x, m),
-// (x_lo, m_lo), v, v_lo.  T threads per row (a power of two; NT / T rows per
-// pass): thread `sub` of a row takes the groups of 4 entries 4 (g T + sub),
+// (x_lo, m_lo), v, v_lo.  T threads per row (T0, a power of two; with SHARE more in
+// a last pass that would leave threads idle, where one thread per row would take a
+// full pass's latency on a few warps; NT / T rows per pass): thread `sub` of a row takes the groups of 4 entries 4 (g T + sub),
 // g = 0, 1, ... (one entry g T + sub at a time in the double-single mode), so the
 // lanes of a warp read consecutive 16-byte words.  The packed pair term is that
 // of force_x2.cuh, folded every 128 terms into (hi, lo) (compensated) or an FP32
@@ -102,9 +103,10 @@ __device__ __forceinline__ void rows_sums_x2(const float *jsm, const int stride_
 // it matters: for the potential, or for a softening too small to keep its
 // zero terms finite.  Every thread of the block calls this function: it holds
 // block barriers.
-template <int MODE, int NT, int STRIDE = 0, bool POT = false, class LoadI, class LoadDS, class Store>
+template <int MODE, int NT, int STRIDE = 0, bool POT = false, bool SHARE = false, class LoadI, class LoadDS,
+          class Store>
 __device__ __forceinline__ void rows_force(const float *jsm, const int stride_rt, const int j0, const int L,
-                                           const int cnt, const int T, const float eps2, const float eps2_lo,
+                                           const int cnt, const int T0, const float eps2, const float eps2_lo,
                                            LoadI &&load_i, LoadDS &&load_ds, Store &&store,
                                            float (*wred)[7][2])
 {
@@ -113,11 +115,16 @@ __device__ __forceinline__ void rows_force(const float *jsm, const int stride_rt
     constexpr bool DSW = MODE == kModeComp || DSM;  // two-word sums
     const int stride = STRIDE > 0 ? STRIDE : stride_rt;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int rpp = NT / T;
-    const int TW = T < 32 ? T : 32;
     const f2_t E2 = f2_pack(eps2, eps2);
     const f2_t NEG3 = f2_pack(-3.0f, -3.0f);
+    int T = T0, rpp = NT / T0;
     for (int q0 = 0; q0 < cnt; q0 += rpp) {
+        if constexpr (SHARE) {  // the rows left for a last, partly filled pass share its threads (two groups
+            if (q0 > 0)         // of 4 j each at least)
+                while (2 * T * (cnt - q0) <= NT && 16 * T <= L) T <<= 1;
+            rpp = NT / T;
+        }
+        const int TW = T < 32 ? T : 32;
         const int rr = q0 + tid / T;
         const int sub = tid % T;
         const bool live = rr < cnt;

@@ -75,7 +75,7 @@ int occupancy(int mode, int threads, int ipt)
 }  // namespace
 
 int force_choose(int mode, int64_t n_act, int64_t n_pad, int sm_count, int req_threads, int req_ipt,
-                 int req_split, ForceConfig *cfg, int req_jsub, int64_t n_pairs)
+                 int req_split, ForceConfig *cfg, int req_jsub, int64_t n_pairs, bool any_rows)
 {
     if (n_pairs > 0 && req_threads == 0 && req_ipt == 0 && req_split <= 0 && req_jsub == 0 &&
         sym_plan(mode, n_act, n_pairs, sm_count, cfg))
@@ -85,7 +85,7 @@ int force_choose(int mode, int64_t n_act, int64_t n_pad, int sm_count, int req_t
     // the slice shape: one CTA per SM over its slice of the stream, for mid-size blocks when the
     // caller fixes no parameter and the slice fits shared memory
     if (NB_PACKED && (mode == kModePlain || mode == kModeComp) && req_threads == 0 && req_ipt == 0 &&
-        req_split <= 0 && req_jsub == 0 && n_act >= NB_SLICE_MIN_ROWS && n_act <= NB_SLICE_MAX_ROWS &&
+        req_split <= 0 && req_jsub == 0 && (any_rows || n_act >= NB_SLICE_MIN_ROWS) && n_act <= NB_SLICE_MAX_ROWS &&
         n_tiles >= kJSubMinTiles && slice_chunk(n_pad, sm_count) > 0) {
         cfg->threads = kSliceThreads;
         cfg->ipt = 1;

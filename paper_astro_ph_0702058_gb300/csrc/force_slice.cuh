@@ -3,11 +3,16 @@
 // entries [g c, (g+1) c), c = ceil(n_pad / CTAs) rounded up to 4.  It copies
 // its slice of every array into shared memory once, then sums the pair terms
 // of all of the block's rows over it (rows_force of block_rows.cuh: T threads
-// per row, T = 1 from 512 rows on, the packed pair term and 128-term folds,
-// the potential included) and writes one partial per row in the layout of the
-// j-range partials (range = CTA), which the two-dimensional reduction adds in
-// CTA order.  For mid-size blocks this replaces many short (i-block, j-range)
-// blocks by one evenly filled wave whose j are read from HBM or L2 once per SM.
+// per row, T = 1 from 512 rows on but for the rows of a last, partly filled pass,
+// the packed pair term and 128-term folds, the potential included) and writes one
+// partial per row in the layout of the j-range partials (range = CTA), which the
+// two-dimensional reduction adds in CTA order.  For mid-size blocks this replaces
+// many short (i-block, j-range) blocks by one evenly filled wave whose j are read
+// from HBM or L2 once per SM.  A last pass whose rows share its threads: 1594 rows
+// at n = 65536 compensated 151 -> 131 us per call.  For small blocks (a force on
+// its own; the block-step graph keeps 64 x 1, one tile per range) a row's j go to
+// up to 32 threads in every CTA instead of one thread per 256 j: one row at n =
+// 65536 32 -> 12 us per call, 32 rows 34 -> 15, 300 rows 58 -> 36 (plain).
 #pragma once
 
 #include "block_rows.cuh"
@@ -88,7 +93,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1) force_slice_kernel(const For
             if (DSW) d[static_cast<size_t>(7 + c) * na] = lw[c];
         }
     };
-    rows_force<MODE, kSliceThreads, SJ, true>(jsm, SJ, lo, L, na, T, P.eps2, 0.0f, load_i, no_ds, store, wred);
+    rows_force<MODE, kSliceThreads, SJ, true, true>(jsm, SJ, lo, L, na, T, P.eps2, 0.0f, load_i, no_ds, store, wred);
 }
 
 template <int MODE, int SJ>

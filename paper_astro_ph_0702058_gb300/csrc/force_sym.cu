@@ -165,6 +165,39 @@ __global__ void __launch_bounds__(256)
         pot[q] = t;
 }
 
+// Few rows with many j-ranges, for a caller's own buffers: the sums and their
+// order are those of reduce_partials_2d_kernel (8 rows x 32 lanes of one
+// component per block); each result goes to the context and to the caller's
+// device buffer in one kernel, where a copy each took ~2 us of a call's 35.
+template <int MODE>
+__global__ void __launch_bounds__(256)
+    force_out_kernel(const float *__restrict__ part, const int split, const int n_act, double *__restrict__ acc,
+                     double *__restrict__ jerk, double *__restrict__ pot, const ForceUser u)
+{
+    constexpr int NC = MODE == kModeComp ? 14 : 7, R = 8, L = 32;
+    __shared__ float2 sh[L][R];
+    const int row = threadIdx.x % R, w = threadIdx.x / R;
+    const int c = blockIdx.y;
+    const int q = blockIdx.x * R + row;
+    float h = 0.0f, l = 0.0f;
+    if (q < n_act)
+#pragma unroll 4
+        for (int sp = w; sp < split; sp += L) {
+            const float *b = part + (static_cast<size_t>(sp) * NC + c) * n_act + q;
+            ds2_add(h, l, b[0], MODE == kModeComp ? b[static_cast<size_t>(7) * n_act] : 0.0f);
+        }
+    sh[w][row] = make_float2(h, l);
+    __syncthreads();
+    if (w != 0 || q >= n_act) return;
+#pragma unroll
+    for (int k = 1; k < L; ++k) ds2_add(h, l, sh[k][row].x, sh[k][row].y);
+    const double t = static_cast<double>(h) + static_cast<double>(l);
+    const size_t e = c < 6 ? 3 * static_cast<size_t>(q) + c % 3 : static_cast<size_t>(q);
+    (c < 3 ? acc : c < 6 ? jerk : pot)[e] = t;
+    double *const o = c < 3 ? u.acc : c < 6 ? u.jerk : u.pot;
+    if (o) o[e] = t;
+}
+
 // Scratch of a context: the general path's row count, the marks, the
 // compaction's counts, then the rows and the other particles (together n).
 struct SymScratch {
@@ -357,6 +390,16 @@ cudaError_t force_sym_launch(int mode, const JStream &js, int64_t n, const int32
     if (e != cudaSuccess) return e;
     ++*launches;
     return force_sym_reduce_launch(mode, P.part, cfg.split, n_act, acc, jerk, pot, P.skip, false, s, launches);
+}
+
+cudaError_t force_out_launch(int mode, const float *part, int split, int64_t n_act, double *acc, double *jerk,
+                             double *pot, const ForceUser &u, cudaStream_t s, int64_t *launches)
+{
+    const int na = static_cast<int>(n_act);
+    auto *kernel = mode == kModeComp ? force_out_kernel<kModeComp> : force_out_kernel<kModePlain>;
+    kernel<<<dim3((na + 7) / 8, 7), 256, 0, s>>>(part, split, na, acc, jerk, pot, u);
+    ++*launches;
+    return cudaGetLastError();
 }
 
 cudaError_t force_sym_reduce_launch(int mode, const float *part, int slots, int64_t n_act, double *acc, double *jerk,

@@ -128,9 +128,12 @@ extern int g_skip_first_copy;  // test hook: force kernels leave out their first
 // req_* > 0 override the automatic choice.
 // req_jsub: 0 automatic, 1 one thread per row, 4 four (256 threads, one i each).
 // n_pairs: the particles the block belongs to when it may take the force by
-// unordered pairs (force_sym_launch), else 0.
+// unordered pairs (force_sym_launch), else 0.  any_rows: the slice shape also
+// for small blocks (a force on its own, which need not take the shape of the
+// block-step graph).
 int force_choose(int mode, int64_t n_act, int64_t n_pad, int sm_count, int req_threads,
-                 int req_ipt, int req_split, ForceConfig *cfg, int req_jsub = 0, int64_t n_pairs = 0);
+                 int req_ipt, int req_split, ForceConfig *cfg, int req_jsub = 0, int64_t n_pairs = 0,
+                 bool any_rows = false);
 // Whether this mode's force kernels honour ForceParams::n_act_dev (the packed kernels).
 bool force_reads_device_rows(int mode);
 // Scratch bytes needed for partial sums when cfg.split > 1 (0 otherwise).
@@ -170,6 +173,15 @@ cudaError_t force_sym_launch(int mode, const JStream &js, int64_t n, const int32
 cudaError_t force_sym_reduce_launch(int mode, const float *part, int slots, int64_t n_act, double *acc, double *jerk,
                                     double *pot, const long long *rows_general, bool general, cudaStream_t s,
                                     int64_t *launches);
+
+// A caller's device buffers for a force, where a kernel may use them as they are (NULL: not).
+struct ForceUser {
+    const int32_t *list;
+    double *acc, *jerk, *pot;
+};
+// Plain and compensated partial sums of many ranges (split >= 8) to acc, jerk and pot and to u's buffers.
+cudaError_t force_out_launch(int mode, const float *part, int split, int64_t n_act, double *acc, double *jerk,
+                             double *pot, const ForceUser &u, cudaStream_t s, int64_t *launches);
 
 // ---- force_ds.cu ----
 int force_occupancy_ds();

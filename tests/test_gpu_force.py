@@ -238,3 +238,31 @@ def test_force_full_size_bench_launch(torch, mode):
     print(f"\nN=2^20 {mode} (4096 rows): " + ", ".join(f"{k} max {v.max():.2e} p50 {np.median(v):.2e} "
                                           f"within {REL[mode]:.0e}: {np.mean(v <= REL[mode]):.3f}"
                                           for k, v in e_all.items()))
+
+
+@pytest.mark.parametrize("mode", ["plain", "comp"])
+@pytest.mark.parametrize("n,n_act", [(16384, 1), (16384, 17), (20001, 511), (65536, 33), (65536, 513), (65536, 1025),
+                                     (65536, 1594), (70000, 300)])
+def test_force_small_blocks_and_device_buffers(torch, mode, n, n_act):
+    """Small blocks in the slice shape and last passes of a few rows; lists and outputs in device memory are used as
+    they are (overlapping outputs are copied one after the other), with the results of host buffers bit for bit."""
+    m, x, v = plummer_sphere(n, 6)
+    act = active_subset(n, n_act, 17)
+    with _sim(m, x, v, EPS2, mode) as sim:
+        sim.predict(0.0)
+        host = gpu_force(sim, act)
+        assert sim.stats()["last_threads"] == 512
+        rows = torch.from_numpy(act).cuda()
+        out = [torch.full((n_act, 3), -7.0, dtype=torch.float64, device="cuda") for _ in range(2)]
+        out.append(torch.full((n_act,), -7.0, dtype=torch.float64, device="cuda"))
+        sim.force(rows, acc=out[0], jerk=out[1], pot=out[2])
+        both = torch.zeros((n_act, 3), dtype=torch.float64, device="cuda")
+        from paper_astro_ph_0702058_gb300._lib import nbody_force
+        nbody_force(sim.handle, rows, n_act, both, both, None)  # the same buffer twice: the later output stays
+        sim.correct(rows)  # the context's own copy of the forces is there
+    for h, d in zip(host, out):
+        assert np.array_equal(h, d.cpu().numpy())
+    assert np.array_equal(both.cpu().numpy(), host[1])
+    idx = np.linspace(0, n_act - 1, min(n_act, 300)).astype(int)
+    check_force(mode, m, x, v, EPS2, act[idx], tuple(h[idx] for h in host), oracle.force(m, x, v, EPS2, act[idx]),
+                f"small n={n} n_act={n_act}")
