@@ -205,7 +205,7 @@ __device__ __forceinline__ void rows_force(const float *jsm, const int stride_rt
 // The corrector of Sect. 2 and Eq. (timestep) for rows q < cnt at tick tb: row q
 // is particle idx[q], its forces fh[q][0..5] (+ fl[q][0..5], two-word sums).  Up
 // to 8 rows run in warp 0 with 4 lanes per row (lanes 0-2 one component each,
-// then the four norms of Eq. (timestep) one per lane: the operations of
+// then the four squared norms of Eq. (timestep) one per lane: the operations of
 // correct_row, in parallel); more rows one per thread q < cnt.  GB300's FP64
 // unit is one per SM and takes ~19 cycles per warp instruction whatever the
 // number of active lanes, so rows are packed into as few warps as possible.
@@ -259,12 +259,12 @@ __device__ __forceinline__ void rows_correct(const State &S, const int *idx, con
             double w[3];
 #pragma unroll
             for (int c = 0; c < 3; ++c) w[c] = part == 0 ? f[c] : part == 1 ? f[3 + c] : part == 2 ? u[c][0] : u[c][1];
-            const double nrm = norm3(w);  // |ap|, |kp|, |a^(2)|, |a^(3)| on lanes 0-3
-            const double an = __shfl_sync(0xffffffffu, nrm, base), kn = __shfl_sync(0xffffffffu, nrm, base + 1);
-            const double a2n = __shfl_sync(0xffffffffu, nrm, base + 2);
-            const double a3n = __shfl_sync(0xffffffffu, nrm, base + 3);
+            const double nrm = square3(w);  // |ap|^2, |kp|^2, |a^(2)|^2, |a^(3)|^2 on lanes 0-3
+            const double aa = __shfl_sync(0xffffffffu, nrm, base), kk = __shfl_sync(0xffffffffu, nrm, base + 1);
+            const double s2 = __shfl_sync(0xffffffffu, nrm, base + 2);
+            const double t2 = __shfl_sync(0xffffffffu, nrm, base + 3);
             if (live && part == 0) {
-                const int l_new = corr_level(an, kn, a2n, a3n, eta, lmin, lmax, ld_state<true>(S.level + r),
+                const int l_new = corr_level(aa, kk, s2, t2, eta, lmin, lmax, ld_state<true>(S.level + r),
                                              static_cast<int64_t>(tb), finite, st);
                 S.t[r] = static_cast<int64_t>(tb);
                 S.level[r] = static_cast<int8_t>(l_new);

@@ -163,18 +163,49 @@ __device__ __forceinline__ void corr_dim(const double x, const double v, const d
     a2e = a2 + a3 * d.dt;  // a^(2) at the end of the step
 }
 
-// Eq. (timestep) from |a|, |k|, |a^(2)|, |a^(3)| at the end of the step, then the
-// level rule: shrink at once, grow one level when the new time allows.  Raises
-// the non-finite and dt_min flags; returns the new level.
-__device__ __forceinline__ int corr_level(const double an, const double kn, const double a2n, const double a3n,
+__device__ __forceinline__ double square3(const double *u) { return __fma_rn(u[2], u[2], __fma_rn(u[1], u[1], u[0] * u[0])); }
+
+// (a b)^(1/2) for a, b >= 0; products far from the middle of the range take the
+// two roots one by one.
+__device__ __forceinline__ double sqrt_product(const double a, const double b)
+{
+    const double p = a * b;
+    const unsigned int ex = (static_cast<unsigned int>(__double2hiint(p)) >> 20) - 123u;
+    return ex <= 1800u ? p * rsqrt_f64(p) : sqrt(a) * sqrt(b);
+}
+
+// Level of Eq. (timestep)'s dt = [eta (|a||a2| + |k|^2) / (|k||a3| + |a2|^2)]^(1/2)
+// (as level_of) from the squared norms.  A level only needs floor(log2 dt): with
+// numerator N and denominator D, floor(log2 (N / D)) is the difference of their
+// exponents, less one where N's fraction is the smaller, and dt's exponent half of
+// that, rounded down.  So neither a division nor the outer root is taken, and two
+// roots of products replace the four norms': ~30 operations on the FP64 pipe (one
+// unit per SM, ~64 cycles each in a dependent chain) where the four norms, the
+// division and the root took over 100.
+__device__ __forceinline__ int crit_level(const double a2, const double k2, const double s2, const double t2,
+                                          const double eta, const int lmin, const int lmax, bool *clamped)
+{
+    const double num = eta * (sqrt_product(a2, s2) + k2), den = sqrt_product(k2, t2) + s2;
+    const long long nb = __double_as_longlong(num), db = __double_as_longlong(den);
+    const int ne = static_cast<int>(nb >> 52), de = static_cast<int>(db >> 52);  // (negative: sign set)
+    if (ne < 1 || ne > 2046 || de < 1 || de > 2046)  // zero, subnormal, infinite, NaN
+        return level_of(den == 0.0 ? static_cast<double>(INFINITY) : sqrt(num / den), lmin, lmax, clamped);
+    const long long frac = (1ll << 52) - 1;
+    const int lq = ne - de - ((nb & frac) < (db & frac) ? 1 : 0);
+    const int L = -(lq >> 1);
+    *clamped = L > lmax;
+    return L < lmin ? lmin : L > lmax ? lmax : L;
+}
+
+// Eq. (timestep) from |a|^2, |k|^2, |a^(2)|^2, |a^(3)|^2 at the end of the step,
+// then the level rule: shrink at once, grow one level when the new time allows.
+// Raises the non-finite and dt_min flags; returns the new level.
+__device__ __forceinline__ int corr_level(const double a2, const double k2, const double s2, const double t2,
                                           const double eta, const int lmin, const int lmax, const int l_old,
                                           const int64_t t_new, const bool finite, DevStatus *st)
 {
-    const double num = an * a2n + kn * kn;
-    const double den = kn * a3n + a2n * a2n;
-    const double dtc = den == 0.0 ? static_cast<double>(INFINITY) : sqrt(eta * num / den);
     bool clamped = false;
-    const int lc = level_of(dtc, lmin, lmax, &clamped);
+    const int lc = crit_level(a2, k2, s2, t2, eta, lmin, lmax, &clamped);
     int l_new;
     if (!finite || lc < 0) {
         l_new = lmax;
@@ -219,7 +250,7 @@ __device__ __forceinline__ int correct_row(const State &S, const int64_t i, cons
         S.k[c][i] = kp[c];
     }
     // Eq. (timestep) with end-of-step quantities.
-    const int l_new = corr_level(norm3(ap), norm3(kp), norm3(a2e), norm3(a3), eta, lmin, lmax,
+    const int l_new = corr_level(square3(ap), square3(kp), square3(a2e), square3(a3), eta, lmin, lmax,
                                  ld_state<CG>(S.level + i), t_new, finite, st);
     S.t[i] = t_new;
     S.level[i] = static_cast<int8_t>(l_new);
