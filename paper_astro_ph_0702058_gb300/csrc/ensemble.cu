@@ -29,8 +29,7 @@
 #include <vector>
 
 #include "arena.h"
-#include "force_x2.cuh"
-#include "step_impl.cuh"
+#include "block_rows.cuh"
 
 namespace nb {
 
@@ -48,13 +47,14 @@ struct EnsDev {
     int32_t *act;          // [n_tot] block lists: cluster c's at act[off[c] ..]
     long long *item_pfx;   // [n_cl + 1] exclusive prefix of work items
     long long *row_pfx;    // [n_cl + 1] exclusive prefix of active rows
+    long long *slot_pfx;   // [n_cl] exclusive prefix of partial sums (rows x j-ranges)
     int *nsplit;           // [n_cl] j-ranges this step
     int *tpr;              // [n_cl] tiles per j-range
     unsigned int *work;    // work-item counter of the force kernel
     int *live;             // [2]: clusters with a block this step, batched steps with work
     long long *blocks;     // [n_cl] block steps taken per cluster
     long long *pairs;      // [n_cl] pair interactions evaluated per cluster
-    float *part;           // partial sums [row][s_max][7 or 14]
+    float *part;           // partial sums: row q of cluster c, range s at (slot_pfx[c] + q nsplit[c] + s) x 7 or 14
     DevStatus *st;
 };
 
@@ -67,38 +67,70 @@ __device__ __forceinline__ unsigned long long ens_due(const State &S, int64_t i,
     return static_cast<unsigned long long>(S.t[i] + (int64_t(1) << (lmax - S.level[i])));
 }
 
-// Block scheduler of Sect. 2 for one cluster per block.
-__global__ void ens_schedule_kernel(const EnsDev E, long long t_end, int lmax)
+// Block scheduler of Sect. 2 for one cluster per block of kSchedThreads.  Up to
+// kSchedKeep particles per thread keep their due tick in registers between the
+// minimum and the ordered list (clusters of up to 8192; further ones read it
+// again); the list's offsets come from one scan over the warps' counts of every
+// round.  256 threads with two passes over the state and a barrier pair per round
+// took 26.7 us per batched step (128 clusters of 256 to 8191).
+constexpr int kSchedThreads = 1024, kSchedKeep = 8;
+
+__global__ void __launch_bounds__(kSchedThreads) ens_schedule_kernel(const EnsDev E, long long t_end, int lmax)
 {
     __shared__ unsigned long long shm[32];
-    __shared__ int warp_tot[32];
+    __shared__ int tot[kSchedKeep][32];
     const int c = blockIdx.x;
     const int64_t lo = E.off[c], hi = E.off[c + 1];
-    unsigned long long m = ~0ull;
-    for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-        const unsigned long long d = ens_due(E.S, i, lmax);
-        m = d < m ? d : m;
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    unsigned long long d[kSchedKeep], m = ~0ull;
+#pragma unroll
+    for (int k = 0; k < kSchedKeep; ++k) {
+        const int64_t i = lo + k * kSchedThreads + threadIdx.x;
+        d[k] = i < hi ? ens_due(E.S, i, lmax) : ~0ull;
+        m = d[k] < m ? d[k] : m;
+    }
+    for (int64_t i = lo + kSchedKeep * kSchedThreads + threadIdx.x; i < hi; i += kSchedThreads) {
+        const unsigned long long t = ens_due(E.S, i, lmax);
+        m = t < m ? t : m;
     }
     m = block_reduce(m, MinOp(), shm, ~0ull);
     if (static_cast<long long>(m) > t_end) {
         if (threadIdx.x == 0) E.n_act[c] = 0;
         return;
     }
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
     int count = 0;
-    for (int64_t base = lo; base < hi; base += blockDim.x) {
-        const int64_t i = base + threadIdx.x;
-        const bool hit = i < hi && ens_due(E.S, i, lmax) == m;
-        const unsigned mask = __ballot_sync(0xffffffffu, hit);
-        if (l == 0) warp_tot[w] = __popc(mask);
-        __syncthreads();
-        int before = 0, round = 0;
-        for (int k = 0; k < nw; ++k) {
-            if (k < w) before += warp_tot[k];
-            round += warp_tot[k];
+    for (int64_t base = lo; base < hi; base += kSchedKeep * kSchedThreads) {
+        unsigned hit[kSchedKeep];
+#pragma unroll
+        for (int k = 0; k < kSchedKeep; ++k) {
+            if (base > lo) {
+                const int64_t i = base + k * kSchedThreads + threadIdx.x;
+                d[k] = i < hi ? ens_due(E.S, i, lmax) : ~0ull;
+            }
+            hit[k] = __ballot_sync(0xffffffffu, d[k] == m);
+            if (l == 0) tot[k][w] = __popc(hit[k]);
         }
-        if (hit) E.act[lo + count + before + __popc(mask & ((1u << l) - 1u))] = static_cast<int32_t>(i);
-        count += round;
+        __syncthreads();
+        int before[kSchedKeep], total[kSchedKeep];  // of this warp in each round, and of the round
+#pragma unroll
+        for (int k = 0; k < kSchedKeep; ++k) {
+            const int v = tot[k][l];
+            int s = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, s, o);
+                if (l >= o) s += u;
+            }
+            before[k] = __shfl_sync(0xffffffffu, s - v, w);
+            total[k] = __shfl_sync(0xffffffffu, s, 31);
+        }
+#pragma unroll
+        for (int k = 0; k < kSchedKeep; ++k) {
+            if (hit[k] >> l & 1u)
+                E.act[lo + count + before[k] + __popc(hit[k] & ((1u << l) - 1u))] =
+                    static_cast<int32_t>(base + k * kSchedThreads + threadIdx.x);
+            count += total[k];
+        }
         __syncthreads();
     }
     if (threadIdx.x == 0) {
@@ -109,24 +141,41 @@ __global__ void ens_schedule_kernel(const EnsDev E, long long t_end, int lmax)
     }
 }
 
-// Work items and row offsets of this step (one block, fixed summation order).
-__global__ void ens_plan_kernel(const EnsDev E, int rows_per_item, int tiles_per_range)
+// j-ranges of a block of na rows in a cluster of n particles: ranges of
+// tiles_per_range tiles, at most s_max; with `share` single tiles where the partial
+// sums of s_max n rows and ranges hold them (na <= n / 4 of 8192 particles: 32
+// ranges), else as many ranges as they hold.  A step's blocks hold some tens of rows
+// per cluster, its time is that of its last items, and long items picked up late
+// were most of it (128 clusters: 0.24 Tpairs/s with ranges of up to 4 tiles).  The
+// rule looks at the cluster alone, so its arithmetic does not depend on the others
+// of the batch.
+constexpr int kEnsMostRanges = 64;
+__device__ __forceinline__ int ens_ranges(const int na, const int64_t n, const int tiles_per_range, const int s_max,
+                                          const bool share, int &tpr)
 {
-    __shared__ long long s_items[1024], s_rows[1024];
-    __shared__ int s_live[1024];
+    const int ntl = static_cast<int>((n + kJTile - 1) / kJTile);
+    int S = min((ntl + tiles_per_range - 1) / tiles_per_range, s_max);
+    if (share) S = max(S, static_cast<int>(min(static_cast<int64_t>(min(ntl, kEnsMostRanges)), s_max * n / na)));
+    tpr = (ntl + S - 1) / S;
+    return (ntl + tpr - 1) / tpr;
+}
+
+// Work items, row and partial-sum offsets of this step (one block, fixed order).
+__global__ void ens_plan_kernel(const EnsDev E, int rows_per_item, int tiles_per_range, bool share)
+{
+    __shared__ long long s_items[32], s_rows[32], s_slots[32];
+    __shared__ int s_live[32];
     const int t = threadIdx.x, nt = blockDim.x;
     const int chunk = (E.n_cl + nt - 1) / nt;
     const int c0 = t * chunk, c1 = min(c0 + chunk, E.n_cl);
-    long long items = 0, rows = 0;
+    long long items = 0, rows = 0, slots = 0;
     int live = 0;
     for (int c = c0; c < c1; ++c) {
         const int na = E.n_act[c];
         int S = 0, tpr = 1;
         if (na > 0) {
-            const int ntl = static_cast<int>((E.off[c + 1] - E.off[c] + kJTile - 1) / kJTile);
-            S = min((ntl + tiles_per_range - 1) / tiles_per_range, E.s_max);
-            tpr = (ntl + S - 1) / S;
-            S = (ntl + tpr - 1) / tpr;
+            S = ens_ranges(na, E.off[c + 1] - E.off[c], tiles_per_range, E.s_max, share, tpr);
+            slots += static_cast<long long>(na) * S;
             items += static_cast<long long>((na + rows_per_item - 1) / rows_per_item) * S;
             rows += na;
             live += 1;
@@ -134,36 +183,60 @@ __global__ void ens_plan_kernel(const EnsDev E, int rows_per_item, int tiles_per
         E.nsplit[c] = S;
         E.tpr[c] = tpr;
     }
-    s_items[t] = items;
-    s_rows[t] = rows;
-    s_live[t] = live;
-    __syncthreads();
-    if (t == 0) {  // sequential exclusive scan over the (<= 1024) per-thread sums
-        long long ai = 0, ar = 0;
-        int al = 0;
-        for (int k = 0; k < nt; ++k) {
-            const long long xi = s_items[k], xr = s_rows[k];
-            s_items[k] = ai;
-            s_rows[k] = ar;
-            ai += xi;
-            ar += xr;
-            al += s_live[k];
+    // exclusive scan over the 1024 threads' sums (one thread adding them in turn took 14 of the kernel's 17.6 us)
+    const int w = t >> 5, l = t & 31;
+    long long xi = items, xr = rows, xs = slots;
+    int xl = live;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long ui = __shfl_up_sync(0xffffffffu, xi, o), ur = __shfl_up_sync(0xffffffffu, xr, o);
+        const long long us = __shfl_up_sync(0xffffffffu, xs, o);
+        const int ul = __shfl_up_sync(0xffffffffu, xl, o);
+        if (l >= o) {
+            xi += ui;
+            xr += ur;
+            xs += us;
+            xl += ul;
         }
-        E.item_pfx[E.n_cl] = ai;
-        E.row_pfx[E.n_cl] = ar;
+    }
+    if (l == 31) {
+        s_items[w] = xi;
+        s_rows[w] = xr;
+        s_slots[w] = xs;
+        s_live[w] = xl;
+    }
+    __syncthreads();
+    long long bi = 0, br = 0, bs = 0;
+    int al = 0;
+    for (int k = 0; k < nt / 32; ++k) {
+        if (k == w) {
+            bi += xi - items;
+            br += xr - rows;
+            bs += xs - slots;
+        } else if (k < w) {
+            bi += s_items[k];
+            br += s_rows[k];
+            bs += s_slots[k];
+        }
+        al += s_live[k];
+    }
+    if (t == nt - 1) {
+        E.item_pfx[E.n_cl] = bi + items;
+        E.row_pfx[E.n_cl] = br + rows;
         E.live[0] = al;
         if (al > 0) E.live[1] += 1;
         E.work[0] = 0u;
     }
-    __syncthreads();
-    long long pi = s_items[t], pr = s_rows[t];
+    long long pi = bi, pr = br, ps = bs;
     for (int c = c0; c < c1; ++c) {
         E.item_pfx[c] = pi;
         E.row_pfx[c] = pr;
+        E.slot_pfx[c] = ps;
         const int na = E.n_act[c];
         if (na > 0) {
             pi += static_cast<long long>((na + rows_per_item - 1) / rows_per_item) * E.nsplit[c];
             pr += na;
+            ps += static_cast<long long>(na) * E.nsplit[c];
         }
     }
 }
@@ -196,14 +269,16 @@ __global__ void ens_predict_kernel(const EnsDev E, double tick, int comp)
         const float hx = d2f_rn(xp[0]), hy = d2f_rn(xp[1]), hz = d2f_rn(xp[2]);
         const float hm = d2f_rn(E.S.m[i]);
         const float hvx = d2f_rn(vp[0]), hvy = d2f_rn(vp[1]), hvz = d2f_rn(vp[2]);
-        E.J.posm[j] = make_float4(hx, hy, hz, hm);
-        E.J.vel[j] = make_float4(hvx, hvy, hvz, 0.f);
+        if (!NB_PACKED) {  // the scalar force kernel's streams
+            E.J.posm[j] = make_float4(hx, hy, hz, hm);
+            E.J.vel[j] = make_float4(hvx, hvy, hvz, 0.f);
+        }
         float lx = 0.f, ly = 0.f, lz = 0.f;
         if (comp) {
             lx = d2f_rn(xp[0] - f2d(hx));
             ly = d2f_rn(xp[1] - f2d(hy));
             lz = d2f_rn(xp[2] - f2d(hz));
-            E.J.poslo[j] = make_float4(lx, ly, lz, 0.f);
+            if (!NB_PACKED) E.J.poslo[j] = make_float4(lx, ly, lz, 0.f);
         }
         float *a = E.J.soa + j;
         const int64_t np = E.J.n_pad;
@@ -222,9 +297,13 @@ __global__ void ens_predict_kernel(const EnsDev E, double tick, int comp)
     }
 }
 
-// Persistent force blocks over the work list of this step.
+// Persistent force blocks over the work list of this step.  share: an item of few
+// rows gives each of them T = 2, 4, .. 32 threads, which take groups of 4 j in turn
+// (rows_sums_x2) and add their sums in a butterfly: most blocks of a cluster hold
+// fewer rows than an item, and an item's time is one thread's j (128 clusters to
+// t = 1/64: the force 22.0 -> 9.4 ms of the run).
 template <int MODE, int NT, int IPT>
-__global__ void __launch_bounds__(NT) ens_force_kernel(const EnsDev E, const float eps2)
+__global__ void __launch_bounds__(NT) ens_force_kernel(const EnsDev E, const float eps2, const bool share)
 {
     constexpr int NARR = (MODE == kModeComp) ? 3 : 2;
     constexpr int NC = (MODE == kModeComp) ? 14 : 7;
@@ -262,6 +341,12 @@ __global__ void __launch_bounds__(NT) ens_force_kernel(const EnsDev E, const flo
         }
     };
     const long long W = E.item_pfx[E.n_cl];
+    // every `stride`-th prefix in shared memory: an item's cluster is found there (and by a few loads among more
+    // than kPfx clusters), not by a chain of loads from L2
+    constexpr int kPfx = 128;
+    __shared__ long long s_pfx[kPfx];
+    const int stride = (E.n_cl + kPfx - 1) / kPfx, n_pfx = (E.n_cl + stride - 1) / stride;
+    for (int k = tid; k < n_pfx; k += NT) s_pfx[k] = E.item_pfx[k * stride];
     unsigned int g = 0;  // tiles this block has consumed: buffer g & 1, phase (g >> 1) & 1
     for (;;) {
         if (tid == 0) s_w = static_cast<long long>(atomicAdd(E.work, 1u));
@@ -269,7 +354,14 @@ __global__ void __launch_bounds__(NT) ens_force_kernel(const EnsDev E, const flo
         const long long w = s_w;
         __syncthreads();
         if (w >= W) break;
-        int lo = 0, hi = E.n_cl;
+        int lo = 0, hi = n_pfx;
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (s_pfx[mid] <= w) lo = mid;
+            else hi = mid;
+        }
+        hi = min(E.n_cl, (lo + 1) * stride);
+        lo *= stride;
         while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
             if (E.item_pfx[mid] <= w) lo = mid;
@@ -284,12 +376,20 @@ __global__ void __launch_bounds__(NT) ens_force_kernel(const EnsDev E, const flo
         const int ntl = static_cast<int>((E.off[c + 1] - roff + kJTile - 1) / kJTile);
         const int t_begin = s * E.tpr[c];
         const int t_end = min(t_begin + E.tpr[c], ntl);
+        const int64_t jt0 = jo / kJTile;
+        if (tid == 0 && t_begin < t_end) issue(jt0 + t_begin, g & 1);  // while the rows are read
 
         float4 xi[IPT], vi[IPT], li[IPT];
         int gi[IPT];
+        int T = 1;  // threads per row
+        if (kPacked && IPT == 1 && share) {
+            const int left = min(NT, nact - blk * NT);
+            while (T < 32 && 2 * T * left <= NT) T <<= 1;
+        }
+        const int row = tid / T, sub = tid % T;
 #pragma unroll
         for (int u = 0; u < IPT; ++u) {
-            const int q = (blk * IPT + u) * NT + tid;
+            const int q = (blk * IPT + u) * NT + row;
             int jidx = -1;
             if (q < nact) {
                 const int64_t i = E.act[roff + q];
@@ -302,9 +402,18 @@ __global__ void __launch_bounds__(NT) ens_force_kernel(const EnsDev E, const flo
             }
             gi[u] = jidx;
             const int64_t l = jidx >= 0 ? jidx : jo;
-            xi[u] = E.J.posm[l];
-            vi[u] = E.J.vel[l];
-            li[u] = (MODE == kModeComp) ? E.J.poslo[l] : make_float4(0.f, 0.f, 0.f, 0.f);
+            if constexpr (kPacked) {
+                const float *a = E.J.soa + l;
+                const int64_t np = E.J.n_pad;
+                xi[u] = make_float4(a[0], a[np], a[2 * np], 0.f);
+                vi[u] = make_float4(a[4 * np], a[5 * np], a[6 * np], 0.f);
+                li[u] = (MODE == kModeComp) ? make_float4(a[7 * np], a[8 * np], a[9 * np], 0.f)
+                                            : make_float4(0.f, 0.f, 0.f, 0.f);
+            } else {
+                xi[u] = E.J.posm[l];
+                vi[u] = E.J.vel[l];
+                li[u] = (MODE == kModeComp) ? E.J.poslo[l] : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
         }
         I2 I[IPT];
         if constexpr (kPacked) {
@@ -329,9 +438,7 @@ __global__ void __launch_bounds__(NT) ens_force_kernel(const EnsDev E, const flo
                 tot[u][k] = 0.0f;
                 lo_[u][k] = 0.0f;
             }
-        const int64_t jt0 = jo / kJTile;
         bool ok = true;
-        if (tid == 0 && t_begin < t_end) issue(jt0 + t_begin, g & 1);
         for (int t = t_begin; t < t_end; ++t, ++g) {
             const int b = g & 1;
             if (tid == 0 && t + 1 < t_end) issue(jt0 + t + 1, b ^ 1);
@@ -345,10 +452,20 @@ __global__ void __launch_bounds__(NT) ens_force_kernel(const EnsDev E, const flo
 #pragma unroll
                 for (int u = 0; u < IPT; ++u)
                     self_tile |= static_cast<unsigned>(gi[u] - j0) < static_cast<unsigned>(kJTile);
-                if (self_tile)
+                if (T > 1) {
+                    if constexpr (IPT == 1) {
+                        if (__any_sync(0xffffffffu, self_tile))
+                            rows_sums_x2<MODE, true, kJTile, true>(soa[b].a[0], kJTile, j0, kJTile / 4 / T, T, sub,
+                                                                   I[0], gi[0], E2, NEG3, tot[0], lo_[0]);
+                        else
+                            rows_sums_x2<MODE, false, kJTile, true>(soa[b].a[0], kJTile, j0, kJTile / 4 / T, T, sub,
+                                                                    I[0], gi[0], E2, NEG3, tot[0], lo_[0]);
+                    }
+                } else if (self_tile) {
                     tile_sums_x2<MODE, IPT, PF, true>(soa[b], j0, I, gi, E2, NEG3, tot, lo_);
-                else
+                } else {
                     tile_sums_x2<MODE, IPT, PF, false>(soa[b], j0, I, gi, E2, NEG3, tot, lo_);
+                }
                 if (__syncthreads_or(!ok)) {
                     if (tid == 0) {
                         mbar_wait_bounded(&bar[b], (g >> 1) & 1);
@@ -379,11 +496,24 @@ __global__ void __launch_bounds__(NT) ens_force_kernel(const EnsDev E, const flo
                 return;
             }
         }
+        if constexpr (IPT == 1) {
+            for (int o = 1; o < T; o <<= 1) {
+#pragma unroll
+                for (int k = 0; k < 7; ++k) {
+                    const float h2 = __shfl_xor_sync(0xffffffffu, tot[0][k], o);
+                    const float l2 = __shfl_xor_sync(0xffffffffu, lo_[0][k], o);
+                    if (MODE == kModeComp)
+                        ds2_add(tot[0][k], lo_[0][k], h2, l2);
+                    else
+                        tot[0][k] = __fadd_rn(tot[0][k], h2);
+                }
+            }
+        }
 #pragma unroll
         for (int u = 0; u < IPT; ++u) {
-            const int q = (blk * IPT + u) * NT + tid;
-            if (q >= nact) continue;
-            float *base = E.part + ((static_cast<size_t>(E.row_pfx[c] + q) * E.s_max) + s) * NC;
+            const int q = (blk * IPT + u) * NT + row;
+            if (q >= nact || sub != 0) continue;
+            float *base = E.part + (static_cast<size_t>(E.slot_pfx[c]) + static_cast<size_t>(q) * S + s) * NC;
 #pragma unroll
             for (int k = 0; k < 7; ++k) {
                 base[k] = tot[u][k];
@@ -391,25 +521,6 @@ __global__ void __launch_bounds__(NT) ens_force_kernel(const EnsDev E, const flo
             }
         }
     }
-}
-
-// Sums a row's j-range partials in ascending range order, as double-single
-// pairs on the FP32 pipe (ds2_add; GB300's FP64 unit is narrow), then hi + lo in
-// FP64.  With one range the result is the range's hi + lo, as the
-// single-system kernel writes it.
-template <int NC>
-__device__ __forceinline__ void ens_row_sums(const EnsDev &E, long long r, int S, double (&f)[7])
-{
-    float h[7], l[7];
-#pragma unroll
-    for (int k = 0; k < 7; ++k) h[k] = l[k] = 0.0f;
-    for (int s = 0; s < S; ++s) {
-        const float *base = E.part + ((static_cast<size_t>(r) * E.s_max) + s) * NC;
-#pragma unroll
-        for (int k = 0; k < 7; ++k) ds2_add(h[k], l[k], base[k], NC == 14 ? base[7 + k] : 0.0f);
-    }
-#pragma unroll
-    for (int k = 0; k < 7; ++k) f[k] = static_cast<double>(h[k]) + static_cast<double>(l[k]);
 }
 
 __device__ __forceinline__ int ens_row_cluster(const EnsDev &E, long long r)
@@ -423,31 +534,64 @@ __device__ __forceinline__ int ens_row_cluster(const EnsDev &E, long long r)
     return lo;
 }
 
-template <int NC>
-__global__ void ens_correct_kernel(const EnsDev E, double tick, double eta, int lmin, int lmax)
+// A block of kRowLanes warps takes 32 active rows: the warps add a row's j-range
+// partials (warp w ranges w, w + kRowLanes, ..., then in warp order; double-single
+// pairs on the FP32 pipe, hi + lo in FP64), and warp 0 goes on with the rows' FP64
+// work (it is alone on its SM's FP64 unit for a few thousand rows a step).  With
+// one range the sum is the range's hi + lo, as the single-system kernel writes it.
+// use(r, c, i, f) takes row r, particle i of cluster c, with its sums.
+constexpr int kRowLanes = 8;
+template <int NC, class Use>
+__device__ __forceinline__ void ens_rows(const EnsDev &E, Use &&use)
 {
+    __shared__ float2 sh[6][kRowLanes][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const long long R = E.row_pfx[E.n_cl];
-    for (long long r = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; r < R;
-         r += static_cast<long long>(gridDim.x) * blockDim.x) {
-        const int c = ens_row_cluster(E, r);
-        const int64_t i = E.act[E.off[c] + (r - E.row_pfx[c])];
-        double f[7];
-        ens_row_sums<NC>(E, r, E.nsplit[c], f);
-        correct_row(E.S, i, f, f + 3, E.t_blk[c], tick, eta, lmin, lmax, E.st);
+    for (long long r0 = blockIdx.x * 32ll; r0 < R; r0 += gridDim.x * 32ll) {
+        const long long r = r0 + lane;
+        const bool live = r < R;
+        const int c = live ? ens_row_cluster(E, r) : 0;
+        const int S = live ? E.nsplit[c] : 0;
+        const long long q = live ? r - E.row_pfx[c] : 0;
+        float h[6], l[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) h[k] = l[k] = 0.0f;
+        const float *base = E.part + (static_cast<size_t>(E.slot_pfx[c]) + static_cast<size_t>(q) * S) * NC;
+        for (int s = w; s < S; s += kRowLanes)
+#pragma unroll
+            for (int k = 0; k < 6; ++k) ds2_add(h[k], l[k], base[s * NC + k], NC == 14 ? base[s * NC + 7 + k] : 0.0f);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) sh[k][w][lane] = make_float2(h[k], l[k]);
+        __syncthreads();
+        if (w == 0 && live) {
+            double f[6];
+            const int nw = min(S, kRowLanes);
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                for (int v = 1; v < nw; ++v) ds2_add(h[k], l[k], sh[k][v][lane].x, sh[k][v][lane].y);
+                f[k] = static_cast<double>(h[k]) + static_cast<double>(l[k]);
+            }
+            use(c, E.act[E.off[c] + q], f);
+        }
+        __syncthreads();
     }
+}
+
+template <int NC>
+__global__ void __launch_bounds__(32 * kRowLanes)
+    ens_correct_kernel(const EnsDev E, double tick, double eta, int lmin, int lmax)
+{
+    ens_rows<NC>(E, [&](const int c, const int64_t i, const double(&f)[6]) {
+        correct_row(E.S, i, f, f + 3, E.t_blk[c], tick, eta, lmin, lmax, E.st);
+    });
 }
 
 // t = 0: a, k from the force on every particle, first levels from Eq. (initTimestep).
 template <int NC>
-__global__ void ens_init_kernel(const EnsDev E, double eta_init, int lmin, int lmax)
+__global__ void __launch_bounds__(32 * kRowLanes)
+    ens_init_kernel(const EnsDev E, double eta_init, int lmin, int lmax)
 {
-    const long long R = E.row_pfx[E.n_cl];
-    for (long long r = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; r < R;
-         r += static_cast<long long>(gridDim.x) * blockDim.x) {
-        const int c = ens_row_cluster(E, r);
-        const int64_t i = E.act[E.off[c] + (r - E.row_pfx[c])];
-        double f[7];
-        ens_row_sums<NC>(E, r, E.nsplit[c], f);
+    ens_rows<NC>(E, [&](const int, const int64_t i, const double(&f)[6]) {
         bool finite = true;
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
@@ -470,7 +614,7 @@ __global__ void ens_init_kernel(const EnsDev E, double eta_init, int lmin, int l
         }
         E.S.t[i] = 0;
         E.S.level[i] = static_cast<int8_t>(L);
-    }
+    });
 }
 
 // phi_i over the particle's own cluster (FP64, ascending j), then per-cluster sums.
@@ -554,12 +698,10 @@ __global__ void ens_pad_kernel(const EnsDev E)
 }  // namespace
 
 // ------------------------------------------------------------------ launchers
-using EnsForceFn = void (*)(EnsDev, float);
-
 template <int MODE, int NT, int IPT>
-void ens_force_instance(const EnsDev &E, float eps2, int grid, cudaStream_t s)
+void ens_force_instance(const EnsDev &E, float eps2, bool share, int grid, cudaStream_t s)
 {
-    ens_force_kernel<MODE, NT, IPT><<<grid, NT, 0, s>>>(E, eps2);
+    ens_force_kernel<MODE, NT, IPT><<<grid, NT, 0, s>>>(E, eps2, share);
 }
 
 // Resident blocks per SM of one force instance (queried once, before any
@@ -595,13 +737,23 @@ void ens_prefetch_occupancy()
     ens_force_occupancy<kModeComp, 128, 2>();
 }
 
-cudaError_t ens_force_launch(int mode, int threads, int ipt, const EnsDev &E, float eps2, int sm_count,
-                             cudaStream_t s, int64_t *launches)
+// Ranges of up to this many tiles share an item's threads among few rows; longer
+// ones (up to the whole stream) keep one thread per row, the single-system
+// kernel's arithmetic with one j-range.
+constexpr int kEnsShareTiles = 8;
+inline bool ens_share(const int ipt, const int tiles_per_range)
 {
+    return NB_PACKED && ipt == 1 && tiles_per_range <= kEnsShareTiles;
+}
+
+cudaError_t ens_force_launch(int mode, int threads, int ipt, int tiles_per_range, const EnsDev &E, float eps2,
+                             int sm_count, cudaStream_t s, int64_t *launches)
+{
+    const bool share = ens_share(ipt, tiles_per_range);
 #define NB_ENS(M, T, I)                                                    \
     if (mode == M && threads == T && ipt == I) {                            \
         const int grid = sm_count * std::max(1, ens_force_occupancy<M, T, I>()); \
-        ens_force_instance<M, T, I>(E, eps2, grid, s);                      \
+        ens_force_instance<M, T, I>(E, eps2, share, grid, s);                      \
         ++*launches;                                                        \
         return cudaGetLastError();                                          \
     }
@@ -633,7 +785,7 @@ struct nbody_ens {
     bool own_stream = false;
     int sm_count = 0;
     int s_max = 8;
-    int threads = 64, ipt = 1, tiles_per_range = 4;
+    int threads = 32, ipt = 1, tiles_per_range = 4;
     std::vector<int64_t> off_h;
     // device memory, in one allocation, and pinned memory in another
     void *dev_base = nullptr, *host_base = nullptr;
@@ -643,7 +795,7 @@ struct nbody_ens {
     float4 *jbuf = nullptr;
     int64_t *off = nullptr, *joff = nullptr;
     int32_t *cl_of = nullptr, *act = nullptr;
-    long long *t_blk = nullptr, *item_pfx = nullptr, *row_pfx = nullptr, *blocks = nullptr, *pairs = nullptr;
+    long long *t_blk = nullptr, *item_pfx = nullptr, *row_pfx = nullptr, *slot_pfx = nullptr, *blocks = nullptr, *pairs = nullptr;
     int *n_act = nullptr, *nsplit = nullptr, *tpr = nullptr, *live = nullptr;
     unsigned int *work = nullptr;
     float *part = nullptr;
@@ -713,18 +865,20 @@ int ens_enqueue_step(nbody_ens *e, long long t_end_tick)
     const int lmax = e->p.lmax;
     const double tick = std::ldexp(1.0, -lmax);
     const int rows = e->threads * e->ipt;
-    ens_schedule_kernel<<<e->n_cl, kEnsThreads, 0, e->s>>>(e->E, t_end_tick, lmax);
-    ens_plan_kernel<<<1, 1024, 0, e->s>>>(e->E, rows, e->tiles_per_range);
+    ens_schedule_kernel<<<e->n_cl, kSchedThreads, 0, e->s>>>(e->E, t_end_tick, lmax);
+    ens_plan_kernel<<<1, 1024, 0, e->s>>>(e->E, rows, e->tiles_per_range, ens_share(e->ipt, e->tiles_per_range));
     const int pg = static_cast<int>(std::min<int64_t>((e->n_tot + 255) / 256, e->sm_count * 16));
     ens_predict_kernel<<<pg, 256, 0, e->s>>>(e->E, tick, e->p.mode == kModeComp);
     NB_ECUDA(cudaGetLastError(), "ensemble step launch");
-    NB_ECUDA(ens_force_launch(e->p.mode, e->threads, e->ipt, e->E, static_cast<float>(e->eps2), e->sm_count, e->s,
+    NB_ECUDA(ens_force_launch(e->p.mode, e->threads, e->ipt, e->tiles_per_range, e->E, static_cast<float>(e->eps2), e->sm_count, e->s,
                               &e->kernel_launches),
              "ensemble force launch");
+    // (a step's rows, a few thousand, over every SM's FP64 unit: 256 rows per block took 24 us)
+    const int cg = static_cast<int>(std::min<int64_t>((e->n_tot + 31) / 32, e->sm_count * 16));
     if (e->p.mode == kModeComp)
-        ens_correct_kernel<14><<<pg, 256, 0, e->s>>>(e->E, tick, e->p.eta, e->p.lmin, lmax);
+        ens_correct_kernel<14><<<cg, 32 * kRowLanes, 0, e->s>>>(e->E, tick, e->p.eta, e->p.lmin, lmax);
     else
-        ens_correct_kernel<7><<<pg, 256, 0, e->s>>>(e->E, tick, e->p.eta, e->p.lmin, lmax);
+        ens_correct_kernel<7><<<cg, 32 * kRowLanes, 0, e->s>>>(e->E, tick, e->p.eta, e->p.lmin, lmax);
     NB_ECUDA(cudaGetLastError(), "ensemble step launch");
     e->kernel_launches += 4;
     return NBODY_OK;
@@ -773,7 +927,7 @@ int nbody_ens_init(nbody_ens **out, int64_t n_clusters, const int64_t *sizes, co
     const int64_t n = off.back();
     if (n > 2147483647LL || jt > 2147483647LL) return efail(NBODY_EINVAL, "nbody_ens_init: too many particles");
 
-    const int sh_t = prm.j_tile ? prm.j_tile : 64, sh_i = prm.i_block ? prm.i_block : 1;
+    const int sh_t = prm.j_tile ? prm.j_tile : 32, sh_i = prm.i_block ? prm.i_block : 1;
     const int sh_p = prm.j_split > 0 ? prm.j_split : 4;
     bool shape_ok = false;
     for (const EnsShape &sh : kEnsShapes) shape_ok |= sh.threads == sh_t && sh.ipt == sh_i;
@@ -822,6 +976,7 @@ int nbody_ens_init(nbody_ens **out, int64_t n_clusters, const int64_t *sizes, co
     dev_mem.add(&e->t_blk, nc * sizeof(long long));
     dev_mem.add(&e->item_pfx, (nc + 1) * sizeof(long long));
     dev_mem.add(&e->row_pfx, (nc + 1) * sizeof(long long));
+    dev_mem.add(&e->slot_pfx, nc * sizeof(long long));
     dev_mem.add(&e->blocks, nc * sizeof(long long));
     dev_mem.add(&e->pairs, nc * sizeof(long long));
     dev_mem.add(&e->n_act, nc * sizeof(int));
@@ -876,6 +1031,7 @@ int nbody_ens_init(nbody_ens **out, int64_t n_clusters, const int64_t *sizes, co
     E.live = e->live;
     E.blocks = e->blocks;
     E.pairs = e->pairs;
+    E.slot_pfx = e->slot_pfx;
     E.part = e->part;
     E.st = e->st;
 
@@ -898,17 +1054,19 @@ int nbody_ens_init(nbody_ens **out, int64_t n_clusters, const int64_t *sizes, co
     ens_pad_kernel<<<std::min(e->n_cl, 1024), 256, 0, s>>>(E);
     // t = 0: everything active, full force per cluster, first levels
     const int pg = static_cast<int>(std::min<int64_t>((n + 255) / 256, e->sm_count * 16));
+    const int cg = static_cast<int>(std::min<int64_t>((n + 31) / 32, e->sm_count * 16));
     ens_all_active_kernel<<<pg, 256, 0, s>>>(E);
-    ens_plan_kernel<<<1, 1024, 0, s>>>(E, e->threads * e->ipt, e->tiles_per_range);
+    ens_plan_kernel<<<1, 1024, 0, s>>>(E, e->threads * e->ipt, e->tiles_per_range,
+                                       ens_share(e->ipt, e->tiles_per_range));
     ens_predict_kernel<<<pg, 256, 0, s>>>(E, std::ldexp(1.0, -prm.lmax), prm.mode == NBODY_MODE_COMP);
     NB_EI(cudaGetLastError(), "init launch");
-    NB_EI(ens_force_launch(prm.mode, e->threads, e->ipt, E, static_cast<float>(eps2), e->sm_count, s,
+    NB_EI(ens_force_launch(prm.mode, e->threads, e->ipt, e->tiles_per_range, E, static_cast<float>(eps2), e->sm_count, s,
                            &e->kernel_launches),
           "init force");
     if (prm.mode == NBODY_MODE_COMP)
-        ens_init_kernel<14><<<pg, 256, 0, s>>>(E, prm.eta_init, prm.lmin, prm.lmax);
+        ens_init_kernel<14><<<cg, 32 * kRowLanes, 0, s>>>(E, prm.eta_init, prm.lmin, prm.lmax);
     else
-        ens_init_kernel<7><<<pg, 256, 0, s>>>(E, prm.eta_init, prm.lmin, prm.lmax);
+        ens_init_kernel<7><<<cg, 32 * kRowLanes, 0, s>>>(E, prm.eta_init, prm.lmin, prm.lmax);
     NB_EI(cudaGetLastError(), "init launch");
     NB_EI(cudaMemsetAsync(e->blocks, 0, nc * sizeof(long long), s), "memset");
     NB_EI(cudaMemsetAsync(e->pairs, 0, nc * sizeof(long long), s), "memset");

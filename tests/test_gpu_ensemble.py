@@ -159,3 +159,35 @@ def test_full_size_c4_sampled_clusters(mode):
     de = np.abs((ek + ep - ek0 - ep0) / (ek0 + ep0))
     print(f"\nC4 {mode}: |dE/E| at t = 1/64 median {np.median(de):.2e} max {de.max():.2e}")
     assert de.max() < 1e-6
+
+
+@pytest.mark.parametrize("mode", ["plain", "comp"])
+def test_automatic_shape_any_batch(mode):
+    """The automatic shape (threads shared among few rows, single-tile ranges for small blocks): a cluster's run does
+    not depend on the other clusters of its batch, also past the 128 clusters whose item offsets sit in shared memory;
+    and its forces at the end are the oracle's within the FP32 bound."""
+    need_gpu()
+    from paper_astro_ph_0702058_gb300 import Ensemble
+    sizes = np.array([700, 1, 33, 2500, 256, 2, 64, 9000] + [5 + 7 * (k % 40) for k in range(150)], dtype=np.int64)
+    parts = [plummer_sphere(int(n), 300 + c) for c, n in enumerate(sizes)]
+
+    def run(pick):
+        m, x, v = (np.concatenate([parts[c][k] for c in pick]) for k in range(3))
+        with Ensemble(sizes[pick], m, x, v, EPS2, eta=0.02, mode=mode) as ens:
+            ens.run(1.0 / 64)
+            s = _state(ens, len(m))
+        off = np.concatenate([[0], np.cumsum(sizes[pick])])
+        return {c: {k: s[k][off[i]:off[i + 1]] for k in ("x", "v", "a", "k")} for i, c in enumerate(pick)}
+
+    whole, few = run(np.arange(len(sizes))), run(np.array([3, 7, 1, 40]))
+    for c in few:
+        for k in few[c]:
+            assert np.array_equal(few[c][k], whole[c][k]), (c, k)
+    for c in (0, 3, 7, 30):
+        mc, n = parts[c][0], int(sizes[c])
+        s = whole[c]
+        rows = np.linspace(0, n - 1, min(n, 200)).astype(int)
+        # a and k are the forces at the predicted state of the last step; at t = 1/64 every particle has been corrected
+        # there, which moves it by the corrector's ~dt^4: compare loosely
+        ra, rk, _ = oracle.force(mc, s["x"], s["v"], EPS2, rows.astype(np.int32))
+        assert np.linalg.norm(s["a"][rows] - ra) <= 1e-4 * np.linalg.norm(ra)
