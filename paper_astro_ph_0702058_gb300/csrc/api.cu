@@ -25,6 +25,7 @@ int g_fail_alloc = 0;    // allocation-failure injection countdown (test hook)
 // replay per block, 2 a device-side loop of blocks in each replay
 int g_step_graphs = 3;
 constexpr int64_t kLoopCap = 1024;  // blocks one replay of the loop may run
+constexpr int64_t kPairsOwnList = 16384;  // rows of a caller's list that may take pairs (plain, compensated)
 constexpr int64_t kRollKeep = int64_t(1) << 30;  // bytes of states a gradient keeps instead of running steps again
 constexpr int64_t kClusterCap = 4096;  // blocks one launch of the cluster or the grid kernel may run
 #ifndef NB_GRID_ROWS
@@ -266,7 +267,7 @@ int force_internal(nbody_ctx *c, int64_t n_act, bool for_step = false, bool asce
                             c->p.j_sub, pairs && c->J.soa ? c->n : 0, user && n_act > 0);
     };
     ForceConfig cfg{};
-    int r = choose(&cfg, true);
+    int r = choose(&cfg, ascending || n_act >= kPairsOwnList || c->p.mode == NBODY_MODE_DS);
     if (r == NBODY_OK && cfg.sym_sb > 0 && !sym_room(c, cfg, n_act)) r = choose(&cfg, false);
     if (r != NBODY_OK) return fail(r, "unsupported force shape: %d threads x %d i per thread", c->p.j_tile, c->p.i_block);
     int64_t launches = 0;

@@ -80,7 +80,7 @@ int force_choose(int mode, int64_t n_act, int64_t n_pad, int sm_count, int req_t
     if (n_pairs > 0 && req_threads == 0 && req_ipt == 0 && req_split <= 0 && req_jsub == 0 &&
         sym_plan(mode, n_act, n_pairs, sm_count, cfg))
         return NBODY_OK;
-    cfg->sym_sb = cfg->sym_ranges = cfg->sym_out_len = 0;
+    cfg->sym_sb = cfg->sym_ranges = 0;
     const int n_tiles = static_cast<int>(n_pad / kJTile);
     // the slice shape: one CTA per SM over its slice of the stream, for mid-size blocks when the
     // caller fixes no parameter and the slice fits shared memory
@@ -228,7 +228,7 @@ cudaError_t force_launch(int mode, const JStream &js, int64_t n, const int32_t *
         return e;
     }
     const ForceConfig &c = cfg;
-    ForceParams P;
+    ForceParams P{};
     P.posm = js.posm;
     P.vel = js.vel;
     P.poslo = js.poslo;

@@ -57,6 +57,9 @@ struct ForceParams {
     double *__restrict__ pot;
     float *__restrict__ part;  // [split][7 or 14][n_act] when split > 1
     DevStatus *st;
+    const float *rows;         // when set: row q is entry q of these arrays (rows_stride floats each), none of them
+    long long rows_stride;     // among the particles of the tiles, and the sums always go to part
+    const long long *skip;     // when set and not zero: nothing to do
     int skip_first_copy;       // test hook: leave the first tile's copy out
     unsigned long long opaque_zero;  // always 0; hides values from the assembler (f2_opaque)
 };

@@ -10,31 +10,35 @@
 
 namespace nb {
 
+cudaError_t force_dispatch_plain(const ForceParams &P, const ForceConfig &cfg, cudaStream_t s);
+cudaError_t force_dispatch_comp(const ForceParams &P, const ForceConfig &cfg, cudaStream_t s);
+
 namespace {
 
 constexpr int kSymMaxSb = 128;             // superblocks
 constexpr int64_t kSymMinRows = 8192;      // rows from which a block may take pairs
+constexpr int64_t kSymMinPart = 20000;     // the same for a part of the particles
 constexpr int64_t kSymDsMin = 4096;        // particles from which the double-single force may
 constexpr int64_t kSymPartCap = int64_t(8) << 30;  // bytes of its slots
 constexpr int kSymThreads = 256;
 constexpr int kSymScan = 4 * kSymThreads;  // particles of a block of the compaction
 
-// Resident warps per SM, and the unroll factor of the pair loop: at n = 262144
-// 12 warps (168 registers) x 4 against 16 (128) x 2 took 44.2 against 45.2 ms in
-// plain mode, 55.2 against 54.4 in compensated mode (128 registers spill there,
-// yet the fourth warp of a scheduler gains more); one-warp CTAs (n <= 32768)
-// are faster with 12 x 4 in both.
+// Resident warps per SM the registers are limited for, and the unroll factor of
+// the pair loop.  Measured at n = 262144, ms: plain 12 warps x 8 43.7, x 4 45.0, 16
+// warps (128 registers) x 4 45.4, x 8 44.9; compensated 16 x 4 53.0 (x 2 56.7, x 8
+// 53.3), 12 x 8 54.1, x 4 54.3; one-warp CTAs (n = 16384, us): plain 12 x 8 235,
+// 16 x 4 231, compensated 12 x 8 280, 16 x 4 291.
 template <int MODE, int W>
 struct SymShape {
     static constexpr bool wide = MODE == kModeComp && W > 1;
-    static constexpr int unroll = wide ? 2 : 4, warps = wide ? 16 : 12;
+    static constexpr int unroll = wide ? 4 : 8, warps = wide ? 16 : 12;
 };
 
 template <int MODE, int W>
 cudaError_t sym_launch(const SymParams &P, const ForceConfig &cfg, cudaStream_t s)
 {
     using Sh = SymShape<MODE, W>;
-    const int units = cfg.sym_sb * (cfg.sym_sb + 1) / 2 + cfg.sym_sb * cfg.sym_ranges;
+    const int units = cfg.sym_sb * (cfg.sym_sb + 1) / 2;
     force_sym_kernel<MODE, W, Sh::unroll, Sh::warps><<<units, 32 * W, 0, s>>>(P);
     return cudaGetLastError();
 }
@@ -106,6 +110,10 @@ __global__ void __launch_bounds__(kSymThreads)
                        const int *__restrict__ mark, const int n, const int *__restrict__ counts,
                        float *__restrict__ out, const long long out_stride, const int n_out)
 {
+    // (and the massless far particles that fill the last tile)
+    for (int e = n_out + static_cast<int>(blockIdx.x * kSymThreads + threadIdx.x); e < out_stride;
+         e += gridDim.x * kSymThreads)
+        for (int a = 0; a < arrays; ++a) out[a * out_stride + e] = a < 3 ? kPadPosition : 0.0f;
     __shared__ int sh[kSymThreads / 32];
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     int before = 0;  // particles of the blocks before this one
@@ -221,16 +229,18 @@ SymScratch sym_scratch(void *p, const int64_t n)
 
 size_t sym_scratch_bytes(int64_t n)
 {
-    return 16 + sizeof(int) * (up4(n) + up4(n / kSymScan + 1)) + sizeof(float) * 16 * (n + 8);
+    return 16 + sizeof(int) * (up4(n) + up4(n / kSymScan + 1)) + sizeof(float) * 16 * (n + 8 + kJTile);
 }
 
-// A block takes pairs from 8192 rows on (full forces at n = 8192, 4096 measured 1.23
-// and 1.0 times the one-sided kernel's rate), when it holds enough of the particles:
-// only pairs within the block are shared, and the one-sided units run at 0.88 of
-// force_kernel_x2's rate (four rows per lane, 12 warps).  Measured, one-sided
-// kernel -> pairs, us: compensated 33536 of 65536 rows 2270 -> 2193, 22000: 1512 ->
-// 1500, 16384: 1142 -> 1140, 40001 of 100003: 4035 -> 4091; plain 40001 of 100003
-// 3396 -> 3242.  So half of the particles compensated, three eighths plain.
+// All particles take pairs from 8192 on (the kernels alone, one-sided -> pairs, us,
+// plain / compensated: n = 8192 82 -> 67 / 96 -> 78; 4096: 30 -> 28 / 34 -> 33, left
+// as it was); a caller's list, which is checked and gathered first (~30 us), from
+// 16384 (251 -> 231 / 301 -> 280 per call).  Only pairs within a block are shared,
+// so a part of the particles gains about 0.2 n_act / n of its time and pays ~25 us
+// for the copies and the second kernel.  Measured (us): compensated 33536 of 65536
+// rows 2228 -> 2129, 22000: 1481 -> 1474, 40001 of 100003 3962 -> 3834, 26000: 2646
+// -> 2563, but 12000 of 32768 433 -> 460; plain 40001 of 100003 3391 -> 3163, 22000
+// of 65536 1248 -> 1252.  So from 20000 rows and a quarter of the particles on.
 // Superblocks are as small as 128 of them allow, for many units (8256 against 2080
 // of twice the size: 4-5 % at n = 65536 and 262144), up to 8 GiB of slots (2^20
 // compensated: 889 ms with 7.6 GB, 920 with 4.3); CTAs of one warp up to 32768
@@ -253,16 +263,23 @@ bool sym_plan(int mode, int64_t n_act, int64_t n, int sm_count, ForceConfig *cfg
         cfg->split = static_cast<int>(sb + 1);
         cfg->tiles_per_split = static_cast<int>(tiles);
         cfg->sym_sb = static_cast<int>(sb);
-        cfg->sym_ranges = cfg->sym_out_len = 0;
+        cfg->sym_ranges = 0;
         return true;
     }
     if (!NB_PACKED || (mode != kModePlain && mode != kModeComp)) return false;
-    if (n_act < kSymMinRows || n_act > n || (mode == kModeComp ? 2 : 8.0 / 3.0) * n_act < n) return false;
+    if (n_act < kSymMinRows || n_act > n || (n_act < n && (n_act < kSymMinPart || 4 * n_act < n))) return false;
     const int nc = two_word_sums(mode) ? 14 : 7;
     const int W = n_act <= 32768 ? 1 : 4;
     const int64_t bt = static_cast<int64_t>(W) * kSymRows;
     const int64_t n_out = n - n_act;
     const int64_t slot_bytes = static_cast<int64_t>(nc) * n_act * sizeof(float);
+    int64_t ranges = 0;  // of the particles outside: as a one-sided force over them takes
+    if (n_out > 0) {
+        ForceConfig out{};
+        if (force_choose(mode, n_act, (n_out + kJTile - 1) / kJTile * kJTile, sm_count, 256, 1, 0, &out) != NBODY_OK)
+            return false;
+        ranges = out.split;
+    }
     const int res = (mode == kModeComp && W > 1 ? 16 : 12) / W;  // resident CTAs per SM (SymShape)
     const int64_t slots = static_cast<int64_t>(res) * sm_count;
     const int64_t t_min = (n_act + bt * kSymMaxSb - 1) / (bt * kSymMaxSb);
@@ -270,15 +287,8 @@ bool sym_plan(int mode, int64_t n_act, int64_t n, int sm_count, ForceConfig *cfg
     double best = 0.0;
     for (int64_t tiles = t_min; !found || tiles <= t_min + t_min / 4; ++tiles) {
         const int64_t sb = (n_act + bt * tiles - 1) / (bt * tiles);
-        // outside ranges: about two units for every resident CTA
-        int64_t ranges = 0, len = 0;
-        if (n_out > 0) {
-            const int64_t want = (2 * slots + sb - 1) / sb;
-            len = ((n_out + want - 1) / want + bt - 1) / bt * bt;
-            ranges = (n_out + len - 1) / len;
-        }
         const int64_t units = sb * (sb + 1) / 2;
-        if (units + sb * ranges < slots) break;  // too few units
+        if (units < slots) break;  // too few units
         if ((sb + 1 + ranges) * slot_bytes > kSymPartCap) continue;
         // the last, partly filled wave: an SM that holds k of res CTAs works at
         // about 0.6, 0.87 and 0.97 of its rate with 1/4, 1/2 and 3/4 of them
@@ -298,7 +308,6 @@ bool sym_plan(int mode, int64_t n_act, int64_t n, int sm_count, ForceConfig *cfg
         cfg->tiles_per_split = static_cast<int>(tiles);
         cfg->sym_sb = static_cast<int>(sb);
         cfg->sym_ranges = static_cast<int>(ranges);
-        cfg->sym_out_len = static_cast<int>(len);
     }
     return found;
 }
@@ -349,8 +358,6 @@ cudaError_t force_sym_launch(int mode, const JStream &js, int64_t n, const int32
     P.n = na;
     P.n_sb = cfg.sym_sb;
     P.tiles = cfg.tiles_per_split;
-    P.n_out = n_out;
-    P.out_len = cfg.sym_out_len;
     P.eps2 = static_cast<float>(eps2);
     P.part = static_cast<float *>(partials);
     P.soa = js.soa;
@@ -371,12 +378,30 @@ cudaError_t force_sym_launch(int mode, const JStream &js, int64_t n, const int32
         }
         if (n_out > 0) {
             float *out = X.rows + kSoaArrays * P.stride;
-            P.out_soa = out;
-            P.out_stride = up4(n_out);
+            const long long out_pad = (n_out + kJTile - 1) / kJTile * kJTile;
             const int nb = (nn + kSymScan - 1) / kSymScan;
             sym_count_kernel<<<nb, kSymThreads, 0, s>>>(X.mark, nn, X.counts);
-            sym_compact_kernel<<<nb, kSymThreads, 0, s>>>(js.soa, js.n_pad, arrays, X.mark, nn, X.counts, out,
-                                                          P.out_stride, n_out);
+            sym_compact_kernel<<<nb, kSymThreads, 0, s>>>(js.soa, js.n_pad, arrays, X.mark, nn, X.counts, out, out_pad,
+                                                          n_out);
+            ForceParams Q{};
+            Q.soa = out;
+            Q.n_act = na;
+            Q.n = nn;
+            Q.n_tiles = static_cast<int>(out_pad / kJTile);
+            Q.eps2 = P.eps2;
+            Q.part = P.part + static_cast<size_t>(cfg.sym_sb + 1) * (mode == kModeComp ? 14 : 7) * na;
+            Q.st = st;
+            Q.rows = X.rows;
+            Q.rows_stride = P.stride;
+            Q.skip = P.skip;
+            ForceConfig oc{};
+            oc.threads = 256;
+            oc.ipt = 1;
+            oc.split = cfg.sym_ranges;
+            oc.n_iblk = (na + 255) / 256;
+            e = mode == kModeComp ? force_dispatch_comp(Q, oc, s) : force_dispatch_plain(Q, oc, s);
+            if (e != cudaSuccess) return e;
+            ++*launches;
             *launches += 2;
         }
         e = cudaGetLastError();

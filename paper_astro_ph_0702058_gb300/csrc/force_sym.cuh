@@ -11,10 +11,11 @@
 //   rows    the block's particles in list order, n of them, as a structure of
 //           arrays (the j-stream itself when the block is all particles, else
 //           a gathered copy); cut into n_sb superblocks of W x 128 x tiles rows.
-//   unit    one CTA per unordered pair (I, J) of superblocks, and one per
-//           (superblock, range of the particles outside the block), whose pairs
-//           give only the row its terms.  Units only share read-only data, so
-//           their order does not matter.
+//   unit    one CTA per unordered pair (I, J) of superblocks.  Units only share
+//           read-only data, so their order does not matter.  The rows' pairs with
+//           the particles outside the block are force_kernel_x2's (as more units
+//           here, one-sided, they ran at 0.88 of its rate: 12 to 16 warps per SM
+//           against 16 to 24).
 //   warp    128 rows i, four per lane in two packed registers, against 128 j in
 //           four turns of 32: in step s of a turn, lane l takes j = (l + s) mod
 //           32 from shared memory; the sums of j move on by one lane per step
@@ -26,10 +27,10 @@
 //   sums    FP32 over 128 terms, folded into (hi, lo) by TwoSum (compensated) or
 //           an FP32 sum (plain), as in force_x2.cuh.  The folded sums live in
 //           the unit's own slots of `part`: the rows of I in slot J, those of J
-//           in slot I (I = J: the second side in slot n_sb), the outside range r
-//           in slot n_sb + 1 + r.  Every row has every slot written once, and
-//           force_sym_reduce adds them in slot order, so results do not depend
-//           on scheduling.
+//           in slot I (I = J: the second side in slot n_sb), the j-ranges outside
+//           in the slots after.  Every row has every slot written once, and
+//           force_sym_reduce_kernel adds them in slot order, so results do not
+//           depend on scheduling.
 // What bounds it: the register file.  A packed FMA of three different registers
 // reads six 32-bit words and issues every 3 cycles, not 2 (measured: 3.01; 2.2
 // where consecutive ones share an operand; scalar FMAs 1.0 each, but mixing
@@ -37,8 +38,8 @@
 // plain).  19 of the 35 operations are such FMAs: 87 cycles for two pairs.
 // Measured against the one-sided kernel (force_kernel_x2) with its reduction,
 // full forces, us: n = 8192 plain 82 -> 67, compensated 96 -> 78; 16384: 251 ->
-// 194, 301 -> 242; 65536: 3566 -> 2804, 4331 -> 3408; 262144: 55672 -> 44243,
-// 66448 -> 54382; 2^20: 880 -> 711 ms, 1060 -> 883 ms.
+// 194, 301 -> 242; 65536: 3566 -> 2816, 4331 -> 3395; 262144: 55672 -> 43727,
+// 66448 -> 53021.
 // Two rows per lane instead of four (96 registers) took 3276 us at n = 65536
 // plain; r^-2 from the MUFU reciprocal instead of a product 0.5-2 % more.
 #pragma once
@@ -55,12 +56,8 @@ struct SymParams {
     int n;                    // rows
     int n_sb;                 // superblocks
     int tiles;                // W x 128-row tiles of a superblock
-    const float *out_soa;     // the particles outside the block, `out_stride` floats each
-    long long out_stride;
-    int n_out;
-    int out_len;              // of them per range (a multiple of W x 128)
     float eps2;
-    float *part;              // [n_sb + 1 + ranges][7 or 14][n]
+    float *part;              // [n_sb + 1][7 or 14][n]
     const long long *skip;    // when set and not zero: nothing to do
     DevStatus *st;
 };
@@ -217,25 +214,6 @@ __device__ __forceinline__ void sym_both(const float *chunk, const SymI &I, cons
     }
 }
 
-// The same rows against a chunk of j that take no force.  (A chunk of values
-// stored twice, read as packed operands without the moves, measured 1.5 % slower.)
-template <int MODE>
-__device__ __forceinline__ void sym_one(const float *chunk, const SymI &I, const f2_t E2, const f2_t NEG3,
-                                        f2_t (&pi)[2][7])
-{
-#pragma unroll 2
-    for (int jl = 0; jl < kSymRows; ++jl) {
-        f2_t v[10];
-        sym_load_j<MODE>(chunk, jl, v);
-#pragma unroll
-        for (int g = 0; g < 2; ++g) {
-            SymT T;
-            sym_term<MODE, false>(v, I, g, E2, NEG3, false, false, T);
-            sym_add(v[3], T, pi[g]);
-        }
-    }
-}
-
 // Element e of array a of a structure of arrays of n; past its end a massless
 // particle far from every other.
 __device__ __forceinline__ float sym_val(const float *soa, const long long stride, const int n, const int a,
@@ -259,29 +237,17 @@ __global__ void __launch_bounds__(32 * W, WARPS / W) force_sym_kernel(const SymP
     const size_t slot = static_cast<size_t>(NC) * n;
     const f2_t E2 = f2_pack(P.eps2, P.eps2), NEG3 = f2_pack(-3.0f, -3.0f);
 
-    // the unit: (I, outside range J), the longer ones, then (I, J) with I <= J
-    const int n_one = P.out_len > 0 ? P.n_sb * ((P.n_out + P.out_len - 1) / P.out_len) : 0;
-    const int u = static_cast<int>(blockIdx.x) - n_one;
-    const bool both = u >= 0;
-    int I_sb, J;
-    if (both) {
-        J = static_cast<int>((sqrtf(8.0f * u + 1.0f) - 1.0f) * 0.5f);
-        while ((J + 1) * (J + 2) / 2 <= u) ++J;
-        while (J * (J + 1) / 2 > u) --J;
-        I_sb = u - J * (J + 1) / 2;
-    } else {
-        I_sb = blockIdx.x % P.n_sb;
-        J = blockIdx.x / P.n_sb;
-    }
-    const bool diag = both && I_sb == J;
-    if (!NB_CHECK(I_sb >= 0 && J >= 0 && (!both || (I_sb <= J && J < P.n_sb)), P.st, 60)) return;
-    float *pi_out = P.part + slot * (both ? J : P.n_sb + 1 + J);
+    // the unit: (I, J) with I <= J
+    const int u = blockIdx.x;
+    int J = static_cast<int>((sqrtf(8.0f * u + 1.0f) - 1.0f) * 0.5f);
+    while ((J + 1) * (J + 2) / 2 <= u) ++J;
+    while (J * (J + 1) / 2 > u) --J;
+    const int I_sb = u - J * (J + 1) / 2;
+    const bool diag = I_sb == J;
+    if (!NB_CHECK(I_sb >= 0 && I_sb <= J && J < P.n_sb, P.st, 60)) return;
+    float *pi_out = P.part + slot * J;
     float *pj_out = P.part + slot * (diag ? P.n_sb : I_sb);
-    // the j of the unit
-    const float *js = both ? P.soa : P.out_soa;
-    const long long js_stride = both ? P.stride : P.out_stride;
-    const int j_begin = both ? J * P.tiles * BT : J * P.out_len;
-    const int j_end = both ? min(n, j_begin + P.tiles * BT) : min(P.n_out, j_begin + P.out_len);
+    const int j_begin = J * P.tiles * BT, j_end = min(n, j_begin + P.tiles * BT);
 
     // j-tiles in groups: the sums of a group's j stay in L2 while every row tile passes
     // over them (large superblocks: 55 MB for all resident CTAs)
@@ -322,7 +288,7 @@ __global__ void __launch_bounds__(32 * W, WARPS / W) force_sym_kernel(const SymP
                 const int k = e % kSymRows;
                 float v[10];
 #pragma unroll
-                for (int a = 0; a < NA; ++a) v[a] = sym_val(js, js_stride, j_end, a, j0 + e);
+                for (int a = 0; a < NA; ++a) v[a] = sym_val(P.soa, P.stride, j_end, a, j0 + e);
                 reinterpret_cast<float4 *>(q)[k] = make_float4(v[0], v[1], v[2], v[3]);
                 reinterpret_cast<float4 *>(q)[kSymRows + k] = make_float4(v[4], v[5], v[6], DSW ? v[7] : 0.0f);
                 if (DSW) reinterpret_cast<float2 *>(q + 8 * kSymRows)[k] = make_float2(v[8], v[9]);
@@ -330,7 +296,7 @@ __global__ void __launch_bounds__(32 * W, WARPS / W) force_sym_kernel(const SymP
             const bool own = diag && j0 == t0;  // the tile of the rows themselves
             const int nk = own ? W / 2 + 1 : W;
             for (int k = 0; k < nk; ++k) {
-                if (k == 0 || both) __syncthreads();
+                __syncthreads();
                 const int c = (k + w) % W;
                 const int jr = j0 + c * kSymRows;
                 // (own: windows 0 .. W/2 meet every pair of chunks, the last one twice)
@@ -341,9 +307,7 @@ __global__ void __launch_bounds__(32 * W, WARPS / W) force_sym_kernel(const SymP
 #pragma unroll
                     for (int q = 0; q < 7; ++q) pi[g][q] = 0ull;
                 const bool jfirst = it == 0 && k == 0;  // (each chunk that exists meets a warp in window 0)
-                if (!both)
-                    sym_one<MODE>(sj + c * CH, I, E2, NEG3, pi);
-                else if (own && k == 0)
+                if (own && k == 0)
                     sym_both<MODE, true, 1>(sj + c * CH, I, lane, E2, NEG3, pi, pj_out + jr, j_end - jr, n, jfirst);
                 else
                     sym_both<MODE, false, UNROLL>(sj + c * CH, I, lane, E2, NEG3, pi, pj_out + jr, j_end - jr, n,

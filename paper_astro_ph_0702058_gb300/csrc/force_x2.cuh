@@ -325,6 +325,7 @@ __global__ void NB_X2_BOUNDS(NT) force_kernel_x2(const ForceParams P)
 
     const int n_act = P.n_act_dev ? static_cast<int>(*P.n_act_dev) : P.n_act;
     if (static_cast<int>(blockIdx.x) * RB * IPT >= n_act) return;  // a launch sized for more rows
+    if (P.skip && *P.skip != 0) return;
     const int tid = threadIdx.x;
     const int row = tid % RB, sub = tid / RB;
     int t_begin, t_end;
@@ -339,7 +340,7 @@ __global__ void NB_X2_BOUNDS(NT) force_kernel_x2(const ForceParams P)
     for (int u = 0; u < IPT; ++u) {
         const int q = (blockIdx.x * IPT + u) * RB + row;
         int idx = -1;
-        if (q < n_act) {
+        if (q < n_act && !P.rows) {
             idx = P.active[q];
             if (idx < 0 || idx >= P.n) {
                 atomicOr(&P.st->flags, kFlagBadIndex);
@@ -351,10 +352,11 @@ __global__ void NB_X2_BOUNDS(NT) force_kernel_x2(const ForceParams P)
         const int l = idx >= 0 ? idx : 0;
         float4 xp, vp, lp = make_float4(0.f, 0.f, 0.f, 0.f);
         if constexpr (SOAIN) {  // the rows from the structure-of-arrays stream, as the tiles
-            const float *a = P.soa + l;
-            xp = make_float4(a[0], a[n_pad], a[2 * n_pad], 0.f);
-            vp = make_float4(a[4 * n_pad], a[5 * n_pad], a[6 * n_pad], 0.f);
-            if (is_ds(MODE)) lp = make_float4(a[7 * n_pad], a[8 * n_pad], a[9 * n_pad], 0.f);
+            const float *a = P.rows ? P.rows + (q < n_act ? q : 0) : P.soa + l;
+            const size_t st = P.rows ? static_cast<size_t>(P.rows_stride) : n_pad;
+            xp = make_float4(a[0], a[st], a[2 * st], 0.f);
+            vp = make_float4(a[4 * st], a[5 * st], a[6 * st], 0.f);
+            if (is_ds(MODE)) lp = make_float4(a[7 * st], a[8 * st], a[9 * st], 0.f);
         } else {
             xp = P.posm[l];
             vp = P.vel[l];
@@ -565,7 +567,7 @@ __global__ void NB_X2_BOUNDS(NT) force_kernel_x2(const ForceParams P)
     for (int u = 0; u < IPT; ++u) {
         const int q = (blockIdx.x * IPT + u) * RB + row;
         if (q >= n_act) continue;
-        if (gridDim.y == 1) {
+        if (gridDim.y == 1 && !P.rows) {
             double r[7];
 #pragma unroll
             for (int c = 0; c < 7; ++c)

@@ -112,8 +112,7 @@ struct ForceConfig {
     int slice = 0;        // 1: the slice shape (one CTA per SM, split = CTAs; force_slice.cuh)
     int sym_sb = 0;       // > 0: by unordered pairs (force_sym.cuh): superblocks of tiles_per_split x threads x ipt
                           // rows, split = slots
-    int sym_ranges = 0;   // ranges of the particles outside the block, of sym_out_len each
-    int sym_out_len = 0;
+    int sym_ranges = 0;   // j-ranges of the particles outside the block
 };
 // The j-subgroup shape: 256 threads, 64 rows of 4 subgroups (packed plain and compensated modes).
 constexpr int kJSubThreads = 256;

@@ -11,7 +11,7 @@ EPS2, LEVEL = (1.0 / 128) ** 2, 9
 
 # one particle, blocks of 32 (component, particle) threads and their edges, several j-ranges, pairs (8192)
 @pytest.mark.parametrize("n,mode", [(1, "plain"), (2, "comp"), (11, "plain"), (33, "comp"), (257, "plain"), (1500, "comp"),
-                                    (8191, "plain"), (8192, "comp"), (20000, "plain"), (300, "ds"), (300, "sumcheck"),
+                                    (8191, "plain"), (16384, "comp"), (20000, "plain"), (300, "ds"), (300, "sumcheck"),
                                     (100, "sorted")])
 def test_rollout_equals_block_steps(n, mode):
     """x_T and v_T of three steps against predict, force and correct called one by one.  Both add the same FP32
