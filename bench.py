@@ -201,13 +201,18 @@ KERNEL_SOURCES = ("paper_astro_ph_0702058_gb300/csrc/force_impl.cuh", "paper_ast
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "force_kernel_traffic_n1048576.json")
 
 
-def kernel_code_digest():
+# the force by unordered pairs (large blocks), recorded likewise
+PAIR_SOURCES = KERNEL_SOURCES + ("paper_astro_ph_0702058_gb300/csrc/force_sym.cuh",)
+ROWS_PER_LANE_BY_PAIRS = 4  # what the library reports as i per thread for a force by unordered pairs
+
+
+def kernel_code_digest(sources=KERNEL_SOURCES):
     """SHA-256 of the force kernel's sources with // comments and blank lines removed, so that
     only code changes invalidate a recorded measurement."""
     import hashlib
     import re
     h = hashlib.sha256()
-    for rel in KERNEL_SOURCES:
+    for rel in sources:
         with open(os.path.join(ROOT, rel)) as f:
             for line in f:
                 code = re.sub(r"//.*", "", line).rstrip()
@@ -225,7 +230,11 @@ def measured_traffic(mode, n, launch=None):
             rec = json.load(f)
     except (OSError, ValueError):
         return None
-    h = hashlib.sha256(kernel_code_digest().encode())
+    if launch is not None and launch[1] == ROWS_PER_LANE_BY_PAIRS:
+        rec = {**rec, **rec.get("by_pairs", {})}
+        h = hashlib.sha256(kernel_code_digest(PAIR_SOURCES).encode())
+    else:
+        h = hashlib.sha256(kernel_code_digest().encode())
     if rec.get("source_sha256") != h.hexdigest() or rec.get("n") != n or mode not in rec:
         return None
     if launch is not None and list(rec[mode].get("launch", [])) != list(launch):
@@ -237,14 +246,17 @@ def roofline(force_ms_avg, n, sm_count, clocks, peaks, mode="comp", launch=None)
     max_mhz = float(peaks.get("sm_max_mhz") or clocks.get("sm_max_mhz") or 2070.0)
     pairs = n * (n - 1)
     achieved = pairs / (force_ms_avg * 1e-3) / 1e9
-    peak = sm_count * FP32_LANES_PER_SM * max_mhz * 1e6 / OPS_PER_PAIR / 1e9
+    ops = OPS_PER_PAIR
+    if launch is not None and launch[1] == ROWS_PER_LANE_BY_PAIRS:
+        ops = 35 / 2  # an unordered pair gives both of its interactions with 35 operations
+    peak = sm_count * FP32_LANES_PER_SM * max_mhz * 1e6 / ops / 1e9
     out = {"bound": "alu", "achieved": round(achieved, 2), "peak": round(peak, 2), "unit": "Gpair/s",
            "frac": round(achieved / peak, 4), "traffic": measured_traffic(mode, n, launch),
            "traffic_unit": "bytes per launch (ncu dram read + write)",
            "peak_basis": f"{sm_count} SM x {FP32_LANES_PER_SM} FP32 lanes x {max_mhz:.0f} MHz / "
-                         f"{OPS_PER_PAIR} FP32 ops per pair (derived from unit counts and the max SM clock)"}
+                         f"{ops} FP32 ops per pair (derived from unit counts and the max SM clock)"}
     if clocks.get("sm_mhz"):
-        at_clock = sm_count * FP32_LANES_PER_SM * clocks["sm_mhz"] * 1e6 / OPS_PER_PAIR / 1e9
+        at_clock = sm_count * FP32_LANES_PER_SM * clocks["sm_mhz"] * 1e6 / ops / 1e9
         out["frac_at_sampled_clock"] = round(achieved / at_clock, 4)
     return out
 
@@ -462,8 +474,9 @@ def force_only(args):
         act = torch.arange(args.n, dtype=torch.int32, device="cuda")
     else:
         act = torch.from_numpy(active_subset(args.n, rows, 2)).to("cuda")
+    shape = dict(zip(("j_tile", "i_block", "j_split"), map(int, args.shape.split(",")))) if args.shape else {}
     for mode in args.modes.split(","):
-        with Simulation(m, x, v, eps2, mode=mode) as sim:
+        with Simulation(m, x, v, eps2, mode=mode, **shape) as sim:
             sim.predict(0.0)
             sim.force(act, rows)
             sim.sync()
@@ -802,6 +815,8 @@ def main(argv=None):
     ap.add_argument("--ens-sample", type=int, default=32,
                     help="clusters run one context each, for comparison (0: skip the comparison)")
     ap.add_argument("--ens-mode", default="comp")
+    ap.add_argument("--shape", default=None, help="--force-only: threads,i per thread,j-ranges of a fixed one-sided "
+                                                  "launch (default: the library's choice)")
     ap.add_argument("--rows", type=int, default=None, help="--force-only: rows of the call (default: all)")
     ap.add_argument("--seed", type=int, default=None, help="--force-only: seed of the sphere (default 3)")
     ap.add_argument("--eps2", type=float, default=None, help="--force-only: softening squared (default 1e-6)")
