@@ -489,8 +489,11 @@ int rollout_impl(const char *who, int64_t n, const double *m, const double *x0, 
                 const int rr = predict_internal(c, 1);
                 if (rr != NBODY_OK) return rr;
             }
+            // (four threads per row below 8192 particles: a step of 1500 is one range's latency, 16 -> 9 us; from
+            // 4096 on the shapes are alike)
             ForceConfig cfg{};
-            const bool parts = packed && force_choose(c->p.mode, n, c->n_pad, c->sm_count, 0, 0, 0, &cfg, 0, n) == NBODY_OK &&
+            const bool parts = packed && force_choose(c->p.mode, n, c->n_pad, c->sm_count, 0, 0, 0, &cfg,
+                                                      n < 8192 ? kJSub : 0, n) == NBODY_OK &&
                                cfg.sym_sb == 0 && cfg.split > 1;
             if (parts) {
                 const int rr = ensure_partials(c, force_partial_bytes(c->p.mode, cfg, n));
