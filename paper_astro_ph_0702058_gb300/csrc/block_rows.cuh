@@ -224,52 +224,48 @@ __device__ __forceinline__ void rows_correct(const State &S, const int *idx, con
             const bool live = q < cnt;
             const int qq = live ? q : 0;
             const int r = idx[qq];
-            double f[6];
-#pragma unroll
-            for (int c = 0; c < 6; ++c) f[c] = DSW ? f2d(fh[qq][c]) + f2d(fl[qq][c]) : f2d(fh[qq][c]);
+            const int c = part < 3 ? part : 2;
+            const int l_old = ld_state<true>(S.level + r);
             const CorrDt d = corr_dt(static_cast<int64_t>(tb) - ld_state<true>(S.t + r), tick, lmax);
-            double a2e = 0.0, a3 = 0.0;
-            bool finite = true;
-            if (part < 3) {
-                const double fa = part == 0 ? f[0] : part == 1 ? f[1] : f[2];
-                const double fk = part == 0 ? f[3] : part == 1 ? f[4] : f[5];
-                double xn, vn;
-                corr_dim(ld_state<true>(S.x[part] + r), ld_state<true>(S.v[part] + r), ld_state<true>(S.a[part] + r),
-                         ld_state<true>(S.k[part] + r), fa, fk, d, xn, vn, a2e, a3);
-                finite = isfinite(xn) && isfinite(vn) && isfinite(fa) && isfinite(fk);
-                if (live) {
-                    S.x[part][r] = xn;
-                    S.v[part][r] = vn;
-                    S.a[part][r] = fa;
-                    S.k[part][r] = fk;
+            double u[4];  // this component of a_p, k_p, a^(2), a^(3)
+            u[0] = DSW ? f2d(fh[qq][c]) + f2d(fl[qq][c]) : f2d(fh[qq][c]);
+            u[1] = DSW ? f2d(fh[qq][3 + c]) + f2d(fl[qq][3 + c]) : f2d(fh[qq][3 + c]);
+            double xn, vn;
+            corr_dim(ld_state<true>(S.x[c] + r), ld_state<true>(S.v[c] + r), ld_state<true>(S.a[c] + r),
+                     ld_state<true>(S.k[c] + r), u[0], u[1], d, xn, vn, u[2], u[3]);
+            const bool ok = finite_f64(xn) && finite_f64(vn) && finite_f64(u[0]) && finite_f64(u[1]);
+            if (live && part < 3) {
+                S.x[part][r] = xn;
+                S.v[part][r] = vn;
+                S.a[part][r] = u[0];
+                S.k[part][r] = u[1];
+            }
+            // (lane 3 of a row repeats lane 2's component)
+            const bool finite = ((__ballot_sync(0xffffffffu, ok) >> base) & 15u) == 15u;
+            // the 4 x 4 transpose: lane p of a row gets quantity p of lanes (components) 0, 1, 2
+#pragma unroll
+            for (int o = 1; o <= 2; o <<= 1)
+#pragma unroll
+                for (int p = 0; p < 2; ++p) {
+                    double &lo = u[o == 1 ? 2 * p : p], &hi = u[o == 1 ? 2 * p + 1 : p + 2];
+                    const double got = __shfl_xor_sync(0xffffffffu, (part & o) ? lo : hi, o);
+                    if (part & o)
+                        lo = got;
+                    else
+                        hi = got;
                 }
-            }
-            double u[3][2];  // a^(2) and a^(3) of the row, every component
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                u[c][0] = __shfl_sync(0xffffffffu, a2e, base + c);
-                u[c][1] = __shfl_sync(0xffffffffu, a3, base + c);
-            }
-            // all four lanes' finiteness (every lane takes part in every shuffle)
-            const int f1 = __shfl_xor_sync(0xffffffffu, static_cast<int>(finite), 1);
-            const int f2 = __shfl_xor_sync(0xffffffffu, static_cast<int>(finite), 2);
-            finite = finite && f1 && f2;
-            const int f3 = __shfl_xor_sync(0xffffffffu, static_cast<int>(finite), 1);
-            finite = finite && f3;
-            double w[3];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) w[c] = part == 0 ? f[c] : part == 1 ? f[3 + c] : part == 2 ? u[c][0] : u[c][1];
-            const double nrm = square3(w);  // |ap|^2, |kp|^2, |a^(2)|^2, |a^(3)|^2 on lanes 0-3
+            const double nrm = square3(u);  // |ap|^2, |kp|^2, |a^(2)|^2, |a^(3)|^2 on lanes 0-3
             const double aa = __shfl_sync(0xffffffffu, nrm, base), kk = __shfl_sync(0xffffffffu, nrm, base + 1);
             const double s2 = __shfl_sync(0xffffffffu, nrm, base + 2);
             const double t2 = __shfl_sync(0xffffffffu, nrm, base + 3);
             if (live && part == 0) {
-                const int l_new = corr_level(aa, kk, s2, t2, eta, lmin, lmax, ld_state<true>(S.level + r),
-                                             static_cast<int64_t>(tb), finite, st);
+                const int l_new = corr_level(aa, kk, s2, t2, eta, lmin, lmax, l_old, static_cast<int64_t>(tb), finite,
+                                             st);
                 S.t[r] = static_cast<int64_t>(tb);
                 S.level[r] = static_cast<int8_t>(l_new);
                 due(q, r, tb + (1ull << (lmax - l_new)));
             }
+            __syncwarp();  // what due() stored is seen by the whole warp
         }
     } else if (tid < cnt) {
         double f[6];

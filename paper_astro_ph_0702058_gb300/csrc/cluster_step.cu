@@ -147,12 +147,14 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_step_kernel(const ClArg
         //    block (unchanged) and the rows it corrected (their new ones), stored into every CTA
         unsigned long long m = (mine && !hit) ? due_c[tid] : ~0ull;
         if (tid < cnt_last) m = due_r[tid] < m ? due_r[tid] : m;
-        m = block_reduce(m, MinOp(), red_u64, ~0ull);
+        m = warp_min(m);
+        if (lane == 0) red_u64[warp] = m;
+        __syncthreads();
+        if (warp == 0) m = warp_min(lane < kClWarps ? red_u64[lane] : ~0ull);
         if (warp == 0 && lane < C) *cl.map_shared_rank(&x_min[rank], lane) = m;
         cl.sync();  // barrier A: every corrector of the last block has finished
         if (rank == 0 && tid == 0) x_flags = __ldcg(&A.st->flags);  // stored into the others below
-        tb = ~0ull;
-        for (int r = 0; r < C; ++r) tb = x_min[r] < tb ? x_min[r] : tb;
+        tb = warp_min(lane < C ? x_min[lane] : ~0ull);
 
         // 2. this CTA's active particles (ascending) and its particles predicted to tb
         {

@@ -157,9 +157,10 @@ __global__ void __launch_bounds__(kGrThreads, 1) grid_step_kernel(const GrArgs A
     int na = 0;
     for (;;) {
         // 1. this CTA's earliest due tick, its particles due then (ascending), published
+        const unsigned flags_now = tid == 0 ? __ldcg(&A.st->flags) : 0u;  // (published below)
         unsigned long long m = ~0ull;
         for (int k = tid; k < nown; k += kGrThreads) m = due_c[k] < m ? due_c[k] : m;
-        m = block_reduce(m, MinOp(), red_u64, ~0ull);
+        m = block_min(m, red_u64);
         int cnt = 0;
         for (int base = 0; base < nown; base += kGrThreads) {
             const int k = base + tid;
@@ -182,7 +183,7 @@ __global__ void __launch_bounds__(kGrThreads, 1) grid_step_kernel(const GrArgs A
         if (tid == 0) {
             A.pub[g].m = m;
             A.pub[g].cnt = cnt;
-            A.pub[g].flags = __ldcg(&A.st->flags);
+            A.pub[g].flags = flags_now;
         }
         if (A.skip_arrival && done == 0 && g == G - 1) break;
         if (!barrier()) break;

@@ -73,6 +73,12 @@ __device__ __forceinline__ double rsqrt_f64(const double x)
     return __fma_rn(__dmul_rn(y0, e), __fma_rn(0.375, e, 0.5), y0);
 }
 
+// Neither infinite nor NaN, on the integer pipe.
+__device__ __forceinline__ bool finite_f64(const double d)
+{
+    return (static_cast<unsigned int>(__double2hiint(d)) & 0x7ff00000u) != 0x7ff00000u;
+}
+
 __device__ __forceinline__ double norm3(const double *u)
 {
     return sqrt(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
@@ -130,13 +136,25 @@ struct CorrDt {
 __device__ __forceinline__ CorrDt corr_dt(const int64_t steps, const double tick, const int lmax)
 {
     CorrDt d;
+    // A step of 2^k ticks of 2^-lmax (every particle of a block): dt = 2^e with
+    // e = k - lmax, and every quantity but dt/3 is a power of two, dt/3 that power
+    // times the rounded 1/3.  They are built from exponent bits on the integer pipe
+    // (the conversion and the products below, ~8 dependent operations of ~64 cycles
+    // on the FP64 pipe, give the same bits).
+    const int e = (__ffsll(steps) - 1) - lmax;
+    if (steps > 0 && (steps & (steps - 1)) == 0 && e >= -250 && e <= 250) {
+        auto pow2 = [](const int k) { return __longlong_as_double(static_cast<long long>(1023 + k) << 52); };
+        d.dt = pow2(e);
+        d.idt = pow2(-e);
+        d.idt2 = pow2(-2 * e);
+        d.dt3 = pow2(3 * e);
+        d.dt4 = pow2(4 * e);
+        d.pd = {d.dt, pow2(e - 1),
+                __longlong_as_double(__double_as_longlong(1.0 / 3.0) + static_cast<long long>(e) * (1ll << 52))};
+        return d;
+    }
     d.dt = static_cast<double>(steps) * tick;
-    // 1/dt: when the step is 2^k ticks of 2^-lmax (every particle of a block) it
-    // is 2^(lmax - k), built from its exponent bits; otherwise an IEEE division.
-    // Both give the same bits.
-    d.idt = (steps > 0 && (steps & (steps - 1)) == 0)
-                ? __longlong_as_double(static_cast<long long>(1023 + lmax - (__ffsll(steps) - 1)) << 52)
-                : 1.0 / d.dt;
+    d.idt = 1.0 / d.dt;
     d.idt2 = d.idt * d.idt;
     d.dt3 = d.dt * d.dt * d.dt;
     d.dt4 = d.dt3 * d.dt;
@@ -216,7 +234,7 @@ __device__ __forceinline__ int corr_level(const double a2, const double k2, cons
     } else {
         // grow one level, only if the new time is a multiple of twice the old step
         const int64_t two_old = int64_t(2) << (lmax - l_old);
-        l_new = (l_old - 1 >= lmin && t_new % two_old == 0) ? l_old - 1 : l_old;
+        l_new = (l_old - 1 >= lmin && (t_new & (two_old - 1)) == 0) ? l_old - 1 : l_old;
     }
     if (clamped) {
         atomicOr(&st->flags, kFlagDtMin);
@@ -233,6 +251,7 @@ __device__ __forceinline__ int correct_row(const State &S, const int64_t i, cons
                                             const double *kp_in, const int64_t t_new, const double tick,
                                             const double eta, const int lmin, const int lmax, DevStatus *st)
 {
+    const int l_old = ld_state<CG>(S.level + i);
     const CorrDt d = corr_dt(t_new - ld_state<CG>(S.t + i), tick, lmax);
     double ap[3], kp[3], a2e[3], a3[3];
     bool finite = true;
@@ -243,7 +262,7 @@ __device__ __forceinline__ int correct_row(const State &S, const int64_t i, cons
         double xn, vn;
         corr_dim(ld_state<CG>(S.x[c] + i), ld_state<CG>(S.v[c] + i), ld_state<CG>(S.a[c] + i),
                  ld_state<CG>(S.k[c] + i), ap[c], kp[c], d, xn, vn, a2e[c], a3[c]);
-        finite = finite && isfinite(xn) && isfinite(vn) && isfinite(ap[c]) && isfinite(kp[c]);
+        finite = finite && finite_f64(xn) && finite_f64(vn) && finite_f64(ap[c]) && finite_f64(kp[c]);
         S.x[c][i] = xn;
         S.v[c][i] = vn;
         S.a[c][i] = ap[c];
@@ -251,7 +270,7 @@ __device__ __forceinline__ int correct_row(const State &S, const int64_t i, cons
     }
     // Eq. (timestep) with end-of-step quantities.
     const int l_new = corr_level(square3(ap), square3(kp), square3(a2e), square3(a3), eta, lmin, lmax,
-                                 ld_state<CG>(S.level + i), t_new, finite, st);
+                                 l_old, t_new, finite, st);
     S.t[i] = t_new;
     S.level[i] = static_cast<int8_t>(l_new);
     return l_new;
@@ -277,6 +296,27 @@ __device__ __forceinline__ T block_reduce(T v, Op op, T *sh, T id)
     v = sh[0];
     __syncthreads();
     return v;
+}
+
+// Minimum over the warp, in every lane: the high words first, then the low words of
+// the lanes that have the smallest (two warp reductions instead of ten shuffles).
+__device__ __forceinline__ unsigned long long warp_min(const unsigned long long v)
+{
+    const unsigned hi = static_cast<unsigned>(v >> 32), lo = static_cast<unsigned>(v);
+    const unsigned mh = __reduce_min_sync(0xffffffffu, hi);
+    const unsigned ml = __reduce_min_sync(0xffffffffu, hi == mh ? lo : ~0u);
+    return static_cast<unsigned long long>(mh) << 32 | ml;
+}
+
+// Minimum over the block, in every thread, with one barrier.  sh: one word per warp,
+// not stored to again before the block's next barrier.
+__device__ __forceinline__ unsigned long long block_min(unsigned long long v, unsigned long long *sh)
+{
+    v = warp_min(v);
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    return warp_min(lane < static_cast<int>(blockDim.x >> 5) ? sh[lane] : ~0ull);
 }
 
 struct MinOp {
