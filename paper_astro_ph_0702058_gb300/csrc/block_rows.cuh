@@ -209,10 +209,11 @@ __device__ __forceinline__ void rows_force(const float *jsm, const int stride_rt
 // correct_row, in parallel); more rows one per thread q < cnt.  GB300's FP64
 // unit is one per SM and takes ~19 cycles per warp instruction whatever the
 // number of active lanes, so rows are packed into as few warps as possible.
-// The state is read through L2 (another CTA of the launch may have written it).
+// R says where the state is (GlobalRows<true> where another CTA of the launch may
+// have written it).
 // due(q, r, t) receives each row's new due tick t (from one thread per row).
-template <bool DSW, class Due>
-__device__ __forceinline__ void rows_correct(const State &S, const int *idx, const float (*fh)[6],
+template <bool DSW, class Rows, class Due>
+__device__ __forceinline__ void rows_correct(const Rows &R, const int *idx, const float (*fh)[6],
                                              const float (*fl)[6], const int cnt, const unsigned long long tb,
                                              const double tick, const double eta, const int lmin, const int lmax,
                                              DevStatus *st, Due &&due)
@@ -225,21 +226,15 @@ __device__ __forceinline__ void rows_correct(const State &S, const int *idx, con
             const int qq = live ? q : 0;
             const int r = idx[qq];
             const int c = part < 3 ? part : 2;
-            const int l_old = ld_state<true>(S.level + r);
-            const CorrDt d = corr_dt(static_cast<int64_t>(tb) - ld_state<true>(S.t + r), tick, lmax);
+            const int l_old = R.level(r);
+            const CorrDt d = corr_dt(static_cast<int64_t>(tb) - R.t(r), tick, lmax);
             double u[4];  // this component of a_p, k_p, a^(2), a^(3)
             u[0] = DSW ? f2d(fh[qq][c]) + f2d(fl[qq][c]) : f2d(fh[qq][c]);
             u[1] = DSW ? f2d(fh[qq][3 + c]) + f2d(fl[qq][3 + c]) : f2d(fh[qq][3 + c]);
             double xn, vn;
-            corr_dim(ld_state<true>(S.x[c] + r), ld_state<true>(S.v[c] + r), ld_state<true>(S.a[c] + r),
-                     ld_state<true>(S.k[c] + r), u[0], u[1], d, xn, vn, u[2], u[3]);
+            corr_dim(R.x(c, r), R.v(c, r), R.a(c, r), R.k(c, r), u[0], u[1], d, xn, vn, u[2], u[3]);
             const bool ok = finite_f64(xn) && finite_f64(vn) && finite_f64(u[0]) && finite_f64(u[1]);
-            if (live && part < 3) {
-                S.x[part][r] = xn;
-                S.v[part][r] = vn;
-                S.a[part][r] = u[0];
-                S.k[part][r] = u[1];
-            }
+            if (live && part < 3) R.put(part, r, xn, vn, u[0], u[1]);
             // (lane 3 of a row repeats lane 2's component)
             const bool finite = ((__ballot_sync(0xffffffffu, ok) >> base) & 15u) == 15u;
             // the 4 x 4 transpose: lane p of a row gets quantity p of lanes (components) 0, 1, 2
@@ -261,8 +256,7 @@ __device__ __forceinline__ void rows_correct(const State &S, const int *idx, con
             if (live && part == 0) {
                 const int l_new = corr_level(aa, kk, s2, t2, eta, lmin, lmax, l_old, static_cast<int64_t>(tb), finite,
                                              st);
-                S.t[r] = static_cast<int64_t>(tb);
-                S.level[r] = static_cast<int8_t>(l_new);
+                R.put_time(r, static_cast<int64_t>(tb), l_new);
                 due(q, r, tb + (1ull << (lmax - l_new)));
             }
             __syncwarp();  // what due() stored is seen by the whole warp
@@ -272,7 +266,7 @@ __device__ __forceinline__ void rows_correct(const State &S, const int *idx, con
 #pragma unroll
         for (int c = 0; c < 6; ++c) f[c] = DSW ? f2d(fh[tid][c]) + f2d(fl[tid][c]) : f2d(fh[tid][c]);
         const int r = idx[tid];
-        const int l_new = correct_row<true>(S, r, f, f + 3, static_cast<int64_t>(tb), tick, eta, lmin, lmax, st);
+        const int l_new = correct_row_at(R, r, f, f + 3, static_cast<int64_t>(tb), tick, eta, lmin, lmax, st);
         due(tid, r, tb + (1ull << (lmax - l_new)));
     }
 }

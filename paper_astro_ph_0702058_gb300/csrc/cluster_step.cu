@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_step_kernel(const ClArg
                 const int o = r / chunk;
                 if (NB_CHECK(o < C && r - o * chunk < chunk, A.st, 6)) *cl.map_shared_rank(&due_c[r - o * chunk], o) = dd;
             };
-            rows_correct<DSW>(S, row_idx, f_hi, f_lo, cnt, tb, A.tick, A.eta, A.lmin, A.lmax, A.st, due);
+            rows_correct<DSW>(GlobalRows<true>{S}, row_idx, f_hi, f_lo, cnt, tb, A.tick, A.eta, A.lmin, A.lmax, A.st, due);
         }
         cnt_last = cnt;
         ++done;

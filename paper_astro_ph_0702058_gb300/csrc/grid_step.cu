@@ -25,7 +25,8 @@
 //   4. each CTA adds the G partials of each of its own rows in CTA order (lanes
 //      over CTAs, then a butterfly: double-single in compensated mode) and
 //      corrects them (rows_correct), keeping their new due ticks.
-// The state of a particle is read and written by its owner only; what crosses
+// The state of a particle is read and written by its owner only (in shared memory
+// where it fits, for the whole launch); what crosses
 // CTAs (published ticks, the list, the row buffer, the partials) is read through
 // L2 after a barrier.  The barriers count arrivals on one counter in global
 // memory (zeroed before each launch) and give up after ~1 s, raising the
@@ -84,10 +85,17 @@ struct GrArgs {
 // offsets; the kernel is built for a few strides, the smallest that holds the
 // chunk is launched), their due ticks and its rows of a block.
 constexpr int kGrStrides[4] = {512, 1024, 2048, kGrMaxChunk};
+// Up to a stride of 1024 there is room for the state of the CTA's particles too (105
+// bytes each, 160 KB in all at 1024 in compensated mode): loaded at the start of the
+// launch, stored when it ends, so that neither the prediction nor the corrector waits
+// for L2 and no barrier for the corrector's stores (a block of 5001 particles 18.3 ->
+// 17.5 us, of 65536 51.0 -> 49.5 us).
+constexpr bool gr_keeps_state(const int sj) { return sj <= 1024; }
 template <int MODE, int SJ>
 constexpr size_t gr_smem()
 {
-    return static_cast<size_t>(SJ) * (SoaTile<MODE>::NA * sizeof(float) + sizeof(unsigned long long) + sizeof(int));
+    return static_cast<size_t>(SJ) * (SoaTile<MODE>::NA * sizeof(float) + sizeof(unsigned long long) + sizeof(int) +
+                                      (gr_keeps_state(SJ) ? kRowWords * sizeof(double) + sizeof(int8_t) : 0));
 }
 
 template <int MODE, int SJ>
@@ -116,11 +124,24 @@ __global__ void __launch_bounds__(kGrThreads, 1) grid_step_kernel(const GrArgs A
     const int nown = max(0, min(lo + CH, n) - lo);
     const int L = (nown + 3) & ~3;  // entries the force reads: own particles, then massless padding
     const int RM = A.rows_max;
+    constexpr bool KEEP = gr_keeps_state(SJ);
+    const auto R = [&] {  // the state of this CTA's particles
+        if constexpr (KEEP)
+            return SharedRows<SJ>{reinterpret_cast<double *>(own + SJ), lo};
+        else
+            return GlobalRows<true>{S};
+    }();
 
+    if constexpr (KEEP)
+        for (int k = tid; k < nown; k += kGrThreads) {
+            const int i = lo + k;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) R.put(c, i, S.x[c][i], S.v[c][i], S.a[c][i], S.k[c][i]);
+            R.put_time(i, S.t[i], S.level[i]);
+        }
     for (int k = tid; k < CH; k += kGrThreads) {
         const bool in = k < nown;
-        due_c[k] = in ? static_cast<unsigned long long>(ld_state<true>(S.t + lo + k) +
-                                                        (int64_t(1) << (A.lmax - ld_state<true>(S.level + lo + k))))
+        due_c[k] = in ? static_cast<unsigned long long>(R.t(lo + k) + (int64_t(1) << (A.lmax - R.level(lo + k))))
                       : ~0ull;
 #pragma unroll
         for (int a = 0; a < NA; ++a) jsm[a * SJ + k] = in ? 0.0f : (a < 3 ? kPadPosition : 0.0f);
@@ -139,12 +160,11 @@ __global__ void __launch_bounds__(kGrThreads, 1) grid_step_kernel(const GrArgs A
     auto predict_own = [&](const unsigned long long t, float *dst, const int64_t stride, const int64_t base) {
         for (int k = tid; k < nown; k += kGrThreads) {
             const int i = lo + k;
-            const PredDt pd = pred_dt(static_cast<double>(static_cast<int64_t>(t) - ld_state<true>(S.t + i)) * A.tick);
+            const PredDt pd = pred_dt(static_cast<double>(static_cast<int64_t>(t) - R.t(i)) * A.tick);
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 double xp, vp;
-                predict_dim(ld_state<true>(S.x[c] + i), ld_state<true>(S.v[c] + i), ld_state<true>(S.a[c] + i),
-                            ld_state<true>(S.k[c] + i), pd, xp, vp);
+                predict_dim(R.x(c, i), R.v(c, i), R.a(c, i), R.k(c, i), pd, xp, vp);
                 const float h = d2f_rn(xp);
                 dst[c * stride + base + k] = h;
                 dst[(4 + c) * stride + base + k] = d2f_rn(vp);
@@ -336,12 +356,27 @@ __global__ void __launch_bounds__(kGrThreads, 1) grid_step_kernel(const GrArgs A
             auto due = [&](const int, const int r, const unsigned long long dd) {
                 if (NB_CHECK(r >= lo && r - lo < nown, A.st, 10)) due_c[r - lo] = dd;
             };
-            rows_correct<DSW>(S, own + q0, f_hi, f_lo, cq, tb, A.tick, A.eta, A.lmin, A.lmax, A.st, due);
+            rows_correct<DSW>(R, own + q0, f_hi, f_lo, cq, tb, A.tick, A.eta, A.lmin, A.lmax, A.st, due);
             __syncthreads();
         }
         ++done;
         rows += na;
         last_t = static_cast<long long>(tb);
+    }
+    if constexpr (KEEP) {
+        __syncthreads();
+        for (int k = tid; k < nown; k += kGrThreads) {
+            const int i = lo + k;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                S.x[c][i] = R.x(c, i);
+                S.v[c][i] = R.v(c, i);
+                S.a[c][i] = R.a(c, i);
+                S.k[c][i] = R.k(c, i);
+            }
+            S.t[i] = R.t(i);
+            S.level[i] = static_cast<int8_t>(R.level(i));
+        }
     }
     if (g == 0 && tid == 0) {
         A.sched_out->t_blk = static_cast<long long>(tb);

@@ -243,16 +243,71 @@ __device__ __forceinline__ int corr_level(const double a2, const double k2, cons
     return l_new;
 }
 
+// Where the corrector and the predictor find particle i's state: the State's global
+// arrays (CG: loads through L2 only), or a copy of the particles lo .. in shared
+// memory, 13 arrays of 8-byte words (x, v, a, k by component, then t) and one of levels.
+template <bool CG>
+struct GlobalRows {
+    const State &S;
+    __device__ __forceinline__ double x(const int c, const int64_t i) const { return ld_state<CG>(S.x[c] + i); }
+    __device__ __forceinline__ double v(const int c, const int64_t i) const { return ld_state<CG>(S.v[c] + i); }
+    __device__ __forceinline__ double a(const int c, const int64_t i) const { return ld_state<CG>(S.a[c] + i); }
+    __device__ __forceinline__ double k(const int c, const int64_t i) const { return ld_state<CG>(S.k[c] + i); }
+    __device__ __forceinline__ int64_t t(const int64_t i) const { return ld_state<CG>(S.t + i); }
+    __device__ __forceinline__ int level(const int64_t i) const { return ld_state<CG>(S.level + i); }
+    __device__ __forceinline__ void put(const int c, const int64_t i, const double x, const double v, const double a,
+                                        const double k) const
+    {
+        S.x[c][i] = x;
+        S.v[c][i] = v;
+        S.a[c][i] = a;
+        S.k[c][i] = k;
+    }
+    __device__ __forceinline__ void put_time(const int64_t i, const int64_t t, const int level) const
+    {
+        S.t[i] = t;
+        S.level[i] = static_cast<int8_t>(level);
+    }
+};
+
+constexpr int kRowWords = 13;  // 8-byte words of a particle's state besides its level
+template <int STRIDE>
+struct SharedRows {
+    double *w;  // word q of particle i at w[q STRIDE + i - lo]
+    int lo;
+    __device__ __forceinline__ double x(const int c, const int64_t i) const { return w[c * STRIDE + static_cast<int>(i) - lo]; }
+    __device__ __forceinline__ double v(const int c, const int64_t i) const { return w[(3 + c) * STRIDE + static_cast<int>(i) - lo]; }
+    __device__ __forceinline__ double a(const int c, const int64_t i) const { return w[(6 + c) * STRIDE + static_cast<int>(i) - lo]; }
+    __device__ __forceinline__ double k(const int c, const int64_t i) const { return w[(9 + c) * STRIDE + static_cast<int>(i) - lo]; }
+    __device__ __forceinline__ int64_t t(const int64_t i) const { return __double_as_longlong(w[12 * STRIDE + static_cast<int>(i) - lo]); }
+    __device__ __forceinline__ int8_t *levels() const { return reinterpret_cast<int8_t *>(w + kRowWords * STRIDE); }
+    __device__ __forceinline__ int level(const int64_t i) const { return levels()[static_cast<int>(i) - lo]; }
+    __device__ __forceinline__ void put(const int c, const int64_t i, const double x, const double v, const double a,
+                                        const double k) const
+    {
+        double *p = w + c * STRIDE + static_cast<int>(i) - lo;
+        p[0] = x;
+        p[3 * STRIDE] = v;
+        p[6 * STRIDE] = a;
+        p[9 * STRIDE] = k;
+    }
+    __device__ __forceinline__ void put_time(const int64_t i, const int64_t t, const int level) const
+    {
+        w[12 * STRIDE + static_cast<int>(i) - lo] = __longlong_as_double(t);
+        levels()[static_cast<int>(i) - lo] = static_cast<int8_t>(level);
+    }
+};
+
 // Corrector of Sect. 2 for particle i (its forces at the predicted state in
 // ap_in[3], kp_in[3]), then Eq. (timestep) and the new level; the step ends
 // at tick t_new.  Updates x, v, a, k, t, level of i and returns the new level.
-template <bool CG = false>
-__device__ __forceinline__ int correct_row(const State &S, const int64_t i, const double *ap_in,
-                                            const double *kp_in, const int64_t t_new, const double tick,
-                                            const double eta, const int lmin, const int lmax, DevStatus *st)
+template <class Rows>
+__device__ __forceinline__ int correct_row_at(const Rows &R, const int64_t i, const double *ap_in, const double *kp_in,
+                                              const int64_t t_new, const double tick, const double eta, const int lmin,
+                                              const int lmax, DevStatus *st)
 {
-    const int l_old = ld_state<CG>(S.level + i);
-    const CorrDt d = corr_dt(t_new - ld_state<CG>(S.t + i), tick, lmax);
+    const int l_old = R.level(i);
+    const CorrDt d = corr_dt(t_new - R.t(i), tick, lmax);
     double ap[3], kp[3], a2e[3], a3[3];
     bool finite = true;
 #pragma unroll
@@ -260,20 +315,21 @@ __device__ __forceinline__ int correct_row(const State &S, const int64_t i, cons
         ap[c] = ap_in[c];
         kp[c] = kp_in[c];
         double xn, vn;
-        corr_dim(ld_state<CG>(S.x[c] + i), ld_state<CG>(S.v[c] + i), ld_state<CG>(S.a[c] + i),
-                 ld_state<CG>(S.k[c] + i), ap[c], kp[c], d, xn, vn, a2e[c], a3[c]);
+        corr_dim(R.x(c, i), R.v(c, i), R.a(c, i), R.k(c, i), ap[c], kp[c], d, xn, vn, a2e[c], a3[c]);
         finite = finite && finite_f64(xn) && finite_f64(vn) && finite_f64(ap[c]) && finite_f64(kp[c]);
-        S.x[c][i] = xn;
-        S.v[c][i] = vn;
-        S.a[c][i] = ap[c];
-        S.k[c][i] = kp[c];
+        R.put(c, i, xn, vn, ap[c], kp[c]);
     }
     // Eq. (timestep) with end-of-step quantities.
-    const int l_new = corr_level(square3(ap), square3(kp), square3(a2e), square3(a3), eta, lmin, lmax,
-                                 l_old, t_new, finite, st);
-    S.t[i] = t_new;
-    S.level[i] = static_cast<int8_t>(l_new);
+    const int l_new = corr_level(square3(ap), square3(kp), square3(a2e), square3(a3), eta, lmin, lmax, l_old, t_new,
+                                 finite, st);
+    R.put_time(i, t_new, l_new);
     return l_new;
+}
+__device__ __forceinline__ int correct_row(const State &S, const int64_t i, const double *ap_in, const double *kp_in,
+                                           const int64_t t_new, const double tick, const double eta, const int lmin,
+                                           const int lmax, DevStatus *st)
+{
+    return correct_row_at(GlobalRows<false>{S}, i, ap_in, kp_in, t_new, tick, eta, lmin, lmax, st);
 }
 
 // Block-wide reduction; `id` is the identity of `op` (pads missing warps).

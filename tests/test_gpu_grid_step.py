@@ -218,3 +218,10 @@ def test_grid_barrier_times_out_and_context_survives(torch):
         assert nb == nb_ref and sim.stats()["grid_blocks"] > 0
     for key in s:
         assert np.array_equal(s[key], s_ref[key]), key
+
+
+@pytest.mark.parametrize("mode", ["plain", "comp"])
+@pytest.mark.parametrize("n", [100003, 160001])
+def test_grid_blocks_of_large_chunks(torch, mode, n):
+    """1024 particles per CTA, the most whose state stays on the chip for the launch, and more of them."""
+    test_grid_blocks_against_the_oracle(torch, mode, n, 3)
