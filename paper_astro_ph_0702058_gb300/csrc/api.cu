@@ -1065,7 +1065,7 @@ int nbody_step(nbody_ctx *c, double t_end, int64_t max_steps, int64_t *n_steps)
     bool grid_pending = false;   // the next block is not scheduled on the host: the grid kernel schedules it
     if (grid && !c->grid_buf) {
         c->grid_rows = static_cast<int>(std::min<int64_t>(kGridRows, c->n));
-        NB_CUDA(dev_alloc(&c->grid_buf, grid_step_bytes(c->p.mode, c->grid_rows, grid_step_size(c->p.mode))),
+        NB_CUDA(dev_alloc(&c->grid_buf, grid_step_bytes(c->p.mode, c->n, c->grid_rows, grid_step_size(c->p.mode))),
                 "grid block-step scratch allocation");
     }
     while (r == NBODY_OK && tb <= tend && !(max_steps > 0 && done >= max_steps)) {

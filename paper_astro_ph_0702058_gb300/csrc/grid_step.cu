@@ -2,7 +2,7 @@
 // the block time-step scheme of Sect. 2 (the next block time and its active
 // particles, the predictor, the force of Eq. (Force) on the active particles,
 // the corrector and Eq. (timestep)) repeated on the device, the CTAs meeting at
-// three bounded grid barriers per block.
+// two bounded grid barriers per block.
 //
 // Past the one-cluster kernel's sizes, a block of a few hundred rows costs more
 // in the separate kernels' latency (three scheduler passes, the predictor, the
@@ -11,14 +11,14 @@
 // [g ch, (g+1) ch), ch = ceil(n / G) rounded up to 4, keeps their due ticks
 // t_i + dt_i and, each block, their prediction in shared memory.  Per block:
 //   1. each CTA takes the earliest due tick over its particles and lists its
-//      particles due then (ascending); it publishes the tick, the count and the
-//      status flags it sees; barrier;
+//      particles due then (ascending); it publishes the tick, the count, the
+//      status flags it sees, and those particles predicted to that tick: the
+//      block's rows if the tick is the earliest of all; barrier;
 //   2. every CTA takes the block time (the minimum), the block size and where
-//      its own rows start in the block's list (the counts of the CTAs before it
-//      that hold the minimum), all alike, and decides alike whether the block
-//      runs; it writes its rows into the list, predicts all of its particles to
-//      the block time into shared memory (structure of arrays) and copies its
-//      rows' predicted data into a row buffer; barrier;
+//      each CTA's rows start in the block's list (the counts of the CTAs before
+//      it that hold the minimum), all alike, and decides alike whether the block
+//      runs; it writes its rows into the list and predicts all of its particles
+//      to the block time into shared memory (structure of arrays);
 //   3. every CTA sums the pair terms of all of the block's rows over its own
 //      particles (T threads per row, rows_force) and writes one partial per row;
 //      barrier;
@@ -49,9 +49,10 @@ namespace {
 
 constexpr int kGrThreads = 512;
 constexpr int kGrWarps = kGrThreads / 32;
+constexpr int kGrMaxCtas = 256;  // CTAs of a launch (eight records per lane of a warp)
 
 // What each CTA publishes before the barrier of step 1.
-struct GrPub {
+struct __align__(16) GrPub {
     unsigned long long m;  // earliest due tick of its particles
     int cnt;               // its particles due then
     unsigned flags;        // the status flags it saw
@@ -63,7 +64,7 @@ struct GrArgs {
     int64_t n_pad;
     const float *mass_j;  // the j-stream's masses (float), n entries
     int chunk;            // particles per CTA, a multiple of 4
-    int rows_max;         // largest block this launch runs; rows of the row buffer
+    int rows_max;         // largest block this launch runs
     float eps2;
     double tick, eta;
     int lmin, lmax;
@@ -74,7 +75,8 @@ struct GrArgs {
     SchedOut *sched_out;
     StepLoop *L;
     int32_t *act_out;         // the block's list (n), for the host too
-    float *ri;                // predicted data of the block's rows: (NA - 1) x rows_max (no masses)
+    float *ri;                // predicted data of each CTA's due particles, from its chunk's start on: (NA - 1) x
+                              // G chunk (no masses)
     float *part;              // partials: rows_max x G x (12 or 6) floats
     GrPub *pub;               // G records
     unsigned long long *bar;  // barrier counter, zero at launch
@@ -110,7 +112,8 @@ __global__ void __launch_bounds__(kGrThreads, 1) grid_step_kernel(const GrArgs A
     __shared__ unsigned long long red_u64[32];
     __shared__ int warp_tot[kGrWarps];
     __shared__ unsigned long long s_tb;
-    __shared__ int s_na, s_off, s_ok;
+    __shared__ int s_ok;
+    __shared__ int s_pfx[kGrMaxCtas + 1];  // where each CTA's rows start in the block's list; then the block size
     __shared__ unsigned s_flags;
 
     const int CH = A.chunk;
@@ -155,23 +158,29 @@ __global__ void __launch_bounds__(kGrThreads, 1) grid_step_kernel(const GrArgs A
         if (tid == 0) atomicOr(&A.st->flags, static_cast<unsigned>(kFlagTimeout));
         return false;
     };
+    // component c of particle i predicted with the factors pd (the predictor kernel's values): x, y, z
+    // at dst[c stride], vx, vy, vz at dst[(VA + c) stride] and, compensated, the lo parts of x, y, z after them
+    auto predict_c = [&](const int i, const int c, const PredDt &pd, float *dst, const int64_t stride, const int VA) {
+        double xp, vp;
+        predict_dim(R.x(c, i), R.v(c, i), R.a(c, i), R.k(c, i), pd, xp, vp);
+        const float h = d2f_rn(xp);
+        dst[c * stride] = h;
+        dst[(VA + c) * stride] = d2f_rn(vp);
+        if (DSW) dst[(VA + 3 + c) * stride] = d2f_rn(xp - f2d(h));  // the difference is exact
+    };
+    auto step_to = [&](const unsigned long long t, const int i) {
+        return pred_dt(static_cast<double>(static_cast<int64_t>(t) - R.t(i)) * A.tick);
+    };
     // this CTA's particles predicted to tick t: array a of particle lo + k at dst[a * stride + base + k]
-    // (x, y, z, vx, vy, vz and, compensated, the lo parts of x, y, z: the predictor kernel's values)
+    // (x, y, z, m (left alone), vx, vy, vz and the lo parts)
     auto predict_own = [&](const unsigned long long t, float *dst, const int64_t stride, const int64_t base) {
         for (int k = tid; k < nown; k += kGrThreads) {
-            const int i = lo + k;
-            const PredDt pd = pred_dt(static_cast<double>(static_cast<int64_t>(t) - R.t(i)) * A.tick);
+            const PredDt pd = step_to(t, lo + k);
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                double xp, vp;
-                predict_dim(R.x(c, i), R.v(c, i), R.a(c, i), R.k(c, i), pd, xp, vp);
-                const float h = d2f_rn(xp);
-                dst[c * stride + base + k] = h;
-                dst[(4 + c) * stride + base + k] = d2f_rn(vp);
-                if (DSW) dst[(7 + c) * stride + base + k] = d2f_rn(xp - f2d(h));  // the difference is exact
-            }
+            for (int c = 0; c < 3; ++c) predict_c(lo + k, c, pd, dst + base + k, stride, 4);
         }
     };
+    const int64_t RS = static_cast<int64_t>(G) * CH;  // entries per array of A.ri
     long long done = 0, rows = 0, last_t = A.last_t, predicted = -1;
     unsigned long long tb = ~0ull;
     int na = 0;
@@ -205,46 +214,62 @@ __global__ void __launch_bounds__(kGrThreads, 1) grid_step_kernel(const GrArgs A
             A.pub[g].cnt = cnt;
             A.pub[g].flags = flags_now;
         }
+        // the block's rows if m is the earliest tick of all, for every CTA, one component per thread: a wasted
+        // prediction elsewhere, but no third barrier for the rows (with barriers by release and acquire instead of
+        // full fences, a block of 5001 particles 17.5 -> 15.4 us)
+        if (cnt <= RM)
+            for (int e = tid; e < 3 * cnt; e += kGrThreads) {
+                const int q = e / 3, i = own[q];
+                predict_c(i, e - 3 * q, step_to(m, i), A.ri + lo + q, RS, 3);
+            }
         if (A.skip_arrival && done == 0 && g == G - 1) break;
         if (!barrier()) break;
 
         // 2. the block time and size, where this CTA's rows start, the decision (all alike)
         if (warp == 0) {
+            constexpr int PER = kGrMaxCtas / 32;
+            const int per = (G + 31) / 32;  // records per lane, in order
+            ulonglong2 rec[PER];            // the tick; the count and, high, the flags
             unsigned long long mm = ~0ull;
-            for (int r = lane; r < G; r += 32) {
-                const unsigned long long v = __ldcg(&A.pub[r].m);
-                mm = v < mm ? v : mm;
+#pragma unroll
+            for (int u = 0; u < PER; ++u) {
+                const int r = lane * per + u;
+                rec[u] = u < per && r < G ? __ldcg(reinterpret_cast<const ulonglong2 *>(A.pub + r)) : ulonglong2{~0ull, 0ull};
             }
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const unsigned long long v = __shfl_xor_sync(0xffffffffu, mm, o);
-                mm = v < mm ? v : mm;
-            }
-            int before = 0, total = 0;
+            for (int u = 0; u < PER; ++u) mm = rec[u].x < mm ? rec[u].x : mm;
+            mm = warp_min(mm);
+            int sum = 0;
             unsigned fl = 0;
-            for (int r = lane; r < G; r += 32) {
-                const int c = __ldcg(&A.pub[r].m) == mm ? __ldcg(&A.pub[r].cnt) : 0;
-                total += c;
-                before += r < g ? c : 0;
-                fl |= __ldcg(&A.pub[r].flags);
-            }
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                total += __shfl_xor_sync(0xffffffffu, total, o);
-                before += __shfl_xor_sync(0xffffffffu, before, o);
-                fl |= __shfl_xor_sync(0xffffffffu, fl, o);
+            for (int u = 0; u < PER; ++u) {
+                sum += rec[u].x == mm ? static_cast<int>(rec[u].y) : 0;
+                fl |= static_cast<unsigned>(rec[u].y >> 32);
             }
+            fl = __reduce_or_sync(0xffffffffu, fl);
+            int incl = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            int at = incl - sum;
+#pragma unroll
+            for (int u = 0; u < PER; ++u) {
+                const int r = lane * per + u;
+                if (u < per && r < G) s_pfx[r] = at;
+                at += rec[u].x == mm ? static_cast<int>(rec[u].y) : 0;
+            }
+            if (lane == 31) s_pfx[G] = incl;
             if (lane == 0) {
                 s_tb = mm;
-                s_na = total;
-                s_off = before;
                 s_flags = fl;
             }
         }
         __syncthreads();
         tb = s_tb;
-        na = s_na;
-        const int off = s_off;
+        na = s_pfx[G];
+        const int off = s_pfx[g];
         const int mine = m == tb ? cnt : 0;
         const bool go = done < A.budget && (s_flags & A.stop_flags) == 0u && static_cast<long long>(tb) <= A.t_end &&
                         na > 0 && na <= RM;
@@ -260,14 +285,6 @@ __global__ void __launch_bounds__(kGrThreads, 1) grid_step_kernel(const GrArgs A
         }
         predict_own(tb, jsm, SJ, 0);  // this CTA's particles predicted to tb, into shared memory
         __syncthreads();
-        for (int q = tid; q < mine; q += kGrThreads) {  // the rows' predicted data for every CTA
-            const int k = own[q] - lo;
-#pragma unroll
-            for (int a = 0; a < NA; ++a)
-                if (a != 3 && NB_CHECK(off + q < RM, A.st, 9))
-                    A.ri[(a < 3 ? a : a - 1) * RM + off + q] = jsm[a * SJ + k];
-        }
-        if (!barrier()) break;
 
         // 3. the pair terms of every row of the block over this CTA's particles: one partial per row
         {
@@ -277,9 +294,15 @@ __global__ void __launch_bounds__(kGrThreads, 1) grid_step_kernel(const GrArgs A
             while (T > 1 && (T * na > kGrThreads || 8 * T > L)) T >>= 1;
             auto load_i = [&](const int rr, const bool live, I2 &I) {
                 const int p = live ? rr : 0;
-                const float *r = A.ri + p;
-                const float x = __ldcg(r), y = __ldcg(r + RM), z = __ldcg(r + 2 * RM);
-                const float vx = __ldcg(r + 3 * RM), vy = __ldcg(r + 4 * RM), vz = __ldcg(r + 5 * RM);
+                int o = 0;  // the CTA that owns the row: the last whose rows start at or before p
+                for (int hi = G; hi - o > 1;) {
+                    const int mid = (o + hi) >> 1;
+                    (s_pfx[mid] <= p ? o : hi) = mid;
+                }
+                const int q = p - s_pfx[o];
+                const float *r = A.ri + (NB_CHECK(q < CH, A.st, 9) ? o * CH + q : 0);
+                const float x = __ldcg(r), y = __ldcg(r + RS), z = __ldcg(r + 2 * RS);
+                const float vx = __ldcg(r + 3 * RS), vy = __ldcg(r + 4 * RS), vz = __ldcg(r + 5 * RS);
                 I.x = f2_pack(x, x);
                 I.y = f2_pack(y, y);
                 I.z = f2_pack(z, z);
@@ -287,12 +310,12 @@ __global__ void __launch_bounds__(kGrThreads, 1) grid_step_kernel(const GrArgs A
                 I.vy = f2_pack(vy, vy);
                 I.vz = f2_pack(vz, vz);
                 if (DSW) {
-                    const float lx = __ldcg(r + 6 * RM), ly = __ldcg(r + 7 * RM), lz = __ldcg(r + 8 * RM);
+                    const float lx = __ldcg(r + 6 * RS), ly = __ldcg(r + 7 * RS), lz = __ldcg(r + 8 * RS);
                     I.lx = f2_pack(lx, lx);
                     I.ly = f2_pack(ly, ly);
                     I.lz = f2_pack(lz, lz);
                 }
-                return live ? __ldcg(A.act_out + p) : -1;
+                return live && o == g ? own[q] : -1;  // (only an own particle is among the entries)
             };
             auto no_ds = [](const int, const bool, dsa::ds (&)[3], dsa::ds (&)[3]) { return -1; };
             auto store = [&](const int rr, const float *tot, const float *lw) {
@@ -412,7 +435,7 @@ int grid_size_for()
             cudaGetLastError();
             return 0;
         }
-        return sms;
+        return sms < kGrMaxCtas ? sms : kGrMaxCtas;
     }();
     return size;
 }
@@ -439,13 +462,14 @@ cudaError_t launch_mode(const cudaLaunchConfig_t &cfg, const GrArgs &A)
 
 // The scratch: barrier counter, published records, row buffer, partials, each
 // starting on a 256-byte boundary; returns the bytes and fills the offsets.
-size_t grid_layout(const int mode, const int rows_max, const int ctas, size_t off[4])
+size_t grid_layout(const int mode, const int64_t n, const int rows_max, const int ctas, size_t off[4])
 {
     const size_t na = mode == kModeComp ? SoaTile<kModeComp>::NA : SoaTile<kModePlain>::NA;
     const size_t pw = mode == kModeComp ? 12 : 6;
     const size_t rm = static_cast<size_t>(rows_max);
     const size_t sizes[4] = {sizeof(unsigned long long), sizeof(GrPub) * static_cast<size_t>(ctas),
-                             sizeof(float) * (na - 1) * rm, sizeof(float) * pw * rm * static_cast<size_t>(ctas)};
+                             sizeof(float) * (na - 1) * static_cast<size_t>(grid_step_chunk(n, ctas)) * static_cast<size_t>(ctas),
+                             sizeof(float) * pw * rm * static_cast<size_t>(ctas)};
     size_t at = 0;
     for (int q = 0; q < 4; ++q) {
         off[q] = at;
@@ -470,10 +494,10 @@ int grid_step_chunk(int64_t n, int ctas)
     return ch <= kGrMaxChunk ? static_cast<int>(ch) : 0;
 }
 
-size_t grid_step_bytes(int mode, int rows_max, int ctas)
+size_t grid_step_bytes(int mode, int64_t n, int rows_max, int ctas)
 {
     size_t off[4];
-    return grid_layout(mode, rows_max, ctas, off);
+    return grid_layout(mode, n, rows_max, ctas, off);
 }
 
 cudaError_t grid_step_launch(int mode, const State &S, const JStream &J, double eps2, double eta, int lmin, int lmax,
@@ -506,7 +530,7 @@ cudaError_t grid_step_launch(int mode, const State &S, const JStream &J, double 
     A.L = L;
     A.act_out = act_out;
     size_t off[4];
-    grid_layout(mode, rows_max, G, off);
+    grid_layout(mode, S.n, rows_max, G, off);
     unsigned char *p = static_cast<unsigned char *>(buf);
     A.bar = reinterpret_cast<unsigned long long *>(p + off[0]);
     A.pub = reinterpret_cast<GrPub *>(p + off[1]);

@@ -268,7 +268,7 @@ cudaError_t cluster_step_launch(int mode, const State &S, const JStream &J, doub
 // ---- grid_step.cu ----
 // Block steps of larger systems (n <= CTAs x kGrMaxChunk) as one cooperative
 // launch of one CTA per SM, packed plain and compensated modes, with the same
-// contract as cluster_step_launch; `buf` is grid_step_bytes(mode, rows_max,
+// contract as cluster_step_launch; `buf` is grid_step_bytes(mode, n, rows_max,
 // grid_step_size(mode)) bytes of device scratch.  When it stops at a block
 // larger than rows_max (with budget left, due by t_end, no stop flag) it also
 // leaves the j-stream (J.soa) predicted to that block's time and sets
@@ -279,7 +279,7 @@ constexpr int kGrMaxChunk = 3584;  // particles per CTA (their prediction is hel
 int grid_step_size(int mode);
 // Particles per CTA for n (ceil(n / ctas) rounded up to 4), or 0 when above kGrMaxChunk.
 int grid_step_chunk(int64_t n, int ctas);
-size_t grid_step_bytes(int mode, int rows_max, int ctas);
+size_t grid_step_bytes(int mode, int64_t n, int rows_max, int ctas);
 cudaError_t grid_step_launch(int mode, const State &S, const JStream &J, double eps2, double eta, int lmin, int lmax,
                              long long t_end, long long budget, int rows_max, long long last_t, unsigned stop_flags,
                              DevStatus *st, SchedOut *sched_out, StepLoop *L, int32_t *act_out, void *buf,

@@ -63,7 +63,7 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
     return false;
 }
 
-// Device-scope acquire load (pairs with the fence before an arrival).
+// Device-scope acquire load (pairs with the release of an arrival).
 __device__ __forceinline__ unsigned long long ld_acquire_gpu(const unsigned long long *p)
 {
     unsigned long long v;
@@ -72,7 +72,8 @@ __device__ __forceinline__ unsigned long long ld_acquire_gpu(const unsigned long
 }
 
 // Barrier of all CTAs of a cooperative launch (all co-resident): thread 0 of
-// each CTA fences the CTA's stores, adds 1 to *ctr (zero at launch) and waits
+// each CTA adds 1 to *ctr (zero at launch) with release order, which covers the
+// stores of the CTA's other threads before __syncthreads, and waits with acquire loads
 // until it reaches `target` + CTAs (target: thread 0's count of arrivals
 // expected so far, advanced here).  Gives up after ~1 s of wall time and
 // returns false (the caller records a timeout); every thread of the CTA calls
@@ -83,8 +84,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned long long *ctr, unsigned l
     __syncthreads();
     if (threadIdx.x == 0) {
         target += ctas;
-        __threadfence();
-        atomicAdd(ctr, 1ull);
+        asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(ctr) : "memory");
         bool ok = false;
         const uint64_t t0 = global_timer_ns();
         for (uint32_t it = 0; it < (1u << 26); ++it) {
@@ -94,7 +94,6 @@ __device__ __forceinline__ bool grid_barrier(unsigned long long *ctr, unsigned l
             }
             if ((it & 63u) == 63u && global_timer_ns() - t0 > 1000000000ull) break;
         }
-        __threadfence();
         *s_ok = ok;
     }
     __syncthreads();
