@@ -117,18 +117,19 @@ __device__ __forceinline__ void rows_force(const float *jsm, const int stride_rt
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const f2_t E2 = f2_pack(eps2, eps2);
     const f2_t NEG3 = f2_pack(-3.0f, -3.0f);
-    int T = T0, rpp = NT / T0;
+    int T = T0, lt = 31 - __clz(T0), rpp = NT >> lt;  // T = 2^lt (an integer division is a chain of ~100 cycles)
     for (int q0 = 0; q0 < cnt; q0 += rpp) {
         if constexpr (SHARE) {  // the rows left for a last, partly filled pass share its threads (two groups
             if (q0 > 0)         // of 4 j each at least)
                 while (2 * T * (cnt - q0) <= NT && 16 * T <= L) T <<= 1;
-            rpp = NT / T;
+            lt = 31 - __clz(T);
+            rpp = NT >> lt;
         }
         const int TW = T < 32 ? T : 32;
-        const int rr = q0 + tid / T;
-        const int sub = tid % T;
+        const int rr = q0 + (tid >> lt);
+        const int sub = tid & (T - 1);
         const bool live = rr < cnt;
-        const bool warp_live = q0 + warp * 32 / T < cnt;  // a warp with no row skips the sums
+        const bool warp_live = q0 + (warp * 32 >> lt) < cnt;  // a warp with no row skips the sums
         float tot[7], lo[7];
 #pragma unroll
         for (int c = 0; c < 7; ++c) tot[c] = lo[c] = 0.0f;
@@ -140,7 +141,7 @@ __device__ __forceinline__ void rows_force(const float *jsm, const int stride_rt
             dsa::ds sum[7];
 #pragma unroll
             for (int c = 0; c < 7; ++c) sum[c] = {0.0f, 0.0f};
-            const int my = warp_live ? (L - sub + T - 1) / T : 0;
+            const int my = warp_live ? (L - sub + T - 1) >> lt : 0;
 #pragma unroll 1
             for (int g = 0; g < my; ++g) {
                 const int e = g * T + sub;
@@ -155,7 +156,7 @@ __device__ __forceinline__ void rows_force(const float *jsm, const int stride_rt
         } else {
             I2 I;
             const int gi = load_i(rr, live, I);
-            const int my = warp_live ? (L / 4 - sub + T - 1) / T : 0;  // this thread's groups of 4 j
+            const int my = warp_live ? (L / 4 - sub + T - 1) >> lt : 0;  // this thread's groups of 4 j
             // with eps > 0 the pair j = i adds exact zeros to the acceleration and jerk (dx = dv = 0,
             // r^2 = eps^2, m r^-3 finite for eps^2 >= 1e-12 and m < 1e20), so only the potential or a
             // tiny or zero eps needs the mask, and only in a warp with a row whose particle is among the
