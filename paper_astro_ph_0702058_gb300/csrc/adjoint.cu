@@ -24,6 +24,20 @@ namespace nb {
 
 namespace {
 
+// The kernels of a rollout's steps are launched with programmatic stream
+// serialisation (launch_after): once every block of this kernel runs, the next
+// one's may be scheduled, and each waits here, before its first read or write of
+// memory, until the kernel before it is complete and its stores are visible.  A
+// step's kernels take 5 to 15 us each, so the 1 to 2 us between two of them
+// count (4096 particles, 64 steps, loss and gradient 7.01 -> 6.72 ms; below 2000
+// particles the host issues no faster than the kernels end).  What these kernels read was written by the one before, so
+// their pointers are not __restrict__ (no read-only loads).
+__device__ __forceinline__ void after_previous()
+{
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 constexpr int kVjpRows = 64;  // rows of a warp
 
 // Sums of a pair that both of its particles need.  Row data packed for two rows
@@ -119,9 +133,8 @@ __device__ __forceinline__ void vjp_fold(float *p, const size_t n, const int c, 
 // 1500 12.8 -> 9.0 us.
 template <int H, bool FOLD>
 __global__ void __launch_bounds__(32, 12)
-    vjp_pairs_kernel(const float4 *__restrict__ posm, const float4 *__restrict__ vel, const float4 *__restrict__ gA,
-                     const float4 *__restrict__ gK, const int n, const float eps2, const int S, const int tiles,
-                     float *__restrict__ part)
+    vjp_pairs_kernel(const float4 *posm, const float4 *vel, const float4 *gA, const float4 *gK, const int n,
+                     const float eps2, const int S, const int tiles, float *part)
 {
     static_assert(!FOLD || H == 1, "tiles of a superblock whole");
     constexpr int NC = FOLD ? 14 : 7;
@@ -139,6 +152,7 @@ __global__ void __launch_bounds__(32, 12)
     const int j_end = min(n, (J + 1) * sb);
     const f2_t E2 = f2_pack(eps2, eps2);
     const float4 far = make_float4(kPadPosition, kPadPosition, kPadPosition, 0.f), zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    after_previous();
     for (int i0 = I * sb; i0 < min(n, (I + 1) * sb); i0 += kVjpRows) {
         const int r0 = i0 + lane, r1 = r0 + 32;
         VjpRow p;
@@ -310,13 +324,15 @@ __global__ void __launch_bounds__(32 * kLanes)
 // the reduction, the corrector, the copy of the state and the predictor
 // (n = 4096: 7.5 + 11.0 + 2 + 4.7 us before).
 template <bool DSW>
-__global__ void __launch_bounds__(32 * kLanes) roll_step_kernel(const double *src, double *dst, const int n, const double *__restrict__ acc,
-                                 const double *__restrict__ jerk, const float *__restrict__ part, const int split,
-                                 const CorrDt d, const bool predict, const JStream J, DevStatus *st)
+__global__ void __launch_bounds__(32 * kLanes)
+    roll_step_kernel(const double *src, double *dst, const int n, const double *acc, const double *jerk,
+                     const float *part, const int split, const CorrDt d, const bool predict, const JStream J,
+                     DevStatus *st)
 {
     const int idx = blockIdx.x * 32 + (threadIdx.x & 31);
     const bool live = idx < 3 * n;
     const int c = live ? idx / n : 0, i = live ? idx - c * n : 0;
+    after_previous();
     double ap, kp;
     if (part) {
         constexpr int NC = DSW ? 14 : 7;
@@ -372,12 +388,14 @@ struct AdjDt {
 // (left in ga, gk); without it the force at t = 0, whose upstream is (ga, gk)
 // itself.  Last, the j-stream the force adjoint reads, at the prediction of
 // that step from its state `src` (dt = 0 at t = 0).
-__global__ void __launch_bounds__(32 * kLanes) adj_step_kernel(const float *__restrict__ part, const VjpSlots V, const DiffGrads G, const int n,
-                                const AdjDt d, const bool corrector, const double *__restrict__ src, const JStream J)
+__global__ void __launch_bounds__(32 * kLanes)
+    adj_step_kernel(const float *part, const VjpSlots V, const DiffGrads G, const int n, const AdjDt d,
+                    const bool corrector, const double *src, const JStream J)
 {
     const int idx = blockIdx.x * 32 + (threadIdx.x & 31);
     const bool live = idx < 3 * n;
     const int c = live ? idx / n : 0, i = live ? idx - c * n : 0;
+    after_previous();
     double t[3];
     if (V.sb > 0)
         column_sums(V.sb * V.parts + 1, [&](int s, int v, float &a, float &b) {
@@ -498,6 +516,23 @@ __global__ void sum_kernel(const double *__restrict__ v, int64_t n, double *out)
     if (threadIdx.x == 0) *out = s[0];
 }
 
+// A launch whose blocks may start while the stream's previous kernel still runs; the
+// kernel waits for that one in after_previous().
+template <class... P, class... A>
+cudaError_t launch_after(void (*kernel)(P...), const unsigned grid, const unsigned block, cudaStream_t s, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 int blocks_of(int64_t n, int t) { return static_cast<int>((n + t - 1) / t); }
 
 }  // namespace
@@ -529,11 +564,10 @@ cudaError_t force_vjp_launch(const JStream &J, const DiffGrads &G, int64_t n, fl
     const unsigned units = static_cast<unsigned>(static_cast<int64_t>(V.sb) * (V.sb + 1) / 2 * V.parts);
     auto *kernel = V.two_word ? vjp_pairs_kernel<1, true> : V.parts == 2 ? vjp_pairs_kernel<2, false>
                                                                          : vjp_pairs_kernel<1, false>;
-    kernel<<<units, 32, 0, s>>>(J.posm, J.vel, G.gA, G.gK, static_cast<int>(n), eps2, V.sb, V.rows / kVjpRows,
-                                static_cast<float *>(scratch));
     ++*launches;
     *slots = V;
-    return cudaGetLastError();
+    return launch_after(kernel, units, 32, s, J.posm, J.vel, G.gA, G.gK, static_cast<int>(n), eps2, V.sb,
+                        V.rows / kVjpRows, static_cast<float *>(scratch));
 }
 
 cudaError_t vjp_finish_launch(const DiffGrads &G, int64_t n, const void *scratch, const VjpSlots &slots, cudaStream_t s,
@@ -558,9 +592,9 @@ cudaError_t roll_step_launch(const double *src, double *dst, int64_t n, const do
     d.dt4 = d.dt3 * dt;
     d.pd = {dt, 0.5 * dt, dt * (1.0 / 3.0)};
     auto *kernel = two_word ? roll_step_kernel<true> : roll_step_kernel<false>;
-    kernel<<<blocks_of(3 * n, 32), 32 * kLanes, 0, s>>>(src, dst, static_cast<int>(n), acc, jerk, part, split, d, predict, J, st);
     ++*launches;
-    return cudaGetLastError();
+    return launch_after(kernel, blocks_of(3 * n, 32), 32 * kLanes, s, src, dst, static_cast<int>(n), acc, jerk, part,
+                        split, d, predict, J, st);
 }
 
 cudaError_t adj_step_launch(const void *scratch, const VjpSlots &slots, const DiffGrads &G, int64_t n, double dt, bool corrector,
@@ -577,10 +611,9 @@ cudaError_t adj_step_launch(const void *scratch, const VjpSlots &slots, const Di
     d.i2 = d.i1 * d.i1;
     d.i3 = d.i2 * d.i1;
     d.pd = {dt, 0.5 * dt, dt * (1.0 / 3.0)};
-    adj_step_kernel<<<blocks_of(3 * n, 32), 32 * kLanes, 0, s>>>(static_cast<const float *>(scratch), slots, G, static_cast<int>(n), d,
-                                                   corrector, src, J);
     ++*launches;
-    return cudaGetLastError();
+    return launch_after(adj_step_kernel, blocks_of(3 * n, 32), 32 * kLanes, s, static_cast<const float *>(scratch),
+                        slots, G, static_cast<int>(n), d, corrector, src, J);
 }
 
 namespace {
