@@ -704,8 +704,8 @@ def diff_workload(args):
         torch.cuda.synchronize()
         ts.append(time.perf_counter() - t0)
     t = statistics.median(ts)
-    # forward (steps + 1 forces), recomputed segments (steps forces), one force VJP per force
-    pair_passes = (steps + 1) + steps + (steps + 1)
+    # forward (steps + 1 forces; at this size every state is kept, so no segment runs again), one force VJP per force
+    pair_passes = 2 * (steps + 1)
     print(json.dumps({"workload": "diff (C5)", "n": n, "steps": steps, "dt": 2.0 ** -level,
                       "checkpoint_every": ck, "ms_per_gradient": t * 1e3, "gradients_per_s": 1.0 / t,
                       "pair_passes": pair_passes, "pairs_per_s": pair_passes * n * (n - 1) / t,

@@ -30,8 +30,9 @@ namespace {
 // memory, until the kernel before it is complete and its stores are visible.  A
 // step's kernels take 5 to 15 us each, so the 1 to 2 us between two of them
 // count (4096 particles, 64 steps, loss and gradient 7.01 -> 6.72 ms; below 2000
-// particles the host issues no faster than the kernels end).  What these kernels read was written by the one before, so
-// their pointers are not __restrict__ (no read-only loads).
+// particles the host issues no faster than the kernels end).  What these kernels
+// read was written by the one before, so their pointers are not __restrict__ (no
+// read-only loads).
 __device__ __forceinline__ void after_previous()
 {
     asm volatile("griddepcontrol.launch_dependents;");
