@@ -24,7 +24,7 @@
 //   window  the W warps of a CTA take the W chunks of 128 j of a tile in turn
 //           (warp w chunk (k + w) mod W in window k), one block barrier per
 //           window, so no two warps add to one j's sums at a time.
-//   sums    FP32 over 128 terms, folded into (hi, lo) by TwoSum (compensated) or
+//   sums    FP32 over 128 terms (compensated: two of 64, added), folded into (hi, lo) by TwoSum (compensated) or
 //           an FP32 sum (plain), as in force_x2.cuh.  The folded sums live in
 //           the unit's own slots of `part`: the rows of I in slot J, those of J
 //           in slot I (I = J: the second side in slot n_sb), the j-ranges outside
@@ -167,14 +167,24 @@ __device__ __forceinline__ void sym_load_j(const float *chunk, const int jl, f2_
 
 // A warp's 128 rows against a chunk of 128 j, both sides.  DIAG: the chunk is
 // the rows themselves, of which only the pairs j > i count.  pj_out: the sums
-// of the chunk's j (jlive of them exist), component stride n.
+// of the chunk's j (jlive of them exist), component stride n.  Compensated: the
+// rows' sums of the first 64 j wait at mid (14 x 32 words of the warp) and are added
+// at the end, so an FP32 sum has 64 terms, as each half of force_x2.cuh's (128 terms
+// in one made the error at n = 30000 11 % larger than the one-sided kernel's; folded
+// twice as often through L2 instead, the full force at 2^20 took 880 ms, not 853).
 template <int MODE, bool DIAG, int UNROLL>
 __device__ __forceinline__ void sym_both(const float *chunk, const SymI &I, const int lane, const f2_t E2,
                                          const f2_t NEG3, f2_t (&pi)[2][7], float *pj_out, const int jlive,
-                                         const size_t n, const bool jfirst)
+                                         const size_t n, const bool jfirst, f2_t *mid)
 {
 #pragma unroll 1
     for (int r = 0; r < kSymRows; r += 32) {
+        if (MODE == kModeComp && r == kSymRows / 2)
+#pragma unroll
+            for (int q = 0; q < 14; ++q) {
+                mid[32 * q + lane] = pi[q / 7][q % 7];
+                pi[q / 7][q % 7] = 0ull;
+            }
         f2_t pj[7];
 #pragma unroll
         for (int c = 0; c < 7; ++c) pj[c] = 0ull;
@@ -212,6 +222,9 @@ __device__ __forceinline__ void sym_both(const float *chunk, const SymI &I, cons
             }
         }
     }
+    if (MODE == kModeComp)
+#pragma unroll
+        for (int q = 0; q < 14; ++q) pi[q / 7][q % 7] = f2_add(pi[q / 7][q % 7], mid[32 * q + lane]);
 }
 
 // Element e of array a of a structure of arrays of n; past its end a massless
@@ -231,6 +244,8 @@ __global__ void __launch_bounds__(32 * W, WARPS / W) force_sym_kernel(const SymP
     constexpr int BT = W * kSymRows;  // rows of a tile
     constexpr int CH = sym_chunk_floats<MODE>();
     __shared__ __align__(16) float sj[W * CH];
+    __shared__ f2_t s_mid[DSW ? W * 14 * 32 : 1];
+    f2_t *mid = s_mid + (DSW ? (threadIdx.x >> 5) * 14 * 32 : 0);
     if (P.skip && *P.skip != 0) return;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int n = P.n;
@@ -308,10 +323,10 @@ __global__ void __launch_bounds__(32 * W, WARPS / W) force_sym_kernel(const SymP
                     for (int q = 0; q < 7; ++q) pi[g][q] = 0ull;
                 const bool jfirst = it == 0 && k == 0;  // (each chunk that exists meets a warp in window 0)
                 if (own && k == 0)
-                    sym_both<MODE, true, 1>(sj + c * CH, I, lane, E2, NEG3, pi, pj_out + jr, j_end - jr, n, jfirst);
+                    sym_both<MODE, true, 1>(sj + c * CH, I, lane, E2, NEG3, pi, pj_out + jr, j_end - jr, n, jfirst, mid);
                 else
                     sym_both<MODE, false, UNROLL>(sj + c * CH, I, lane, E2, NEG3, pi, pj_out + jr, j_end - jr, n,
-                                                  jfirst);
+                                                  jfirst, mid);
 #pragma unroll
                 for (int g = 0; g < 2; ++g) {
                     const int r0 = i0 + lane + 64 * g, r1 = r0 + 32;
