@@ -24,14 +24,13 @@ constexpr int kSymThreads = 256;
 constexpr int kSymScan = 4 * kSymThreads;  // particles of a block of the compaction
 
 // Resident warps per SM the registers are limited for, and the unroll factor of
-// the pair loop.  Measured at n = 262144, ms: plain 12 warps x 8 43.7, x 4 45.0, 16
-// warps (128 registers) x 4 45.4, x 8 44.9; compensated 16 x 4 53.0 (x 2 56.7, x 8
-// 53.3), 12 x 8 54.1, x 4 54.3; one-warp CTAs (n = 16384, us): plain 12 x 8 235,
-// 16 x 4 231, compensated 12 x 8 280, 16 x 4 291.
+// the pair loop.  Measured at n = 262144, ms: plain (with r^-3 first, sym_add_both) 12
+// warps x 8 43.7, x 4 45.0, 16 warps (128 registers) x 4 45.4, x 8 44.9; compensated
+// 16 x 8 53.1, x 4 54.3, 12 x 8 55.0, x 4 56.0; one-warp CTAs (n = 16384, us): plain
+// 12 x 8 235, 16 x 4 231, compensated 12 x 8 280, 16 x 4 291.
 template <int MODE, int W>
 struct SymShape {
-    static constexpr bool wide = MODE == kModeComp && W > 1;
-    static constexpr int unroll = wide ? 4 : 8, warps = wide ? 16 : 12;
+    static constexpr int unroll = 8, warps = MODE == kModeComp && W > 1 ? 16 : 12;
 };
 
 template <int MODE, int W>

@@ -1,10 +1,10 @@
 // Force of a large block by pairs: an unordered pair (i, j) of active particles
 // is formed once and gives both particles their terms of Eq. (Force).
 //
-// The differences, r^2, r^-1, r^-3 and 3 (dx.dv) r^-2 of Appendix A's pair term
+// The differences, r^2, r^-1, r^-2 and 3 (dx.dv) r^-2 of Appendix A's pair term
 // are the same for (i, j) and (j, i) but for signs that cancel or flip, so the
-// second force of a pair costs 8 more FP32 operations instead of 27 (33 in
-// compensated mode): 35 (41) operations per unordered pair, packed two pairs to
+// second force of a pair costs 9 more FP32 operations instead of 27 (33 in
+// compensated mode): 36 (42) operations per unordered pair, packed two pairs to
 // an instruction as in force_x2.cuh.
 //
 // Layout:
@@ -35,11 +35,11 @@
 // reads six 32-bit words and issues every 3 cycles, not 2 (measured: 3.01; 2.2
 // where consecutive ones share an operand; scalar FMAs 1.0 each, but mixing
 // them with packed ones costs their switch, 3344 against 2947 us at n = 65536
-// plain).  19 of the 35 operations are such FMAs: 87 cycles for two pairs.
+// plain).  17 of the 36 operations are such FMAs.
 // Measured against the one-sided kernel (force_kernel_x2) with its reduction,
 // full forces, us: n = 8192 plain 82 -> 67, compensated 96 -> 78; 16384: 251 ->
-// 194, 301 -> 242; 65536: 3566 -> 2816, 4331 -> 3395; 262144: 55672 -> 43727,
-// 66448 -> 53021.
+// 194, 301 -> 242; 65536: 3566 -> 2840, 4331 -> 3403; 262144: 55672 -> 44100,
+// 66448 -> 53130.
 // Two rows per lane instead of four (96 registers) took 3276 us at n = 65536
 // plain; r^-2 from the MUFU reciprocal instead of a product 0.5-2 % more.
 #pragma once
@@ -69,10 +69,10 @@ struct SymI {
 
 // What two pair terms leave for the sums of both sides.
 struct SymT {
-    f2_t dx, dy, dz, ux, uy, uz, y, y3;
+    f2_t dx, dy, dz, ux, uy, uz, y, y2;
 };
 
-// Pair terms of two rows and one j: dx = x_j - x_i, y = r^-1, y3 = r^-3 and
+// Pair terms of two rows and one j: dx = x_j - x_i, y = r^-1, y2 = r^-2 and
 // u = dv - 3 (dx.dv) r^-2 dx.  ma, mb: pairs to leave out (their terms are zero).
 template <int MODE, bool MASK>
 __device__ __forceinline__ void sym_term(const f2_t (&v)[10], const SymI &I, const int g, const f2_t E2,
@@ -97,26 +97,59 @@ __device__ __forceinline__ void sym_term(const f2_t (&v)[10], const SymI &I, con
     }
     T.y = f2_pack(rsqrt_mufu(a), rsqrt_mufu(b));
     const f2_t xv = f2_fma(T.dz, dvz, f2_fma(T.dy, dvy, f2_mul(T.dx, dvx)));
-    const f2_t y2 = f2_mul(T.y, T.y);
-    T.y3 = f2_mul(T.y, y2);
-    const f2_t w = f2_mul(f2_mul(xv, y2), NEG3);
+    T.y2 = f2_mul(T.y, T.y);
+    const f2_t w = f2_mul(f2_mul(xv, T.y2), NEG3);
     T.ux = f2_fma(w, T.dx, dvx);
     T.uy = f2_fma(w, T.dy, dvy);
     T.uz = f2_fma(w, T.dz, dvz);
 }
 
-// m r^-3 dx, m r^-3 u and m r^-1 added to the sums of one side (the signs of
-// the j side and of the potential are applied when the sums are folded).
-__device__ __forceinline__ void sym_add(const f2_t m, const SymT &T, f2_t (&p)[7])
+// m r^-3 dx, m r^-3 u and m r^-1 added to the sums of both sides (the signs of
+// the j side and of the potential are applied when the sums are folded).  The
+// mass comes first, as in force_x2.cuh: r^-3 alone leaves FP32's range for r
+// above 2^42 or below 2^-42, where m r^-1 r^-2 need not (a cluster in metres).
+// That is 6 products and additions of two registers where r^-3 first took 3 and
+// 2 FMAs of three.  Compensated, every product before the FMAs: at the 128
+// registers of 16 warps the sides one after the other spill more (n = 262144,
+// ms: 53.1 against 56.2 at an unroll of 4, 53.1 with r^-3 first); plain, which
+// has 168, they are faster so (44.1 against 45.0, 43.7 with r^-3 first).
+__device__ __forceinline__ void sym_add(const f2_t s, const SymT &T, f2_t (&p)[7])
 {
-    const f2_t s = f2_mul(m, T.y3);
     p[0] = f2_fma(s, T.dx, p[0]);
     p[1] = f2_fma(s, T.dy, p[1]);
     p[2] = f2_fma(s, T.dz, p[2]);
     p[3] = f2_fma(s, T.ux, p[3]);
     p[4] = f2_fma(s, T.uy, p[4]);
     p[5] = f2_fma(s, T.uz, p[5]);
-    p[6] = f2_fma(T.y, m, p[6]);
+}
+template <int MODE>
+__device__ __forceinline__ void sym_add_both(const f2_t mj, const f2_t mi, const SymT &T, f2_t (&pi)[7], f2_t (&pj)[7])
+{
+    if constexpr (MODE == kModeComp) {
+        const f2_t a = f2_mul(mj, T.y), b = f2_mul(mi, T.y);
+        pi[6] = f2_add(pi[6], a);
+        pj[6] = f2_add(pj[6], b);
+        const f2_t s = f2_mul(a, T.y2), t = f2_mul(b, T.y2);
+        pi[0] = f2_fma(s, T.dx, pi[0]);
+        pj[0] = f2_fma(t, T.dx, pj[0]);
+        pi[1] = f2_fma(s, T.dy, pi[1]);
+        pj[1] = f2_fma(t, T.dy, pj[1]);
+        pi[2] = f2_fma(s, T.dz, pi[2]);
+        pj[2] = f2_fma(t, T.dz, pj[2]);
+        pi[3] = f2_fma(s, T.ux, pi[3]);
+        pj[3] = f2_fma(t, T.ux, pj[3]);
+        pi[4] = f2_fma(s, T.uy, pi[4]);
+        pj[4] = f2_fma(t, T.uy, pj[4]);
+        pi[5] = f2_fma(s, T.uz, pi[5]);
+        pj[5] = f2_fma(t, T.uz, pj[5]);
+    } else {
+        const f2_t a = f2_mul(mj, T.y);
+        sym_add(f2_mul(a, T.y2), T, pi);
+        pi[6] = f2_add(pi[6], a);
+        const f2_t b = f2_mul(mi, T.y);
+        sym_add(f2_mul(b, T.y2), T, pj);
+        pj[6] = f2_add(pj[6], b);
+    }
 }
 
 // Adds x to the sum of component c kept at p (component stride n).
@@ -199,10 +232,7 @@ __device__ __forceinline__ void sym_both(const float *chunk, const SymI &I, cons
                 sym_term<MODE, DIAG>(v, I, g, E2, NEG3, DIAG && jl <= lane + 64 * g, DIAG && jl <= lane + 64 * g + 32,
                                      T[g]);
 #pragma unroll
-            for (int g = 0; g < 2; ++g) {
-                sym_add(v[3], T[g], pi[g]);
-                sym_add(I.m[g], T[g], pj);
-            }
+            for (int g = 0; g < 2; ++g) sym_add_both<MODE>(v[3], I.m[g], T[g], pi[g], pj);
             // j goes to the next lane down, and its sums with it
 #pragma unroll
             for (int c = 0; c < 7; ++c) {

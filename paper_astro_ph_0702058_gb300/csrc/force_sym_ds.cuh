@@ -124,7 +124,6 @@ __device__ __forceinline__ void sym_ds_pair(const dsx::Row &I, const dsx::Row &J
     const f2_t half = f2_pack(0.5f, 0.5f), c38 = f2_pack(0.375f, 0.375f);
     const d2 y = fast_sum(y0, f2_mul(y0, f2_mul(rho, f2_fma(c38, rho, half))));
     const d2 y2 = fast_sum(p, f2_fma(p, f2_fma(rho, rho, rho), pe));
-    const d2 y3 = norm(prod(y, y2, sign));
     // -3 (dx.dv) r^-2
     const f2_t m3 = f2_pack(-3.0f, -3.0f);
     prod2 q3;
@@ -136,7 +135,9 @@ __device__ __forceinline__ void sym_ds_pair(const dsx::Row &I, const dsx::Row &J
     add(xv, prod(dx[2], dv[2], sign));
     xv = fast_sum(xv.h, xv.l);
     const d2 w = norm(prod(xv, norm(q3), sign));
-    const d2 sI = norm(prod(J.m, y3, sign)), sJ = norm(prod(I.m, y3, sign));
+    // (the mass first, as in ds_pair_term: r^-3 alone leaves FP32's range sooner)
+    const prod2 mrI = prod(J.m, y, sign), mrJ = prod(I.m, y, sign);
+    const d2 sI = norm(prod(norm(mrI), y2, sign)), sJ = norm(prod(norm(mrJ), y2, sign));
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         d2 u = dv[c];
@@ -147,8 +148,8 @@ __device__ __forceinline__ void sym_ds_pair(const dsx::Row &I, const dsx::Row &J
         add(sj[c], prod(sJ, dx[c], sign));
         add(sj[3 + c], prod(sJ, u, sign));
     }
-    add(si[6], prod(J.m, y, sign));
-    add(sj[6], prod(I.m, y, sign));
+    add(si[6], mrI);
+    add(sj[6], mrJ);
 }
 
 struct SymDsParams {

@@ -135,3 +135,26 @@ def test_double_single(torch, n, eps2):
         e = errors(*(u[rows] for u in g), *oracle.force(m, x, v, eps2, a[rows]))
         for k in ("acc", "jerk", "pot"):
             assert e[k].max() <= 1e-10, (k, e[k].max())
+
+
+# Units of length and mass that are powers of two change the exponents of every value and nothing else, so the forces
+# scale exactly while every intermediate stays within FP32's range; r^-3 by itself does not (2^-159 and 2^156 in plain
+# and compensated mode; in double-single mode its low words, 2^-132 with 24 bits, do not).
+@pytest.mark.parametrize("mode,n,length,mass", [("plain", 8192, 53, 80), ("comp", 8200, 53, 80), ("plain", 40000, 53, 80),
+                                                ("comp", 33000, 53, 80), ("plain", 8192, -44, -30),
+                                                ("comp", 8192, -44, -30), ("ds", 4096, 36, 72), ("ds", 4100, 36, 72)])
+def test_units_of_any_size(torch, mode, n, length, mass):
+    m, x, v = plummer_sphere(n, 12)
+    act = np.arange(n, dtype=np.int32)
+    got = []
+    for ln, ms in ((0, 0), (length, mass)):
+        lu, mu = 2.0 ** ln, 2.0 ** ms
+        with _sim(m * mu, x * lu, v * lu, EPS2 * lu * lu, mode) as sim:  # (velocities: the unit of time stays)
+            s = {k: np.zeros((n, 3)) for k in ("a", "k")}
+            sim.get_state(**s)  # the set-up's force, by pairs
+            assert sim.stats()["last_i_per_thread"] == (2 if mode == "ds" else 4)
+            sim.predict(0.0)
+            pot = gpu_force(sim, act)[2]
+        got.append((s["a"] * (lu * lu / mu), s["k"] * (lu * lu / mu), pot * (lu / mu)))
+    for one, other in zip(*got):
+        assert np.array_equal(one, other)
