@@ -259,6 +259,11 @@ const char *nbody_last_error(void);
  * (k >= 1; 0 disables).  Lets the out-of-memory paths be exercised. */
 void nbody_debug_fail_alloc(int k);
 
+/* Test hook, host arithmetic only: the bytes of partial sums that a force on
+ * n_act of n particles by unordered pairs would take on a GPU of sm_count SMs,
+ * or 0 where the rule on sizes leaves it to the one-sided kernels. */
+int64_t nbody_debug_pairs_bytes(int mode, int64_t n_act, int64_t n, int sm_count);
+
 /* Test hook: while on (nonzero), force kernels launched from this process do
  * not issue the copy of their first j-tile, so each block's bounded wait for
  * that tile gives up after about 2 s; the kernel records the timeout and

@@ -39,7 +39,7 @@ NBODY_MODE_DS = 4
 EXPORTS = ("nbody_default_params", "nbody_init", "nbody_next_block", "nbody_predict", "nbody_force",
            "nbody_correct", "nbody_step", "nbody_sync", "nbody_energy", "nbody_energy_ds", "nbody_get_state",
            "nbody_set_state", "nbody_get_predicted", "nbody_get_stats", "nbody_free", "nbody_strerror", "nbody_last_error",
-           "nbody_debug_fail_alloc", "nbody_debug_skip_tile_copy", "nbody_debug_step_graphs", "nbody_force_noalloc",
+           "nbody_debug_fail_alloc", "nbody_debug_pairs_bytes", "nbody_debug_skip_tile_copy", "nbody_debug_step_graphs", "nbody_force_noalloc",
            "nbody_ens_init", "nbody_ens_set_shape", "nbody_ens_tune", "nbody_ens_step", "nbody_ens_run",
            "nbody_ens_energy", "nbody_ens_get_state", "nbody_ens_get_stats", "nbody_ens_free",
            "nbody_diff_rollout", "nbody_rollout", "nbody_rollout_vjp")
@@ -103,6 +103,8 @@ def lib():
             L.nbody_last_error.restype = C.c_char_p
             L.nbody_debug_fail_alloc.argtypes = [C.c_int]
             L.nbody_debug_fail_alloc.restype = None
+            L.nbody_debug_pairs_bytes.argtypes = [C.c_int, C.c_int64, C.c_int64, C.c_int]
+            L.nbody_debug_pairs_bytes.restype = C.c_int64
             L.nbody_debug_skip_tile_copy.argtypes = [C.c_int]
             L.nbody_debug_skip_tile_copy.restype = None
             L.nbody_debug_step_graphs.argtypes = [C.c_int]
@@ -282,6 +284,10 @@ def nbody_last_error() -> str:
 
 def nbody_debug_fail_alloc(k: int) -> None:
     lib().nbody_debug_fail_alloc(int(k))
+
+
+def nbody_debug_pairs_bytes(mode: int, n_act: int, n: int, sm_count: int) -> int:
+    return lib().nbody_debug_pairs_bytes(int(mode), int(n_act), int(n), int(sm_count))
 
 
 def nbody_debug_skip_tile_copy(on: bool) -> None:

@@ -1360,6 +1360,12 @@ const char *nbody_last_error(void) { return g_err; }
 
 void nbody_debug_fail_alloc(int k) { g_fail_alloc = k > 0 ? k : 0; }
 
+int64_t nbody_debug_pairs_bytes(int mode, int64_t n_act, int64_t n, int sm_count)
+{
+    ForceConfig cfg{};
+    return sym_plan(mode, n_act, n, sm_count, &cfg) ? static_cast<int64_t>(force_partial_bytes(mode, cfg, n_act)) : 0;
+}
+
 void nbody_debug_skip_tile_copy(int on) { nb::g_skip_first_copy = on ? 1 : 0; }
 
 void nbody_debug_step_graphs(int level) { g_step_graphs = level < 0 ? 0 : (level > 3 ? 3 : level); }

@@ -252,8 +252,11 @@ bool sym_plan(int mode, int64_t n_act, int64_t n, int sm_count, ForceConfig *cfg
         if (n_act != n || n < kSymDsMin) return false;
         const int64_t slot = 14 * n * static_cast<int64_t>(sizeof(float));
         int64_t tiles = (n + kSymDsRows * kSymMaxSb - 1) / (kSymDsRows * kSymMaxSb), sb;
-        while (sb = (n + kSymDsRows * tiles - 1) / (kSymDsRows * tiles), (sb + 1) * slot > kSymPartCap) ++tiles;
-        if (sb * (sb + 1) / 2 < 12LL * sm_count) return false;
+        for (;; ++tiles) {  // fewer superblocks until their slots fit; too few units end it at any n
+            sb = (n + kSymDsRows * tiles - 1) / (kSymDsRows * tiles);
+            if (sb * (sb + 1) / 2 < 12LL * sm_count) return false;
+            if ((sb + 1) * slot <= kSymPartCap) break;
+        }
         cfg->threads = 32;
         cfg->ipt = 2;
         cfg->jsub = 1;
