@@ -112,6 +112,7 @@ struct nbody_ctx {
     double *stage = nullptr;  // 6 n doubles: external forces / AoS staging
     void *partials = nullptr;
     size_t partials_cap = 0;
+    int64_t scratch_gen = 0;  // counts the buffers partials has been: an address may come back with less room
     void *sym_buf = nullptr;  // scratch of the force by unordered pairs (sym_scratch_bytes), on first use
     void *sched_scratch = nullptr;
     SchedOut *sched_out = nullptr;
@@ -136,7 +137,7 @@ struct nbody_ctx {
     cudaGraphExec_t step_graph = nullptr;
     int64_t graph_rows = 0;
     ForceConfig graph_cfg{};
-    void *graph_partials = nullptr;
+    int64_t graph_scratch = -1;  // scratch_gen of the buffer it was captured with
     int64_t graph_launches = 0;  // kernel nodes per block step of a replay
     bool graph_loop = false;
     unsigned char *graph_fits = nullptr;  // graph_rows + 1 flags: block size na takes the graph's shape
@@ -217,15 +218,34 @@ int sync_and_check(nbody_ctx *c)
 int ensure_partials(nbody_ctx *c, size_t bytes)
 {
     if (bytes <= c->partials_cap) return NBODY_OK;
-    if (c->partials) {
+    auto drop = [&]() -> int {
+        if (!c->partials) return NBODY_OK;
         NB_CUDA(cudaStreamSynchronize(c->s), "stream synchronise");
         cudaFree(c->partials);
         c->partials = nullptr;
         c->partials_cap = 0;
-    }
+        ++c->scratch_gen;
+        return NBODY_OK;
+    };
+    // the new one first, so that a refusal leaves the old; without it where there is no room for both
     const size_t cap = std::max(bytes, static_cast<size_t>(1) << 20);
-    NB_CUDA(dev_alloc(&c->partials, cap), "partial-sum scratch allocation");
+    void *p = nullptr;
+    cudaError_t e = dev_alloc(&p, cap);
+    if (e == cudaErrorMemoryAllocation && c->partials) {
+        cudaGetLastError();
+        const int r = drop();
+        if (r != NBODY_OK) return r;
+        e = dev_alloc(&p, cap);
+    }
+    NB_CUDA(e, "partial-sum scratch allocation");
+    const int r = drop();
+    if (r != NBODY_OK) {
+        cudaFree(p);
+        return r;
+    }
+    c->partials = p;
     c->partials_cap = cap;
+    ++c->scratch_gen;
     return NBODY_OK;
 }
 
@@ -994,10 +1014,10 @@ int set_graph_fits(nbody_ctx *c)
     return NBODY_OK;
 }
 
-// Captures the graph once (and again when the partial-sum scratch moved).
+// Captures the graph once (and again when the partial-sum scratch is another buffer).
 int build_step_graph(nbody_ctx *c)
 {
-    if (c->step_graph && c->graph_partials == c->partials) return NBODY_OK;
+    if (c->step_graph && c->graph_scratch == c->scratch_gen) return NBODY_OK;
     if (c->step_graph) {
         cudaGraphExecDestroy(c->step_graph);
         c->step_graph = nullptr;
@@ -1028,7 +1048,7 @@ int build_step_graph(nbody_ctx *c)
         c->step_graph = nullptr;
         return cuda_fail(e, "step graph capture");
     }
-    c->graph_partials = c->partials;
+    c->graph_scratch = c->scratch_gen;
     c->graph_launches = launches;
     c->graph_loop = loop;
     return NBODY_OK;

@@ -90,3 +90,40 @@ def test_device_loop_stops_at_the_strict_error_block(torch):
     assert st0["graph_blocks"] == 0 and st2["graph_blocks"] == st2["blocks"]
     for key in s0:
         assert np.array_equal(s0[key], s2[key]), key
+
+
+@pytest.mark.parametrize("mode", ["plain", "comp"])
+def test_graph_after_its_scratch_was_replaced(torch, mode):
+    """A force between two steps that asks for much more partial-sum scratch, or is refused it, leaves the captured
+    block step on a buffer of the size it was captured with: the run goes on with the same bits."""
+    from paper_astro_ph_0702058_gb300 import Simulation, nbody_debug_fail_alloc, nbody_debug_step_graphs
+    n = 65536
+    m, x, v = plummer_sphere(n, 21)
+    every = np.arange(n, dtype=np.int32)
+    got = []
+    nbody_debug_step_graphs(2)
+    try:
+        for refused in (None, 1, 2, 3):  # which allocation of the force between the steps
+            nbody_debug_fail_alloc(3)  # the set-up's force one-sided: no scratch of the pairs yet
+            with Simulation(m, x, v, EPS2, eta=0.02, mode=mode) as sim:
+                nbody_debug_fail_alloc(0)
+                sim.step(1.0 / 64, 60)
+                if refused is not None:
+                    sim.predict(sim.next_block()[0])
+                    out = [np.zeros((n, 3)), np.zeros((n, 3)), np.zeros(n)]
+                    nbody_debug_fail_alloc(refused)
+                    sim.force(every, acc=out[0], jerk=out[1], pot=out[2])
+                    nbody_debug_fail_alloc(0)
+                    assert all(np.all(np.isfinite(o)) for o in out)
+                sim.step(1.0 / 64, 60)
+                s = dict(x=np.zeros((n, 3)), v=np.zeros((n, 3)), a=np.zeros((n, 3)), k=np.zeros((n, 3)),
+                         t_tick=np.zeros(n, dtype=np.int64), level=np.zeros(n, dtype=np.int8))
+                sim.get_state(**s)
+                assert sim.stats()["graph_blocks"] > 0
+            got.append(s)
+    finally:
+        nbody_debug_fail_alloc(0)
+        nbody_debug_step_graphs(3)
+    for other in got[1:]:
+        for key in other:
+            assert np.array_equal(other[key], got[0][key]), key
