@@ -122,6 +122,16 @@ void nbody_default_params(nbody_params *p);
  * m[n] masses, x[n*3] positions, v[n*3] velocities (copied; host or device),
  * softening eps2 >= 0.  Computes the full force on all particles at t = 0
  * and each particle's first level from dt = eta_init |a| / |k|.
+ * Device memory: about 340 n bytes for the life of the context, up to 110 n
+ * bytes and some tens of MB of scratch on first use, and, for forces by unordered pairs (blocks
+ * of >= 8192 rows, all particles from 4096 in the double-single mode), slots
+ * of partial sums: about 3.6 KB per row in plain mode, 7.2 KB in the others,
+ * 8 GiB at most, and only where they are no more than half of the free memory
+ * (else the one-sided kernels run; the results differ in the last bits).
+ * Slots up to 2 GiB stay for the next force; larger ones are given back when
+ * nbody_init, nbody_step or nbody_sync returns, unless a force was captured
+ * into a graph of the caller's, and all of them where another allocation of
+ * the context would fail.
  * On success *out receives the context (free with nbody_free).
  * Errors: EINVAL (null pointer, n < 1 or n > 2^31 - 1, eps2 < 0, bad levels or
  * mode), ENOMEM, ECUDA, ENONFINITE (non-finite input or initial force). */

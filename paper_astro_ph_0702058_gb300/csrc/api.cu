@@ -26,6 +26,10 @@ int g_fail_alloc = 0;    // allocation-failure injection countdown (test hook)
 int g_step_graphs = 3;
 constexpr int64_t kLoopCap = 1024;  // blocks one replay of the loop may run
 constexpr int64_t kPairsOwnList = 16384;  // rows of a caller's list that may take pairs (plain, compensated)
+// Slots of the force by pairs (up to 8 GiB) above this go back to the device when a call that waits ends: the next
+// force that takes them pays ~0.2 ms per GiB for the allocation and 0.5 for the free, 0.6 % of a full force at 2^20
+// particles (7.1 GiB, compensated), 2 % at 300000 (2 GiB), more below.
+constexpr size_t kSlotsKeep = size_t(2) << 30;
 constexpr int64_t kRollKeep = int64_t(1) << 30;  // bytes of states a gradient keeps instead of running steps again
 constexpr int64_t kClusterCap = 4096;  // blocks one launch of the cluster or the grid kernel may run
 #ifndef NB_GRID_ROWS
@@ -114,6 +118,9 @@ struct nbody_ctx {
     size_t partials_cap = 0;
     int64_t scratch_gen = 0;  // counts the buffers partials has been: an address may come back with less room
     void *sym_buf = nullptr;  // scratch of the force by unordered pairs (sym_scratch_bytes), on first use
+    void *slots = nullptr;    // and its partial sums; what holds more than kSlotsKeep is given back (give_back)
+    size_t slots_cap = 0;
+    bool slots_captured = false;  // a graph of the caller's may hold them: kept until nbody_free
     void *sched_scratch = nullptr;
     SchedOut *sched_out = nullptr;
     DevStatus *st = nullptr;
@@ -156,7 +163,7 @@ namespace {
 void release(nbody_ctx *c)
 {
     if (c->step_graph) cudaGraphExecDestroy(c->step_graph);
-    void *dev[] = {c->dev_base, c->partials, c->graph_fits, c->grid_buf, c->sym_buf};
+    void *dev[] = {c->dev_base, c->partials, c->graph_fits, c->grid_buf, c->sym_buf, c->slots};
     for (void *d : dev)
         if (d) cudaFree(d);
     if (c->host_base) cudaFreeHost(c->host_base);
@@ -215,6 +222,32 @@ int sync_and_check(nbody_ctx *c)
     return absorb_status(c);
 }
 
+// Frees the slots of the force by pairs (after the work that uses them).
+void drop_slots(nbody_ctx *c)
+{
+    if (!c->slots || c->slots_captured) return;
+    cudaStreamSynchronize(c->s);
+    cudaFree(c->slots);
+    c->slots = nullptr;
+    c->slots_cap = 0;
+}
+
+// At the end of a call that has waited: large slots back to the device.
+void give_back(nbody_ctx *c)
+{
+    if (c->slots_cap > kSlotsKeep) drop_slots(c);
+}
+
+// Device memory that a call cannot do without: the slots, which one can, make room for it.
+cudaError_t ctx_alloc(nbody_ctx *c, void **p, size_t bytes)
+{
+    const cudaError_t e = dev_alloc(p, bytes);
+    if (e != cudaErrorMemoryAllocation || !c->slots || c->slots_captured) return e;
+    cudaGetLastError();
+    drop_slots(c);
+    return dev_alloc(p, bytes);
+}
+
 int ensure_partials(nbody_ctx *c, size_t bytes)
 {
     if (bytes <= c->partials_cap) return NBODY_OK;
@@ -230,7 +263,7 @@ int ensure_partials(nbody_ctx *c, size_t bytes)
     // the new one first, so that a refusal leaves the old; without it where there is no room for both
     const size_t cap = std::max(bytes, static_cast<size_t>(1) << 20);
     void *p = nullptr;
-    cudaError_t e = dev_alloc(&p, cap);
+    cudaError_t e = ctx_alloc(c, &p, cap);
     if (e == cudaErrorMemoryAllocation && c->partials) {
         cudaGetLastError();
         const int r = drop();
@@ -261,14 +294,33 @@ bool own_device_ptr(const nbody_ctx *c, const void *p, const uintptr_t align)
     return a.type == cudaMemoryTypeDevice && a.device == c->dev;
 }
 
-// Scratch of the force by unordered pairs (cfg), or false where the device has no room for it.
+// Scratch and slots of the force by unordered pairs (cfg), or false where the device refuses them, where the slots
+// would take more than half of its free memory, or where a capture on the stream allows no allocation.
 bool sym_room(nbody_ctx *c, const ForceConfig &cfg, int64_t n_act)
 {
+    const size_t bytes = force_partial_bytes(c->p.mode, cfg, n_act);
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->s, &cs) != cudaSuccess) cudaGetLastError();
+    if (cs != cudaStreamCaptureStatusNone) {
+        if (!c->sym_buf || bytes > c->slots_cap) return false;
+        c->slots_captured = true;
+        return true;
+    }
     if (!c->sym_buf && dev_alloc(&c->sym_buf, sym_scratch_bytes(c->n)) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    return ensure_partials(c, force_partial_bytes(c->p.mode, cfg, n_act)) == NBODY_OK;
+    if (bytes <= c->slots_cap) return true;
+    if (c->slots && c->slots_captured) return false;
+    drop_slots(c);
+    size_t free_bytes = 0, all_bytes = 0;
+    if (cudaMemGetInfo(&free_bytes, &all_bytes) != cudaSuccess || bytes > free_bytes / 2 ||
+        dev_alloc(&c->slots, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    c->slots_cap = bytes;
+    return true;
 }
 
 // Force on a device list already in act_force.  With for_step, a shape whose
@@ -310,7 +362,7 @@ int force_internal(nbody_ctx *c, int64_t n_act, bool for_step = false, bool asce
             if (r != NBODY_OK) return r;
         }
         NB_CUDA(force_sym_launch(c->p.mode, c->J, c->n, c->act_force, n_act, c->eps2, cfg, ascending, c->f_acc,
-                                 c->f_jerk, c->f_pot, c->partials, c->sym_buf, &rows_general, c->st, c->s, &launches),
+                                 c->f_jerk, c->f_pot, c->slots, c->sym_buf, &rows_general, c->st, c->s, &launches),
                 "force kernel launch");
         if (rows_general) {  // (nothing to do for a list of distinct particles: ~5 us)
             NB_CUDA(force_launch(c->p.mode, c->J, c->n, c->act_force, n_act, c->eps2, general, c->f_acc, c->f_jerk,
@@ -553,7 +605,7 @@ int rollout_impl(const char *who, int64_t n, const double *m, const double *x0, 
         mem.add(&dloss, sizeof(double));
         mem.add(&g4, 2 * npad * sizeof(float4));
         mem.add(&vjp, vjp_bytes);
-        return mem.commit(&mem_base, dev_alloc);
+        return mem.commit(&mem_base, [&](void **p, size_t b) { return ctx_alloc(c, p, b); });
     };
     cudaError_t er = room();
     if (er == cudaErrorMemoryAllocation && keep) {
@@ -774,6 +826,7 @@ int nbody_init(nbody_ctx **out, int64_t n, const double *m, const double *x, con
     r = sync_and_check(c);
     if (r == NBODY_EDTMIN) r = NBODY_OK;  // the first steps may be clamped; counted, not fatal here
     if (r != NBODY_OK) return bail(r);
+    give_back(c);
     c->stats.n = n;
     c->stats.n_pad = c->n_pad;
     c->stats.mode = c->p.mode;
@@ -1008,7 +1061,7 @@ int set_graph_fits(nbody_ctx *c)
         fits[na] = force_choose(c->p.mode, na, c->n_pad, c->sm_count, c->p.j_tile, c->p.i_block, c->p.j_split,
                                 &cfg, c->p.j_sub) == NBODY_OK && same_shape(cfg, c->graph_cfg);
     }
-    NB_CUDA(dev_alloc(reinterpret_cast<void **>(&c->graph_fits), static_cast<size_t>(len)), "graph table allocation");
+    NB_CUDA(ctx_alloc(c, reinterpret_cast<void **>(&c->graph_fits), static_cast<size_t>(len)), "graph table allocation");
     NB_CUDA(cudaMemcpy(c->graph_fits, fits.data(), static_cast<size_t>(len), cudaMemcpyHostToDevice),
             "graph table upload");
     return NBODY_OK;
@@ -1085,7 +1138,7 @@ int nbody_step(nbody_ctx *c, double t_end, int64_t max_steps, int64_t *n_steps)
     bool grid_pending = false;   // the next block is not scheduled on the host: the grid kernel schedules it
     if (grid && !c->grid_buf) {
         c->grid_rows = static_cast<int>(std::min<int64_t>(kGridRows, c->n));
-        NB_CUDA(dev_alloc(&c->grid_buf, grid_step_bytes(c->p.mode, c->n, c->grid_rows, grid_step_size(c->p.mode))),
+        NB_CUDA(ctx_alloc(c, &c->grid_buf, grid_step_bytes(c->p.mode, c->n, c->grid_rows, grid_step_size(c->p.mode))),
                 "grid block-step scratch allocation");
     }
     while (r == NBODY_OK && tb <= tend && !(max_steps > 0 && done >= max_steps)) {
@@ -1228,13 +1281,17 @@ int nbody_step(nbody_ctx *c, double t_end, int64_t max_steps, int64_t *n_steps)
     }
     if (n_steps) *n_steps = done;
     if (r != NBODY_OK) return r;
-    return sync_and_check(c);
+    r = sync_and_check(c);
+    give_back(c);
+    return r;
 }
 
 int nbody_sync(nbody_ctx *c)
 {
     if (!c) return fail(NBODY_EINVAL, "nbody_sync: null context");
-    return sync_and_check(c);
+    const int r = sync_and_check(c);
+    give_back(c);
+    return r;
 }
 
 int nbody_energy(nbody_ctx *c, double *ekin, double *epot)

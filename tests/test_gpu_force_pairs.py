@@ -158,3 +158,75 @@ def test_units_of_any_size(torch, mode, n, length, mass):
         got.append((s["a"] * (lu * lu / mu), s["k"] * (lu * lu / mu), pot * (lu / mu)))
     for one, other in zip(*got):
         assert np.array_equal(one, other)
+
+
+def test_slots_are_given_back(torch):
+    """Slots above 2 GiB leave the device with the calls that wait, smaller ones stay; a refused allocation of them
+    leaves the one-sided kernels, for that call only."""
+    from paper_astro_ph_0702058_gb300 import Simulation, nbody_debug_fail_alloc, nbody_debug_pairs_bytes
+    n = 320000
+    plan = nbody_debug_pairs_bytes(1, n, n, torch.cuda.get_device_properties(0).multi_processor_count)
+    assert plan > 2 << 30
+    small = 512 << 20  # the context's other memory and more
+    m, x, v = plummer_sphere(n, 13)
+    act = torch.arange(n, dtype=torch.int32, device="cuda")
+    new = lambda: [torch.zeros(n, 3, dtype=torch.float64, device="cuda") for _ in range(2)] + [  # noqa: E731
+        torch.zeros(n, dtype=torch.float64, device="cuda")]
+    got, refused = new(), new()
+    free0 = torch.cuda.mem_get_info()[0]
+    held = lambda: free0 - torch.cuda.mem_get_info()[0]  # noqa: E731
+    with Simulation(m, x, v, EPS2, mode="comp") as sim:
+        assert sim.stats()["last_i_per_thread"] == 4 and held() < small
+        sim.predict(0.0)
+        nbody_debug_fail_alloc(1)
+        sim.force(act, acc=refused[0], jerk=refused[1], pot=refused[2])
+        nbody_debug_fail_alloc(0)
+        assert sim.stats()["last_i_per_thread"] == 1
+        for _ in range(2):
+            sim.force(act, acc=got[0], jerk=got[1], pot=got[2])
+            assert sim.stats()["last_i_per_thread"] == 4 and held() > plan
+        sim.sync()
+        assert held() < small
+        s = {k: np.zeros((n, 3)) for k in ("a", "k")}
+        sim.get_state(**s)
+        assert np.array_equal(got[0].cpu().numpy(), s["a"]) and np.array_equal(got[1].cpu().numpy(), s["k"])
+        for a, b in zip(got, refused):  # two summations of the same FP32 terms (64 each, then compensated)
+            assert (a - b).norm() <= 64 * 2.0 ** -24 * b.norm()
+        sim.step(1.0 / 64, 1)
+        assert held() < small
+    n = 40000
+    with Simulation(m[:n], x[:n], v[:n], EPS2, mode="comp") as sim:
+        sim.sync()
+        assert held() > nbody_debug_pairs_bytes(1, n, n, 152)
+
+
+def test_slots_of_a_captured_force_stay(torch):
+    """A caller's graph of a force keeps the slots it was captured with, whatever waits in between."""
+    from paper_astro_ph_0702058_gb300 import Simulation
+    n = 320000
+    m, x, v = plummer_sphere(n, 14)
+    stream = torch.cuda.Stream()
+    act = torch.arange(n, dtype=torch.int32, device="cuda")
+    out = [torch.zeros(n, 3, dtype=torch.float64, device="cuda") for _ in range(2)]
+    torch.cuda.synchronize()
+    with Simulation(m, x, v, EPS2, mode="comp", stream=stream) as sim:
+        sim.predict(0.0)
+        sim.force(act, acc=out[0], jerk=out[1])
+        sim.sync()
+        ref = [o.clone() for o in out]
+        sim.force(act, acc=out[0], jerk=out[1])  # (the capture allocates nothing)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream, capture_error_mode="thread_local"):
+            sim.force(act, acc=out[0], jerk=out[1])
+        assert sim.stats()["last_i_per_thread"] == 4
+        for _ in range(2):
+            sim.sync()  # would give the slots back
+            for o in out:
+                o.zero_()
+            torch.cuda.synchronize()
+            g.replay()
+            torch.cuda.synchronize()
+            for a, b in zip(out, ref):
+                assert torch.equal(a, b)
+        del g
