@@ -374,8 +374,8 @@ typedef struct nbody_ens nbody_ens; /* opaque; owns all of its device memory */
  * in the layout of nbody_init.  Every cluster starts at t = 0 with its full
  * force and first levels (Eq. initTimestep).  p as for nbody_init, except that
  * j_tile, i_block and j_split give the ensemble's force shape (threads per
- * block, i per thread, tiles per j-range; 0 = 64, 1, 4; see
- * nbody_ens_set_shape).  The ensemble runs on p->stream (which must allow
+ * block, i per thread, tiles per j-range; 0 = 32, 1, and 1 or, with i_block 2,
+ * 4; see nbody_ens_set_shape).  The ensemble runs on p->stream (which must allow
  * stream capture: not the legacy default stream) or, if that is NULL, on a
  * stream of its own.
  * Errors: EINVAL, ENOMEM, ECUDA, ENONFINITE. */
@@ -383,8 +383,11 @@ int nbody_ens_init(nbody_ens **out, int64_t n_clusters, const int64_t *sizes, co
                    const double *x, const double *v, double eps2, const nbody_params *p);
 
 /* Force launch shape: threads per block (32, 64 or 128), i-particles per thread
- * (1 or 2), and j-tiles of 256 particles per work item (>= 1; each cluster is
- * cut into at most 8 j-ranges).  Errors: EINVAL for unsupported shapes. */
+ * (1 or 2), and j-tiles of 256 particles per work item (>= 1), longer items where
+ * a cluster would be cut into more than 8 j-ranges.  With one i per thread and up
+ * to 8 tiles per item, rows fewer than an item's threads share them, and a block
+ * of n_act of a cluster's n particles may have 8 n / n_act ranges, at most 64.
+ * Errors: EINVAL for unsupported shapes. */
 int nbody_ens_set_shape(nbody_ens *e, int threads, int i_block, int tiles_per_range);
 
 /* Autotuner: times `steps` batched steps towards t_end for every supported

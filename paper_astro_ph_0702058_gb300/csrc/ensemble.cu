@@ -142,20 +142,20 @@ __global__ void __launch_bounds__(kSchedThreads) ens_schedule_kernel(const EnsDe
 }
 
 // j-ranges of a block of na rows in a cluster of n particles: ranges of
-// tiles_per_range tiles, at most s_max; with `share` single tiles where the partial
-// sums of s_max n rows and ranges hold them (na <= n / 4 of 8192 particles: 32
-// ranges), else as many ranges as they hold.  A step's blocks hold some tens of rows
-// per cluster, its time is that of its last items, and long items picked up late
-// were most of it (128 clusters: 0.24 Tpairs/s with ranges of up to 4 tiles).  The
-// rule looks at the cluster alone, so its arithmetic does not depend on the others
-// of the batch.
+// tiles_per_range tiles (longer ones where they would be too many), at most s_max;
+// with `share` as many as the partial sums of s_max n rows and ranges hold (na <=
+// n / 4 of 8192 particles: all 32 single tiles), at most kEnsMostRanges.  A step's
+// blocks hold some tens of rows per cluster, its time is that of its last items,
+// and long items picked up late were most of it (128 clusters: 0.24 Tpairs/s with
+// ranges of up to 4 tiles), so single tiles are the default.  The rule looks at the
+// cluster alone, so its arithmetic does not depend on the others of the batch.
 constexpr int kEnsMostRanges = 64;
 __device__ __forceinline__ int ens_ranges(const int na, const int64_t n, const int tiles_per_range, const int s_max,
                                           const bool share, int &tpr)
 {
     const int ntl = static_cast<int>((n + kJTile - 1) / kJTile);
-    int S = min((ntl + tiles_per_range - 1) / tiles_per_range, s_max);
-    if (share) S = max(S, static_cast<int>(min(static_cast<int64_t>(min(ntl, kEnsMostRanges)), s_max * n / na)));
+    const int most = share ? static_cast<int>(min(static_cast<int64_t>(kEnsMostRanges), s_max * n / na)) : s_max;
+    const int S = min((ntl + tiles_per_range - 1) / tiles_per_range, most);
     tpr = (ntl + S - 1) / S;
     return (ntl + tpr - 1) / tpr;
 }
@@ -746,6 +746,9 @@ inline bool ens_share(const int ipt, const int tiles_per_range)
     return NB_PACKED && ipt == 1 && tiles_per_range <= kEnsShareTiles;
 }
 
+// Tiles per range where the caller names none.
+inline int ens_default_tiles(const int ipt) { return NB_PACKED && ipt == 1 ? 1 : 4; }
+
 cudaError_t ens_force_launch(int mode, int threads, int ipt, int tiles_per_range, const EnsDev &E, float eps2,
                              int sm_count, cudaStream_t s, int64_t *launches)
 {
@@ -785,7 +788,7 @@ struct nbody_ens {
     bool own_stream = false;
     int sm_count = 0;
     int s_max = 8;
-    int threads = 32, ipt = 1, tiles_per_range = 4;
+    int threads = 32, ipt = 1, tiles_per_range = 1;
     std::vector<int64_t> off_h;
     // device memory, in one allocation, and pinned memory in another
     void *dev_base = nullptr, *host_base = nullptr;
@@ -928,7 +931,7 @@ int nbody_ens_init(nbody_ens **out, int64_t n_clusters, const int64_t *sizes, co
     if (n > 2147483647LL || jt > 2147483647LL) return efail(NBODY_EINVAL, "nbody_ens_init: too many particles");
 
     const int sh_t = prm.j_tile ? prm.j_tile : 32, sh_i = prm.i_block ? prm.i_block : 1;
-    const int sh_p = prm.j_split > 0 ? prm.j_split : 4;
+    const int sh_p = prm.j_split > 0 ? prm.j_split : ens_default_tiles(sh_i);
     bool shape_ok = false;
     for (const EnsShape &sh : kEnsShapes) shape_ok |= sh.threads == sh_t && sh.ipt == sh_i;
     if (!shape_ok) return efail(NBODY_EINVAL, "nbody_ens_init: unsupported force shape %d x %d", sh_t, sh_i);

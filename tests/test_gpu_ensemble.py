@@ -191,3 +191,27 @@ def test_automatic_shape_any_batch(mode):
         # there, which moves it by the corrector's ~dt^4: compare loosely
         ra, rk, _ = oracle.force(mc, s["x"], s["v"], EPS2, rows.astype(np.int32))
         assert np.linalg.norm(s["a"][rows] - ra) <= 1e-4 * np.linalg.norm(ra)
+
+
+@pytest.mark.parametrize("mode", ["plain", "comp"])
+def test_tiles_per_range_is_what_the_caller_asks(mode):
+    """The t = 0 forces of clusters whose rows fill their items: with ranges as long as the cluster they are the bits
+    of a single system's one j-range, and with single tiles those of one range per tile."""
+    need_gpu()
+    from paper_astro_ph_0702058_gb300 import Ensemble, Simulation
+    sizes = [2048, 1024, 512]  # 8, 4 and 2 tiles
+    parts, m, x, v = _clusters(sizes, 170)
+    off = np.concatenate([[0], np.cumsum(sizes)])
+    for threads in (32, 64):
+        for tiles, split in ((8, lambda n: 1), (4, lambda n: max(n // 1024, 1)), (1, lambda n: n // 256)):
+            with Ensemble(sizes, m, x, v, EPS2, mode=mode, threads=threads, i_block=1, tiles_per_range=tiles) as ens:
+                got = _state(ens, len(m))
+            for c, (mc, xc, vc) in enumerate(parts):
+                with Simulation(mc, xc, vc, EPS2, mode=mode, j_tile=64, i_block=1, j_sub=1, j_split=split(len(mc))) as sim:
+                    ref = _state(sim, len(mc))
+                for key in ("a", "k"):
+                    a, b = got[key][off[c]:off[c + 1]], ref[key]
+                    if split(len(mc)) == 1:  # (the sums of several ranges are added in another order, in double-single)
+                        assert np.array_equal(a, b), (threads, tiles, c, key)
+                    else:
+                        assert np.linalg.norm(a - b) <= 2.0 ** -40 * np.linalg.norm(b), (threads, tiles, c, key)
