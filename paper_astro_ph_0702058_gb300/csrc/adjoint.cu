@@ -287,7 +287,8 @@ __device__ __forceinline__ void column_sums(const int count, At &&at, double (&s
 }
 
 // Value of component c of particle i in slot s (zero where the slot has none).
-__device__ __forceinline__ void vjp_at_slot(const float *__restrict__ part, const VjpSlots V, const int n, const int c,
+// (part: written by the kernel before, see after_previous.)
+__device__ __forceinline__ void vjp_at_slot(const float *part, const VjpSlots V, const int n, const int c,
                                             const int i, const int s, float &a, float &b)
 {
     if (V.parts == 2 && s < 2 * (i / V.rows) && (s & 1)) return;  // (as the j of an earlier superblock: one slot)
