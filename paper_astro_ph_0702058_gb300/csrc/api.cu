@@ -584,10 +584,15 @@ int rollout_impl(const char *who, int64_t n, const double *m, const double *x0, 
         }
         return NBODY_OK;
     };
+    // (the steps flag single components, so the report does not count rows)
+    auto finish = [&]() -> int {
+        const int rr = sync_and_check(c);
+        return rr == NBODY_ENONFINITE ? fail(rr, "%s: non-finite force or state during the steps", who) : rr;
+    };
     if (!backward) {
         r = run(xvak, steps, [&](int64_t) { return xvak; });
         if (r == NBODY_OK) r = copy_final();
-        if (r == NBODY_OK) r = sync_and_check(c);
+        if (r == NBODY_OK) r = finish();
         return done(r);
     }
     // Every state is kept where kRollKeep holds them; else checkpoints every checkpoint_every steps, and the
@@ -692,7 +697,7 @@ int rollout_impl(const char *who, int64_t n, const double *m, const double *x0, 
               "gradient copy");
     }
     if (g_m) NB_DR(cudaMemcpyAsync(g_m, G.gm, nd * sizeof(double), cudaMemcpyDefault, s), "gradient copy");
-    r = sync_and_check(c);
+    r = finish();
 #undef NB_DR
     return done(r);
 }

@@ -82,3 +82,21 @@ def test_segments_where_the_states_are_too_many_to_keep():
         nbody_rollout_vjp(n, m, x, v, EPS2, LEVEL, steps, every, 0, g[0], g[1], *out[-1])
     for a, b in zip(*out):
         assert np.all(np.isfinite(a)) and np.array_equal(a, b)
+
+
+def test_nonfinite_steps_are_reported():
+    """A run whose velocities leave FP32's range after its first step fails, without a count of rows that is not one."""
+    import re
+    need_gpu()
+    from paper_astro_ph_0702058_gb300 import NBodyError
+    from paper_astro_ph_0702058_gb300._lib import nbody_rollout, nbody_rollout_vjp
+    n, steps = 2, 3
+    m, x, v = np.full(n, 1e25), np.array([[5e-4, 0, 0], [-5e-4, 0, 0]]), np.zeros((n, 3))
+    out = [np.zeros((n, 3)), np.zeros((n, 3))]
+    for call in (lambda: nbody_rollout(n, m, x, v, 1e-8, 0, steps, 0, *out),
+                 lambda: nbody_rollout_vjp(n, m, x, v, 1e-8, 0, steps, 16, 0, np.ones((n, 3)), None, *out, None)):
+        with pytest.raises(NBodyError) as e:
+            call()
+        assert e.value.code == -5 and "non-finite" in str(e.value)
+        rows = re.search(r"(\d+) rows", str(e.value))
+        assert rows is None or int(rows.group(1)) <= n * steps, str(e.value)
