@@ -144,3 +144,37 @@ def test_rollout_autograd_inside_a_larger_program():
     torch.testing.assert_close(xt.grad, gx, rtol=1e-12, atol=0)
     torch.testing.assert_close(vt.grad, gv, rtol=1e-12, atol=0)
     torch.testing.assert_close(mt.grad, gm, rtol=1e-12, atol=0)
+
+
+@pytest.mark.parametrize("n,mode", [(96, "plain"), (700, "plain"), (700, "comp"), (301, "ds"), (96, "sumcheck"), (64, "sorted")])
+def test_states_run_again_give_the_bits_of_kept_ones(n, mode):
+    """Where the states of a run cannot be kept, the steps of a segment run again: the loss, its gradient and a
+    vector-Jacobian product are the same bits, whatever the segments' length.  (The buffer of all states is the first
+    allocation of these sizes whose refusal the call survives.)"""
+    need_gpu()
+    from paper_astro_ph_0702058_gb300 import MODES, NBodyError, nbody_debug_fail_alloc
+    from paper_astro_ph_0702058_gb300._lib import nbody_rollout_vjp
+    m, x, v = plummer_sphere(n, 61)
+    steps = 37
+    g = np.random.default_rng(4).standard_normal((2, n, 3))
+
+    def vjp(ck):
+        out = np.zeros((n, 3)), np.zeros((n, 3)), np.zeros(n)
+        nbody_rollout_vjp(n, m, x, v, EPS2, LEVEL, steps, ck, MODES[mode], g[0], g[1], *out)
+        return out
+
+    for call in (lambda ck: _gpu_grad(m, x, v, steps=steps, ck=ck, mode=MODES[mode]), vjp):
+        kept = call(16)
+        for ck in (1, 7, 16, 36, 37, 50):
+            for k in range(1, 12):
+                nbody_debug_fail_alloc(k)
+                try:
+                    again = call(ck)
+                    break
+                except NBodyError as e:
+                    assert e.code == -2
+                finally:
+                    nbody_debug_fail_alloc(0)
+            assert 3 <= k <= 6  # (a context's device and pinned memory and the set-up's scratch come before)
+            for a, b in zip(kept, again):
+                assert np.array_equal(a, b), (ck, k)
