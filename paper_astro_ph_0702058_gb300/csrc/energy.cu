@@ -10,9 +10,9 @@
 // FP64 potential.  GB300's SM has one FP64 unit that takes ~19 cycles per warp
 // instruction, so the pair term is written to use few of its operations: 6 for
 // the differences and r^2; then, from the MUFU's approximate y0 (rsqrt.approx.f64,
-// a relative error below 2^-20), the root by one step of third order in the
+// a relative error of 2^-20), the root by one step of third order in the
 // residual e = 1 - r^2 y0^2, y = y0 (1 + e/2 + 3 e^2/8) (the binomial series of
-// (1 - e)^(-1/2); the next term is 5 e^3/16 < 2^-61), 5; and the product with m_j
+// (1 - e)^(-1/2); the next term is 5 e^3/16 < 2^-58.7), 5; and the product with m_j
 // into the sum, 1.  A pair costs 12 FP64 operations, where an IEEE square root
 // and division per ordered pair took about 2 x 28: n = 65536 240 -> 46.5 ms (49 by
 // 12 operations of 2^31 pairs at 1.68 per clock per SM).
