@@ -248,7 +248,7 @@ def roofline(force_ms_avg, n, sm_count, clocks, peaks, mode="comp", launch=None)
     achieved = pairs / (force_ms_avg * 1e-3) / 1e9
     ops = OPS_PER_PAIR
     if launch is not None and launch[1] == ROWS_PER_LANE_BY_PAIRS:
-        ops = 35 / 2  # an unordered pair gives both of its interactions with 35 operations
+        ops = 36 / 2  # an unordered pair gives both of its interactions with 36 operations
     peak = sm_count * FP32_LANES_PER_SM * max_mhz * 1e6 / ops / 1e9
     out = {"bound": "alu", "achieved": round(achieved, 2), "peak": round(peak, 2), "unit": "Gpair/s",
            "frac": round(achieved / peak, 4), "traffic": measured_traffic(mode, n, launch),
@@ -714,7 +714,8 @@ def diff_workload(args):
 
 def pipe_probe(args):
     """The roofline's unit rates, measured: FP32 FMA / ADD / MUL, packed FP32x2 FMA and MUFU rsqrt
-    results per SM per clock (csrc/pipe_probe.cu, chains of independent accumulators), the FP64 FMA and
+    results per SM per clock (csrc/pipe_probe.cu, chains of independent accumulators; the packed FMA also with registers of its own
+    in every operation, the register file's bound), the FP64 FMA and
     conversion rates, and the cycles per operation of one dependent FP64 chain (FMA, square root,
     division) in one block of 1 to 16 warps."""
     from paper_astro_ph_0702058_gb300 import build as nb_build

@@ -1,6 +1,7 @@
 // Throughput probes of the GPU pipes that bound the pair loop: chains of
-// FP32 FMA, ADD and MUL, the packed FP32x2 FMA, and the MUFU reciprocal
-// square root; and of the pipes that bound the FP64 predictor and corrector:
+// FP32 FMA, ADD and MUL, the packed FP32x2 FMA (whose rate depends on how many of
+// its three registers differ from those of the operation before), and the MUFU
+// reciprocal square root; and of the pipes that bound the FP64 predictor and corrector:
 // FP64 FMA and the double -> float -> double conversions.  Then the latency of
 // one dependent FP64 chain (FMA, square root + add, division + add) in one
 // block of 1, 4 or 16 warps with 1 or 32 active lanes: the cycles each
@@ -59,17 +60,25 @@ __global__ void scalar_chain(float *out, long long *cyc, int iters, float a, flo
     if (threadIdx.x == 0) cyc[blockIdx.x] = clock64() - c0;
 }
 
-__global__ void packed_chain(float *out, long long *cyc, int iters, float a, float b)
+// Packed FMA chains.  OWN 0: every accumulator with the same multiplier and addend, each
+// one value in both halves; 1: a multiplier of its own each, the addend shared; 2:
+// multiplier and addend of its own each, so of an operation's three 64-bit registers
+// none is among those of the one before.
+template <int OWN>
+__global__ void __launch_bounds__(256, OWN == 0 ? 8 : 4) packed_chain(float *out, long long *cyc, int iters, float a, float b)
 {
     const long long c0 = clock64();
-    unsigned long long r[kChains];
-    for (int i = 0; i < kChains; ++i) r[i] = pack2(threadIdx.x * 1e-3f + i, i * 0.5f);
-    const unsigned long long A = pack2(a, a), B = pack2(b, b);
+    unsigned long long r[kChains], A[kChains], B[kChains];
+    for (int i = 0; i < kChains; ++i) {
+        r[i] = pack2(threadIdx.x * 1e-3f + i, i * 0.5f);
+        A[i] = OWN == 0 ? pack2(a, a) : pack2(a - threadIdx.x * 1e-6f - i * 1e-5f, a - i * 1e-4f);
+        B[i] = OWN == 0 ? pack2(b, b) : pack2(b + threadIdx.x * 1e-6f + i * 1e-5f, b + i * 1e-4f);
+    }
     for (int it = 0; it < iters; ++it) {
 #pragma unroll
         for (int u = 0; u < kInner; ++u)
 #pragma unroll
-            for (int i = 0; i < kChains; ++i) r[i] = fma2(r[i], A, B);
+            for (int i = 0; i < kChains; ++i) r[i] = fma2(r[i], A[OWN > 0 ? i : 0], B[OWN > 1 ? i : 0]);
     }
     unsigned long long s = 0;
     for (int i = 0; i < kChains; ++i) s ^= r[i];
@@ -157,7 +166,7 @@ int main()
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     double ops_per_thread = static_cast<double>(iters) * kInner * kChains;
-    const double threads_total = static_cast<double>(blocks) * threads;
+    int grid = blocks;  // all resident at once, so that a block's clocks are the kernel's
     long long *cyc_h = new long long[blocks];
     auto run = [&](const char *name, double results_per_op, auto launch) {
         launch();  // warm-up
@@ -170,8 +179,9 @@ int main()
         cudaEventElapsedTime(&ms, e0, e1);
         cudaMemcpy(cyc_h, cyc, blocks * sizeof(long long), cudaMemcpyDeviceToHost);
         long long cmax = 0;
-        for (int i = 0; i < blocks; ++i) cmax = cyc_h[i] > cmax ? cyc_h[i] : cmax;
+        for (int i = 0; i < grid; ++i) cmax = cyc_h[i] > cmax ? cyc_h[i] : cmax;
         const double clk = static_cast<double>(cmax) / (ms * 1e-3);  // SM clock seen by the busiest block
+        const double threads_total = static_cast<double>(grid) * threads;
         const double per_sm_clk = ops_per_thread * threads_total * results_per_op / (ms * 1e-3) / sm / clk;
         std::printf("\"%s\": {\"per_sm_per_clk\": %.2f, \"sm_mhz\": %.0f}, ", name, per_sm_clk, clk * 1e-6);
     };
@@ -179,7 +189,12 @@ int main()
     run("ffma", 1.0, [&] { scalar_chain<0><<<blocks, threads>>>(out, cyc, iters, 1.0001f, 1e-6f); });
     run("fadd", 1.0, [&] { scalar_chain<1><<<blocks, threads>>>(out, cyc, iters, 1e-6f, 1e-6f); });
     run("fmul", 1.0, [&] { scalar_chain<2><<<blocks, threads>>>(out, cyc, iters, 1.0000001f, 1e-6f); });
-    run("ffma2_fp32_results", 2.0, [&] { packed_chain<<<blocks, threads>>>(out, cyc, iters, 1.0001f, 1e-6f); });
+    run("ffma2_fp32_results", 2.0, [&] { packed_chain<0><<<grid, threads>>>(out, cyc, iters, 0.9999f, 1e-6f); });
+    grid = sm * 4;  // (up to 64 registers a thread)
+    run("ffma2_own_multiplier", 2.0, [&] { packed_chain<1><<<grid, threads>>>(out, cyc, iters, 0.9999f, 1e-6f); });
+    run("ffma2_three_own_registers", 2.0,
+        [&] { packed_chain<2><<<grid, threads>>>(out, cyc, iters, 0.9999f, 1e-6f); });
+    grid = blocks;
     run("mufu_rsqrt", 1.0, [&] { mufu_chain<<<blocks, threads>>>(out, cyc, iters); });
     const int iters64 = iters / 20;  // the FP64 pipes are narrow: fewer trips
     ops_per_thread = static_cast<double>(iters64) * kInner * kChains;

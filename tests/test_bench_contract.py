@@ -41,3 +41,14 @@ def test_traffic_record_matches_the_kernel_sources():
     for mode in ("plain", "comp"):
         t = bench.measured_traffic(mode, 1 << 20, [256, 1, 2])
         assert t is not None and t > 0, mode
+
+
+def test_traffic_record_of_the_force_by_pairs_matches_its_sources():
+    """Likewise the record of the full force by unordered pairs, the launch the benchmark makes by default."""
+    import bench
+    for mode, words in (("plain", 7), ("comp", 14)):
+        t = bench.measured_traffic(mode, 1 << 20, [128, 4, 129])
+        # at least the slots' half that cannot wait in L2, at most every slot once per tile of 512 rows
+        assert t is not None, mode
+        slots = 129 * words * 4 * (1 << 20)
+        assert slots / 2 < t < 2 * 16 * slots
