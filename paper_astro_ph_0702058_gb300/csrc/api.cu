@@ -30,6 +30,9 @@ constexpr int64_t kPairsOwnList = 16384;  // rows of a caller's list that may ta
 // force that takes them pays ~0.2 ms per GiB for the allocation and 0.5 for the free, 0.6 % of a full force at 2^20
 // particles (7.1 GiB, compensated), 2 % at 300000 (2 GiB), more below.
 constexpr size_t kSlotsKeep = size_t(2) << 30;
+// Partial sums that a context whose set-up leaves none (its force goes by pairs) holds from the start, for blocks of up
+// to ~1900 rows compensated: within the context's one allocation, where a first block's own takes 50 to 150 us.
+constexpr size_t kPartialsBase = size_t(16) << 20;
 constexpr int64_t kRollKeep = int64_t(1) << 30;  // bytes of states a gradient keeps instead of running steps again
 constexpr int64_t kClusterCap = 4096;  // blocks one launch of the cluster or the grid kernel may run
 #ifndef NB_GRID_ROWS
@@ -116,6 +119,7 @@ struct nbody_ctx {
     double *stage = nullptr;  // 6 n doubles: external forces / AoS staging
     void *partials = nullptr;
     size_t partials_cap = 0;
+    void *partials_base = nullptr;  // within dev_base: what partials is until it has to grow (kPartialsBase)
     int64_t scratch_gen = 0;  // counts the buffers partials has been: an address may come back with less room
     void *sym_buf = nullptr;  // scratch of the force by unordered pairs (sym_scratch_bytes), on first use
     void *slots = nullptr;    // and its partial sums; what holds more than kSlotsKeep is given back (give_back)
@@ -163,6 +167,7 @@ namespace {
 void release(nbody_ctx *c)
 {
     if (c->step_graph) cudaGraphExecDestroy(c->step_graph);
+    if (c->partials == c->partials_base) c->partials = nullptr;
     void *dev[] = {c->dev_base, c->partials, c->graph_fits, c->grid_buf, c->sym_buf, c->slots};
     for (void *d : dev)
         if (d) cudaFree(d);
@@ -254,7 +259,7 @@ int ensure_partials(nbody_ctx *c, size_t bytes)
     auto drop = [&]() -> int {
         if (!c->partials) return NBODY_OK;
         NB_CUDA(cudaStreamSynchronize(c->s), "stream synchronise");
-        cudaFree(c->partials);
+        if (c->partials != c->partials_base) cudaFree(c->partials);
         c->partials = nullptr;
         c->partials_cap = 0;
         ++c->scratch_gen;
@@ -264,7 +269,7 @@ int ensure_partials(nbody_ctx *c, size_t bytes)
     const size_t cap = std::max(bytes, static_cast<size_t>(1) << 20);
     void *p = nullptr;
     cudaError_t e = ctx_alloc(c, &p, cap);
-    if (e == cudaErrorMemoryAllocation && c->partials) {
+    if (e == cudaErrorMemoryAllocation && c->partials && c->partials != c->partials_base) {
         cudaGetLastError();
         const int r = drop();
         if (r != NBODY_OK) return r;
@@ -355,21 +360,29 @@ int force_internal(nbody_ctx *c, int64_t n_act, bool for_step = false, bool asce
     if (cfg.sym_sb > 0) {
         const long long *rows_general = nullptr;
         ForceConfig general{};
+        void *general_part = nullptr;
         if (!ascending) {
             r = choose(&general, false);
             if (r != NBODY_OK) return r;
-            r = ensure_partials(c, force_partial_bytes(c->p.mode, general, n_act));
-            if (r != NBODY_OK) return r;
+            // (one of the two computes: the pairs of distinct particles, the general path of others)
+            const size_t bytes = force_partial_bytes(c->p.mode, general, n_act);
+            if (bytes <= c->slots_cap) {
+                general_part = c->slots;
+            } else {
+                r = ensure_partials(c, bytes);
+                if (r != NBODY_OK) return r;
+                general_part = c->partials;
+            }
         }
         NB_CUDA(force_sym_launch(c->p.mode, c->J, c->n, c->act_force, n_act, c->eps2, cfg, ascending, c->f_acc,
                                  c->f_jerk, c->f_pot, c->slots, c->sym_buf, &rows_general, c->st, c->s, &launches),
                 "force kernel launch");
         if (rows_general) {  // (nothing to do for a list of distinct particles: ~5 us)
             NB_CUDA(force_launch(c->p.mode, c->J, c->n, c->act_force, n_act, c->eps2, general, c->f_acc, c->f_jerk,
-                                 c->f_pot, c->partials, c->st, c->s, &launches, rows_general, false),
+                                 c->f_pot, general_part, c->st, c->s, &launches, rows_general, false),
                     "force kernel launch");
             if (general.split > 1)
-                NB_CUDA(force_sym_reduce_launch(c->p.mode, static_cast<float *>(c->partials), general.split, n_act,
+                NB_CUDA(force_sym_reduce_launch(c->p.mode, static_cast<float *>(general_part), general.split, n_act,
                                                 c->f_acc, c->f_jerk, c->f_pot, rows_general, true, c->s, &launches),
                         "force kernel launch");
         }
@@ -778,11 +791,17 @@ int nbody_init(nbody_ctx **out, int64_t n, const double *m, const double *x, con
     host_mem.add(&c->st_host, sizeof(DevStatus));
     host_mem.add(&c->e_host, 2 * sizeof(double));
     host_mem.add(&c->trange_host, 2 * sizeof(unsigned long long));
+    ForceConfig all{};
+    const bool base = prm.j_tile == 0 && prm.i_block == 0 && prm.j_split <= 0 && prm.j_sub == 0 &&
+                      sym_plan(prm.mode, n, n, c->sm_count, &all);
+    if (base) dev_mem.add(&c->partials_base, kPartialsBase);
     dev_mem.add(&c->loop_dev, sizeof(StepLoop));
     host_mem.add(&c->loop_host, sizeof(StepLoop));
     NB_INIT(dev_mem.commit(&c->dev_base, dev_alloc), "context allocation");
     NB_INIT(host_mem.commit(&c->host_base, host_alloc), "pinned allocation");
     std::memset(c->st_host, 0, sizeof(DevStatus));
+    c->partials = c->partials_base;
+    c->partials_cap = base ? kPartialsBase : 0;
 
     State &S = c->S;
     S.n = n;
