@@ -106,10 +106,13 @@ typedef struct {
                          blocks of 512 to 8191 rows when j_tile and i_block are 0, else 1);
                          1 = one thread per row; 4 = 256 threads as 64 rows x 4 threads,
                          each taking a quarter of every j-tile (j_tile, i_block ignored).
-                         With all four force-tuning fields 0, blocks of 512 to 8191 rows of
-                         streams of 16384 to 3584 x SMs particles take the slice shape
-                         instead: one block of 512 threads per SM over its contiguous
-                         slice of the j-stream held in shared memory, j_split = SMs       */
+                         With all four force-tuning fields 0, streams of 16384 to
+                         3584 x SMs particles take the slice shape instead for blocks of
+                         512 to 8191 rows (in nbody_force of 1 to 8191): one block of 512
+                         threads per SM over its contiguous slice of the j-stream held in
+                         shared memory, j_split = SMs; and blocks of >= 8192 rows that are
+                         all particles (a caller's list: >= 16384), or >= 20000 and a
+                         quarter of them, go by unordered pairs                          */
     void *stream;     /* cudaStream_t for all work of the context, or NULL                  */
 } nbody_params;
 
@@ -196,10 +199,11 @@ int nbody_energy(nbody_ctx *ctx, double *ekin, double *epot);
 /* The same diagnostic with the potential in double-single arithmetic on the
  * FP32 pipe: positions, masses and eps2 split into (hi, lo) float pairs,
  * 1/r from the MUFU seed and one Newton step with a double-single residual,
- * each 256-particle tile's terms summed in double-single and the tile sums
- * in FP64.  Agrees with nbody_energy to ~1e-13 relative and avoids an FP64
- * square root and division per pair, which make nbody_energy take about a
- * minute at n = 2^20 on GB300.  E_kin is FP64 as in nbody_energy.
+ * each unordered pair once, the terms of at most 128 j summed in
+ * double-single and those sums in FP64.  Agrees with nbody_energy to ~1e-13
+ * relative and takes 2.1 s at n = 2^20 on GB300, where nbody_energy (12 FP64
+ * operations per unordered pair) takes about 12 s.  E_kin is FP64 as in
+ * nbody_energy.
  * Synchronises the stream.  Errors: ENOTSYNC as nbody_energy. */
 int nbody_energy_ds(nbody_ctx *ctx, double *ekin, double *epot);
 
@@ -306,13 +310,13 @@ void nbody_debug_skip_tile_copy(int on);
  *      blocks per launch).  Larger plain and compensated systems (n up to
  *      3584 per SM, automatic shapes) run their blocks of up to 4095 rows in
  *      one cooperative launch of one CTA per SM that repeats the same steps,
- *      its CTAs meeting at three grid barriers per block (each gives up after
+ *      its CTAs meeting at two grid barriers per block (each gives up after
  *      about 1 s and raises NBODY_ETIMEOUT); a larger block ends the launch
  *      and runs as at level 2.  Both kernels' forces are the same pair terms
  *      summed in another order, so their results differ from levels 0-2 in
  *      the last bits.
  * A context captures its graph in the form of the level in force when it
- * builds it (once, and again only if its scratch buffer moves); a loop graph
+ * builds it (once, and again only if its scratch buffer is replaced); a loop graph
  * run at level 1 stops after each block.
  * The graph is used only when its launch shape is the one the separate
  * launches would take, so levels 0-2 give the same results bit for bit.

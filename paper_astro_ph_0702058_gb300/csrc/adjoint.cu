@@ -540,7 +540,7 @@ int blocks_of(int64_t n, int t) { return static_cast<int>((n + t - 1) / t); }
 }  // namespace
 
 // Superblocks of 64 rows up to n = 8192 (128 of them), each pair of them in two
-// parts while that leaves fewer warps than the GPU holds (n = 4096 and below);
+// parts while that leaves fewer warps than the GPU holds (up to n = 3776 on 152 SMs);
 // more tiles per superblock beyond, their sums folded in double-single.
 VjpSlots vjp_slots(int64_t n, int sm_count)
 {

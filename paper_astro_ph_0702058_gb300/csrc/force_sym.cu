@@ -242,7 +242,8 @@ size_t sym_scratch_bytes(int64_t n)
 // of 65536 1248 -> 1252.  So from 20000 rows and a quarter of the particles on.
 // Superblocks are as small as 128 of them allow, for many units (8256 against 2080
 // of twice the size: 4-5 % at n = 65536 and 262144), up to 8 GiB of slots (2^20
-// compensated: 889 ms with 7.6 GB, 920 with 4.3); CTAs of one warp up to 32768
+// compensated, before the pair loop's last changes: 889 ms with 7.6 GB, 920 with 4.3;
+// now 853); CTAs of one warp up to 32768
 // rows, of four above (n = 16384: 194 against 240 us plain; 65536: 2894 against 2804).
 bool sym_plan(int mode, int64_t n_act, int64_t n, int sm_count, ForceConfig *cfg)
 {

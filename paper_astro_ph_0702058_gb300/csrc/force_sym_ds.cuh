@@ -11,10 +11,10 @@
 //
 // An unordered pair takes about 410 FP32 operations, 205 per interaction (the
 // one-sided loop 325, 396 before its products joined their sums unnormalised).
-// Bound by the FMA pipe and its operand reads (force_sym.cuh): 818 + 90 cycles of
-// two pairs' 1150 measured; 8 to 12 resident warps make no difference.  Full
-// forces, one-sided -> pairs, us: n = 4096 303 -> 196, 16384 3340 -> 1984, 30000
-// 11151 -> 6656.
+// Bound by the FMA pipe and its operand reads (force_sym.cuh): about 815 + 90 cycles
+// of two pairs' 1140 measured; 8 to 12 resident warps make no difference.  Full
+// forces, one-sided -> pairs, us: n = 4096 303 -> 196, 16384 3340 -> 1967, 30000
+// 11151 -> 6656 (before the mass came first).
 //
 // The assembler fuses a packed product into a packed addition that uses it, also
 // where both are written as separate round-to-nearest instructions; a product
