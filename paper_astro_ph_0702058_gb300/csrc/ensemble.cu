@@ -67,16 +67,18 @@ __device__ __forceinline__ unsigned long long ens_due(const State &S, int64_t i,
     return static_cast<unsigned long long>(S.t[i] + (int64_t(1) << (lmax - S.level[i])));
 }
 
-// Block scheduler of Sect. 2 for one cluster per block of kSchedThreads.  Up to
+// Block scheduler of Sect. 2 for one cluster per block of NT threads.  Up to
 // kSchedKeep particles per thread keep their due tick in registers between the
-// minimum and the ordered list (clusters of up to 8192; further ones read it
-// again); the list's offsets come from one scan over the warps' counts of every
-// round.  256 threads with two passes over the state and a barrier pair per round
-// took 26.7 us per batched step (128 clusters of 256 to 8191).
-constexpr int kSchedThreads = 1024, kSchedKeep = 8;
+// minimum and the ordered list (with 1024 threads clusters of up to 8192; further
+// ones read it again); the list's offsets come from one scan over the warps' counts
+// of every round.  256 threads with two passes over the state and a barrier pair per
+// round took 26.7 us per batched step (128 clusters of 256 to 8191), this 7.
+constexpr int kSchedKeep = 8;
 
-__global__ void __launch_bounds__(kSchedThreads) ens_schedule_kernel(const EnsDev E, long long t_end, int lmax)
+template <int NT>
+__global__ void __launch_bounds__(NT) ens_schedule_kernel(const EnsDev E, long long t_end, int lmax)
 {
+    constexpr int kSchedThreads = NT;
     __shared__ unsigned long long shm[32];
     __shared__ int tot[kSchedKeep][32];
     const int c = blockIdx.x;
@@ -114,7 +116,7 @@ __global__ void __launch_bounds__(kSchedThreads) ens_schedule_kernel(const EnsDe
         int before[kSchedKeep], total[kSchedKeep];  // of this warp in each round, and of the round
 #pragma unroll
         for (int k = 0; k < kSchedKeep; ++k) {
-            const int v = tot[k][l];
+            const int v = l < NT / 32 ? tot[k][l] : 0;
             int s = v;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -746,6 +748,28 @@ inline bool ens_share(const int ipt, const int tiles_per_range)
     return NB_PACKED && ipt == 1 && tiles_per_range <= kEnsShareTiles;
 }
 
+// Threads of a scheduler block: no more than the largest cluster's particles fill, and
+// no more than 4 waves of resident threads over all clusters (as long as that leaves
+// 128).  A block of 1024 for each of 20000 clusters of 8 took 238 us per batched step
+// where 64 threads take 16.5 (their run to t = 1/64 73.4 -> 26.6 ms; 2000 clusters of
+// 100 9.6 -> 7.0, 3000 of 1500 132-158 -> 107, 600 of 1000 13.2 -> 12.2).
+inline int ens_sched_threads(const int64_t n_most, const int64_t n_cl, const int sm_count)
+{
+    int t = 64;
+    while (t < 1024 && kSchedKeep * t < n_most && (t < 128 || 2 * t * n_cl <= 4ll * 2048 * sm_count)) t *= 2;
+    return t;
+}
+cudaError_t ens_schedule_launch(const int threads, const EnsDev &E, long long t_end, int lmax, cudaStream_t s)
+{
+    auto *kernel = threads == 64    ? ens_schedule_kernel<64>
+                   : threads == 128 ? ens_schedule_kernel<128>
+                   : threads == 256 ? ens_schedule_kernel<256>
+                   : threads == 512 ? ens_schedule_kernel<512>
+                                    : ens_schedule_kernel<1024>;
+    kernel<<<E.n_cl, threads, 0, s>>>(E, t_end, lmax);
+    return cudaGetLastError();
+}
+
 // Tiles per range where the caller names none.
 inline int ens_default_tiles(const int ipt) { return NB_PACKED && ipt == 1 ? 1 : 4; }
 
@@ -789,6 +813,7 @@ struct nbody_ens {
     int sm_count = 0;
     int s_max = 8;
     int threads = 32, ipt = 1, tiles_per_range = 1;
+    int sched_threads = 1024;
     std::vector<int64_t> off_h;
     // device memory, in one allocation, and pinned memory in another
     void *dev_base = nullptr, *host_base = nullptr;
@@ -868,7 +893,7 @@ int ens_enqueue_step(nbody_ens *e, long long t_end_tick)
     const int lmax = e->p.lmax;
     const double tick = std::ldexp(1.0, -lmax);
     const int rows = e->threads * e->ipt;
-    ens_schedule_kernel<<<e->n_cl, kSchedThreads, 0, e->s>>>(e->E, t_end_tick, lmax);
+    NB_ECUDA(ens_schedule_launch(e->sched_threads, e->E, t_end_tick, lmax, e->s), "ensemble step launch");
     ens_plan_kernel<<<1, 1024, 0, e->s>>>(e->E, rows, e->tiles_per_range, ens_share(e->ipt, e->tiles_per_range));
     const int pg = static_cast<int>(std::min<int64_t>((e->n_tot + 255) / 256, e->sm_count * 16));
     ens_predict_kernel<<<pg, 256, 0, e->s>>>(e->E, tick, e->p.mode == kModeComp);
@@ -964,6 +989,7 @@ int nbody_ens_init(nbody_ens **out, int64_t n_clusters, const int64_t *sizes, co
     int dev = 0;
     NB_EI(cudaGetDevice(&dev), "cudaGetDevice");
     NB_EI(cudaDeviceGetAttribute(&e->sm_count, cudaDevAttrMultiProcessorCount, dev), "SM count");
+    e->sched_threads = ens_sched_threads(*std::max_element(sz.begin(), sz.end()), n_clusters, e->sm_count);
     const size_t nd = static_cast<size_t>(n), nc = static_cast<size_t>(n_clusters);
     const size_t NC = prm.mode == NBODY_MODE_COMP ? 14 : 7;
     Arena dev_mem, host_mem;

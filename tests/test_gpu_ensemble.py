@@ -215,3 +215,25 @@ def test_tiles_per_range_is_what_the_caller_asks(mode):
                         assert np.array_equal(a, b), (threads, tiles, c, key)
                     else:
                         assert np.linalg.norm(a - b) <= 2.0 ** -40 * np.linalg.norm(b), (threads, tiles, c, key)
+
+
+@pytest.mark.parametrize("sizes", [[512, 1, 33], [513, 1024, 7], [1025, 2048], [2049, 300], [4096, 4097, 5],
+                                   [3000, 1200, 129] + [4] * 5000])
+def test_scheduler_of_any_cluster_size(sizes):
+    """Scheduler blocks of 64 to 1024 threads by the largest cluster, and of fewer than it fills where there are many
+    clusters: a cluster's run is the bits of its run alone (whose block fits it)."""
+    need_gpu()
+    from paper_astro_ph_0702058_gb300 import Ensemble
+    parts = [plummer_sphere(int(n), 500 + c % 7 if n == 4 else 400 + c) for c, n in enumerate(sizes)]
+    m, x, v = (np.concatenate([p[k] for p in parts]) for k in range(3))
+    with Ensemble(sizes, m, x, v, EPS2, eta=0.02) as ens:
+        ens.run(1.0 / 64)
+        got, blocks = _state(ens, len(m)), ens.stats()["blocks"]
+    off = np.concatenate([[0], np.cumsum(sizes)])
+    for c in range(min(len(sizes), 4)):
+        with Ensemble([sizes[c]], *parts[c], EPS2, eta=0.02) as one:
+            one.run(1.0 / 64)
+            ref = _state(one, sizes[c])
+            assert one.stats()["blocks"][0] == blocks[c]
+        for key in ref:
+            assert np.array_equal(got[key][off[c]:off[c + 1]], ref[key]), (c, key)
