@@ -109,10 +109,13 @@ __device__ __forceinline__ void sym_term(const f2_t (&v)[10], const SymI &I, con
 // mass comes first, as in force_x2.cuh: r^-3 alone leaves FP32's range for r
 // above 2^42 or below 2^-42, where m r^-1 r^-2 need not (a cluster in metres).
 // That is 6 products and additions of two registers where r^-3 first took 3 and
-// 2 FMAs of three.  Compensated, every product before the FMAs: at the 128
-// registers of 16 warps the sides one after the other spill more (n = 262144,
-// ms: 53.1 against 56.2 at an unroll of 4, 53.1 with r^-3 first); plain, which
-// has 168, they are faster so (44.1 against 45.0, 43.7 with r^-3 first).
+// 2 FMAs of three.  ORDER is the order the compiler does best with at the
+// kernel's registers: 0 one side after the other (plain, four warps: n = 262144 44.1
+// ms, 45.0 in order 2), 1 every product first and the sides' FMAs in turn
+// (compensated, four warps at 128 registers: 53.1 ms, 53.7 in order 2, 56.2 and more
+// spills in order 0), 2 every product first, then side by side (one-warp CTAs: n =
+// 32000 plain 746 us, 758 in orders 0 and 1, compensated 886, 888 in order 1).  With
+// r^-3 first they took 43.7 and 53.1 ms, 737 and 874 us.
 __device__ __forceinline__ void sym_add(const f2_t s, const SymT &T, f2_t (&p)[7])
 {
     p[0] = f2_fma(s, T.dx, p[0]);
@@ -122,33 +125,38 @@ __device__ __forceinline__ void sym_add(const f2_t s, const SymT &T, f2_t (&p)[7
     p[4] = f2_fma(s, T.uy, p[4]);
     p[5] = f2_fma(s, T.uz, p[5]);
 }
-template <int MODE>
+template <int ORDER>
 __device__ __forceinline__ void sym_add_both(const f2_t mj, const f2_t mi, const SymT &T, f2_t (&pi)[7], f2_t (&pj)[7])
 {
-    if constexpr (MODE == kModeComp) {
-        const f2_t a = f2_mul(mj, T.y), b = f2_mul(mi, T.y);
-        pi[6] = f2_add(pi[6], a);
-        pj[6] = f2_add(pj[6], b);
-        const f2_t s = f2_mul(a, T.y2), t = f2_mul(b, T.y2);
-        pi[0] = f2_fma(s, T.dx, pi[0]);
-        pj[0] = f2_fma(t, T.dx, pj[0]);
-        pi[1] = f2_fma(s, T.dy, pi[1]);
-        pj[1] = f2_fma(t, T.dy, pj[1]);
-        pi[2] = f2_fma(s, T.dz, pi[2]);
-        pj[2] = f2_fma(t, T.dz, pj[2]);
-        pi[3] = f2_fma(s, T.ux, pi[3]);
-        pj[3] = f2_fma(t, T.ux, pj[3]);
-        pi[4] = f2_fma(s, T.uy, pi[4]);
-        pj[4] = f2_fma(t, T.uy, pj[4]);
-        pi[5] = f2_fma(s, T.uz, pi[5]);
-        pj[5] = f2_fma(t, T.uz, pj[5]);
-    } else {
+    if constexpr (ORDER == 0) {
         const f2_t a = f2_mul(mj, T.y);
         sym_add(f2_mul(a, T.y2), T, pi);
         pi[6] = f2_add(pi[6], a);
         const f2_t b = f2_mul(mi, T.y);
         sym_add(f2_mul(b, T.y2), T, pj);
         pj[6] = f2_add(pj[6], b);
+    } else {
+        const f2_t a = f2_mul(mj, T.y), b = f2_mul(mi, T.y);
+        pi[6] = f2_add(pi[6], a);
+        pj[6] = f2_add(pj[6], b);
+        const f2_t s = f2_mul(a, T.y2), t = f2_mul(b, T.y2);
+        if constexpr (ORDER == 2) {
+            sym_add(s, T, pi);
+            sym_add(t, T, pj);
+        } else {
+            pi[0] = f2_fma(s, T.dx, pi[0]);
+            pj[0] = f2_fma(t, T.dx, pj[0]);
+            pi[1] = f2_fma(s, T.dy, pi[1]);
+            pj[1] = f2_fma(t, T.dy, pj[1]);
+            pi[2] = f2_fma(s, T.dz, pi[2]);
+            pj[2] = f2_fma(t, T.dz, pj[2]);
+            pi[3] = f2_fma(s, T.ux, pi[3]);
+            pj[3] = f2_fma(t, T.ux, pj[3]);
+            pi[4] = f2_fma(s, T.uy, pi[4]);
+            pj[4] = f2_fma(t, T.uy, pj[4]);
+            pi[5] = f2_fma(s, T.uz, pi[5]);
+            pj[5] = f2_fma(t, T.uz, pj[5]);
+        }
     }
 }
 
@@ -205,7 +213,7 @@ __device__ __forceinline__ void sym_load_j(const float *chunk, const int jl, f2_
 // at the end, so an FP32 sum has 64 terms, as each half of force_x2.cuh's (128 terms
 // in one made the error at n = 30000 11 % larger than the one-sided kernel's; folded
 // twice as often through L2 instead, the full force at 2^20 took 880 ms, not 853).
-template <int MODE, bool DIAG, int UNROLL>
+template <int MODE, bool DIAG, int UNROLL, int ORDER>
 __device__ __forceinline__ void sym_both(const float *chunk, const SymI &I, const int lane, const f2_t E2,
                                          const f2_t NEG3, f2_t (&pi)[2][7], float *pj_out, const int jlive,
                                          const size_t n, const bool jfirst, f2_t *mid)
@@ -232,7 +240,7 @@ __device__ __forceinline__ void sym_both(const float *chunk, const SymI &I, cons
                 sym_term<MODE, DIAG>(v, I, g, E2, NEG3, DIAG && jl <= lane + 64 * g, DIAG && jl <= lane + 64 * g + 32,
                                      T[g]);
 #pragma unroll
-            for (int g = 0; g < 2; ++g) sym_add_both<MODE>(v[3], I.m[g], T[g], pi[g], pj);
+            for (int g = 0; g < 2; ++g) sym_add_both<ORDER>(v[3], I.m[g], T[g], pi[g], pj);
             // j goes to the next lane down, and its sums with it
 #pragma unroll
             for (int c = 0; c < 7; ++c) {
@@ -273,6 +281,7 @@ __global__ void __launch_bounds__(32 * W, WARPS / W) force_sym_kernel(const SymP
     constexpr int NC = DSW ? 14 : 7, NA = DSW ? 10 : 7;
     constexpr int BT = W * kSymRows;  // rows of a tile
     constexpr int CH = sym_chunk_floats<MODE>();
+    constexpr int ORDER = W == 1 ? 2 : DSW ? 1 : 0;  // (sym_add_both)
     __shared__ __align__(16) float sj[W * CH];
     __shared__ f2_t s_mid[DSW ? W * 14 * 32 : 1];
     f2_t *mid = s_mid + (DSW ? (threadIdx.x >> 5) * 14 * 32 : 0);
@@ -353,10 +362,11 @@ __global__ void __launch_bounds__(32 * W, WARPS / W) force_sym_kernel(const SymP
                     for (int q = 0; q < 7; ++q) pi[g][q] = 0ull;
                 const bool jfirst = it == 0 && k == 0;  // (each chunk that exists meets a warp in window 0)
                 if (own && k == 0)
-                    sym_both<MODE, true, 1>(sj + c * CH, I, lane, E2, NEG3, pi, pj_out + jr, j_end - jr, n, jfirst, mid);
+                    sym_both<MODE, true, 1, ORDER>(sj + c * CH, I, lane, E2, NEG3, pi, pj_out + jr, j_end - jr, n,
+                                                   jfirst, mid);
                 else
-                    sym_both<MODE, false, UNROLL>(sj + c * CH, I, lane, E2, NEG3, pi, pj_out + jr, j_end - jr, n,
-                                                  jfirst, mid);
+                    sym_both<MODE, false, UNROLL, ORDER>(sj + c * CH, I, lane, E2, NEG3, pi, pj_out + jr, j_end - jr, n,
+                                                         jfirst, mid);
 #pragma unroll
                 for (int g = 0; g < 2; ++g) {
                     const int r0 = i0 + lane + 64 * g, r1 = r0 + 32;
